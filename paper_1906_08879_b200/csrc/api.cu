@@ -20,7 +20,7 @@ struct placeto_graph {
     DeviceInfo info{};
     int *d_ints = nullptr;       // one allocation for all int arrays
     int4 *d_packed = nullptr;    // per direction lvl4[n_levels], pos4[n] (see DevLevels)
-    int *d_child_ptr = nullptr, *d_child = nullptr, *d_n_parents = nullptr;   // inside d_ints
+    int *d_child_ptr = nullptr, *d_child = nullptr, *d_child_entry = nullptr;   // inside d_ints
     int *d_parent_ptr = nullptr, *d_parent = nullptr;                          // inside d_ints
     uint8_t *d_relation = nullptr;
     DevLevels lv[2]{};
@@ -381,8 +381,8 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
                                        p.nbr.size(), p.own_slot.size(), p.nbr_slot.size()};
         for (int k = 0; k < kArrays; ++k) { offs[dir][k] = total; total += (sizes[k] + 3) & ~size_t(3); }
     }
-    // and, by node id: children, parent counts (runtime simulator), parents (policy gradient)
-    const std::vector<int32_t> *extra[5] = {&g->host.child_ptr, &g->host.child, &g->host.n_parents,
+    // and, by node id: children and their entries in the parent lists (runtime simulator), parents (policy gradient)
+    const std::vector<int32_t> *extra[5] = {&g->host.child_ptr, &g->host.child, &g->host.child_entry,
                                             &g->host.parent_ptr, &g->host.parent};
     size_t sim_off[5];
     for (int k = 0; k < 5; ++k) { sim_off[k] = total; total += (extra[k]->size() + 3) & ~size_t(3); }
@@ -410,7 +410,7 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
         g->lv[dir].n_nbr = static_cast<int>(p.nbr.size());
     }
     {
-        int **dst[5] = {&g->d_child_ptr, &g->d_child, &g->d_n_parents, &g->d_parent_ptr, &g->d_parent};
+        int **dst[5] = {&g->d_child_ptr, &g->d_child, &g->d_child_entry, &g->d_parent_ptr, &g->d_parent};
         for (int k = 0; k < 5; ++k) {
             *dst[k] = g->d_ints + sim_off[k];
             if (!extra[k]->empty() &&
@@ -829,7 +829,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
 
 size_t placeto_simulator_workspace_bytes(const placeto_graph *g, int32_t P, int32_t m) {
     if (!g || P < 1 || m < 1 || m > PLACETO_MAX_M) return 0;
-    return sim_workspace_bytes(g->host.n, (int)g->host.n_edges, m, P);
+    return sim_workspace_bytes(g->host.n, (int)g->host.n_edges, P, g->on_device ? g->info : DeviceInfo{148, 227 * 1024});
 }
 
 placeto_status placeto_simulate_placements(const placeto_graph *g, const float *cost, const float *bytes,
@@ -847,18 +847,18 @@ placeto_status placeto_simulate_placements(const placeto_graph *g, const float *
         (runtime && !aligned16(runtime)) || (peak_memory && !aligned16(peak_memory)) ||
         (penalised && !aligned16(penalised)))
         return PLACETO_ERR_INVALID_ARG;
-    if (workspace_bytes < sim_workspace_bytes(g->host.n, (int)g->host.n_edges, m, P))
+    if (workspace_bytes < sim_workspace_bytes(g->host.n, (int)g->host.n_edges, P, g->info))
         return PLACETO_ERR_WORKSPACE;
     SimArgs a;
     a.n = g->host.n; a.n_edges = (int)g->host.n_edges; a.m = m; a.P = P;
-    a.child_ptr = g->d_child_ptr; a.child = g->d_child; a.n_parents = g->d_n_parents;
+    a.child_ptr = g->d_child_ptr; a.child = g->d_child; a.child_entry = g->d_child_entry;
     a.parent_ptr = g->d_parent_ptr; a.parent = g->d_parent;
     a.cost = cost; a.bytes = bytes; a.dev = dev;
     a.bandwidth = bandwidth;
     a.mem_limit = mem_limit; a.mem_scale = mem_scale;
     a.runtime = runtime; a.peak_memory = peak_memory; a.penalised = penalised;
     a.workspace = static_cast<char *>(workspace);
-    return cuda_status(launch_simulator(a, static_cast<cudaStream_t>(stream)));
+    return cuda_status(launch_simulator(a, g->info, static_cast<cudaStream_t>(stream)));
 }
 
 placeto_status placeto_simulate_runtime(const placeto_graph *g, const float *cost, const float *bytes,

@@ -163,8 +163,9 @@ struct EpisodeArgs {
 
 struct SimArgs {
     int n, n_edges, m, P;
-    const int *child_ptr, *child, *n_parents;   // by node id
+    const int *child_ptr, *child;               // by node id
     const int *parent_ptr, *parent;             // by node id, ascending
+    const int *child_entry;                     // [n_edges] entry in `parent` of the edge at this entry of `child`
     const float *cost, *bytes;                  // [n]
     const uint8_t *dev;                         // [P][n]
     double bandwidth;
@@ -294,9 +295,9 @@ cudaError_t launch_episode_end_compact(int n, int E, const uint8_t *state, uint8
 // true when an episode step on these shapes runs on kernels that take compact states
 bool pool_head_takes_compact(const PoolArgs &a);
 
-// simulator.cu: event-based run time of P placements, one thread each
-size_t sim_workspace_bytes(int n, int n_edges, int m, int P);
-cudaError_t launch_simulator(const SimArgs &a, cudaStream_t stream);
+// simulator.cu: event-based run time of P placements, a group of lanes each
+size_t sim_workspace_bytes(int n, int n_edges, int P, const DeviceInfo &di);
+cudaError_t launch_simulator(const SimArgs &a, const DeviceInfo &di, cudaStream_t stream);
 
 // gradient.cu: gradient of the policy objective with respect to all weights
 bool policy_gradient_applicable(const GradArgs &a);

@@ -119,11 +119,9 @@ placeto_status build_plan(int32_t n, int64_t n_edges, const int32_t *src, const 
         assign_slots(n, level_up, plan.dir[1]);
         plan.child_ptr.assign(n + 1, 0);
         plan.child.clear();
-        plan.n_parents.assign(n, 0);
         for (int32_t v = 0; v < n; ++v) {
             plan.child.insert(plan.child.end(), chi[v].begin(), chi[v].end());
             plan.child_ptr[v + 1] = static_cast<int32_t>(plan.child.size());
-            plan.n_parents[v] = static_cast<int32_t>(par[v].size());
         }
         plan.parent_ptr.assign(n + 1, 0);
         plan.parent.clear();
@@ -131,6 +129,11 @@ placeto_status build_plan(int32_t n, int64_t n_edges, const int32_t *src, const 
             plan.parent.insert(plan.parent.end(), par[v].begin(), par[v].end());
             plan.parent_ptr[v + 1] = static_cast<int32_t>(plan.parent.size());
         }
+        // parents are visited in ascending order by every child: walking the children in ascending
+        // order fills each parent's child list front to back
+        plan.child_entry.assign(plan.child.size(), 0);
+        std::vector<int32_t> at(plan.child_ptr.begin(), plan.child_ptr.end() - 1);
+        for (int32_t e = 0; e < static_cast<int32_t>(plan.parent.size()); ++e) plan.child_entry[at[plan.parent[e]]++] = e;
         plan.max_level_width = 0;
         for (int dir = 0; dir < 2; ++dir)
             for (int32_t l = 0; l < plan.dir[dir].n_levels; ++l)

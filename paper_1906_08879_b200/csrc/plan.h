@@ -31,9 +31,10 @@ struct HostPlan {
     int32_t max_degree = 0;          // largest neighbour set, both directions
     LevelPlan dir[2];                // 0 top-down, 1 bottom-up
     std::vector<uint8_t> relation;   // [n * n], see placeto_graph_host_view
-    // by node id, for the runtime simulator: children (ascending) and number of parents
-    std::vector<int32_t> child_ptr, child, n_parents;
-    std::vector<int32_t> parent_ptr, parent;   // by node id, ascending (the policy gradient's gathers)
+    // by node id, ascending, for the runtime simulator and the policy gradient's gathers: children and parents;
+    // child_entry[e] is the entry in `parent` of the edge at entry e of `child`
+    std::vector<int32_t> child_ptr, child, child_entry;
+    std::vector<int32_t> parent_ptr, parent;
 };
 
 // Validates the edge list and fills `plan`. Returns PLACETO_OK,

@@ -6,15 +6,26 @@
 // device; a transfer takes size / bandwidth; the result is the time stamp of the
 // last Op-done event.
 //
-// One thread simulates one placement (the event loop is serial by nature; the
-// batch of placements is the parallel dimension). At most one Op-done event per
-// device and one Transfer-done event per bus are outstanding, so the event set is
-// two arrays of m time stamps scanned for the earliest (equal stamps: the event
-// created first). Queues are linked lists threaded through per-placement arrays
-// in the workspace, which is interleaved by placement (element i of placement p
-// at [i * P + p]) so that neighbouring threads touch neighbouring words. All
-// times are doubles and are added and divided in the order the model states, so
-// results are reproducible bit for bit.
+// A group of 8, 16 or 32 lanes (the fewest that give every device a lane; two
+// devices per lane beyond 32) simulates one placement. The event loop is serial by
+// nature and bound by the latency of its dependent steps and by the instructions
+// they take, so several placements share a warp and walk their events in lockstep:
+// the code below has no branch on what a placement's event is (an operation or a
+// transfer that ends; which device), only predicates, and its loops run until the
+// last group of the warp is through. Lane d keeps the whole state of device d (what
+// it runs, what its bus sends, its queues' ends, its memory) in registers, the
+// earliest event is found with a butterfly over the group, and the children
+// (parents) of the operation are looked at one per lane. Queues are linked lists
+// threaded through per-placement arrays of 16-bit ids, which live in shared memory
+// together with the graph; what does not fit there (large graphs) keeps the arrays in the
+// workspace as 32-bit words. All times are doubles and are added and divided in
+// the order the model states, so results are reproducible bit for bit.
+//
+// Measured on a B200 (279-node graph of multi-branch modules, 4096 placements on 4 devices, about
+// 500 events each): 0.79 ms; one thread per placement with the devices' state in local memory
+// and the queues in the workspace took 2.88 ms. What is left is latency: 7 warps per SM, an
+// instruction of a warp every 6.1 cycles, about 500 per event of the four placements
+// of a warp. One placement per warp was slower (0.91 ms: bound by instruction issue).
 //
 // Readings where the paper is silent: one run time per operation; a tensor is
 // sent once to each distinct device hosting a child; a free device or bus starts
@@ -39,168 +50,393 @@ namespace placeto {
 
 namespace {
 
-constexpr int kThreads = 64;
-constexpr int kMaxM = PLACETO_MAX_M;
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kMaxThreads = 256;
 
-// per placement: ints  pending[n], op_next[n], tr_op[T], tr_dst[T], tr_next[T], sent_mark[m * ?]
-// with T = min(n_edges, n * (m - 1)) transfer records at most
-__host__ __device__ inline size_t sim_ints(int n, int n_edges) {
-    return 3 * (size_t)n + 3 * (size_t)n_edges;     // + tr_left[n]: transfers of a tensor not yet done
+// Per placement, T = n_edges transfer records at most (one per tensor and device it is sent to):
+//   pending[n]   inputs an operation still waits for          next[n]     queue link of an operation
+//   local[n]     its children on its own device still to run  tr_left[n]  its transfers not yet done
+//   tr_op[T], tr_dst[T], tr_next[T], and tr_kids[T]: children at the destination still to run
+//   rec[n_edges] by parent-list entry: the record that brings this input, if it comes from elsewhere
+// As 32-bit words in the workspace:
+__host__ __device__ inline size_t sim_ints(int n, int n_edges) { return 4 * (size_t)n + 5 * (size_t)n_edges; }
+
+// The same in shared memory, packed (ids and counts below 65535, devices and transfers below 256), with
+// the placement's device row; and what the placements of a block share: cost, transfer time, size,
+// the child and parent lists and, per child-list entry, the parent-list entry of the same edge.
+struct SimPlan {
+    int per_block;          // placements per block
+    int graph_bytes;        // shared by the block
+    int state_bytes;        // per placement
+};
+__host__ __device__ inline int round16(int v) { return (v + 15) & ~15; }
+inline int sim_state_bytes(int n, int n_edges) {
+    return round16(3 * 2 * n + 4 * 2 * n_edges + n_edges + 2 * n);
+}
+inline int sim_graph_bytes(int n, int n_edges) {
+    return round16(8 * n + 2 * 4 * n + 2 * 4 * (n + 1) + 3 * 2 * n_edges);
 }
 
-__global__ void __launch_bounds__(kThreads)
-simulate_kernel(const SimArgs a) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.P) return;
-    const int n = a.n, m = a.m, P = a.P;
-    int *base = reinterpret_cast<int *>(a.workspace);
-    auto at = [&](size_t i) -> int & { return base[i * P + p]; };
-    const size_t o_pending = 0, o_next = n, o_trop = 2 * (size_t)n, o_trdst = o_trop + a.n_edges,
-                 o_trnext = o_trdst + a.n_edges, o_trleft = o_trnext + a.n_edges;
-    constexpr int kFinished = -1;            // value of pending[] once the operation has run
-    const uint8_t *dev = a.dev + (size_t)p * n;
+// An order-preserving map from doubles (no NaN) to unsigned integers.
+__device__ __forceinline__ unsigned long long time_key(double t) {
+    const long long b = __double_as_longlong(t);
+    return (unsigned long long)(b ^ ((b >> 63) | (long long)0x8000000000000000ull));
+}
 
-    // small per-device state in local memory
-    int q_head[kMaxM], q_tail[kMaxM], t_head[kMaxM], t_tail[kMaxM];
-    int run_op[kMaxM], run_tr[kMaxM];        // what the device / bus is busy with, -1 = free
-    int op_seq[kMaxM], tr_seq[kMaxM];
-    double op_end[kMaxM], tr_end[kMaxM];
-    int sent[kMaxM];                          // last operation whose output was queued for the device
-    double mem[kMaxM], peak[kMaxM];           // bytes held now / at most
-    for (int d = 0; d < m; ++d) {
-        q_head[d] = q_tail[d] = t_head[d] = t_tail[d] = -1;
-        run_op[d] = run_tr[d] = -1;
-        sent[d] = -1;
-        mem[d] = peak[d] = 0.0;
-    }
-    auto hold = [&](int d, int o) {
-        mem[d] += (double)a.bytes[o];
-        if (mem[d] > peak[d]) peak[d] = mem[d];
-    };
-    // the copy of u's output on device d goes once no child there and no transfer needs it
-    auto maybe_release = [&](int u, int d) {
-        const int e0 = a.child_ptr[u], e1 = a.child_ptr[u + 1];
-        if (e0 == e1) return;
-        for (int e = e0; e < e1; ++e) {
-            const int c = a.child[e];
-            if (dev[c] == d && at(o_pending + c) != kFinished) return;
+__device__ __forceinline__ double key_time(unsigned long long key) {
+    return __longlong_as_double((long long)(key ^ (key >> 63 ? 0x8000000000000000ull : ~0ull)));
+}
+
+// Where a placement's arrays live: kShared packs them, otherwise all are ints in the workspace.
+template <bool kShared> struct SimTypes { typedef unsigned short id; typedef unsigned char small; };
+template <> struct SimTypes<false> { typedef int id; typedef int small; };
+
+// kGroup lanes per placement, kPerLane devices per lane: lane l of a group keeps device l (and l + 32).
+template <bool kShared, int kGroup, int kPerLane>
+__global__ void __launch_bounds__(kMaxThreads)
+simulate_kernel(const SimArgs a, const SimPlan plan) {
+    static_assert(kPerLane == 1 || kGroup == 32, "the second device of a lane is lane + 32");
+    typedef typename SimTypes<kShared>::id Id;
+    typedef typename SimTypes<kShared>::small Small;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, gl = lane & (kGroup - 1), g0 = lane & ~(kGroup - 1);
+    const unsigned group_bits = kGroup == 32 ? kFull : (1u << (kGroup & 31)) - 1;
+    const int n = a.n, m = a.m, E = a.n_edges;
+    const int slot = threadIdx.x / kGroup;                // placement of the block
+    const int p = blockIdx.x * plan.per_block + slot;
+    const bool live = slot < plan.per_block && p < a.P;
+    const int none = kShared ? 0xffff : -1;               // end of a list
+
+    // ---- the graph
+    const float *cost = a.cost, *bytes = a.bytes;
+    const int *child_ptr = a.child_ptr, *parent_ptr = a.parent_ptr;
+    const double *xfer = nullptr;                         // transfer time of every output tensor
+    const unsigned short *child16 = nullptr, *parent16 = nullptr, *same16 = nullptr;
+    if (kShared) {
+        double *x = reinterpret_cast<double *>(smem);
+        float *c = reinterpret_cast<float *>(x + n), *s = c + n;
+        int *cp = reinterpret_cast<int *>(s + n), *pp = cp + n + 1;
+        unsigned short *ch = reinterpret_cast<unsigned short *>(pp + n + 1), *pa = ch + E, *sa = pa + E;
+        for (int v = threadIdx.x; v < n; v += blockDim.x) {
+            c[v] = a.cost[v];
+            s[v] = a.bytes[v];
+            x[v] = (double)a.bytes[v] / a.bandwidth;
         }
-        if (d == dev[u] && at(o_trleft + u) > 0) return;
-        mem[d] -= (double)a.bytes[u];
-    };
-    int seq = 0, n_tr = 0, done = 0;
+        for (int v = threadIdx.x; v <= n; v += blockDim.x) { cp[v] = a.child_ptr[v]; pp[v] = a.parent_ptr[v]; }
+        for (int e = threadIdx.x; e < E; e += blockDim.x) {
+            ch[e] = (unsigned short)a.child[e];
+            pa[e] = (unsigned short)a.parent[e];
+            sa[e] = (unsigned short)a.child_entry[e];
+        }
+        cost = c; bytes = s; xfer = x; child_ptr = cp; parent_ptr = pp; child16 = ch; parent16 = pa; same16 = sa;
+        __syncthreads();
+    }
+    auto child = [&](int e) -> int { return kShared ? (int)child16[e] : a.child[e]; };
+    auto parent = [&](int e) -> int { return kShared ? (int)parent16[e] : a.parent[e]; };
+    auto entry = [&](int e) -> int { return kShared ? (int)same16[e] : a.child_entry[e]; };
+
+    // ---- the placement's arrays
+    const uint8_t *dev = a.dev + (size_t)(live ? p : 0) * n;
+    Id *pending, *next, *local, *tr_op, *tr_next, *tr_kids, *rec;
+    Small *tr_dst, *tr_left;
+    {
+        Id *base = kShared ? reinterpret_cast<Id *>(smem + plan.graph_bytes + (size_t)(live ? slot : 0) * plan.state_bytes)
+                           : reinterpret_cast<Id *>(a.workspace) + (size_t)(live ? p : 0) * sim_ints(n, E);
+        pending = base;
+        next = pending + n;
+        local = next + n;
+        tr_op = local + n;
+        tr_next = tr_op + E;
+        tr_kids = tr_next + E;
+        rec = tr_kids + E;
+        tr_dst = reinterpret_cast<Small *>(rec + E);
+        tr_left = tr_dst + E;
+        if (kShared) {
+            uint8_t *copy = reinterpret_cast<uint8_t *>(tr_left + n);
+            if (live)
+                for (int v = gl; v < n; v += kGroup) copy[v] = dev[v];
+            dev = copy;
+        }
+    }
+
+    // ---- device state: element [d >> 5] in lane d & 31 of the group
+    constexpr unsigned long long kIdle = ~0ull;           // key of nothing outstanding
+    int q_head[kPerLane], q_tail[kPerLane], t_head[kPerLane], t_tail[kPerLane];
+    int run_op[kPerLane], run_tr[kPerLane];               // what the device / bus is busy with, -1 = free
+    unsigned op_tag[kPerLane], tr_tag[kPerLane];          // order of creation among all events, the lowest bit 1 for a transfer
+    unsigned long long op_key[kPerLane], tr_key[kPerLane];// its time stamp as an ordered integer
+    double mem[kPerLane], peak[kPerLane];
+#pragma unroll
+    for (int k = 0; k < kPerLane; ++k) {
+        q_head[k] = q_tail[k] = t_head[k] = t_tail[k] = none;
+        run_op[k] = run_tr[k] = -1;
+        op_tag[k] = tr_tag[k] = kFull;
+        op_key[k] = tr_key[k] = kIdle;
+        mem[k] = peak[k] = 0.0;
+    }
+    int n_tr = 0, done = 0;
     double last = 0.0;
 
-    auto push_op = [&](int d, int v) {
-        at(o_next + v) = -1;
-        if (q_tail[d] < 0) q_head[d] = v; else at(o_next + q_tail[d]) = v;
-        q_tail[d] = v;
+    // All lanes run these; `who` is a device of the lane's group, or -1 where the group has nothing to do.
+    auto in_group = [&](bool v) { return (__ballot_sync(kFull, v) >> g0) & group_bits; };
+    auto push_op = [&](int who, int v) {
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k)
+            if (gl + 32 * k == who) {
+                next[v] = (Id)none;
+                if (q_tail[k] == none) q_head[k] = v; else next[q_tail[k]] = (Id)v;
+                q_tail[k] = v;
+            }
     };
-    auto start_op = [&](int d, double now) {
-        const int v = q_head[d];
-        q_head[d] = at(o_next + v);
-        if (q_head[d] < 0) q_tail[d] = -1;
-        run_op[d] = v;
-        hold(d, v);
-        op_end[d] = now + (double)a.cost[v];
-        op_seq[d] = seq++;
+    auto outstanding = [&](double t) { return t < DBL_MAX ? time_key(t) : kIdle; };      // (not for NaN or infinity)
+    // Device od starts the head of its queue, if it is free and has one.
+    auto start_op = [&](int od, double now, unsigned tag) {
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k)
+            if (gl + 32 * k == od && run_op[k] < 0 && q_head[k] != none) {
+                const int v = q_head[k];
+                q_head[k] = next[v];
+                if (q_head[k] == none) q_tail[k] = none;
+                run_op[k] = v;
+                op_key[k] = outstanding(now + (double)cost[v]);
+                op_tag[k] = tag;
+                mem[k] += (double)bytes[v];               // its output occupies the device from now on
+                if (mem[k] > peak[k]) peak[k] = mem[k];
+            }
     };
-    auto start_transfer = [&](int d, double now) {
-        const int r = t_head[d];
-        t_head[d] = at(o_trnext + r);
-        if (t_head[d] < 0) t_tail[d] = -1;
-        run_tr[d] = r;
-        hold(at(o_trdst + r), at(o_trop + r));
-        tr_end[d] = now + (double)a.bytes[at(o_trop + r)] / a.bandwidth;
-        tr_seq[d] = seq++;
+    // The bus of device td starts the head of its queue, if it is free and has one.
+    auto start_transfer = [&](int td, double now, unsigned tag) {
+        int sent = -1, to = 0;
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k)
+            if (gl + 32 * k == td && run_tr[k] < 0 && t_head[k] != none) {
+                const int r = t_head[k];
+                t_head[k] = tr_next[r];
+                if (t_head[k] == none) t_tail[k] = none;
+                run_tr[k] = r;
+                sent = tr_op[r];
+                to = tr_dst[r];
+                tr_key[k] = outstanding(now + (kShared ? xfer[sent] : (double)bytes[sent] / a.bandwidth));
+                tr_tag[k] = tag;
+            }
+        if (!__any_sync(kFull, sent >= 0)) return;
+        const int from = td < 0 ? 0 : td & 31;
+        sent = __shfl_sync(kFull, sent, from, kGroup);
+        to = __shfl_sync(kFull, to, from, kGroup);
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k)
+            if (sent >= 0 && gl + 32 * k == to) {         // the copy occupies the destination from now on
+                mem[k] += (double)bytes[sent];
+                if (mem[k] > peak[k]) peak[k] = mem[k];
+            }
     };
 
-    for (int v = 0; v < n; ++v) {
-        at(o_pending + v) = a.n_parents[v];
-        at(o_trleft + v) = 0;
-        if (a.n_parents[v] == 0 && dev[v] < m) push_op(dev[v], v);
+    __syncwarp();
+    for (int v0 = 0; v0 < n; v0 += kGroup) {
+        const int v = v0 + gl;
+        bool root = false;
+        if (live && v < n) {
+            const int np = parent_ptr[v + 1] - parent_ptr[v], dv = dev[v];
+            int here = 0;
+            for (int e = child_ptr[v]; e < child_ptr[v + 1]; ++e) here += dev[child(e)] == dv;
+            local[v] = (Id)here;
+            pending[v] = (Id)np;
+            tr_left[v] = 0;
+            root = np == 0 && dv < m;
+        }
+        unsigned bits = in_group(root);
+        while (__any_sync(kFull, bits != 0)) {
+            const int r = bits ? v0 + __ffs(bits) - 1 : 0;
+            push_op(bits ? (int)dev[r] : -1, r);
+            bits &= bits - 1;
+        }
     }
-    for (int d = 0; d < m; ++d)
-        if (q_head[d] >= 0) start_op(d, 0.0);
+    __syncwarp();
+    for (int d = 0; d < m; ++d) start_op(live ? d : -1, 0.0, 2 * d);
 
     // every operation and every transfer is one event: the loop is bounded
-    const long long max_events = (long long)n + a.n_edges + 1;
-    for (long long it = 0; it < max_events; ++it) {
+    const long long max_events = (long long)n + E + 1;
+    unsigned tag_base = 4 * 64;                           // tags of the events that this event creates
+    for (long long it = 0; it < max_events; ++it, tag_base += 4) {
         // the earliest outstanding event; equal time stamps: the one created first
-        int kind = -1, who = -1, best_seq = 0;
-        double now = DBL_MAX;
-        for (int d = 0; d < m; ++d) {
-            if (run_op[d] >= 0 && (op_end[d] < now || (op_end[d] == now && op_seq[d] < best_seq))) {
-                now = op_end[d]; kind = 0; who = d; best_seq = op_seq[d];
+        unsigned long long key = kIdle;
+        unsigned tag = kFull;
+        int where = 0, which = 0;
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k) {
+            if (op_key[k] < key || (op_key[k] == key && op_tag[k] < tag)) { key = op_key[k]; tag = op_tag[k]; where = gl + 32 * k; which = run_op[k]; }
+            if (tr_key[k] < key || (tr_key[k] == key && tr_tag[k] < tag)) { key = tr_key[k]; tag = tr_tag[k]; where = gl + 32 * k; which = run_tr[k]; }
+        }
+        const unsigned own_tag = tag;
+#pragma unroll
+        for (int o = kGroup / 2; o > 0; o >>= 1) {
+            const unsigned long long key2 = __shfl_xor_sync(kFull, key, o);
+            const unsigned tag2 = __shfl_xor_sync(kFull, tag, o);
+            if (key2 < key || (key2 == key && tag2 < tag)) { key = key2; tag = tag2; }
+        }
+        const bool alive = key != kIdle;
+        if (!__any_sync(kFull, alive)) break;
+        const unsigned owners = in_group(alive && own_tag == tag);      // tags are unique among what is outstanding
+        const int owner = owners ? __ffs(owners) - 1 : 0;
+        const int d = __shfl_sync(kFull, where, owner, kGroup);         // device or bus
+        which = __shfl_sync(kFull, which, owner, kGroup);               // operation or transfer record
+        const double now = key_time(key);
+        const bool is_op = alive && !(tag & 1), is_tr = alive && (tag & 1);
+        const int o = is_tr ? (int)tr_op[which] : (alive ? which : 0);
+        const int to = is_tr ? (int)tr_dst[which] : d;    // the device whose children of o this event serves
+        const int c0 = child_ptr[o], c1 = alive ? child_ptr[o + 1] : c0;
+        const int p0 = parent_ptr[o], p1 = is_op ? parent_ptr[o + 1] : p0;
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k)
+            if (alive && gl + 32 * k == d) {
+                if (is_op) { run_op[k] = -1; op_key[k] = kIdle; op_tag[k] = kFull; }
+                else { run_tr[k] = -1; tr_key[k] = kIdle; tr_tag[k] = kFull; }
             }
-            if (run_tr[d] >= 0 && (tr_end[d] < now || (tr_end[d] == now && tr_seq[d] < best_seq))) {
-                now = tr_end[d]; kind = 1; who = d; best_seq = tr_seq[d];
+        if (is_op) { ++done; last = now; }
+        // Copies on device d that may go: of the inputs that an operation read (a lane per parent; it
+        // was the last child there, and at the producer no transfer is left), of the tensor that a transfer sent.
+        for (int e = p0 + gl; __any_sync(kFull, e - gl < p1 || (is_tr && e - gl == p0)); e += kGroup) {
+            bool gone = false;
+            int u = o;
+            if (e < p1) {
+                u = parent(e);
+                const bool home = (int)dev[u] == d;
+                Id *count = home ? local + u : tr_kids + rec[e];
+                const int left = (int)*count - 1;
+                *count = (Id)left;
+                gone = left == 0 && !(home && tr_left[u] > 0);
+            } else if (is_tr && e == p0) {
+                const int left = (int)tr_left[o] - 1;
+                tr_left[o] = (Small)left;
+                gone = left == 0 && (int)local[o] == 0;
+            }
+            unsigned bits = in_group(gone);
+            while (__any_sync(kFull, bits != 0)) {        // subtracted in ascending order
+                const int x = __shfl_sync(kFull, u, bits ? __ffs(bits) - 1 : 0, kGroup);
+#pragma unroll
+                for (int k = 0; k < kPerLane; ++k)
+                    if (bits && gl + 32 * k == d) mem[k] -= (double)bytes[x];
+                bits &= bits - 1;
             }
         }
-        if (kind < 0) break;
-        if (kind == 0) {                        // Op-done on device `who`
-            const int d = who, o = run_op[d];
-            run_op[d] = -1;
-            ++done;
-            last = now;
-            at(o_pending + o) = kFinished;
-            for (int e = a.parent_ptr[o]; e < a.parent_ptr[o + 1]; ++e)      // the inputs o read here
-                if (dev[a.parent[e]] < m) maybe_release(a.parent[e], d);
-            for (int e = a.child_ptr[o]; e < a.child_ptr[o + 1]; ++e) {
-                const int c = a.child[e], dc = dev[c];
-                if (dc >= m) continue;
-                if (dc != d) {
-                    if (sent[dc] != o && n_tr < a.n_edges) {   // the tensor goes to each device once
-                        sent[dc] = o;
-                        const int r = n_tr++;
-                        at(o_trop + r) = o;
-                        at(o_trdst + r) = dc;
-                        at(o_trnext + r) = -1;
-                        at(o_trleft + o) += 1;
-                        if (t_tail[d] < 0) t_head[d] = r; else at(o_trnext + t_tail[d]) = r;
-                        t_tail[d] = r;
-                    }
-                } else if (--at(o_pending + c) == 0) {
-                    push_op(d, c);
+        // The children of o: those on device `to` have one input less to wait for, those elsewhere get o's
+        // output sent, once per device, in child order.
+        for (int e = c0 + gl; __any_sync(kFull, e - gl < c1); e += kGroup) {
+            const int c = e < c1 ? child(e) : 0, dc = e < c1 ? (int)dev[c] : 0xff;
+            bool ready = false;
+            if (dc == to) {
+                const int left = (int)pending[c] - 1;
+                pending[c] = (Id)left;
+                ready = left == 0;
+            }
+            unsigned bits = in_group(ready);
+            while (__any_sync(kFull, bits != 0)) {
+                const int x = __shfl_sync(kFull, c, bits ? __ffs(bits) - 1 : 0, kGroup);
+                push_op(bits ? to : -1, x);
+                bits &= bits - 1;
+            }
+            unsigned away = in_group(is_op && dc < m && dc != d);
+            while (__any_sync(kFull, away != 0)) {
+                const int x = __shfl_sync(kFull, dc, away ? __ffs(away) - 1 : 0, kGroup);
+                const unsigned same = in_group(dc == x) & away;
+                away &= ~same;
+                // children beyond one per lane: the record may have been made by an earlier pass
+                int r = n_tr;
+                if (e - gl > c0 && same)
+                    for (int q = n_tr - (int)tr_left[o]; q < n_tr; ++q)
+                        if ((int)tr_dst[q] == x) r = q;
+                if (dc == x && same) rec[entry(e)] = (Id)r;
+                __syncwarp();
+                if (same) {
+#pragma unroll
+                    for (int k = 0; k < kPerLane; ++k)
+                        if (gl + 32 * k == d) {
+                            if (r == n_tr) {
+                                tr_op[r] = (Id)o;
+                                tr_dst[r] = (Small)x;
+                                tr_next[r] = (Id)none;
+                                tr_kids[r] = (Id)__popc(same);
+                                tr_left[o] = (Small)(tr_left[o] + 1);
+                                if (t_tail[k] == none) t_head[k] = r; else tr_next[t_tail[k]] = (Id)r;
+                                t_tail[k] = r;
+                            } else {
+                                tr_kids[r] = (Id)(tr_kids[r] + __popc(same));
+                            }
+                        }
+                    n_tr += r == n_tr;
                 }
+                __syncwarp();
             }
-            if (run_tr[d] < 0 && t_head[d] >= 0) start_transfer(d, now);
-            if (q_head[d] >= 0) start_op(d, now);
-        } else {                                // Transfer-done on the bus of device `who`
-            const int d = who, r = run_tr[d];
-            run_tr[d] = -1;
-            const int o = at(o_trop + r), to = at(o_trdst + r);
-            at(o_trleft + o) -= 1;
-            maybe_release(o, d);
-            for (int e = a.child_ptr[o]; e < a.child_ptr[o + 1]; ++e) {
-                const int c = a.child[e];
-                if (dev[c] == to && --at(o_pending + c) == 0) push_op(to, c);
-            }
-            if (run_op[to] < 0 && q_head[to] >= 0) start_op(to, now);
-            if (t_head[d] >= 0) start_transfer(d, now);
         }
+        __syncwarp();
+        // an ending operation creates the transfer's event first, an ending transfer the operation's (the
+        // two touch the memory of one device only in the second case)
+        start_op(alive ? to : -1, now, tag_base + (is_op ? 2 : 0));
+        start_transfer(alive ? d : -1, now, tag_base + (is_op ? 0 : 2) + 1);
+        __syncwarp();
     }
     // a device id outside [0, m) leaves operations unplaced: report NaN
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     const bool ok = done == n;
-    if (a.runtime) a.runtime[p] = ok ? last : nan;
     double top = 0.0;
-    for (int d = 0; d < m; ++d) {
-        if (a.peak_memory) a.peak_memory[(size_t)p * m + d] = ok ? peak[d] : nan;
-        top = peak[d] > top ? peak[d] : top;
+#pragma unroll
+    for (int k = 0; k < kPerLane; ++k) {
+        const int d = gl + 32 * k;
+        if (live && d < m) {
+            if (a.peak_memory) a.peak_memory[(size_t)p * m + d] = ok ? peak[k] : nan;
+            top = peak[k] > top ? peak[k] : top;
+        }
     }
-    if (a.penalised) a.penalised[p] = !ok ? nan : (top <= a.mem_limit ? last : last + a.mem_scale * (top - a.mem_limit));
+#pragma unroll
+    for (int o = kGroup / 2; o > 0; o >>= 1) {
+        const double other = __shfl_xor_sync(kFull, top, o);
+        top = other > top ? other : top;
+    }
+    if (live && gl == 0) {
+        if (a.runtime) a.runtime[p] = ok ? last : nan;
+        if (a.penalised) a.penalised[p] = !ok ? nan : (top <= a.mem_limit ? last : last + a.mem_scale * (top - a.mem_limit));
+    }
 }
 
 }  // namespace
 
-size_t sim_workspace_bytes(int n, int n_edges, int m, int P) {
-    (void)m;
+namespace {
+// placements per block whose arrays fit in shared memory beside the graph; 0: the arrays go to the workspace
+int sim_shared_fit(int n, int n_edges, const DeviceInfo &di) {
+    if (n_edges >= 0xffff) return 0;
+    const int budget = std::min(di.max_smem_optin, 227 * 1024) - 1024;
+    const int fit = (budget - sim_graph_bytes(n, n_edges)) / sim_state_bytes(n, n_edges);
+    return fit >= 4 ? fit : 0;
+}
+}  // namespace
+
+size_t sim_workspace_bytes(int n, int n_edges, int P, const DeviceInfo &di) {
+    if (sim_shared_fit(n, n_edges, di) > 0) return 256;
     return std::max<size_t>(sim_ints(n, n_edges) * (size_t)P * sizeof(int), 256);
 }
 
-cudaError_t launch_simulator(const SimArgs &a, cudaStream_t stream) {
-    simulate_kernel<<<(a.P + kThreads - 1) / kThreads, kThreads, 0, stream>>>(a);
+cudaError_t launch_simulator(const SimArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    SimPlan plan;
+    plan.graph_bytes = sim_graph_bytes(a.n, a.n_edges);
+    plan.state_bytes = sim_state_bytes(a.n, a.n_edges);
+    const int group = a.m <= 8 ? 8 : a.m <= 16 ? 16 : 32;
+    const int fit = sim_shared_fit(a.n, a.n_edges, di);
+    const bool shared = fit > 0;
+    const int most = shared ? std::min(fit, kMaxThreads / group) : kMaxThreads / group;
+    // the placements spread evenly over the SMs, and over the waves of blocks where one does not hold them
+    const int waves = (a.P + most * di.sm_count - 1) / (most * di.sm_count);
+    plan.per_block = (a.P + waves * di.sm_count - 1) / (waves * di.sm_count);
+    const int grid = (a.P + plan.per_block - 1) / plan.per_block;
+    const int threads = (plan.per_block * group + 31) & ~31;
+    const size_t smem = shared ? (size_t)plan.graph_bytes + (size_t)plan.per_block * plan.state_bytes : 0;
+    typedef void (*Kernel)(const SimArgs, const SimPlan);
+    const Kernel kernels[2][4] = {
+        {simulate_kernel<false, 8, 1>, simulate_kernel<false, 16, 1>, simulate_kernel<false, 32, 1>, simulate_kernel<false, 32, 2>},
+        {simulate_kernel<true, 8, 1>, simulate_kernel<true, 16, 1>, simulate_kernel<true, 32, 1>, simulate_kernel<true, 32, 2>}};
+    const Kernel kern = kernels[shared][a.m <= 8 ? 0 : a.m <= 16 ? 1 : a.m <= 32 ? 2 : 3];
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    kern<<<grid, threads, smem, stream>>>(a, plan);
     count_launch();
     return cudaGetLastError();
 }

@@ -147,3 +147,25 @@ def test_workload_graph_memory():
     np.testing.assert_array_equal(rt.cpu().numpy()[sel], want_rt)
     np.testing.assert_array_equal(peak.cpu().numpy()[sel], want_peak)
     np.testing.assert_array_equal(pen.cpu().numpy()[sel], want_pen)
+
+
+@pytest.mark.parametrize("n,m,P,p", [(7, 40, 5, 0.3), (90, 60, 200, 0.9), (1200, 33, 3, 0.05), (450, 2, 40, 0.7), (1, 1, 1, 0.0),
+                                     (40, 32, 5000, 0.4)])
+def test_devices_per_lane_fan_out_and_arrays_in_the_workspace(n, m, P, p):
+    """A lane keeps two devices beyond 32; nodes with more than 32 children take several passes; graphs whose arrays
+    (n = 1200 and 450 with tens of thousands of edges) do not fit in shared memory keep them in the workspace; more
+    placements than one block per SM holds."""
+    r = rng(n + m)
+    src, dst = random_dag(r, n, p)
+    cost = r.integers(1, 5, n).astype(np.float32)        # many equal time stamps
+    size = r.integers(1, 5, n).astype(np.float32)
+    devs = r.integers(0, m, size=(P, n))
+    g = placeto.Graph(n, src, dst)
+    rt, peak, pen = placeto.placeto_simulate_placements(g, dev_t(cost), dev_t(size), dev_t(devs.astype(np.uint8)), m, 2.0,
+                                                        6.0, 2.0)
+    torch.cuda.synchronize()
+    sel = np.arange(0, P, max(1, P // 4))
+    want_rt, want_peak, want_pen = simulator.placements(n, src, dst, cost, size, devs[sel], m, 2.0, 6.0, 2.0)
+    np.testing.assert_array_equal(rt.cpu().numpy()[sel], want_rt)
+    np.testing.assert_array_equal(peak.cpu().numpy()[sel], want_peak)
+    np.testing.assert_array_equal(pen.cpu().numpy()[sel], want_pen)
