@@ -123,9 +123,9 @@ Layout make_layout(const placeto_graph *g, const placeto_weights *w, int B, plac
         L.total = off;
         return L;
     }
-    if (w->F >= 4 && w->F <= 16 && (w->F & 3) == 0) {
+    if (w->F <= 16) {
         if (w->d == 32) pool_d32_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
-        if (w->d == 64) pool_d64_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
+        if (w->d == 64 && (w->F & 3) == 0) pool_d64_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
         if (w->d == 64) pool_tc_chunks((int)n, B, g->info, &L.chunk_nodes_tc, &L.chunks_tc);
     }
     if (call == PLACETO_CALL_LOGITS || (call >= PLACETO_CALL_FORWARD && call <= PLACETO_CALL_EPISODE))
@@ -777,7 +777,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
     // episode) is the whole state, and the head kernel makes the transition itself.
     bool compact_path = false;
     if (!(flags & (PLACETO_GENERIC | PLACETO_TENSOR | PLACETO_PER_LEVEL | PLACETO_COOPERATIVE)) && w->m < 63 &&
-        L.chunks32 > 0) {
+        L.chunks32 > 0 && (w->F & 3) == 0) {
         EmbedArgs ea;
         ea.lv[0] = g->lv[0]; ea.lv[1] = g->lv[1];
         ea.f[0] = to_dev(w->f_down); ea.f[1] = to_dev(w->f_up);

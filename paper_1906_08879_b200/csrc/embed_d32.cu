@@ -1,12 +1,16 @@
 // Step 2 of the policy (Sec. 2.2 step 2 of the Placeto paper) specialised for
-// embedding width d = 32 with two-layer ReLU networks of hidden width 32:
+// embedding width d = 32 with ReLU networks of one layer (the paper's own, Appendix A.7)
+// or two layers of hidden width 32:
 //   h_v = g( sum_{u in nbr(v)} m_u ),   m_u = f([h_u || x_u]).
 //
 // Design (one block = one direction x one slice of the state batch, walking all
 // levels with __syncthreads() between levels; states never interact):
 //   - Lane j of every warp keeps column j of all four weight matrices of the
 //     direction in registers (32 + 32 + (32 + F) + 32 values), so a warp carries
-//     a row (node, state) through gather -> g1 -> g2 -> f1 -> f2 on its own.
+//     a row (node, state) through gather -> g1 -> g2 -> f1 -> f2 on its own. With
+//     single-layer networks the second layers drop out at compile time: half
+//     the dependent chain of a level (whole path on a 279-node graph, 132 levels, 250
+//     states, two devices, B200: 106 us; 618 us on the dimension-generic kernels).
 //     Between layers the 32 outputs are exchanged through a per-warp shared
 //     buffer and read back as broadcast 128-bit loads: 4 FMAs per shared load,
 //     issued as two packed fma.rn.f32x2 against weights kept in register pairs.
@@ -99,7 +103,7 @@ struct Weights32 {
 // gather -> g -> store h -> f -> store m. The R rows share the node, so the
 // schedule lookups are done once. A, Bf: the warp's exchange buffers, R rows of
 // KF floats each. All shared-memory offsets are 32-bit.
-template <int R, int KF>
+template <int R, int KF, int L>   // L layers per network
 __device__ __forceinline__ void run_node(const Weights32 &w, const pair_t (&wf1)[KF / 2], int pos,
                                          int q, int s0, bool last_live, int nb, int S, int F,
                                          int lane, const int4 *meta, const int *nbr_slot,
@@ -148,10 +152,12 @@ __device__ __forceinline__ void run_node(const Weights32 &w, const pair_t (&wf1)
     __syncwarp();
     matvec<R, kD>(w.g1, w.bg1, A, KF, acc);
 after_g1:
+    if constexpr (L == 2) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
-    __syncwarp();
-    matvec<R, kD>(w.g2, w.bg2, Bf, KF, acc);
+        for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
+        __syncwarp();
+        matvec<R, kD>(w.g2, w.bg2, Bf, KF, acc);
+    }
     float *hrow = H + ((size_t)v * B + b_first + s0) * kD + lane;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -159,23 +165,26 @@ after_g1:
         if (r == 0 || last_live) hrow[r * kD] = acc[r];
     }
     if (slot < 0) return;                   // nobody consumes this node's message
+    float *in = L == 2 ? A : Bf;            // the buffer that the last product did not read
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        A[r * KF + lane] = acc[r];
-        if (lane < KF - kD) A[r * KF + kD + lane] = x[r];
+        in[r * KF + lane] = acc[r];
+        if (lane < KF - kD) in[r * KF + kD + lane] = x[r];
     }
     __syncwarp();
-    matvec<R, KF>(wf1, w.bf1, A, KF, acc);
+    matvec<R, KF>(wf1, w.bf1, in, KF, acc);
+    if constexpr (L == 2) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
-    __syncwarp();
-    matvec<R, kD>(w.f2, w.bf2, Bf, KF, acc);
+        for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
+        __syncwarp();
+        matvec<R, kD>(w.f2, w.bf2, Bf, KF, acc);
+    }
 #pragma unroll
     for (int r = 0; r < R; ++r)
         if (r == 0 || last_live) msg[((slot * S) + st[r]) * kD + lane] = fmaxf(acc[r], 0.f);
 }
 
-template <int F4, bool kCompact>   // feature width padded to 4 * F4; features built from compact states
+template <int F4, bool kCompact, int L>   // feature width padded to 4 * F4; features built from compact states; layers
 __global__ void __launch_bounds__(kThreads, 1)
 embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     constexpr int KF = kD + 4 * F4;      // padded input width of f's first layer
@@ -225,14 +234,17 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
 #pragma unroll
     for (int k = 0; k < kD; k += 2) {
         w.g1[k / 2] = pack2(g.W1[k * kD + lane], g.W1[(k + 1) * kD + lane]);
-        w.g2[k / 2] = pack2(g.W2[k * kD + lane], g.W2[(k + 1) * kD + lane]);
-        w.f2[k / 2] = pack2(f.W2[k * kD + lane], f.W2[(k + 1) * kD + lane]);
+        if constexpr (L == 2) {
+            w.g2[k / 2] = pack2(g.W2[k * kD + lane], g.W2[(k + 1) * kD + lane]);
+            w.f2[k / 2] = pack2(f.W2[k * kD + lane], f.W2[(k + 1) * kD + lane]);
+        }
     }
 #pragma unroll
     for (int k = 0; k < KF; k += 2)
         wf1[k / 2] = pack2(k < kD + F ? f.W1[k * kD + lane] : 0.f,
                            k + 1 < kD + F ? f.W1[(k + 1) * kD + lane] : 0.f);
-    w.bg1 = g.b1[lane]; w.bg2 = g.b2[lane]; w.bf1 = f.b1[lane]; w.bf2 = f.b2[lane];
+    w.bg1 = g.b1[lane]; w.bf1 = f.b1[lane];
+    if constexpr (L == 2) { w.bg2 = g.b2[lane]; w.bf2 = f.b2[lane]; }
     const float *__restrict__ X = a.X;
     float *__restrict__ H = a.H[dir];
     __syncthreads();
@@ -285,7 +297,7 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
             if (warp < rows) {
                 const int q = nb == 1 ? warp : (int)__umulhi((unsigned)warp, magic_nb);
                 const int s0 = warp - q * nb;
-                run_node<1, KF>(w, wf1, p0 + q, q, s0, true, nb, p.S, F, lane, meta, nbr_slot, msg,
+                run_node<1, KF, L>(w, wf1, p0 + q, q, s0, true, nb, p.S, F, lane, meta, nbr_slot, msg,
                                 xs, H, B, b_first, A, Bf);
             }
         } else {
@@ -294,7 +306,7 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
             for (int item = warp; item < width * ppn; item += kWarps) {
                 const int q = ppn == 1 ? item : (int)__umulhi((unsigned)item, magic_ppn);
                 const int s0 = (item - q * ppn) * 2;
-                run_node<2, KF>(w, wf1, p0 + q, q, s0, s0 + 1 < nb, nb, p.S, F, lane, meta, nbr_slot,
+                run_node<2, KF, L>(w, wf1, p0 + q, q, s0, s0 + 1 < nb, nb, p.S, F, lane, meta, nbr_slot,
                                 msg, xs, H, B, b_first, A, Bf);
             }
         }
@@ -303,8 +315,8 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     }
 }
 
-bool relu2x32(const DevMlp &m, int in) {
-    return m.n_layers == 2 && m.in_dim == in && m.hidden_dim == kD && m.out_dim == kD &&
+bool relu32(const DevMlp &m, int in, int layers) {
+    return m.n_layers == layers && m.in_dim == in && m.hidden_dim == kD && m.out_dim == kD &&
            m.act == 0 && m.final_act == 1;
 }
 
@@ -313,7 +325,7 @@ bool relu2x32(const DevMlp &m, int in) {
 bool embed_d32_applicable(const EmbedArgs &a) {
     if (a.d != kD || a.F < 1 || a.F > 16) return false;
     for (int dir = 0; dir < 2; ++dir)
-        if (!relu2x32(a.f[dir], kD + a.F) || !relu2x32(a.g[dir], kD)) return false;
+        if (!relu32(a.f[dir], kD + a.F, a.f[0].n_layers) || !relu32(a.g[dir], kD, a.f[0].n_layers)) return false;
     return true;
 }
 
@@ -366,15 +378,13 @@ cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStrea
     D32Plan p;
     if (!plan_d32(a, di, &p)) return cudaErrorNotSupported;
     const int F4 = (a.F + 3) / 4;
-    void (*kern)(const EmbedArgs, const D32Plan) = nullptr;
-    const bool compact = a.compact.state != nullptr;
-    switch (F4) {
-        case 1: kern = compact ? embed_d32_kernel<1, true> : embed_d32_kernel<1, false>; break;
-        case 2: kern = compact ? embed_d32_kernel<2, true> : embed_d32_kernel<2, false>; break;
-        case 3: kern = compact ? embed_d32_kernel<3, true> : embed_d32_kernel<3, false>; break;
-        case 4: kern = compact ? embed_d32_kernel<4, true> : embed_d32_kernel<4, false>; break;
-        default: return cudaErrorNotSupported;
-    }
+    typedef void (*Kernel)(const EmbedArgs, const D32Plan);
+    static const Kernel kernels[2][2][4] = {     // [layers][compact][F4]
+        {{embed_d32_kernel<1, false, 1>, embed_d32_kernel<2, false, 1>, embed_d32_kernel<3, false, 1>, embed_d32_kernel<4, false, 1>},
+         {embed_d32_kernel<1, true, 1>, embed_d32_kernel<2, true, 1>, embed_d32_kernel<3, true, 1>, embed_d32_kernel<4, true, 1>}},
+        {{embed_d32_kernel<1, false, 2>, embed_d32_kernel<2, false, 2>, embed_d32_kernel<3, false, 2>, embed_d32_kernel<4, false, 2>},
+         {embed_d32_kernel<1, true, 2>, embed_d32_kernel<2, true, 2>, embed_d32_kernel<3, true, 2>, embed_d32_kernel<4, true, 2>}}};
+    const Kernel kern = kernels[a.f[0].n_layers - 1][a.compact.state != nullptr][F4 - 1];
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)p.smem_bytes);
     if (err != cudaSuccess) return err;

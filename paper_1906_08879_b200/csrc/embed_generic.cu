@@ -261,7 +261,7 @@ cudaError_t launch_embed_generic(const EmbedArgs &a, const DeviceInfo &di, unsig
 // direction (msg[2 * dir], msg[2 * dir + 1]).
 cudaError_t launch_embed_rounds(const EmbedArgs &a, const DeviceInfo &di, int rounds, float *const msg[4],
                                 cudaStream_t stream) {
-    if (embed_d32_applicable(a)) {
+    if (embed_d32_applicable(a) && a.f[0].n_layers == 2) {
         const cudaError_t e = launch_embed_rounds_d32(a, di, rounds, msg, stream);
         if (e != cudaErrorNotSupported) return e;
     }

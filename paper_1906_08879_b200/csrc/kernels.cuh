@@ -317,12 +317,12 @@ cudaError_t launch_embed_generic(const EmbedArgs &a, const DeviceInfo &di, unsig
 cudaError_t launch_embed_rounds(const EmbedArgs &a, const DeviceInfo &di, int rounds, float *const msg[4],
                                 cudaStream_t stream);
 
-// embed_rounds_d32.cu: the same rounds for the shapes of embed_d32_applicable (throughput kernel)
+// embed_rounds_d32.cu: the same rounds for the two-layer shapes of embed_d32_applicable (throughput kernel)
 cudaError_t launch_embed_rounds_d32(const EmbedArgs &a, const DeviceInfo &di, int rounds,
                                     float *const msg[4], cudaStream_t stream);
 
-// embed_d32.cu: specialised message passing for d = 32 with two-layer ReLU
-// networks of hidden width 32; returns cudaErrorNotSupported when the shapes or
+// embed_d32.cu: specialised message passing for d = 32 with ReLU networks of one
+// layer or of two with hidden width 32; returns cudaErrorNotSupported when the shapes or
 // the shared-memory budget do not fit (the caller then uses the generic kernel).
 bool embed_d32_applicable(const EmbedArgs &a);
 bool embed_d32_fits(const EmbedArgs &a, const DeviceInfo &di);   // applicable and within shared memory
@@ -370,7 +370,7 @@ cudaError_t launch_policy_generic(const PoolArgs &a, const DeviceInfo &di, cudaS
 // adds the chunk partial sums, applies h_i, the head and the softmax (one block per state)
 cudaError_t launch_pool_head(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream);
 
-// policy_d32.cu: specialised partial sums for d = 32, F a multiple of 4, single-layer ReLU l_i
+// policy_d32.cu: specialised partial sums for d = 32, F <= 16, single-layer ReLU l_i
 bool pool_d32_applicable(const PoolArgs &a);
 bool pool_d32_fits(const PoolArgs &a, const DeviceInfo &di);      // applicable (a.chunk_nodes set) and within shared memory
 void pool_d32_chunks(int n, int B, int F, const DeviceInfo &di, int *chunk_nodes, int *chunks);

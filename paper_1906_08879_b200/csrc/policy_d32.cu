@@ -87,11 +87,14 @@ pool_d32_kernel(const PoolArgs a, const Pool32Plan p) {
     // (16 states x 32 floats of H_down and H_up, 16 states x F of X are contiguous
     // both in global and in shared memory), all reporting to one mbarrier
     __shared__ __align__(8) unsigned long long bar;
-    const unsigned w_bytes = (unsigned)(E * kD * sizeof(float));      // F == FP here: no padding rows
+    const unsigned w_bytes = (unsigned)((2 * kD + F) * kD * sizeof(float));
+    // The raw features of a node's 16 states are a whole number of 16-byte pieces only when F is a
+    // multiple of 4; otherwise (and with compact states) the threads write them, zero padded.
+    const bool bulk_x = !kCompact && F == FP;
     const unsigned h_bytes = (unsigned)(nb * kD * sizeof(float)), x_bytes = (unsigned)(nb * F * sizeof(float));
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
-        mbar_expect(&bar, 3 * w_bytes + (unsigned)nu * (2 * h_bytes + (kCompact ? 0u : x_bytes)));
+        mbar_expect(&bar, 3 * w_bytes + (unsigned)nu * (2 * h_bytes + (bulk_x ? x_bytes : 0u)));
     }
     if (threadIdx.x < 3 * kD) bs[threadIdx.x] = a.l[threadIdx.x / kD].b1[threadIdx.x % kD];
     __syncthreads();
@@ -103,13 +106,23 @@ pool_d32_kernel(const PoolArgs a, const Pool32Plan p) {
         const size_t row = (size_t)(u0 + q) * B + b0;
         if (which == 0) bulk_load(hd + (size_t)q * kWarps * kD, a.H[0] + row * kD, h_bytes, &bar);
         else if (which == 1) bulk_load(hu + (size_t)q * kWarps * kD, a.H[1] + row * kD, h_bytes, &bar);
-        else if (!kCompact) bulk_load(xs + (size_t)q * kWarps * FP, a.X + row * F, x_bytes, &bar);
+        else if (bulk_x) bulk_load(xs + (size_t)q * kWarps * FP, a.X + row * F, x_bytes, &bar);
     }
     if (kCompact) {
         // no X tensor: the tile's features from one byte per (node, state)
         for (int i = threadIdx.x; i < nu * nb; i += kThreads) {     // one (node, state) pair per thread
             const int q = i / nb, st = i - q * nb;
             compact_features(a.compact, u0 + q, b0 + st, B, xs + (size_t)q * kWarps * FP + st * FP);
+        }
+        __syncthreads();
+    } else if (!bulk_x) {
+        for (int i = threadIdx.x; i < nu * nb * FP; i += kThreads) {
+            const int q = i / (nb * FP), r = i - q * (nb * FP), st = r / FP, k = r - st * FP;
+            xs[(size_t)q * kWarps * FP + r] = k < F ? a.X[((size_t)(u0 + q) * B + b0 + st) * F + k] : 0.f;
+        }
+        for (int i = threadIdx.x; i < 3 * (FP - F) * kD; i += kThreads) {      // weight rows past 64 + F
+            const int set = i / ((FP - F) * kD), r = i - set * ((FP - F) * kD);
+            Ws[(set * E + 2 * kD + F) * kD + r] = 0.f;
         }
         __syncthreads();
     }
@@ -173,7 +186,7 @@ bool relu1(const DevMlp &m, int in) {
 }  // namespace
 
 bool pool_d32_applicable(const PoolArgs &a) {
-    if (a.d != kD || a.F < 4 || a.F > 16 || (a.F & 3)) return false;
+    if (a.d != kD || a.F < 1 || a.F > 16) return false;
     for (int i = 0; i < 3; ++i)
         if (!relu1(a.l[i], 2 * kD + a.F)) return false;
     return true;
@@ -181,7 +194,7 @@ bool pool_d32_applicable(const PoolArgs &a) {
 
 // Nodes per chunk and number of chunks for a batch of B states.
 void pool_d32_chunks(int n, int B, int F, const DeviceInfo &di, int *chunk_nodes, int *chunks) {
-    const int E = 2 * kD + F;
+    const int E = 2 * kD + ((F + 3) & ~3);
     const size_t budget = (size_t)std::min(di.max_smem_optin, 227 * 1024) - 1024;
     const size_t fixed = (size_t)(3 * E * kD + 3 * kD) * sizeof(float);
     const size_t per_node = (size_t)kWarps * E * sizeof(float);
@@ -196,7 +209,7 @@ void pool_d32_chunks(int n, int B, int F, const DeviceInfo &di, int *chunk_nodes
 }
 
 bool pool_d32_fits(const PoolArgs &a, const DeviceInfo &di) {
-    const int E = 2 * kD + a.F;
+    const int E = 2 * kD + ((a.F + 3) & ~3);
     const size_t bytes = ((size_t)(3 * E * kD + 3 * kD) + (size_t)a.chunk_nodes * kWarps * E) * sizeof(float);
     return pool_d32_applicable(a) && a.chunk_nodes > 0 && bytes <= (size_t)di.max_smem_optin;
 }
@@ -206,11 +219,11 @@ cudaError_t launch_pool_d32(const PoolArgs &a, const DeviceInfo &di, cudaStream_
     Pool32Plan p;
     p.chunk_nodes = a.chunk_nodes;
     p.chunks = a.chunks;
-    const int E = 2 * kD + a.F;
+    const int E = 2 * kD + ((a.F + 3) & ~3);
     p.smem_bytes = ((size_t)(3 * E * kD + 3 * kD) + (size_t)p.chunk_nodes * kWarps * E) * sizeof(float);
     if (p.smem_bytes > (size_t)di.max_smem_optin) return cudaErrorNotSupported;
     void (*kern)(const PoolArgs, const Pool32Plan) = nullptr;
-    switch (a.F / 4) {
+    switch ((a.F + 3) / 4) {
         case 1: kern = a.compact.state ? pool_d32_kernel<1, true> : pool_d32_kernel<1, false>; break;
         case 2: kern = a.compact.state ? pool_d32_kernel<2, true> : pool_d32_kernel<2, false>; break;
         case 3: kern = a.compact.state ? pool_d32_kernel<3, true> : pool_d32_kernel<3, false>; break;

@@ -354,16 +354,39 @@ pool_head_kernel(const PoolArgs a, int tmp_floats, int stage_floats) {
 }
 
 // The same finish for the common shapes (single-layer h_i of width d, two-layer
-// head whose hidden width is a multiple of 4) with HS states per block, HS chosen
-// so that the blocks cover the device: a small batch is spread over many SMs
-// instead of eight states sharing one. Nothing is staged: weights are read once
-// per block straight from L2 as 128-bit loads, a thread of the first head layer
+// head) with HS states per block, HS chosen so that the blocks cover the device: a
+// small batch is spread over many SMs instead of eight states sharing one. Nothing
+// is staged: weights are read once per block straight from L2, as 128-bit loads
+// where the hidden width keeps the rows of the head's first matrix aligned for
+// them (VEC = 4), as 64- or 32-bit ones otherwise (odd device counts: F = m + 4 is
+// then no multiple of 4); a thread of the first head layer
 // owns a (states x 4 columns) register tile and one part of the inner dimension,
 // and activations sit transposed in shared memory ([k][state]) so that a tile's
 // states come with one broadcast load. Parts are added in a fixed order.
 constexpr int kFastThreads = 512;
 
-template <int HS>
+// four consecutive floats of a row, of which the first `left` exist (left >= 1)
+template <int VEC>
+__device__ __forceinline__ float4 load_row4(const float *__restrict__ p, int left) {
+    if (VEC == 4) return __ldg(reinterpret_cast<const float4 *>(p));
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (VEC == 2) {                         // `left` is even
+        const float2 lo = __ldg(reinterpret_cast<const float2 *>(p));
+        v.x = lo.x; v.y = lo.y;
+        if (left > 2) {
+            const float2 hi = __ldg(reinterpret_cast<const float2 *>(p + 2));
+            v.z = hi.x; v.w = hi.y;
+        }
+    } else {
+        v.x = __ldg(p);
+        if (left > 1) v.y = __ldg(p + 1);
+        if (left > 2) v.z = __ldg(p + 2);
+        if (left > 3) v.w = __ldg(p + 3);
+    }
+    return v;
+}
+
+template <int HS, int VEC>
 __global__ void __launch_bounds__(kFastThreads, 1)
 pool_head_fast_kernel(const PoolArgs a) {
     constexpr int SR = HS < 4 ? HS : 4;     // states of a thread tile
@@ -371,11 +394,12 @@ pool_head_fast_kernel(const PoolArgs a) {
     extern __shared__ __align__(16) float smem[];
     const int d = a.d, F = a.F, B = a.B, m = a.m;
     const int E = 2 * d + F, Z = 5 * d + F, Hd = a.head.hidden_dim;
+    const int Hp = (Hd + 3) & ~3;                  // hidden units in whole groups of four columns
     float *zt = smem;                              // [Z][HS]: e_c, then the three h_i outputs
     float *sum = zt + Z * HS;                      // [HS][3 d]
-    float *hid = sum + HS * 3 * d;                 // [Hd][HS]
-    float *lg = hid + Hd * HS;                     // [HS][m]
-    float *red = lg + ((HS * m + 3) & ~3);         // [parts][Hd][HS]
+    float *hid = sum + HS * 3 * d;                 // [Hp][HS]
+    float *lg = hid + Hp * HS;                     // [HS][m]
+    float *red = lg + ((HS * m + 3) & ~3);         // [parts][Hp][HS]
     const int b0 = blockIdx.x * HS;
     prefetch_l2(a.head.W1, (size_t)Z * Hd);
     prefetch_l2(a.head.W2, (size_t)Hd * m);
@@ -418,7 +442,7 @@ pool_head_fast_kernel(const PoolArgs a) {
         const DevMlp &nt = a.h[set];
         const float *__restrict__ W = nt.W1 + 4 * cq;
         const float *v = sum + s * 3 * d + set * d;
-        float4 acc = *reinterpret_cast<const float4 *>(nt.b1 + 4 * cq);
+        float4 acc = *reinterpret_cast<const float4 *>(nt.b1 + 4 * cq), odd = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int kb = 0; kb < d; kb += 16) {   // sixteen weight rows in flight (d is a multiple of 4)
             float4 w[16];
 #pragma unroll
@@ -426,12 +450,15 @@ pool_head_fast_kernel(const PoolArgs a) {
                 w[t] = kb + t < d ? __ldg(reinterpret_cast<const float4 *>(W + (size_t)(kb + t) * d))
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                const float x = kb + t < d ? v[kb + t] : 0.f;
-                acc.x = fmaf(x, w[t].x, acc.x); acc.y = fmaf(x, w[t].y, acc.y);
-                acc.z = fmaf(x, w[t].z, acc.z); acc.w = fmaf(x, w[t].w, acc.w);
+            for (int t = 0; t < 16; t += 2) {      // two chains: shorter, and less rounding in each
+                const float x = kb + t < d ? v[kb + t] : 0.f, y = kb + t + 1 < d ? v[kb + t + 1] : 0.f;
+                acc.x = fmaf(x, w[t].x, acc.x); odd.x = fmaf(y, w[t + 1].x, odd.x);
+                acc.y = fmaf(x, w[t].y, acc.y); odd.y = fmaf(y, w[t + 1].y, odd.y);
+                acc.z = fmaf(x, w[t].z, acc.z); odd.z = fmaf(y, w[t + 1].z, odd.z);
+                acc.w = fmaf(x, w[t].w, acc.w); odd.w = fmaf(y, w[t + 1].w, odd.w);
             }
         }
+        acc.x += odd.x; acc.y += odd.y; acc.z += odd.z; acc.w += odd.w;
         if (nt.act == 0 && nt.final_act) {
             acc.x = fmaxf(acc.x, 0.f); acc.y = fmaxf(acc.y, 0.f);
             acc.z = fmaxf(acc.z, 0.f); acc.w = fmaxf(acc.w, 0.f);
@@ -441,7 +468,7 @@ pool_head_fast_kernel(const PoolArgs a) {
     }
     __syncthreads();
     // head, first layer
-    const int CG = Hd >> 2, tiles = SG * CG;
+    const int CG = Hp >> 2, tiles = SG * CG;
     const int parts = max(1, min((int)blockDim.x / tiles, Z));
     const int per = (Z + parts - 1) / parts;
     if ((int)threadIdx.x < tiles * parts) {
@@ -459,7 +486,7 @@ pool_head_fast_kernel(const PoolArgs a) {
             float4 w[16];
 #pragma unroll
             for (int t = 0; t < 16; ++t)
-                w[t] = kb + t < k1 ? __ldg(reinterpret_cast<const float4 *>(W + (size_t)(kb + t) * Hd))
+                w[t] = kb + t < k1 ? load_row4<VEC>(W + (size_t)(kb + t) * Hd, Hd - 4 * cg)
                                    : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int t = 0; t < 16; ++t) {
@@ -487,13 +514,13 @@ pool_head_fast_kernel(const PoolArgs a) {
         for (int c = 0; c < 4; ++c)
 #pragma unroll
             for (int s = 0; s < SR; ++s)
-                red[((size_t)part * Hd + 4 * cg + c) * HS + sg * SR + s] = acc[s][c];
+                red[((size_t)part * Hp + 4 * cg + c) * HS + sg * SR + s] = acc[s][c];
     }
     __syncthreads();
     const bool relu = a.head.act == 0;
     for (int i = threadIdx.x; i < Hd * HS; i += blockDim.x) {
         float acc = a.head.b1[i / HS];
-        for (int q = 0; q < parts; ++q) acc += red[(size_t)q * Hd * HS + i];
+        for (int q = 0; q < parts; ++q) acc += red[(size_t)q * Hp * HS + i];
         hid[i] = relu ? fmaxf(acc, 0.f) : acc;
     }
     __syncthreads();
@@ -554,8 +581,8 @@ pool_head_fast_kernel(const PoolArgs a) {
 }
 
 bool head_fast_applicable(const PoolArgs &a) {
-    if ((a.d & 3) || a.head.n_layers != 2 || (a.head.hidden_dim & 3)) return false;
-    if (a.head.hidden_dim / 4 * 2 > kFastThreads) return false;
+    if ((a.d & 3) || a.head.n_layers != 2) return false;
+    if ((a.head.hidden_dim + 3) / 4 * 2 > kFastThreads) return false;
     for (int i = 0; i < 3; ++i)
         if (a.h[i].n_layers != 1 || a.h[i].in_dim != a.d || a.h[i].out_dim != a.d) return false;
     return true;
@@ -563,7 +590,7 @@ bool head_fast_applicable(const PoolArgs &a) {
 
 template <int HS>
 cudaError_t launch_head_fast(const PoolArgs &a, cudaStream_t stream) {
-    const int Z = 5 * a.d + a.F, Hd = a.head.hidden_dim;
+    const int Z = 5 * a.d + a.F, Hd = (a.head.hidden_dim + 3) & ~3;
     constexpr int SR = HS < 4 ? HS : 4;
     const int tiles = (HS / SR) * (Hd / 4);
     const int parts = std::max(1, std::min(kFastThreads / tiles, Z));
@@ -571,11 +598,13 @@ cudaError_t launch_head_fast(const PoolArgs &a, cudaStream_t stream) {
                           (size_t)parts * Hd * HS;
     const size_t bytes = floats * sizeof(float);
     if (bytes > 200 * 1024) return cudaErrorNotSupported;
-    cudaError_t err = cudaFuncSetAttribute(pool_head_fast_kernel<HS>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    void (*kern)(const PoolArgs) = (a.head.hidden_dim & 3) == 0   ? pool_head_fast_kernel<HS, 4>
+                                   : (a.head.hidden_dim & 1) == 0 ? pool_head_fast_kernel<HS, 2>
+                                                                  : pool_head_fast_kernel<HS, 1>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (err != cudaSuccess) return err;
     // always preceded by one of this library's pooling kernels on the same stream
-    err = launch_overlapped(true, pool_head_fast_kernel<HS>, dim3((a.B + HS - 1) / HS), dim3(kFastThreads),
+    err = launch_overlapped(true, kern, dim3((a.B + HS - 1) / HS), dim3(kFastThreads),
                             bytes, stream, a);
     count_launch();
     return err;

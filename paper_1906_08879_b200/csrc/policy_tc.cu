@@ -152,6 +152,12 @@ __device__ __forceinline__ void store_split4(unsigned char *head_at, int tail_by
     *reinterpret_cast<float4 *>(head_at + tail_bytes) = t;
 }
 
+__device__ __forceinline__ void store_split2(unsigned char *head_at, int tail_bytes, float x, float y) {
+    const float hx = __uint_as_float(tf32_round(x)), hy = __uint_as_float(tf32_round(y));
+    *reinterpret_cast<float2 *>(head_at) = make_float2(hx, hy);
+    *reinterpret_cast<float2 *>(head_at + tail_bytes) = make_float2(x - hx, y - hy);
+}
+
 __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const PoolArgs a, const PoolTcPlan p) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ unsigned long long bar_full[kStages], bar_buf_free[kStages], bar_acc_full[kStages], bar_acc_free[kStages];
@@ -268,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const PoolArgs a, 
     } else if (warp < kIssueWarp) {
         // ------------------------------------------------------------ producer warps
         const int pw = warp - kEpiWarps, ptid = tid - kEpiThreads;
-        const int f4 = F >> 2;
+        const int f4 = max(1, F >> 2);
         dependency_wait();          // the embeddings may come from a kernel that is still running
         // An item's row of the relation matrix is scanned once per set: keep the block's rows in
         // shared memory when they fit.
@@ -329,7 +335,11 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const PoolArgs a, 
         // fenced (the fence would wait for loads in flight) and arrive while the warp waits
         // for a free tile.
         float4 hv[kRowsPerWarp], xv;
-        const int xj = lane / f4, xpiece = lane - xj * f4;      // f4 <= 4: lanes 0 .. 4 f4 - 1 are in use
+        // F a multiple of 4: 16-byte pieces, lanes 0 .. 4 f4 - 1 are in use; otherwise rows of X are not
+        // 16-byte aligned and eight lanes take a row two words at a time (padding words as zeros).
+        const bool vec_x = (F & 3) == 0;
+        const int xj = vec_x ? lane / f4 : lane >> 3, xpiece = vec_x ? lane - xj * f4 : lane & 7;
+        const bool x_lane = xj < kRowsPerWarp && (vec_x || 2 * xpiece < F);
         auto prefetch = [&](const int *rows_of_tile, int rows, int b) {
 #pragma unroll
             for (int j = 0; j < kRowsPerWarp; ++j) {
@@ -340,8 +350,15 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const PoolArgs a, 
                 }
             }
             const int rx = pw + xj * kProdWarps;
-            if (xj < kRowsPerWarp && rx < rows)
-                xv = reinterpret_cast<const float4 *>(a.X + ((size_t)rows_of_tile[rx] * B + b) * F)[xpiece];
+            if (x_lane && rx < rows) {
+                const float *x = a.X + ((size_t)rows_of_tile[rx] * B + b) * F;
+                if (vec_x) {
+                    xv = reinterpret_cast<const float4 *>(x)[xpiece];
+                } else {
+                    xv.x = x[2 * xpiece];
+                    xv.y = 2 * xpiece + 1 < F ? x[2 * xpiece + 1] : 0.f;
+                }
+            }
         };
         unsigned tc = 0;
         bool ok = true;
@@ -375,8 +392,11 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const PoolArgs a, 
                         if (r < rows) store_split4(tile + (r >> 3) * SBO + (r & 7) * 16 + lane * LBO, tail_bytes, hv[j]);
                     }
                     const int rx = pw + xj * kProdWarps;
-                    if (xj < kRowsPerWarp && rx < rows)
-                        store_split4(tile + (rx >> 3) * SBO + (rx & 7) * 16 + (32 + xpiece) * LBO, tail_bytes, xv);
+                    if (x_lane && rx < rows) {
+                        unsigned char *x_at = tile + (rx >> 3) * SBO + (rx & 7) * 16;
+                        if (vec_x) store_split4(x_at + (32 + xpiece) * LBO, tail_bytes, xv);
+                        else store_split2(x_at + (32 + (xpiece >> 1)) * LBO + 8 * (xpiece & 1), tail_bytes, xv.x, xv.y);
+                    }
                     if (ptid == 0) {
                         int flags = 0;
                         if (t == n_tiles - 1) flags |= kLastOfItem | ((k + 1) % my_items == 0 ? kLastOfSet : 0);
@@ -459,7 +479,7 @@ bool relu1x64(const DevMlp &m, int in) {
 }  // namespace
 
 bool pool_tc_applicable(const PoolArgs &a) {
-    if (a.d != kD || a.F < 4 || a.F > 16 || (a.F & 3)) return false;
+    if (a.d != kD || a.F < 1 || a.F > 16) return false;
     for (int i = 0; i < 3; ++i)
         if (!relu1x64(a.l[i], 2 * kD + a.F)) return false;
     return true;

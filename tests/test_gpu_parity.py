@@ -331,6 +331,16 @@ def test_single_layer_networks_as_in_the_paper():
         _small_case(30, src, dst, d=16, m=4, B=12, layers=1, seed=3, schedule=sched)
 
 
+@pytest.mark.parametrize("d,m,B", [(32, 2, 1), (32, 3, 90), (32, 4, 300), (32, 5, 77), (32, 12, 150), (64, 2, 1), (64, 3, 90),
+                                   (64, 8, 300), (64, 5, 600)])
+def test_single_layer_networks_at_the_specialised_widths(d, m, B):
+    """Single-layer f, g at d = 32 and 64: one state per block, levels of one row per warp and of several, a ragged last
+    slice; feature widths that are and are not multiples of 4 (rows of X and of the head's first matrix unaligned)."""
+    r = rng(B + m)
+    src, dst = random_dag(r, 45, 0.12)
+    _small_case(45, src, dst, d=d, m=m, B=B, layers=1, seed=B + d)
+
+
 def test_identity_activation_and_path_counting():
     one = net([[1.0], [1.0]], [0.0], act=1)
     idn = net([[1.0]], [0.0], act=1)
