@@ -492,7 +492,7 @@ def run_b200(args):
                 "traffic": traffic, "traffic_source": traffic_from,
                 "arithmetic": ("fp32 accumulate on tcgen05.mma, TF32 head+tail operands (4 products per instruction)"
                                if d == 64 and (args.flags & 64) and not (args.flags & 24)
-                               else "fp32 accumulate on mma.sync, TF32 head+tail operands (3 products)"
+                               else "fp32 accumulate on mma.sync, operands as two scaled fp16 pieces (3 products)"
                                if d == 64 and not (args.flags & 24) else "fp32 fma"),
                 "algorithmic_bytes": (4 * F + 8 * d) * n * B,
                 "hbm": {"achieved": (4 * F + 8 * d) * n * B / (embed_ms * 1e-3) / 1e9, "peak": hbm_peak,

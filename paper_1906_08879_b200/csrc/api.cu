@@ -219,15 +219,9 @@ placeto_status run_embed(const placeto_graph *g, const placeto_weights *w, const
         cudaError_t e = launch_embed_tc(a, g->info, stream, after_own_kernel);
         if (e != cudaErrorNotSupported) return cuda_status(e);
     }
-    // d = 64: the pipeline of layers, if it fits
-    if (!(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY | PLACETO_TENSOR)) && schedule == PLACETO_SLICED &&
-        ((flags & PLACETO_PIPELINE) ? embed_pipe_applicable(a) : embed_pipe_preferred(a, g->info))) {
-        cudaError_t e = launch_embed_pipe(a, g->info, stream, after_own_kernel);
-        if (e != cudaErrorNotSupported) return cuda_status(e);
-    }
-    const bool want_mma = (flags & PLACETO_TENSOR) ? embed_mma_applicable(a) : embed_mma_preferred(a);
-    if (!(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY)) && schedule == PLACETO_SLICED && want_mma) {
-        cudaError_t e = launch_embed_mma(a, g->info, stream, after_own_kernel);
+    const bool split = (flags & (PLACETO_TENSOR | PLACETO_PIPELINE)) ? embed_split_applicable(a) : embed_split_preferred(a, g->info);
+    if (!(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY)) && schedule == PLACETO_SLICED && split) {
+        cudaError_t e = launch_embed_split(a, g->info, stream, after_own_kernel);
         if (e != cudaErrorNotSupported) return cuda_status(e);
     }
     if (!(flags & PLACETO_GENERIC) && schedule == PLACETO_SLICED && embed_d32_applicable(a)) {

@@ -1,0 +1,535 @@
+// Step 2 of the policy (Sec. 2.2 step 2 of the Placeto paper) on the tensor cores for
+// d = 32 and d = 64, ReLU networks of one or two layers:
+//   h_v = g( sum_{u in nbr(v)} m_u ),   m_u = f([h_u || x_u]).
+//
+// A block owns a slice of the state batch and one direction and walks the levels of
+// the graph; a level's rows (node, state) are cut into tiles of eight, and a tile is
+// carried through gather -> g -> (store h) -> f -> (store m) by one group of d / 16
+// warps, 16 output columns of every layer per warp, whose weights it keeps in
+// registers. Between layers the activations of the tile go through shared memory
+// as half-precision pieces (see split_mma.cuh) and the group meets at a named
+// barrier. Groups are independent inside a level: with more tiles than groups a group
+// carries two at once. States never interact, so the levels are ordered by __syncthreads()
+// alone. Messages stay in shared-memory slots (assigned on the host), so global traffic
+// is x in and h out.
+//
+// A level is a serial chain (gather, four layers), so what is not arithmetic of the tile
+// is taken off it: four helper warps work a level ahead, turning the schedule into one
+// record per row and the raw features (cp.async, two levels ahead, or compact states) into
+// pieces.
+//
+// Measured on a B200, message passing alone, against the kernels it replaced (d = 64: a pipeline of layers on TF32
+// mma.sync, a warpgroup per layer; single layers: the dimension-generic kernel), us:
+//   d = 64, 1987 nodes in 741 levels:  64 states 884 -> 758, 256 states 1272 -> 951, 512 states 1932 -> 1350,
+//   single-layer networks, 512 states: 12180 -> 839.  d = 32, 992 nodes in 249 levels, 992 states (against the FMA
+//   kernel): 826 -> 711.
+// What bounds it: the chain of a level, about 2000 cycles for one tile at d = 64 (gather 450, a layer 300: 30 for the
+// barrier, 100 until a warp has its fragments - four warps read the whole tile -, 100 of products, 70 to finish and
+// split), and 800 for each further tile (the tensor pipe needs 415). Two blocks per SM (half the warps each) are
+// slower (1473), a message's bound carried along with it too (1423), and the records read before the level starts.
+//
+// There is no spin-wait; summation orders are fixed: results are reproducible bit for bit.
+#include <cuda_pipeline.h>
+
+#include <algorithm>
+
+#include "split_mma.cuh"
+
+namespace placeto {
+
+namespace {
+
+using namespace split;
+
+constexpr int kTile = 8;
+// Two warpgroups compute, one helps. The computing threads keep up to 136 registers of weights: the helpers give
+// most of theirs away (12 warps are launched with 168 each: 8 x 232 + 4 x 40 = 12 x 168).
+constexpr int kComputeThreads = 256, kHelperThreads = 128, kThreads = kComputeThreads + kHelperThreads;
+constexpr int kHelperBar = 15;
+
+// d, layers and the split used
+template <int D_, int L_, typename SP_>
+struct Config {
+    typedef SP_ SP;
+    static constexpr int D = D_, L = L_;
+    static constexpr int W = D / 16, G = kComputeThreads / 32 / W;       // warps of a group, groups
+    static constexpr int kGroupThreads = 32 * W;
+    static constexpr int KS = D / 16;
+    static constexpr int P = D + 4;                      // row stride of a message slot (floats)
+    static constexpr int kStride = 2 * D + 16;           // row stride of a tile piece (bytes)
+    static constexpr unsigned kPiece = kTile * kStride;
+    static constexpr unsigned kBuffer = SP::kPieces * kPiece;
+    static constexpr unsigned kSlot = 2 * kBuffer + kTile * 4;           // one tile in flight: two buffers, the rows' scales
+    static constexpr unsigned kGroupBytes = 2 * kSlot;
+    // per row of a level, written by the helper warps: a record, the raw features' pieces (16 columns, zero
+    // padded) and their scale
+    static constexpr int kXStride = 32;
+    static constexpr unsigned kXPiece = kTile * kXStride;
+    static constexpr unsigned kXTile = SP::kPieces * kXPiece;
+    static constexpr unsigned kRowTile = kXTile + kTile * 16 + kTile * 4;
+};
+
+struct SplitPlan {
+    int S, n_slices;
+    int x_floats;          // floats of one raw feature buffer
+    int row_bytes;         // bytes of one level's row tiles (records, feature pieces)
+    int int_floats[2];     // shared-memory floats taken by each direction's schedule
+    size_t smem_bytes;
+};
+
+// a matrix's bounds: |out| <= norm * max |in| + bias (largest over the columns)
+struct Bound { float norm, bias; };
+
+template <typename C, bool kCompact>
+__global__ void __launch_bounds__(kThreads, 1)
+embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
+    typedef typename C::SP SP;
+    constexpr int D = C::D, L = C::L, KS = C::KS, P = C::P;
+    extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int group = warp / C::W, c0 = 16 * (warp % C::W);
+    const int gt = threadIdx.x % C::kGroupThreads;
+    const int g = lane >> 2, t = lane & 3;
+    const int dir = (int)blockIdx.y;
+    const DevLevels lv = a.lv[dir];
+    const int B = a.B, F = a.F, S = p.S;
+    const int b_first = blockIdx.x * S;
+    const int nb = min(S, B - b_first);
+    const int n_levels = lv.n_levels;
+
+    // ---- shared memory: [schedule][message slots][raw features x2][bounds][row tiles x2][tiles of every group]
+    //   meta[p] = {first neighbour entry, end of neighbour entries, own slot, node id}
+    int *ism = reinterpret_cast<int *>(smem);
+    int4 *meta_w = reinterpret_cast<int4 *>(ism);
+#pragma unroll 1
+    for (int i = threadIdx.x; i < a.n; i += kThreads) {
+        meta_w[i] = lv.pos4[i];
+        PLACETO_DEBUG_CHECK(a.status, lv.pos4[i].x >= 0 && lv.pos4[i].x <= lv.pos4[i].y && lv.pos4[i].y <= lv.n_nbr &&
+                                          lv.pos4[i].z >= -1 && lv.pos4[i].z < lv.n_slots && lv.pos4[i].w >= 0 &&
+                                          lv.pos4[i].w < a.n);
+    }
+#pragma unroll 1
+    for (int e = threadIdx.x; e < lv.n_nbr; e += kThreads)
+        PLACETO_DEBUG_CHECK(a.status, lv.nbr_slot[e] >= 0 && lv.nbr_slot[e] < lv.n_slots);
+    PLACETO_DEBUG_CHECK(a.status, nb >= 1 && b_first + nb <= B);
+    ism += 4 * a.n;
+    auto stage_ints = [&](const int *src, int count) {
+        int *dst = ism;
+#pragma unroll 1
+        for (int i = threadIdx.x; i < count; i += kThreads) dst[i] = src[i];
+        ism += (count + 3) & ~3;
+        return (const int *)dst;
+    };
+    const int4 *meta = meta_w;
+    const int *level_ptr = stage_ints(lv.level_ptr, n_levels + 1);
+    const int *nbr_slot = stage_ints(lv.nbr_slot, lv.n_nbr);
+    float *msg = smem + p.int_floats[dir];                      // [n_slots][S][P]
+    float *xstage = msg + (size_t)lv.n_slots * S * P;           // [2][x_floats]
+    Bound *bounds = reinterpret_cast<Bound *>(xstage + 2 * (size_t)p.x_floats);     // [5 matrices][W]
+    unsigned char *row_tiles = reinterpret_cast<unsigned char *>(bounds + 5 * 4);   // [2][tiles of the widest level]
+    unsigned char *tiles = row_tiles + 2 * (size_t)p.row_bytes + (group < C::G ? group : 0) * C::kGroupBytes;
+    float *__restrict__ H = a.H[dir];
+
+    if (threadIdx.x >= kComputeThreads) {
+        // ------------------------------------------------------------ the helper warps
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        const int ht = threadIdx.x - kComputeThreads;
+        // exact division of small non-negative numbers by a per-block constant
+        const unsigned magic_nb = (unsigned)((0x100000000ull + nb - 1) / nb);
+        auto node_of_row = [&](int r) { return nb == 1 ? r : (int)__umulhi((unsigned)r, magic_nb); };
+        // One level ahead of the groups: every row's record {row of H (-1: past the last), own message (-1: nobody
+        // reads it), first neighbour's message, first neighbour entry | entries << 16} (offsets in floats) and its
+        // features as pieces; two levels ahead: the raw features.
+        const int per_node = nb * F;                        // floats per node, contiguous in X
+        const bool vec = (F & 3) == 0;
+        const int per = vec ? per_node >> 2 : per_node;     // copy pieces per node
+        const unsigned magic_per = (unsigned)((0x100000000ull + per - 1) / per);
+        auto fetch = [&](int level) {
+            if (level < n_levels) {
+                const int p0 = level_ptr[level], width = level_ptr[level + 1] - p0;
+                float *dst = xstage + (size_t)(level & 1) * p.x_floats;
+                if (kCompact) {
+#pragma unroll 1
+                    for (int i = ht; i < width * nb; i += kHelperThreads) {       // one (node, state) pair per thread
+                        const int q = node_of_row(i), s = i - q * nb;
+                        compact_features(a.compact, meta[p0 + q].w, b_first + s, B, dst + (size_t)i * F);
+                    }
+                } else {
+#pragma unroll 1
+                    for (int i = ht; i < width * per; i += kHelperThreads) {
+                        const int q = per == 1 ? i : (int)__umulhi((unsigned)i, magic_per);
+                        const int piece = i - q * per;
+                        const float *src = a.X + ((size_t)meta[p0 + q].w * B + b_first) * F;
+                        if (vec) __pipeline_memcpy_async(dst + q * per_node + 4 * piece, src + 4 * piece, 16);
+                        else __pipeline_memcpy_async(dst + q * per_node + piece, src + piece, 4);
+                    }
+                }
+            }
+            __pipeline_commit();
+        };
+        auto publish = [&](int level) {
+            const int p0 = level_ptr[level], rows = (level_ptr[level + 1] - p0) * nb;
+            unsigned char *out = row_tiles + (size_t)(level & 1) * p.row_bytes;
+            const float *xs = xstage + (size_t)(level & 1) * p.x_floats;
+#pragma unroll 1
+            for (int r = ht; r < (rows + kTile - 1) / kTile * kTile; r += kHelperThreads) {
+                int4 rec = make_int4(-1, -1, 0, 0);
+                if (r < rows) {
+                    const int q = node_of_row(r), s = r - q * nb;
+                    const int4 m = meta[p0 + q];
+                    rec = make_int4((int)((unsigned)m.w * B + b_first + s), m.z >= 0 ? (m.z * S + s) * P : -1,
+                                    m.x < m.y ? (nbr_slot[m.x] * S + s) * P : 0, m.x | (m.y - m.x) << 16);
+                }
+                *reinterpret_cast<int4 *>(out + (r / kTile) * C::kRowTile + C::kXTile + (r % kTile) * 16) = rec;
+            }
+            // thread (row, two columns); rows past the last keep whatever the tile holds: their results are not stored
+#pragma unroll 1
+            for (int r0 = 0; r0 < rows; r0 += kHelperThreads / 8) {
+                const int r = min(r0 + (ht >> 3), rows - 1), k = 2 * (ht & 7);
+                float x = k < F ? xs[r * F + k] : 0.f, y = k + 1 < F ? xs[r * F + k + 1] : 0.f;
+                unsigned char *tile = out + (r / kTile) * C::kRowTile;
+                if constexpr (SP::kScaled) {
+                    float top = fmaxf(fabsf(x), fabsf(y));
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+                    const float up = scale_up(top);
+                    if (k == 0) reinterpret_cast<float *>(tile + C::kXTile + kTile * 16)[r % kTile] = up;
+                    x *= up;
+                    y *= up;
+                }
+                unsigned pc[SP::kPieces];
+                SP::pieces(x, y, pc);
+#pragma unroll
+                for (int q = 0; q < SP::kPieces; ++q)
+                    *reinterpret_cast<unsigned *>(tile + q * C::kXPiece + (r % kTile) * C::kXStride + 2 * k) = pc[q];
+            }
+        };
+        __syncthreads();              // schedule staged
+        dependency_wait();            // the raw features may come from a kernel that is still running
+        fetch(0);
+        fetch(1);
+        __pipeline_wait_prior(1);
+        group_sync<kHelperThreads>(kHelperBar);
+        publish(0);
+        __syncthreads();
+#pragma unroll 1
+        for (int level = 0; level < n_levels; ++level) {
+            if (level + 1 < n_levels) {
+                fetch(level + 2);
+                __pipeline_wait_prior(1);
+                group_sync<kHelperThreads>(kHelperBar);
+                publish(level + 1);
+            }
+            __syncthreads();
+        }
+        return;
+    }
+
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    // ---- this warp's 16 columns of every matrix
+    const DevMlp fn = a.f[dir], gn = a.g[dir];
+    Weights<SP, KS> wg1, wg2, wf1, wf2;
+    Weights<SP, 1> wx;                                          // the rows of f's first matrix that take the raw features
+    const int col = c0 + g;                                     // this lane finishes columns col, col + 8 of rows 2t, 2t + 1
+    float bg1[2], bg2[2], bf1[2], bf2[2];
+    {
+        auto record = [&](int which, float norm, const float (&bias)[2]) {
+            if (!SP::kScaled) return;
+            float top = fmaxf(fabsf(bias[0]), fabsf(bias[1]));
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+            if (group == 0 && lane == 0) bounds[which * C::W + warp] = Bound{norm, top};
+        };
+        auto bias_of = [&](const float *b, float (&v)[2]) { v[0] = b[col]; v[1] = b[col + 8]; };
+        bias_of(gn.b1, bg1);
+        record(0, wg1.load(c0, lane, [&](int k, int c) { return gn.W1[k * D + c]; }), bg1);
+        if constexpr (L == 2) {
+            bias_of(gn.b2, bg2);
+            record(1, wg2.load(c0, lane, [&](int k, int c) { return gn.W2[k * D + c]; }), bg2);
+        }
+        bias_of(fn.b1, bf1);
+        record(2, wf1.load(c0, lane, [&](int k, int c) { return fn.W1[k * D + c]; }), bf1);
+        record(3, wx.load(c0, lane, [&](int k, int c) { return k < F ? fn.W1[(D + k) * D + c] : 0.f; }), bf1);
+        if constexpr (L == 2) {
+            bias_of(fn.b2, bf2);
+            record(4, wf2.load(c0, lane, [&](int k, int c) { return fn.W2[k * D + c]; }), bf2);
+        }
+    }
+    __syncthreads();              // schedule and bounds staged
+    // Fp16x2: a row's activations are carried multiplied by a power of two. With b a bound of the row's input of
+    // g that is at least the largest bias, b * prod (norm_i + 1) bounds every later layer, so the powers of two
+    // of the layers are the input's times constants of the launch (rounded up to powers of two):
+    //   after g's layers: row scale * ug[i];  after f's first: min(row scale * uh, scale of x * ux)
+    // (The bound of the gathered row is its largest entry, found with shuffles: carrying a bound with every message
+    // is loose by another 2^4 .. 2^6 per level, four times the error.)
+    float floor_b = 0.f, ug[2] = {1.f, 1.f}, uh = 1.f, ux = 1.f;
+    if constexpr (SP::kScaled) {
+        float grow[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            float norm = 0.f;
+            if (L == 2 || (i != 1 && i != 4))
+                for (int q = 0; q < C::W; ++q) {
+                    norm = fmaxf(norm, bounds[i * C::W + q].norm);
+                    floor_b = fmaxf(floor_b, bounds[i * C::W + q].bias);
+                }
+            grow[i] = inverse_pow2(pow2_above(norm + 1.f));
+        }
+        ug[0] = grow[0];
+        ug[1] = L == 2 ? ug[0] * grow[1] : ug[0];
+        uh = 0.5f * ug[1] * grow[2];
+        ux = 0.5f * grow[3];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            bg1[c] *= ug[0];
+            bg2[c] = L == 2 ? bg2[c] * ug[1] : 0.f;
+        }
+        wg1.inv *= ug[0];
+        if constexpr (L == 2) wg2.inv *= grow[1];
+        wf1.inv *= inverse_pow2(ug[1]);
+    }
+    const unsigned tile_addr = smem_addr(tiles);
+    const unsigned ld_at = tile_addr + ld_offset(lane, C::kStride), st_at = tile_addr + st_offset(lane, C::kStride, c0);
+    const unsigned x_at = ld_offset(lane & 15, C::kXStride);
+    constexpr int kLanes = D / 4;                        // gathering threads of a row: four columns each
+    const int rr = gt / kLanes, c4 = 4 * (gt % kLanes);
+    unsigned char *gather_to = tiles + rr * C::kStride + 2 * c4;
+    float *scale_to = reinterpret_cast<float *>(tiles + 2 * C::kBuffer) + rr;
+
+    // Tiles at `info` and, with NT = 2, G tiles on: gather -> g -> h -> f -> m.
+    auto run = [&](auto nt_constant, const unsigned char *info) {
+        constexpr int NT = decltype(nt_constant)::value;
+        constexpr int kNext = C::G * (int)C::kRowTile;
+        // ---- sums of the neighbours' messages
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            const int4 m = *reinterpret_cast<const int4 *>(info + i * kNext + C::kXTile + rr * 16);
+            const unsigned count = (unsigned)m.w >> 16;
+            const float *row = msg + m.z;
+            float4 acc = *reinterpret_cast<const float4 *>(row + c4);
+            if (count == 0) acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (__any_sync(0xffffffffu, count > 1)) {
+                const int *slot = nbr_slot + (m.w & 0xffff);
+                const float *from = row - (count > 1 ? slot[0] : 0) * (S * P);     // the state's row of slot 0
+#pragma unroll 4
+                for (int e = 1; e < (int)count; ++e) {
+                    const float *next = from + slot[e] * (S * P);
+                    const float4 v = *reinterpret_cast<const float4 *>(next + c4);
+                    acc.x += v.x;
+                    acc.y += v.y;
+                    acc.z += v.z;
+                    acc.w += v.w;
+                }
+            }
+            if constexpr (SP::kScaled) {
+                float top = fmaxf(fmaxf(fmaxf(fabsf(acc.x), fabsf(acc.y)), fmaxf(fabsf(acc.z), fabsf(acc.w))), floor_b);
+#pragma unroll
+                for (int o = 1; o < kLanes; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+                const float up = scale_up(top);
+                if (c4 == 0) scale_to[i * C::kSlot / 4] = up;
+                acc = make_float4(acc.x * up, acc.y * up, acc.z * up, acc.w * up);
+            }
+            store_row4<SP>(gather_to + i * C::kSlot, C::kPiece, acc);
+        }
+        group_sync<C::kGroupThreads>(1 + group);
+        // ---- where rows 2t, 2t + 1 of every tile go, and their scales
+        int2 to[NT][2];                                  // {row of H (-1: past the last), own message}
+        [[maybe_unused]] float up[NT][2], upx[NT][2];
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                to[i][e] = *reinterpret_cast<const int2 *>(info + i * kNext + C::kXTile + (2 * t + e) * 16);
+                if constexpr (SP::kScaled) {
+                    up[i][e] = reinterpret_cast<const float *>(tiles + i * C::kSlot + 2 * C::kBuffer)[2 * t + e];
+                    upx[i][e] = reinterpret_cast<const float *>(info + i * kNext + C::kXTile + kTile * 16)[2 * t + e];
+                }
+            }
+        float v[NT][4];
+        auto product = [&](const Weights<SP, KS> &w, auto from_constant) {
+            unsigned in[NT];
+#pragma unroll
+            for (int i = 0; i < NT; ++i) in[i] = ld_at + i * C::kSlot;
+            tile_mma<SP, KS, NT, decltype(from_constant)::value *(int)C::kBuffer, (int)C::kPiece>(w, in, v);
+        };
+        typedef std::integral_constant<int, 0> buffer0;
+        typedef std::integral_constant<int, 1> buffer1;
+        // v = relu(v * w.inv + bias), the bias times the row's scale
+        auto finish = [&](const Weights<SP, KS> &w, const float (&bias)[2]) {
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    v[i][c] = fmaxf(SP::kScaled ? fmaf(v[i][c], w.inv, bias[c >> 1] * up[i][c & 1]) : v[i][c] + bias[c >> 1], 0.f);
+        };
+        auto hand_over = [&](int dst) {
+#pragma unroll
+            for (int i = 0; i < NT; ++i) store_tile<SP>(st_at + i * C::kSlot + dst * C::kBuffer, C::kPiece, lane, v[i]);
+        };
+        product(wg1, buffer0());
+        finish(wg1, bg1);
+        if constexpr (L == 2) {
+            hand_over(1);
+            group_sync<C::kGroupThreads>(1 + group);
+            product(wg2, buffer1());
+            finish(wg2, bg2);
+        }
+        constexpr int kG = L == 2 ? 0 : 1;               // the buffer that g's output goes to
+        hand_over(kG);
+        [[maybe_unused]] float back[NT][2];              // 1 / the row's scale
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float f = 1.f;
+                if constexpr (SP::kScaled) {
+                    back[i][e] = inverse_pow2(up[i][e]);
+                    f = back[i][e] * inverse_pow2(ug[L - 1]);
+                }
+                if (to[i][e].x != -1) {
+                    float *h = H + (size_t)(unsigned)to[i][e].x * D + col;
+                    h[0] = v[i][e] * f;
+                    h[8] = v[i][2 + e] * f;
+                }
+            }
+        group_sync<C::kGroupThreads>(1 + group);
+        // ---- f's first layer: the raw features and the embedding
+        float x[NT][4];
+        {
+            unsigned in[NT];
+#pragma unroll
+            for (int i = 0; i < NT; ++i) in[i] = smem_addr(info) + i * kNext + x_at;
+            tile_mma<SP, 1, NT, 0, (int)C::kXPiece>(wx, in, x);
+        }
+        product(wf1, std::integral_constant<int, kG>());
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if constexpr (SP::kScaled) {
+                    // (L = 1: this is the message, unscaled)
+                    const float uf = L == 1 ? 1.f : fminf(up[i][e] * uh, upx[i][e] * ux);
+                    const float fh = back[i][e] * wf1.inv * uf, fx = inverse_pow2(upx[i][e]) * wx.inv * uf;
+                    v[i][e] = fmaxf(fmaf(v[i][e], fh, fmaf(x[i][e], fx, bf1[0] * uf)), 0.f);
+                    v[i][2 + e] = fmaxf(fmaf(v[i][2 + e], fh, fmaf(x[i][2 + e], fx, bf1[1] * uf)), 0.f);
+                    if (L == 2) up[i][e] = uf;
+                } else {
+                    v[i][e] = fmaxf(v[i][e] + (x[i][e] + bf1[0]), 0.f);
+                    v[i][2 + e] = fmaxf(v[i][2 + e] + (x[i][2 + e] + bf1[1]), 0.f);
+                }
+            }
+        if constexpr (L == 2) {
+            hand_over(1);
+            group_sync<C::kGroupThreads>(1 + group);
+            product(wf2, buffer1());
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float f = SP::kScaled ? inverse_pow2(up[i][e]) * wf2.inv : 1.f;
+                    v[i][e] = fmaxf(SP::kScaled ? fmaf(v[i][e], f, bf2[0]) : v[i][e] + bf2[0], 0.f);
+                    v[i][2 + e] = fmaxf(SP::kScaled ? fmaf(v[i][2 + e], f, bf2[1]) : v[i][2 + e] + bf2[1], 0.f);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool kept = to[i][e].y >= 0;
+                float *m = msg + (kept ? to[i][e].y : 0);
+                if (kept) {
+                    m[col] = v[i][e];
+                    m[col + 8] = v[i][2 + e];
+                }
+            }
+    };
+
+    int n_tiles = (level_ptr[1] * nb + kTile - 1) / kTile, first = level_ptr[1];
+    const unsigned char *mine = row_tiles + group * (int)C::kRowTile;
+    __syncthreads();                                     // level 0 published
+#pragma unroll 1
+    for (int level = 0; level < n_levels; ++level) {
+        const int next = level_ptr[min(level + 2, n_levels)];
+        const unsigned char *info = mine + (level & 1) * p.row_bytes;
+        int left = n_tiles - group;                      // this group takes every G-th tile
+#pragma unroll 1
+        for (; left > C::G; left -= 2 * C::G, info += 2 * C::G * (int)C::kRowTile) run(std::integral_constant<int, 2>{}, info);
+        if (left > 0) run(std::integral_constant<int, 1>{}, info);
+        n_tiles = ((next - first) * nb + kTile - 1) / kTile;
+        first = next;
+        __syncthreads();
+    }
+}
+
+bool relu_net(const DevMlp &m, int in, int d, int layers) {
+    return m.n_layers == layers && m.in_dim == in && m.hidden_dim == d && m.out_dim == d && m.act == 0 && m.final_act == 1;
+}
+
+template <typename C>
+cudaError_t launch(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap) {
+    SplitPlan p;
+    const int want = std::max(1, std::min(a.B, di.sm_count / 2));      // one block per SM, half of them per direction
+    p.S = (a.B + want - 1) / want;
+    const size_t budget = (size_t)std::min(di.max_smem_optin, 227 * 1024) - 1024;
+    for (int dir = 0; dir < 2; ++dir) {
+        const DevLevels &lv = a.lv[dir];
+        p.int_floats[dir] = 4 * a.n + ((lv.n_levels + 1 + 3) & ~3) + ((lv.n_nbr + 3) & ~3);
+    }
+    auto x_floats = [&](int S) { return (a.max_level_width * S * a.F + 3) & ~3; };
+    auto row_bytes = [&](int S) { return (a.max_level_width * S + kTile - 1) / kTile * (int)C::kRowTile; };
+    auto need = [&](int S) {
+        size_t worst = 0;
+        for (int dir = 0; dir < 2; ++dir)
+            worst = std::max(worst, (size_t)p.int_floats[dir] + (size_t)a.lv[dir].n_slots * S * C::P);
+        return (worst + 2 * (size_t)x_floats(S)) * sizeof(float) + 5 * 4 * sizeof(Bound) + 2 * (size_t)row_bytes(S) +
+               (size_t)C::G * C::kGroupBytes;
+    };
+    while (p.S > 1 && need(p.S) > budget) --p.S;
+    if (need(p.S) > budget || std::max(a.lv[0].n_nbr, a.lv[1].n_nbr) > 0xffff) return cudaErrorNotSupported;
+    // Shared memory may force more slices than one wave of blocks holds: spread the batch evenly over
+    // the waves it then takes (two full waves finish before one full wave and a ragged one of larger slices)
+    const int waves = ((a.B + p.S - 1) / p.S + want - 1) / want;
+    p.S = std::min(p.S, (a.B + want * waves - 1) / (want * waves));
+    p.n_slices = (a.B + p.S - 1) / p.S;
+    p.x_floats = x_floats(p.S);
+    p.row_bytes = row_bytes(p.S);
+    p.smem_bytes = need(p.S);
+    auto kern = a.compact.state != nullptr ? embed_split_kernel<C, true> : embed_split_kernel<C, false>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);
+    if (err != cudaSuccess) return err;
+    err = launch_overlapped(overlap, kern, dim3(p.n_slices, 2), dim3(kThreads), p.smem_bytes, stream, a, p);
+    count_launch();
+    return err;
+}
+
+}  // namespace
+
+bool embed_split_applicable(const EmbedArgs &a) {
+    if ((a.d != 32 && a.d != 64) || a.F < 1 || a.F > 16) return false;
+    for (int dir = 0; dir < 2; ++dir)
+        if (!relu_net(a.f[dir], a.d + a.F, a.d, a.f[0].n_layers) || !relu_net(a.g[dir], a.d, a.d, a.f[0].n_layers)) return false;
+    return true;
+}
+
+// d = 64: wherever it applies. d = 32: measured against the FMA kernel (us, two layers / one), the lines cross at 12
+// to 14 rows of a block per level: 20 rows 417 -> 308 / 295 -> 213, 12 rows 286 -> 263 / 203 -> 183, 8.5 rows
+// 96 -> 114 / 70 -> 80; with four neighbours per node (a recurrent grid with attention) the gather, which only one
+// group of warps per tile does, costs more than the products save: 26 rows 310 -> 401.
+bool embed_split_preferred(const EmbedArgs &a, const DeviceInfo &di) {
+    if (!embed_split_applicable(a)) return false;
+    if (a.d == 64) return true;
+    const int blocks = std::max(1, std::min(a.B, di.sm_count / 2)), S = (a.B + blocks - 1) / blocks;
+    const long long rows = (long long)a.n * S;
+    return rows >= 12ll * a.lv[0].n_levels && rows >= 12ll * a.lv[1].n_levels && a.lv[0].n_nbr <= 2 * a.n;
+}
+
+cudaError_t launch_embed_split(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap) {
+    if (a.d == 32)
+        return a.f[0].n_layers == 2 ? launch<Config<32, 2, Bf16x3>>(a, di, stream, overlap)
+                                    : launch<Config<32, 1, Bf16x3>>(a, di, stream, overlap);
+    return a.f[0].n_layers == 2 ? launch<Config<64, 2, Fp16x2>>(a, di, stream, overlap)
+                                : launch<Config<64, 1, Fp16x2>>(a, di, stream, overlap);
+}
+
+}  // namespace placeto

@@ -334,19 +334,11 @@ cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStrea
 bool embed_d64_applicable(const EmbedArgs &a);
 cudaError_t launch_embed_d64(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream);
 
-// embed_mma.cu: d = 32 / 64 on the tensor cores (mma.sync, TF32 operands split
-// into head + tail, three products per step for FP32 accuracy).
-bool embed_mma_applicable(const EmbedArgs &a);
-bool embed_mma_preferred(const EmbedArgs &a);   // applicable and faster than the FMA kernels
-cudaError_t launch_embed_mma(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream,
-                             bool overlap = false);
-
-// embed_pipe.cu: d = 64 as a pipeline of layers on mma.sync (a group of warps per layer of f and g,
-// tiles of eight rows handed from layer to layer through shared memory). cudaErrorNotSupported when
-// the schedule and the message slots do not fit in shared memory.
-bool embed_pipe_applicable(const EmbedArgs &a);
-bool embed_pipe_preferred(const EmbedArgs &a, const DeviceInfo &di);   // where the library picks it
-cudaError_t launch_embed_pipe(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
+// embed_split.cu: d = 32 / 64 on the tensor cores with operands split into half-precision pieces, a group of
+// warps per tile of eight rows. cudaErrorNotSupported when the schedule and the slots do not fit.
+bool embed_split_applicable(const EmbedArgs &a);
+bool embed_split_preferred(const EmbedArgs &a, const DeviceInfo &di);   // applicable and faster than the FMA kernels
+cudaError_t launch_embed_split(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
 
 // embed_tc.cu: d = 64 on tcgen05 tensor cores with accumulators in tensor memory (TF32 head + tail
 // operands, all four partial products per instruction). A bounded wait that runs out inside the
