@@ -167,7 +167,9 @@ typedef struct {
 #define PLACETO_TCGEN05 64u    /* d = 64: take the kernel built on tcgen05.mma with accumulators in tensor
                                   memory instead of the warp-level (mma.sync) tensor-core kernel that is
                                   the default there (measured slower at the configured batch sizes) */
-#define PLACETO_PIPELINE 128u  /* another name of PLACETO_TENSOR */
+#define PLACETO_PIPELINE 128u  /* d = 64, two layers: take the kernel that runs the four layers of g and f as a
+                                  pipeline on TF32 operands (a group of warps per layer, tiles of eight rows).
+                                  It is what placeto_embed_forward picks there anyway; the flag pins the choice. */
 
 typedef enum {
     PLACETO_CALL_EMBED = 0,       /* placeto_embed_forward */

@@ -198,7 +198,7 @@ placeto_status cuda_status(cudaError_t e) {
 placeto_status run_embed(const placeto_graph *g, const placeto_weights *w, const float *X, int B,
                          float *H_down, float *H_up, char *ws, const Layout &L, uint32_t flags,
                          cudaStream_t stream, const StatusSlot &status, bool after_own_kernel = false,
-                         const CompactState *compact = nullptr) {
+                         const CompactState *compact = nullptr, bool embeddings_returned = false) {
     EmbedArgs a;
     a.status = status;
     a.compact = compact ? *compact : CompactState{};
@@ -219,8 +219,19 @@ placeto_status run_embed(const placeto_graph *g, const placeto_weights *w, const
         cudaError_t e = launch_embed_tc(a, g->info, stream, after_own_kernel);
         if (e != cudaErrorNotSupported) return cuda_status(e);
     }
-    const bool split = (flags & (PLACETO_TENSOR | PLACETO_PIPELINE)) ? embed_split_applicable(a) : embed_split_preferred(a, g->info);
-    if (!(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY)) && schedule == PLACETO_SLICED && split) {
+    // The embeddings of placeto_embed_forward go to the caller and from there to the policy gradient, whose ReLU masks
+    // are the signs of what is computed: a last bit that changes flips a mask now and then, and at d = 64 one flip moves a
+    // weight gradient by up to 4e-4 of its norm (100 states of a 531-node graph, as much as a gradient differs from
+    // FP64 for the same reason). So that call keeps the kernels whose bits users have (for two layers: the FMA kernel at
+    // d = 32, the TF32 pipeline at d = 64: 303 us there, 260 on the split kernel), and the calls that keep H to
+    // themselves take the fastest.
+    const bool tensor = !(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY)) && schedule == PLACETO_SLICED;
+    if (tensor && ((flags & PLACETO_PIPELINE) || (embeddings_returned && !(flags & PLACETO_TENSOR))) && embed_pipe_applicable(a)) {
+        cudaError_t e = launch_embed_pipe(a, g->info, stream, after_own_kernel);
+        if (e != cudaErrorNotSupported) return cuda_status(e);
+    }
+    const bool keep = embeddings_returned && a.d == 32;
+    if (tensor && ((flags & PLACETO_TENSOR) ? embed_split_applicable(a) : !keep && embed_split_preferred(a, g->info))) {
         cudaError_t e = launch_embed_split(a, g->info, stream, after_own_kernel);
         if (e != cudaErrorNotSupported) return cuda_status(e);
     }
@@ -542,7 +553,7 @@ placeto_status placeto_embed_forward(const placeto_graph *g, const placeto_weigh
         return PLACETO_ERR_INVALID_ARG;
     char *ws = static_cast<char *>(workspace);
     return run_embed(g, w, X, B, H_down, H_up, ws, L, flags, static_cast<cudaStream_t>(stream),
-                     new_status_slot(g, ws, L));
+                     new_status_slot(g, ws, L), false, nullptr, true);
 }
 
 placeto_status placeto_policy_logits(const placeto_graph *g, const placeto_weights *w,

@@ -340,6 +340,11 @@ bool embed_split_applicable(const EmbedArgs &a);
 bool embed_split_preferred(const EmbedArgs &a, const DeviceInfo &di);   // applicable and faster than the FMA kernels
 cudaError_t launch_embed_split(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
 
+// embed_pipe.cu: d = 64, two layers, as a pipeline of layers on mma.sync (TF32 head + tail operands, a group of warps
+// per layer of f and g). cudaErrorNotSupported when the schedule and the message slots do not fit in shared memory.
+bool embed_pipe_applicable(const EmbedArgs &a);
+cudaError_t launch_embed_pipe(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
+
 // embed_tc.cu: d = 64 on tcgen05 tensor cores with accumulators in tensor memory (TF32 head + tail
 // operands, all four partial products per instruction). A bounded wait that runs out inside the
 // kernel is reported through a.status as PLACETO_ERR_TIMEOUT.

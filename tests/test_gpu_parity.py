@@ -341,6 +341,25 @@ def test_single_layer_networks_at_the_specialised_widths(d, m, B):
     _small_case(45, src, dst, d=d, m=m, B=B, layers=1, seed=B + d)
 
 
+@pytest.mark.parametrize("d,m,B,layers", [(64, 8, 1, 2), (64, 3, 90, 2), (64, 8, 600, 2), (64, 5, 300, 1), (32, 4, 1, 2), (32, 8, 1500, 2),
+                                          (32, 3, 900, 1)])
+def test_split_sweep_kernel_over_tiles(d, m, B, layers):
+    """The split tensor-core kernel (whole path, and pinned by the flag): levels of one partial tile, of one tile per
+    group, of more tiles than groups (a group carries two at once); nodes of many neighbours; feature rows that are
+    and are not 16-byte aligned."""
+    r = rng(B + d)
+    src, dst = random_dag(r, 37, 0.15)
+    _small_case(37, src, dst, d=d, m=m, B=B, layers=layers, seed=B + m, schedule=placeto.PLACETO_TENSOR)
+    cfg = {"n": 37, "src": src, "dst": dst, "m": m, "d": d, "F": m + 4}
+    cfg["cost"], cfg["bytes"] = states.node_costs(r, 37, normalise=True)
+    cfg["dev"], cfg["cur"], cfg["placed"] = states.random_states(r, 37, m, B)
+    cfg["weights"] = states.policy_weights(r, d, m + 4, m, layers, 0, 0.1)
+    g, w = placeto.Graph(37, src, dst), placeto.Weights(cfg["weights"])
+    logits, _ = placeto.placeto_policy_forward(g, w, *(dev_t(cfg[k]) for k in ("cost", "bytes", "dev", "cur", "placed")))
+    torch.cuda.synchronize()
+    assert_close(logits, oracle.forward(cfg)["logits"], "logits")
+
+
 def test_identity_activation_and_path_counting():
     one = net([[1.0], [1.0]], [0.0], act=1)
     idn = net([[1.0]], [0.0], act=1)
