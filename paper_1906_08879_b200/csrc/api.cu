@@ -916,6 +916,7 @@ placeto_status placeto_policy_gradient(const placeto_graph *g, const placeto_wei
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     a.n = g->host.n; a.B = B; a.d = w->d; a.F = w->F; a.m = w->m;
     a.relation = g->d_relation;
+    a.max_level_width = g->host.max_level_width;
     a.lv[0] = g->lv[0]; a.lv[1] = g->lv[1];
     a.child_ptr = g->d_child_ptr; a.child = g->d_child;
     a.parent_ptr = g->d_parent_ptr; a.parent = g->d_parent;

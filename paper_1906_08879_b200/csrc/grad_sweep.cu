@@ -1,0 +1,550 @@
+// The policy gradient's passes over the node-state rows for d = 32 and d = 64 with two-layer f and g
+// of hidden width d (a single layer widened by an identity layer counts as two): what every
+// row's forward values are, and the reverse of the two message-passing sweeps.
+//
+//   row kernels : all rows are independent. The first recomputes f's hidden layer and message from
+//                 H and X, the second the sum of a node's messages and g's hidden layer; both also
+//                 leave one bit per ReLU (positive or not) for the sweep.
+//   sweep kernel: the reverse of the top-down pass walks the bottom-up levels (a node after all its
+//                 consumers) and the other way round, so it is the forward sweep with transposed
+//                 matrices: gather ds of the consumers -> mask m -> W_f2^T -> mask f hidden -> W_f1^T,
+//                 + d/dh -> mask h -> W_g2^T -> mask g hidden -> W_g1^T -> ds. It runs on the tensor
+//                 cores as embed_split.cu does: a tile of eight rows per group of d / 16 warps, bf16
+//                 pieces (exact, six products: gradients need the exponent range of FP32), ds in the
+//                 shared-memory slots of the schedule, helper warps for records and masks.
+// Measured on a B200, us, against the dimension-generic kernels of gradient.cu (which serve every other shape and did
+// all of this in the sweep, one phase after another in shared memory): 279 nodes, 132 levels, d = 32, 256 states:
+// sweep 966 -> 133, rows 120 -> 104; 531 nodes, 235 levels, d = 64, 100 states: sweep 2216 -> 330, rows 294 -> 164. The
+// sweep is bound by the chain of a level (2000 cycles at d = 32, as the forward kernel), the row kernels by their
+// shared-memory loads (one per four FMAs).
+#include <cuda_pipeline.h>
+
+#include <algorithm>
+
+#include "split_mma.cuh"
+
+namespace placeto {
+
+namespace {
+
+using namespace split;
+
+// ------------------------------------------------------------------ row kernels
+constexpr int kRowWarps = 8, kRowThreads = 32 * kRowWarps;
+constexpr int kRowsPerWarp = 8;
+
+// acc[r][c] += in[r][0 .. K) . W[.][lane + 32 c], k ascending: W [K][D] and the rows in shared memory. K a multiple
+// of 4 (zero padded). A weight load serves eight rows, a row's broadcast load four weights.
+template <int D>
+__device__ __forceinline__ void row_products(const float *W, const float *in, int stride, int K, int lane,
+                                             float (&acc)[kRowsPerWarp][D / 32]) {
+    constexpr int C = D / 32;
+    for (int k = 0; k < K; k += 4) {
+        float w[4][C];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < C; ++c) w[q][c] = W[(k + q) * D + lane + 32 * c];
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            const float4 x = *reinterpret_cast<const float4 *>(in + r * stride + k);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                acc[r][c] = fmaf(x.x, w[0][c], acc[r][c]);
+                acc[r][c] = fmaf(x.y, w[1][c], acc[r][c]);
+                acc[r][c] = fmaf(x.z, w[2][c], acc[r][c]);
+                acc[r][c] = fmaf(x.w, w[3][c], acc[r][c]);
+            }
+        }
+    }
+}
+
+// masks [row][4][D / 32]: bit j % 32 of word j / 32 is set where m, f's hidden layer, h, g's hidden layer is positive
+enum { kMaskM, kMaskF, kMaskH, kMaskG };
+
+template <int D>
+__global__ void __launch_bounds__(kRowThreads)
+grad_rows_f_kernel(const GradArgs a) {
+    constexpr int C = D / 32;
+    extern __shared__ __align__(16) float smem[];
+    const int dir = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const DevMlp f = a.f[dir];
+    const int F = a.F, K = (D + F + 3) & ~3;
+    float *W1 = smem, *W2 = W1 + K * D;                  // [K][D] zero padded, [D][D]
+    float *in = W2 + D * D + warp * kRowsPerWarp * (K + D), *hid = in + kRowsPerWarp * K;
+    for (int i = threadIdx.x; i < K * D; i += kRowThreads) W1[i] = i < (D + F) * D ? f.W1[i] : 0.f;
+    for (int i = threadIdx.x; i < D * D; i += kRowThreads) W2[i] = f.W2[i];
+    __syncthreads();
+    float b1[C], b2[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) { b1[c] = f.b1[lane + 32 * c]; b2[c] = f.b2[lane + 32 * c]; }
+    const float *H = a.H[dir];
+    unsigned *masks = a.masks[dir];
+    const size_t R = (size_t)a.n * a.B;
+    const size_t step = (size_t)gridDim.x * kRowWarps * kRowsPerWarp;
+    for (size_t r0 = ((size_t)blockIdx.x * kRowWarps + warp) * kRowsPerWarp; r0 < R; r0 += step) {
+        const int rows = (int)min((size_t)kRowsPerWarp, R - r0);
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            const size_t row = r0 + min(r, rows - 1);    // rows past the last repeat it
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const float h = H[row * D + lane + 32 * c];
+                in[r * K + lane + 32 * c] = h;
+                const unsigned bits = __ballot_sync(0xffffffffu, h > 0.f);
+                if (lane == 0 && r < rows) masks[(row * 4 + kMaskH) * C + c] = bits;
+            }
+            if (lane < K - D) in[r * K + D + lane] = lane < F ? a.X[row * F + lane] : 0.f;
+        }
+        __syncwarp();
+        float acc[kRowsPerWarp][C];
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[r][c] = b1[c];
+        row_products<D>(W1, in, K, K, lane, acc);
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const float v = fmaxf(acc[r][c], 0.f);
+                hid[r * D + lane + 32 * c] = v;
+                const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
+                if (r < rows) {
+                    a.FH[dir][(r0 + r) * D + lane + 32 * c] = v;
+                    if (lane == 0) masks[((r0 + r) * 4 + kMaskF) * C + c] = bits;
+                }
+                acc[r][c] = b2[c];
+            }
+        __syncwarp();
+        row_products<D>(W2, hid, D, D, lane, acc);
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const float v = fmaxf(acc[r][c], 0.f);
+                const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
+                if (r < rows) {
+                    a.M[dir][(r0 + r) * D + lane + 32 * c] = v;
+                    if (lane == 0) masks[((r0 + r) * 4 + kMaskM) * C + c] = bits;
+                }
+            }
+    }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kRowThreads)
+grad_rows_g_kernel(const GradArgs a) {
+    constexpr int C = D / 32;
+    extern __shared__ __align__(16) float smem[];
+    const int dir = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const DevMlp gn = a.g[dir];
+    float *W1 = smem, *in = W1 + D * D + warp * kRowsPerWarp * D;
+    for (int i = threadIdx.x; i < D * D; i += kRowThreads) W1[i] = gn.W1[i];
+    __syncthreads();
+    float b1[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) b1[c] = gn.b1[lane + 32 * c];
+    const int *nbr_ptr = dir == 0 ? a.parent_ptr : a.child_ptr, *nbr = dir == 0 ? a.parent : a.child;
+    const float *M = a.M[dir];
+    const int B = a.B;
+    const size_t R = (size_t)a.n * B;
+    const size_t step = (size_t)gridDim.x * kRowWarps * kRowsPerWarp;
+    for (size_t r0 = ((size_t)blockIdx.x * kRowWarps + warp) * kRowsPerWarp; r0 < R; r0 += step) {
+        const int rows = (int)min((size_t)kRowsPerWarp, R - r0);
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            const size_t row = r0 + min(r, rows - 1);
+            const int u = (int)(row / B), b = (int)(row - (size_t)u * B);
+            float s[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) s[c] = 0.f;
+            for (int e = nbr_ptr[u]; e < nbr_ptr[u + 1]; ++e)
+#pragma unroll
+                for (int c = 0; c < C; ++c) s[c] += M[((size_t)nbr[e] * B + b) * D + lane + 32 * c];
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                in[r * D + lane + 32 * c] = s[c];
+                if (r < rows) a.Sg[dir][row * D + lane + 32 * c] = s[c];
+            }
+        }
+        __syncwarp();
+        float acc[kRowsPerWarp][C];
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[r][c] = 0.f;
+        row_products<D>(W1, in, D, D, lane, acc);
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const float v = fmaxf(acc[r][c] + b1[c], 0.f);
+                const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
+                if (r < rows) {
+                    a.T1[dir][(r0 + r) * D + lane + 32 * c] = v;
+                    if (lane == 0) a.masks[dir][((r0 + r) * 4 + kMaskG) * C + c] = bits;
+                }
+            }
+    }
+}
+
+// ------------------------------------------------------------------ reverse sweep
+constexpr int kTile = 8;
+constexpr int kComputeThreads = 256, kHelperThreads = 128, kThreads = kComputeThreads + kHelperThreads;
+
+template <int D_>
+struct SweepConfig {
+    static constexpr int D = D_, W = D / 16, G = kComputeThreads / 32 / W, KS = D / 16;
+    static constexpr int kGroupThreads = 32 * W;
+    static constexpr int P = D + 4;                      // row stride of a slot (floats)
+    static constexpr int kStride = 2 * D + 16;           // row stride of a tile piece (bytes)
+    static constexpr unsigned kPiece = kTile * kStride, kBuffer = 3 * kPiece;
+    static constexpr unsigned kGroupBytes = 2 * kBuffer;
+    static constexpr int kMaskBytes = 4 * D / 8;         // a row's masks
+    static constexpr unsigned kRowTile = kTile * (16 + kMaskBytes);      // records, then masks
+    static constexpr unsigned kTailBytes = 4 * W * KS * 32 * 16;         // third pieces of the four matrices
+};
+
+struct SweepPlan {
+    int S, n_slices;
+    int row_bytes;
+    int int_floats[2];
+    size_t smem_bytes;
+};
+
+// One warp's 16 output columns of a D x D matrix: two pieces in registers, the third in shared memory (`tail`:
+// [k-step][lane], 16 bytes each), where it is read once per product.
+template <int KS>
+struct WeightsTail {
+    unsigned a[2][KS][4];
+    template <typename At>
+    __device__ __forceinline__ void load(int c0, int lane, bool store, uint4 *tail, At at) {
+        const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+            unsigned l[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int k = 16 * ks + 2 * t + 8 * (i >> 1), c = c0 + g + 8 * (i & 1);
+                unsigned p[3];
+                Bf16x3::pieces(at(k, c), at(k + 1, c), p);
+                a[0][ks][i] = p[0];
+                a[1][ks][i] = p[1];
+                l[i] = p[2];
+            }
+            if (store) tail[ks * 32 + lane] = make_uint4(l[0], l[1], l[2], l[3]);
+        }
+    }
+};
+// out = the tile's product with this warp's columns: six products of bf16 pieces per k-step in three chains
+template <int KS, int OFF, int PIECE>
+__device__ __forceinline__ void tail_mma(const WeightsTail<KS> &w, const uint4 *tail, unsigned tile, int lane, float (&out)[4]) {
+    float A[4], Bc[4], C[4];
+#pragma unroll
+    for (int kp = 0; kp < KS / 2; ++kp) {
+        unsigned b[3][4];
+        if (kp == 0) {
+            ldmatrix4<OFF>(b[0], tile);
+            ldmatrix4<OFF + PIECE>(b[1], tile);
+            ldmatrix4<OFF + 2 * PIECE>(b[2], tile);
+        } else {
+            ldmatrix4<OFF + 64>(b[0], tile);
+            ldmatrix4<OFF + PIECE + 64>(b[1], tile);
+            ldmatrix4<OFF + 2 * PIECE + 64>(b[2], tile);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int ks = 2 * kp + j;
+            const uint4 l4 = tail[ks * 32 + lane];
+            const unsigned l[4] = {l4.x, l4.y, l4.z, l4.w};
+            const unsigned b0[2] = {b[0][2 * j], b[0][2 * j + 1]}, b1[2] = {b[1][2 * j], b[1][2 * j + 1]},
+                           b2[2] = {b[2][2 * j], b[2][2 * j + 1]};
+            auto step = [&](auto first) {
+                constexpr bool z = decltype(first)::value;
+                chain<Bf16x3, z>(A, w.a[0][ks], b0);
+                chain<Bf16x3, z>(Bc, w.a[0][ks], b1);
+                chain<Bf16x3, z>(C, w.a[0][ks], b2);
+                chain<Bf16x3, false>(Bc, w.a[1][ks], b0);
+                chain<Bf16x3, false>(C, w.a[1][ks], b1);
+                chain<Bf16x3, false>(C, l, b0);
+            };
+            if (ks == 0) step(std::true_type());
+            else step(std::false_type());
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) out[c] = A[c] + (Bc[c] + C[c]);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1)
+grad_sweep_split_kernel(const GradArgs a, const SweepPlan p) {
+    typedef SweepConfig<D> C;
+    constexpr int KS = C::KS, P = C::P;
+    extern __shared__ __align__(16) float smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int group = warp / C::W, c0 = 16 * (warp % C::W);
+    const int gt = threadIdx.x % C::kGroupThreads;
+    const int g = lane >> 2, t = lane & 3;
+    const int dir = (int)blockIdx.y;
+    const DevLevels lv = a.lv[1 - dir];                  // consumers of a node come before it
+    const int B = a.B, S = p.S;
+    const int b_first = blockIdx.x * S;
+    const int nb = min(S, B - b_first);
+    const int n_levels = lv.n_levels;
+
+    // ---- shared memory: [schedule][ds slots][third weight pieces][row tiles x3][tiles of every group]
+    int *ism = reinterpret_cast<int *>(smem);
+    int4 *meta_w = reinterpret_cast<int4 *>(ism);
+#pragma unroll 1
+    for (int i = threadIdx.x; i < a.n; i += kThreads) meta_w[i] = lv.pos4[i];
+    ism += 4 * a.n;
+    auto stage_ints = [&](const int *src, int count) {
+        int *dst = ism;
+#pragma unroll 1
+        for (int i = threadIdx.x; i < count; i += kThreads) dst[i] = src[i];
+        ism += (count + 3) & ~3;
+        return (const int *)dst;
+    };
+    const int4 *meta = meta_w;
+    const int *level_ptr = stage_ints(lv.level_ptr, n_levels + 1);
+    const int *nbr_slot = stage_ints(lv.nbr_slot, lv.n_nbr);
+    float *msg = smem + p.int_floats[dir];                      // [n_slots][S][P]
+    uint4 *tails = reinterpret_cast<uint4 *>(msg + (size_t)lv.n_slots * S * P);
+    unsigned char *row_tiles = reinterpret_cast<unsigned char *>(tails) + C::kTailBytes;
+    unsigned char *tiles = row_tiles + 3 * (size_t)p.row_bytes + (group < C::G ? group : 0) * C::kGroupBytes;
+
+    if (threadIdx.x >= kComputeThreads) {
+        // ------------------------------------------------------------ the helper warps, two levels ahead: every row's
+        // record {row (-1: past the last), own slot (-1: nobody reads it), first consumer's ds, first entry | entries << 16}
+        // and, by cp.async, its masks
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        const int ht = threadIdx.x - kComputeThreads;
+        const unsigned magic_nb = (unsigned)((0x100000000ull + nb - 1) / nb);
+        constexpr int kParts = C::kMaskBytes / 16;
+        auto publish = [&](int level) {
+            if (level < n_levels) {
+                const int p0 = level_ptr[level], rows = (level_ptr[level + 1] - p0) * nb;
+                unsigned char *out = row_tiles + (size_t)(level % 3) * p.row_bytes;
+#pragma unroll 1
+                for (int r = ht; r < (rows + kTile - 1) / kTile * kTile; r += kHelperThreads) {
+                    unsigned char *tile = out + (r / kTile) * C::kRowTile;
+                    int4 rec = make_int4(-1, -1, 0, 0);
+                    if (r < rows) {
+                        const int q = nb == 1 ? r : (int)__umulhi((unsigned)r, magic_nb), s = r - q * nb;
+                        const int4 m = meta[p0 + q];
+                        rec = make_int4((int)((unsigned)m.w * B + b_first + s), m.z >= 0 ? (m.z * S + s) * P : -1,
+                                        m.x < m.y ? (nbr_slot[m.x] * S + s) * P : 0, m.x | (m.y - m.x) << 16);
+                        const unsigned char *from = reinterpret_cast<const unsigned char *>(a.masks[dir]) +
+                                                    (size_t)(unsigned)rec.x * C::kMaskBytes;
+                        unsigned char *to = tile + kTile * 16 + (r % kTile) * C::kMaskBytes;
+#pragma unroll
+                        for (int i = 0; i < kParts; ++i) __pipeline_memcpy_async(to + 16 * i, from + 16 * i, 16);
+                    }
+                    *reinterpret_cast<int4 *>(tile + (r % kTile) * 16) = rec;
+                }
+            }
+            __pipeline_commit();
+        };
+        __syncthreads();              // schedule staged
+        publish(0);
+        publish(1);
+        __pipeline_wait_prior(1);
+        __syncthreads();
+#pragma unroll 1
+        for (int level = 0; level < n_levels; ++level) {
+            publish(level + 2);
+            __pipeline_wait_prior(1);                    // the next level's masks have landed
+            __syncthreads();
+        }
+        return;
+    }
+
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    const DevMlp fn = a.f[dir], gn = a.g[dir];
+    WeightsTail<KS> wf2, wf1, wg2, wg1;                  // transposed: column c of the product reads row c of the matrix
+    auto tail_of = [&](int which) { return tails + (which * C::W + warp % C::W) * KS * 32; };
+    const bool first_group = group == 0;
+    wf2.load(c0, lane, first_group, tail_of(0), [&](int k, int c) { return fn.W2[c * D + k]; });
+    wf1.load(c0, lane, first_group, tail_of(1), [&](int k, int c) { return fn.W1[c * D + k]; });
+    wg2.load(c0, lane, first_group, tail_of(2), [&](int k, int c) { return gn.W2[c * D + k]; });
+    wg1.load(c0, lane, first_group, tail_of(3), [&](int k, int c) { return gn.W1[c * D + k]; });
+    const int col = c0 + g;
+    const unsigned tile_addr = smem_addr(tiles);
+    const unsigned ld_at = tile_addr + ld_offset(lane, C::kStride), st_at = tile_addr + st_offset(lane, C::kStride, c0);
+    constexpr int kLanes = D / 4;
+    const int rr = gt / kLanes, c4 = 4 * (gt % kLanes);
+    unsigned char *gather_to = tiles + rr * C::kStride + 2 * c4;
+    __syncthreads();                  // schedule and third pieces staged
+
+    auto run = [&](const unsigned char *info) {
+        // ---- this lane's d/dh from the pooling, asked for well before it is used
+        int2 to[2];                                      // rows 2t, 2t + 1: {row, own slot}
+        float dh[4];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            to[e] = *reinterpret_cast<const int2 *>(info + (2 * t + e) * 16);
+            const float *at = a.DH[dir] + (size_t)(unsigned)(to[e].x != -1 ? to[e].x : 0) * D + col;
+            dh[e] = at[0];
+            dh[2 + e] = at[8];
+        }
+        // ---- sums of the consumers' ds, through the message's ReLU
+        {
+            const int4 m = *reinterpret_cast<const int4 *>(info + rr * 16);
+            const unsigned bits = reinterpret_cast<const unsigned *>(info + kTile * 16 + rr * C::kMaskBytes)[kMaskM * (D / 32) + (c4 >> 5)] >> (c4 & 31);
+            const unsigned count = (unsigned)m.w >> 16;
+            float4 acc = *reinterpret_cast<const float4 *>(msg + m.z + c4);
+            if (count == 0) acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (__any_sync(0xffffffffu, count > 1)) {
+                const int *slot = nbr_slot + (m.w & 0xffff);
+                const float *from = msg + m.z + c4 - (count > 1 ? slot[0] : 0) * (S * P);
+#pragma unroll 4
+                for (int e = 1; e < (int)count; ++e) {
+                    const float4 v = *reinterpret_cast<const float4 *>(from + slot[e] * (S * P));
+                    acc.x += v.x;
+                    acc.y += v.y;
+                    acc.z += v.z;
+                    acc.w += v.w;
+                }
+            }
+            acc = make_float4(bits & 1 ? acc.x : 0.f, bits & 2 ? acc.y : 0.f, bits & 4 ? acc.z : 0.f, bits & 8 ? acc.w : 0.f);
+            store_row4<Bf16x3>(gather_to, C::kPiece, acc);
+            if (m.x != -1) *reinterpret_cast<float4 *>(a.DPRE_F2[dir] + (size_t)(unsigned)m.x * D + c4) = acc;
+        }
+        group_sync<C::kGroupThreads>(1 + group);
+        float v[4];
+        // v through the ReLUs of mask `which`, stored for the weight gradients and handed to the next product
+        auto pass_on = [&](int which, float *out, auto buffer_constant) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const unsigned bits = reinterpret_cast<const unsigned *>(info + kTile * 16 + (2 * t + e) * C::kMaskBytes)[which * (D / 32) + (c0 >> 5)] >> (col & 31);
+                if (!(bits & 1)) v[e] = 0.f;
+                if (!(bits & 256)) v[2 + e] = 0.f;
+            }
+            store_tile<Bf16x3>(st_at + decltype(buffer_constant)::value * C::kBuffer, C::kPiece, lane, v);
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                if (to[e].x != -1) {
+                    float *at = out + (size_t)(unsigned)to[e].x * D + col;
+                    at[0] = v[e];
+                    at[8] = v[2 + e];
+                }
+            group_sync<C::kGroupThreads>(1 + group);
+        };
+        typedef std::integral_constant<int, 0> buffer0;
+        typedef std::integral_constant<int, 1> buffer1;
+        tail_mma<KS, 0, (int)C::kPiece>(wf2, tail_of(0), ld_at, lane, v);
+        pass_on(kMaskF, a.DFH[dir], buffer1());
+        tail_mma<KS, (int)C::kBuffer, (int)C::kPiece>(wf1, tail_of(1), ld_at, lane, v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] += dh[c];
+        pass_on(kMaskH, a.DPRE_G2[dir], buffer0());
+        tail_mma<KS, 0, (int)C::kPiece>(wg2, tail_of(2), ld_at, lane, v);
+        pass_on(kMaskG, a.DT1[dir], buffer1());
+        tail_mma<KS, (int)C::kBuffer, (int)C::kPiece>(wg1, tail_of(3), ld_at, lane, v);
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            if (to[e].y >= 0) {
+                float *m = msg + to[e].y + col;
+                m[0] = v[e];
+                m[8] = v[2 + e];
+            }
+    };
+
+    int n_tiles = (level_ptr[1] * nb + kTile - 1) / kTile, first = level_ptr[1], buffer = 0;
+    const unsigned char *mine = row_tiles + group * (int)C::kRowTile;
+    __syncthreads();                  // levels 0 and 1 published, level 0's masks landed
+#pragma unroll 1
+    for (int level = 0; level < n_levels; ++level) {
+        const int next = level_ptr[min(level + 2, n_levels)];
+        const unsigned char *info = mine + buffer * p.row_bytes;
+#pragma unroll 1
+        for (int left = n_tiles - group; left > 0; left -= C::G, info += C::G * (int)C::kRowTile) run(info);
+        n_tiles = ((next - first) * nb + kTile - 1) / kTile;
+        first = next;
+        buffer = buffer == 2 ? 0 : buffer + 1;
+        __syncthreads();
+    }
+}
+
+template <int D>
+bool plan_sweep(const GradArgs &a, const DeviceInfo &di, SweepPlan *out) {
+    typedef SweepConfig<D> C;
+    SweepPlan p;
+    const int want = std::max(1, std::min(a.B, di.sm_count / 2));
+    p.S = (a.B + want - 1) / want;
+    const size_t budget = (size_t)std::min(di.max_smem_optin, 227 * 1024) - 1024;
+    int width = 1;
+    for (int dir = 0; dir < 2; ++dir) {
+        const DevLevels &lv = a.lv[1 - dir];
+        p.int_floats[dir] = 4 * a.n + ((lv.n_levels + 1 + 3) & ~3) + ((lv.n_nbr + 3) & ~3);
+        if (lv.n_nbr > 0xffff) return false;
+        width = std::max(width, a.max_level_width);
+    }
+    auto row_bytes = [&](int S) { return (width * S + kTile - 1) / kTile * (int)C::kRowTile; };
+    auto need = [&](int S) {
+        size_t worst = 0;
+        for (int dir = 0; dir < 2; ++dir)
+            worst = std::max(worst, (size_t)p.int_floats[dir] + (size_t)a.lv[1 - dir].n_slots * S * C::P);
+        return worst * sizeof(float) + C::kTailBytes + 3 * (size_t)row_bytes(S) + (size_t)C::G * C::kGroupBytes;
+    };
+    while (p.S > 1 && need(p.S) > budget) --p.S;
+    if (need(p.S) > budget) return false;
+    const int waves = ((a.B + p.S - 1) / p.S + want - 1) / want;
+    p.S = std::min(p.S, (a.B + want * waves - 1) / (want * waves));
+    p.n_slices = (a.B + p.S - 1) / p.S;
+    p.row_bytes = row_bytes(p.S);
+    p.smem_bytes = need(p.S);
+    *out = p;
+    return true;
+}
+
+template <int D>
+cudaError_t launch_rows(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    const size_t R = (size_t)a.n * a.B;
+    const int blocks = (int)std::min<size_t>((R + kRowWarps * kRowsPerWarp - 1) / (kRowWarps * kRowsPerWarp), 2 * (size_t)di.sm_count);
+    const int K = (D + a.F + 3) & ~3;
+    const size_t smem_f = ((size_t)(K + D) * D + (size_t)kRowThreads / 32 * kRowsPerWarp * (K + D)) * sizeof(float);
+    const size_t smem_g = ((size_t)D * D + (size_t)kRowThreads / 32 * kRowsPerWarp * D) * sizeof(float);
+    cudaError_t err = cudaFuncSetAttribute(grad_rows_f_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f);
+    if (err != cudaSuccess) return err;
+    grad_rows_f_kernel<D><<<dim3(blocks, 2), kRowThreads, smem_f, stream>>>(a);
+    count_launch();
+    grad_rows_g_kernel<D><<<dim3(blocks, 2), kRowThreads, smem_g, stream>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t launch_sweep(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    SweepPlan p;
+    if (!plan_sweep<D>(a, di, &p)) return cudaErrorNotSupported;
+    cudaError_t err = cudaFuncSetAttribute(grad_sweep_split_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);
+    if (err != cudaSuccess) return err;
+    grad_sweep_split_kernel<D><<<dim3(p.n_slices, 2), kThreads, p.smem_bytes, stream>>>(a, p);
+    count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool grad_split_applicable(const GradArgs &a, const DeviceInfo &di) {
+    if ((a.d != 32 && a.d != 64) || a.F < 1 || a.F > 16) return false;
+    for (int dir = 0; dir < 2; ++dir)
+        if (a.f[dir].hidden_dim != a.d || a.g[dir].hidden_dim != a.d) return false;
+    SweepPlan p;
+    return a.d == 32 ? plan_sweep<32>(a, di, &p) : plan_sweep<64>(a, di, &p);
+}
+
+cudaError_t launch_grad_rows(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    return a.d == 32 ? launch_rows<32>(a, di, stream) : launch_rows<64>(a, di, stream);
+}
+
+cudaError_t launch_grad_sweep_split(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    return a.d == 32 ? launch_sweep<32>(a, di, stream) : launch_sweep<64>(a, di, stream);
+}
+
+}  // namespace placeto

@@ -598,7 +598,8 @@ size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int H
     // chunk partials of all sixteen layer products side by side
     const size_t widest = 2 * (((size_t)d + F + 1) * Hf + ((size_t)Hf + 1) * d + ((size_t)d + 1) * Hg + ((size_t)Hg + 1) * d) +
                           3 * ((E + 1) * (size_t)d + ((size_t)d + 1) * d) + (Z + 1) * (size_t)Hh + ((size_t)Hh + 1) * m;
-    return total + (size_t)kGradChunks * widest + 256;
+    const size_t masks = 2 * R * (((size_t)d + 31) / 32) * 4;
+    return total + masks + (size_t)kGradChunks * widest + 256;
 }
 
 cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, cudaStream_t stream) {
@@ -618,12 +619,17 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
     for (int i = 0; i < 3; ++i) a.DPRE_L[i] = take(R * d);
     a.Zbuf = take((size_t)B * Z); a.HID = take((size_t)B * Hh); a.DHID = take((size_t)B * Hh);
     a.DLOG = take((size_t)B * m); a.Sbuf = take((size_t)B * 3 * d); a.DPRE_H = take((size_t)B * 3 * d);
+    for (int dir = 0; dir < 2; ++dir) a.masks[dir] = reinterpret_cast<unsigned *>(take(R * (((size_t)d + 31) / 32) * 4));
     float *partial = p;
+    const bool split = grad_split_applicable(a, di);
 
     cudaError_t err = cudaMemsetAsync(a.DPRE_L[0], 0, 3 * ((R * d + 3) & ~size_t(3)) * sizeof(float), stream);
     if (err != cudaSuccess) return err;
     // 1. messages
-    {
+    if (split) {
+        err = launch_grad_rows(a, di, stream);
+        if (err != cudaSuccess) return err;
+    } else {
         const int Hf = std::max(a.f[0].hidden_dim, a.f[1].hidden_dim);
         const size_t smem = (size_t)kRows * (d + F + Hf) * sizeof(float);
         err = cudaFuncSetAttribute(grad_messages_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -645,7 +651,10 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
         count_launch();
     }
     // 3. reverse sweeps
-    {
+    if (split) {
+        err = launch_grad_sweep_split(a, di, stream);
+        if (err != cudaSuccess) return err;
+    } else {
         const int slices = std::max(1, std::min(B, di.sm_count / 2));
         const int S = (B + slices - 1) / slices;
         int W = d;

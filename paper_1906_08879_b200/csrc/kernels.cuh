@@ -192,6 +192,8 @@ struct GradArgs {
     int accumulate;            // 1: gradients are added to the output buffers
     float *FH[2], *DFH[2], *T1[2], *DT1[2], *M[2], *DS[2], *DPRE_F2[2], *DPRE_G2[2], *Sg[2], *DH[2];
     float *DPRE_L[3], *Zbuf, *HID, *DHID, *DLOG, *Sbuf, *DPRE_H;
+    unsigned *masks[2];        // one bit per ReLU of every row (grad_sweep.cu)
+    int max_level_width;
     GradOut gf[2], gg[2], gl[3], gh[3], ghead;
 };
 
@@ -303,6 +305,12 @@ cudaError_t launch_simulator(const SimArgs &a, const DeviceInfo &di, cudaStream_
 bool policy_gradient_applicable(const GradArgs &a);
 size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh);
 cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, cudaStream_t stream);
+
+// grad_sweep.cu: the passes over the node-state rows for d = 32 / 64 with hidden width d: forward values and masks of
+// every row, then the reverse sweeps on the tensor cores
+bool grad_split_applicable(const GradArgs &a, const DeviceInfo &di);
+cudaError_t launch_grad_rows(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream);
+cudaError_t launch_grad_sweep_split(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream);
 
 // writes the d x d identity matrix followed by d zeros (an identity layer: W2 = I, b2 = 0)
 cudaError_t launch_identity_layer(float *dst, int d, cudaStream_t stream);

@@ -131,3 +131,15 @@ def test_single_layer_networks_as_in_the_paper(d, m):
     cfg["weights"] = states.policy_weights(r, d, m + 4, m, 1, 0, 0.2)
     grads = gpu_gradient(cfg, actions, adv, 0.05)
     compare(cfg, grads, gradient.gradient(cfg, actions, adv, 0.05))
+
+
+@pytest.mark.parametrize("d,m,B,layers", [(32, 4, 1, 2), (32, 2, 160, 2), (32, 12, 75, 1), (64, 3, 1, 2), (64, 8, 155, 2), (64, 5, 76, 1)])
+def test_split_sweep_over_tiles(d, m, B, layers):
+    """The tensor-core reverse sweep: one state per block, levels of one partial tile and of more tiles than groups of
+    warps, a ragged last slice, nodes of many consumers, feature widths that are no multiple of 4."""
+    cfg, actions, adv = small_case(7 * d + B, n=33, m=m, d=d, B=B, p=0.12)
+    r = rng(B)
+    cfg["weights"] = states.policy_weights(r, d, m + 4, m, layers, 0, 0.2)
+    adv = adv.astype(np.float32).astype(np.float64)
+    grads = gpu_gradient(cfg, actions, adv, 0.1)
+    compare(cfg, grads, gradient.gradient(cfg, actions, adv, 0.1))
