@@ -1,0 +1,455 @@
+// The policy gradient through the pooling networks l_i (d = 32 and 64, single ReLU layers): the
+// pooled sums and the sign of every pre-activation, then - once the head has turned the sums into
+// their gradients - d/dh of every node, and the weight gradients of all networks applied per row.
+//
+// Everything here is a product over independent node-state rows, so the kernels are throughput
+// loops: the three networks (or their transposes) stay in shared memory, a block takes (state,
+// chunk of nodes) items, compacts the chunk's nodes by set and gives each warp eight rows of one
+// set at a time. Sums are stored per batch and added in order: no atomics, reproducible bit for bit.
+#include <cuda_pipeline.h>
+
+#include <algorithm>
+
+#include "grad_rows.cuh"
+
+namespace placeto {
+
+namespace {
+
+// The chunk's nodes by set relative to the state's current node, in ascending order; the batches of eight of set i
+// are numbers first[i] .. first[i + 1).
+struct Lists {
+    unsigned short *node;      // [3][chunk_nodes]
+    int *count;                // [3]
+};
+__device__ __forceinline__ void build_lists(const Lists &l, const uint8_t *rel, int u0, int nu, int chunk_nodes, bool valid,
+                                            int warp, int lane) {
+    if (warp < 3) {
+        int cnt = 0;
+        for (int base = 0; base < nu; base += 32) {
+            const int q = base + lane;
+            const bool in = valid && q < nu && rel[u0 + q] == warp;
+            const unsigned bits = __ballot_sync(0xffffffffu, in);
+            if (in) l.node[warp * chunk_nodes + cnt + __popc(bits & ((1u << lane) - 1))] = (unsigned short)(u0 + q);
+            cnt += __popc(bits);
+        }
+        if (lane == 0) l.count[warp] = cnt;
+    }
+}
+// batch `k` of the item: its set, first list entry and rows; false past the last
+__device__ __forceinline__ bool find_batch(const Lists &l, int k, int &set, int &at, int &rows) {
+    for (set = 0; set < 3; ++set) {
+        const int n = (l.count[set] + kRowsPerWarp - 1) / kRowsPerWarp;
+        if (k < n) {
+            at = k * kRowsPerWarp;
+            rows = min(kRowsPerWarp, l.count[set] - at);
+            return true;
+        }
+        k -= n;
+    }
+    return false;
+}
+
+// relu(l_i(e_u)) of every row: sums per (chunk, state, set), and one bit per column, positive or not
+template <int D>
+__global__ void __launch_bounds__(kRowThreads)
+grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
+    constexpr int C = D / 32;
+    extern __shared__ __align__(16) float smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = a.n, B = a.B, F = a.F, E = 2 * D + F, Ep = (E + 3) & ~3;
+    float *W = smem;                                     // [3][Ep][D], zero padded
+    float *in = W + 3 * Ep * D + warp * kRowsPerWarp * Ep;
+    float *sums = W + 3 * Ep * D + kRowWarps * kRowsPerWarp * Ep;       // [batch][D]
+    const int max_batches = chunk_nodes / kRowsPerWarp + 3;
+    Lists l;
+    l.count = reinterpret_cast<int *>(sums + max_batches * D);
+    l.node = reinterpret_cast<unsigned short *>(l.count + 4);
+    for (int i = 0; i < 3; ++i)
+        for (int t = threadIdx.x; t < Ep * D; t += kRowThreads) W[i * Ep * D + t] = t < E * D ? a.l[i].W1[t] : 0.f;
+    __syncthreads();
+    const int items = B * chunks;
+    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+        const int b = item % B, chunk = item / B;
+        const int u0 = chunk * chunk_nodes, nu = min(n, u0 + chunk_nodes) - u0;
+        const int c = a.cur[b];
+        const bool valid = c >= 0 && c < n;
+        build_lists(l, a.relation + (size_t)(valid ? c : 0) * n, u0, nu, chunk_nodes, valid, warp, lane);
+        __syncthreads();
+        int set, at, rows;
+        for (int k = warp; find_batch(l, k, set, at, rows); k += kRowWarps) {
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < kRowsPerWarp; ++r) {
+                const size_t row = (size_t)l.node[set * chunk_nodes + at + min(r, rows - 1)] * B + b;
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    in[r * Ep + lane + 32 * q] = a.H[0][row * D + lane + 32 * q];
+                    in[r * Ep + D + lane + 32 * q] = a.H[1][row * D + lane + 32 * q];
+                }
+                if (lane < Ep - 2 * D) in[r * Ep + 2 * D + lane] = lane < F ? a.X[row * F + lane] : 0.f;
+            }
+            __syncwarp();
+            float acc[kRowsPerWarp][C];
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                const float bias = a.l[set].b1[lane + 32 * q];
+#pragma unroll
+                for (int r = 0; r < kRowsPerWarp; ++r) acc[r][q] = bias;
+            }
+            row_products<D>(W + set * Ep * D, in, Ep, Ep, lane, acc);
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                float s = 0.f;
+#pragma unroll
+                for (int r = 0; r < kRowsPerWarp; ++r) {
+                    const unsigned bits = __ballot_sync(0xffffffffu, acc[r][q] > 0.f);
+                    if (r < rows) {
+                        s += fmaxf(acc[r][q], 0.f);
+                        if (lane == 0) a.l_masks[((size_t)l.node[set * chunk_nodes + at + r] * B + b) * C + q] = bits;
+                    }
+                }
+                sums[k * D + lane + 32 * q] = s;
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 * D; i += kRowThreads) {
+            const int s = i / D, j = i - s * D;
+            int first = 0;
+            for (int q = 0; q < s; ++q) first += (l.count[q] + kRowsPerWarp - 1) / kRowsPerWarp;
+            const int last = first + (l.count[s] + kRowsPerWarp - 1) / kRowsPerWarp;
+            float total = 0.f;
+            for (int q = first; q < last; ++q) total += sums[q * D + j];
+            a.pool_partial[((size_t)chunk * B + b) * 3 * D + i] = total;
+        }
+        __syncthreads();
+    }
+}
+
+// dpre_l = dS of the row's set where the pre-activation was positive; d/dh = dpre_l W_l^T (its embedding columns)
+template <int D>
+__global__ void __launch_bounds__(kRowThreads)
+grad_pool_backward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
+    constexpr int C = D / 32;
+    extern __shared__ __align__(16) float smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = a.n, B = a.B;
+    float *Wt = smem;                                    // [3][D][2 D]
+    float *in = Wt + 3 * D * 2 * D + warp * kRowsPerWarp * D;
+    Lists l;
+    l.count = reinterpret_cast<int *>(Wt + 3 * D * 2 * D + kRowWarps * kRowsPerWarp * D);
+    l.node = reinterpret_cast<unsigned short *>(l.count + 4);
+    for (int i = 0; i < 3; ++i)
+        for (int t = threadIdx.x; t < 2 * D * D; t += kRowThreads) {
+            // a warp reads 4 rows x 8 columns: whole sectors, stores to eight rows
+            const int q = t >> 5, j = q % (D / 8) * 8 + (t & 7), k = q / (D / 8) * 4 + (t >> 3 & 3);
+            Wt[(i * D + j) * 2 * D + k] = a.l[i].W1[k * D + j];
+        }
+    __syncthreads();
+    const int items = B * chunks;
+    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+        const int b = item % B, chunk = item / B;
+        const int u0 = chunk * chunk_nodes, nu = min(n, u0 + chunk_nodes) - u0;
+        const int c = a.cur[b];
+        const bool valid = c >= 0 && c < n;
+        build_lists(l, a.relation + (size_t)(valid ? c : 0) * n, u0, nu, chunk_nodes, valid, warp, lane);
+        // the current node's embedding enters the head directly; a state without one contributes nothing
+        if (valid && c >= u0 && c < u0 + nu && warp == kRowWarps - 1) {
+#pragma unroll
+            for (int q = 0; q < 2 * C; ++q)
+                a.DH[q / C][((size_t)c * B + b) * D + lane + 32 * (q % C)] = a.dZ[(size_t)b * 2 * D + lane + 32 * q];
+        }
+        if (!valid)
+            for (int i = threadIdx.x; i < nu * D; i += kRowThreads) {
+                const size_t at = ((size_t)(u0 + i / D) * B + b) * D + i % D;
+                a.DH[0][at] = 0.f;
+                a.DH[1][at] = 0.f;
+            }
+        __syncthreads();
+        int set, at, rows;
+        for (int k = warp; find_batch(l, k, set, at, rows); k += kRowWarps) {
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                const float ds = a.dS[((size_t)b * 3 + set) * D + lane + 32 * q];
+#pragma unroll
+                for (int r = 0; r < kRowsPerWarp; ++r) {
+                    const size_t row = (size_t)l.node[set * chunk_nodes + at + min(r, rows - 1)] * B + b;
+                    const float v = a.l_masks[row * C + q] >> lane & 1 ? ds : 0.f;
+                    in[r * D + lane + 32 * q] = v;
+                    if (r < rows) a.DPRE_L[0][row * D + lane + 32 * q] = v;
+                }
+            }
+            __syncwarp();
+            float acc[kRowsPerWarp][2 * C];
+#pragma unroll
+            for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+                for (int q = 0; q < 2 * C; ++q) acc[r][q] = 0.f;
+            row_products<2 * D>(Wt + set * 2 * D * D, in, D, D, lane, acc);
+#pragma unroll
+            for (int r = 0; r < kRowsPerWarp; ++r)
+                if (r < rows) {
+                    const size_t row = (size_t)l.node[set * chunk_nodes + at + r] * B + b;
+#pragma unroll
+                    for (int q = 0; q < 2 * C; ++q) a.DH[q / C][row * D + lane + 32 * (q % C)] = acc[r][q];
+                }
+        }
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------ weight gradients
+// partial[chunk][K + 1][J] = sum over rows of [in || 1]^T dp. A thread owns TK x 4 outputs; the rows arrive in stages
+// of 32 by cp.async while the stage before is multiplied.
+constexpr int kStageRows = 32;
+
+// One stage of the product: the staged rows' inputs [32][Kp] and gradients [32][D].
+template <int D, int TK>
+__device__ __forceinline__ void stage_product(const float *in, const float *dp, int Kp, int rows, int tk, int tj, float (&acc)[TK][4]) {
+    const float *pa = in + TK * tk, *pb = dp + 4 * tj;
+#pragma unroll 4
+    for (int r = 0; r < rows; ++r) {
+        float x[TK];
+#pragma unroll
+        for (int i = 0; i < TK; i += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(pa + r * Kp + i);
+            x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+        }
+        const float4 y = *reinterpret_cast<const float4 *>(pb + r * D);
+#pragma unroll
+        for (int i = 0; i < TK; ++i) {
+            acc[i][0] = fmaf(x[i], y.x, acc[i][0]);
+            acc[i][1] = fmaf(x[i], y.y, acc[i][1]);
+            acc[i][2] = fmaf(x[i], y.z, acc[i][2]);
+            acc[i][3] = fmaf(x[i], y.w, acc[i][3]);
+        }
+    }
+}
+template <int D, int TK>
+__device__ __forceinline__ void write_partial(float *out, int K, int tk, int tj, const float (&acc)[TK][4]) {
+#pragma unroll
+    for (int i = 0; i < TK; ++i)
+        if (TK * tk + i <= K)
+            *reinterpret_cast<float4 *>(out + (size_t)(TK * tk + i) * D + 4 * tj) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+}
+
+// The eight layers of f and g: blockIdx.y = job, blockIdx.x = chunk of the rows.
+struct RowJob {
+    const float *in, *x, *dp;      // [R][D], [R][F] or null, [R][D]
+    float *partial;
+};
+struct RowJobs { RowJob job[8]; };
+
+template <int D, int TK>
+__global__ void __launch_bounds__(D == 64 ? 192 : 128)
+grad_weight_rows_kernel(const RowJobs jobs, size_t R, int F, int chunks) {
+    extern __shared__ __align__(16) float smem[];
+    const RowJob w = jobs.job[blockIdx.y];
+    const int K = D + (w.x ? F : 0), Kp = (K + TK) / TK * TK;
+    const int stage = kStageRows * (Kp + D);
+    const int threads = blockDim.x;
+    const int tiles_j = D / 4;
+    const int tk = threadIdx.x / tiles_j, tj = threadIdx.x % tiles_j;
+    const bool live = TK * tk < Kp;
+    const size_t per = ((R + chunks - 1) / chunks + kStageRows - 1) / kStageRows * kStageRows;
+    const size_t r_begin = min(R, (size_t)blockIdx.x * per), r_end = min(R, r_begin + per);
+    for (int i = threadIdx.x; i < 2 * kStageRows * (Kp - K); i += threads) {       // the ones of the bias, the padding
+        const int r = i / (Kp - K), k = i - r * (Kp - K);
+        smem[(r / kStageRows) * stage + (r % kStageRows) * Kp + K + k] = k == 0 ? 1.f : 0.f;
+    }
+    auto load = [&](size_t r0, int buffer) {
+        float *in = smem + buffer * stage, *dp = in + kStageRows * Kp;
+        const int rows = (int)min((size_t)kStageRows, r_end - r0);
+        for (int i = threadIdx.x; i < rows * (D / 4); i += threads) {
+            const int r = i / (D / 4), q = 4 * (i % (D / 4));
+            __pipeline_memcpy_async(dp + r * D + q, w.dp + (r0 + r) * D + q, 16);
+            __pipeline_memcpy_async(in + r * Kp + q, w.in + (r0 + r) * D + q, 16);
+        }
+        if (w.x)
+            for (int i = threadIdx.x; i < kStageRows * F; i += threads) {
+                const int r = i % kStageRows, k = i / kStageRows;
+                if (r < rows) __pipeline_memcpy_async(in + r * Kp + D + k, w.x + (r0 + r) * F + k, 4);
+            }
+        __pipeline_commit();
+    };
+    float acc[TK][4];
+#pragma unroll
+    for (int i = 0; i < TK; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+    if (r_begin < r_end) load(r_begin, 0);
+    int buffer = 0;
+    for (size_t r0 = r_begin; r0 < r_end; r0 += kStageRows, buffer ^= 1) {
+        if (r0 + kStageRows < r_end) load(r0 + kStageRows, buffer ^ 1);
+        else __pipeline_commit();
+        __pipeline_wait_prior(1);
+        __syncthreads();
+        const float *in = smem + buffer * stage;
+        if (live) stage_product<D, TK>(in, in + kStageRows * Kp, Kp, (int)min((size_t)kStageRows, r_end - r0), tk, tj, acc);
+        __syncthreads();
+    }
+    if (live) write_partial<D, TK>(w.partial + (size_t)blockIdx.x * (K + 1) * D, K, tk, tj, acc);
+}
+
+// The three l_i: blockIdx.y = set, blockIdx.x = chunk of the nodes; the rows of the set, node after node. (State after
+// state is ten times less accurate: the terms of a state have one sign and cancel only between states.)
+template <int D, int TK>
+__global__ void __launch_bounds__(D == 64 ? 320 : 192)
+grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const partial1, float *const partial2, int chunks) {
+    extern __shared__ __align__(16) float smem[];
+    const int set = blockIdx.y;
+    const int n = a.n, B = a.B, F = a.F, K = 2 * D + F, Kp = (K + TK) / TK * TK;
+    const int stage = kStageRows * (Kp + D);
+    const int threads = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tiles_j = D / 4;
+    const int tk = threadIdx.x / tiles_j, tj = threadIdx.x % tiles_j;
+    const bool live = TK * tk < Kp;
+    int *list = reinterpret_cast<int *>(smem + 2 * stage);           // rows waiting: fewer than 32 left over, then a node's
+    __shared__ int have_s;
+    for (int i = threadIdx.x; i < 2 * kStageRows * (Kp - K); i += threads) {
+        const int r = i / (Kp - K), k = i - r * (Kp - K);
+        smem[(r / kStageRows) * stage + (r % kStageRows) * Kp + K + k] = k == 0 ? 1.f : 0.f;
+    }
+    auto load = [&](int first, int rows, int buffer) {
+        float *in = smem + buffer * stage, *dp = in + kStageRows * Kp;
+        for (int i = threadIdx.x; i < rows * (D / 4); i += threads) {
+            const int r = i / (D / 4), q = 4 * (i % (D / 4));
+            const size_t row = (size_t)(unsigned)list[first + r] * D + q;
+            __pipeline_memcpy_async(in + r * Kp + q, a.H[0] + row, 16);
+            __pipeline_memcpy_async(in + r * Kp + D + q, a.H[1] + row, 16);
+            __pipeline_memcpy_async(dp + r * D + q, a.DPRE_L[0] + row, 16);
+        }
+        for (int i = threadIdx.x; i < kStageRows * F; i += threads) {
+            const int r = i % kStageRows, k = i / kStageRows;
+            if (r < rows) __pipeline_memcpy_async(in + r * Kp + 2 * D + k, a.X + (size_t)(unsigned)list[first + r] * F + k, 4);
+        }
+        __pipeline_commit();
+    };
+    float acc[TK][4];
+#pragma unroll
+    for (int i = 0; i < TK; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+    const int per = (n + chunks - 1) / chunks;
+    const int u0 = blockIdx.x * per, u1 = min(n, u0 + per);
+    int have = 0;
+    for (int u = u0; u < u1; ++u) {
+        if (warp == 0) {
+            int cnt = have;
+            for (int base = 0; base < B; base += 128) {          // four loads in flight
+                int s[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int b = base + 32 * q + lane, c = b < B ? a.cur[b] : -1;
+                    s[q] = c >= 0 && c < n ? a.relation[(size_t)c * n + u] : 3;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const unsigned bits = __ballot_sync(0xffffffffu, s[q] == set);
+                    if (s[q] == set) list[cnt + __popc(bits & ((1u << lane) - 1))] = u * B + base + 32 * q + lane;
+                    cnt += __popc(bits);
+                }
+            }
+            if (lane == 0) have_s = cnt;
+        }
+        __syncthreads();
+        have = have_s;
+        const int use = u + 1 < u1 ? have / kStageRows * kStageRows : have;
+        if (use > 0) load(0, min(kStageRows, use), 0);
+        int buffer = 0;
+        for (int r0 = 0; r0 < use; r0 += kStageRows, buffer ^= 1) {
+            if (r0 + kStageRows < use) load(r0 + kStageRows, min(kStageRows, use - r0 - kStageRows), buffer ^ 1);
+            else __pipeline_commit();
+            __pipeline_wait_prior(1);
+            __syncthreads();
+            const float *in = smem + buffer * stage;
+            if (live) stage_product<D, TK>(in, in + kStageRows * Kp, Kp, min(kStageRows, use - r0), tk, tj, acc);
+            __syncthreads();
+        }
+        const int left = have - use;
+        int keep = 0;
+        if ((int)threadIdx.x < left) keep = list[use + threadIdx.x];
+        __syncthreads();
+        if ((int)threadIdx.x < left) list[threadIdx.x] = keep;
+        have = left;
+        __syncthreads();
+    }
+    float *out = set == 0 ? partial0 : set == 1 ? partial1 : partial2;
+    if (live) write_partial<D, TK>(out + (size_t)blockIdx.x * (K + 1) * D, K, tk, tj, acc);
+}
+
+size_t forward_smem(int D, int F, int chunk_nodes) {
+    const int Ep = (2 * D + F + 3) & ~3;
+    return ((size_t)3 * Ep * D + (size_t)kRowWarps * kRowsPerWarp * Ep + (size_t)(chunk_nodes / kRowsPerWarp + 3) * D + 4) * sizeof(float) +
+           (size_t)3 * chunk_nodes * 2;
+}
+size_t backward_smem(int D, int chunk_nodes) {
+    return ((size_t)6 * D * D + (size_t)kRowWarps * kRowsPerWarp * D + 4) * sizeof(float) + (size_t)3 * chunk_nodes * 2;
+}
+
+template <int D>
+cudaError_t launch_forward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    const size_t smem = forward_smem(D, a.F, a.pool_chunk_nodes);
+    cudaError_t err = cudaFuncSetAttribute(grad_pool_forward_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    const int grid = std::min(a.B * a.pool_chunks, (D == 32 ? 3 : 1) * di.sm_count);
+    grad_pool_forward_kernel<D><<<grid, kRowThreads, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
+    count_launch();
+    return cudaGetLastError();
+}
+template <int D>
+cudaError_t launch_backward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    const size_t smem = backward_smem(D, a.pool_chunk_nodes);
+    cudaError_t err = cudaFuncSetAttribute(grad_pool_backward_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    const int grid = std::min(a.B * a.pool_chunks, (D == 32 ? 4 : 1) * di.sm_count);
+    grad_pool_backward_kernel<D><<<grid, kRowThreads, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
+    count_launch();
+    return cudaGetLastError();
+}
+
+template <int D, int TK>
+cudaError_t launch_weights(const GradArgs &a, float *const (&rows)[8], int row_chunks, float *const (&pool)[3], int pool_chunks,
+                           cudaStream_t stream) {
+    RowJobs jobs;
+    for (int dir = 0; dir < 2; ++dir) {
+        const RowJob j[4] = {{a.H[dir], a.X, a.DFH[dir], rows[4 * dir]},
+                             {a.FH[dir], nullptr, a.DPRE_F2[dir], rows[4 * dir + 1]},
+                             {a.Sg[dir], nullptr, a.DT1[dir], rows[4 * dir + 2]},
+                             {a.T1[dir], nullptr, a.DPRE_G2[dir], rows[4 * dir + 3]}};
+        for (int k = 0; k < 4; ++k) jobs.job[4 * dir + k] = j[k];
+    }
+    const int Kp = (D + a.F + TK) / TK * TK, Lp = (2 * D + a.F + TK) / TK * TK;
+    const int threads = (Kp / TK * (D / 4) + 31) & ~31, pool_threads = (Lp / TK * (D / 4) + 31) & ~31;
+    size_t smem = (size_t)2 * kStageRows * (Kp + D) * sizeof(float);
+    cudaError_t err = cudaFuncSetAttribute(grad_weight_rows_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    grad_weight_rows_kernel<D, TK><<<dim3(row_chunks, 8), threads, smem, stream>>>(jobs, (size_t)a.n * a.B, a.F, row_chunks);
+    count_launch();
+    smem = (size_t)2 * kStageRows * (Lp + D) * sizeof(float) + (size_t)(a.B + kStageRows) * sizeof(int);
+    err = cudaFuncSetAttribute(grad_weight_pool_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    grad_weight_pool_kernel<D, TK><<<dim3(pool_chunks, 3), pool_threads, smem, stream>>>(a, pool[0], pool[1], pool[2], pool_chunks);
+    count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Chunks of at most 256 nodes, more of them while the batch alone does not fill the device.
+void grad_pool_chunks(int n, int B, const DeviceInfo &di, int *chunk_nodes, int *chunks) {
+    int c = (n + 255) / 256;
+    c = std::max(c, std::min((2 * di.sm_count + B - 1) / B, (n + 63) / 64));
+    *chunk_nodes = (n + c - 1) / c;
+    *chunks = (n + *chunk_nodes - 1) / *chunk_nodes;
+}
+cudaError_t launch_grad_pool_forward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    return a.d == 32 ? launch_forward<32>(a, di, stream) : launch_forward<64>(a, di, stream);
+}
+cudaError_t launch_grad_pool_backward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
+    return a.d == 32 ? launch_backward<32>(a, di, stream) : launch_backward<64>(a, di, stream);
+}
+cudaError_t launch_grad_weights_split(const GradArgs &a, float *const (&rows)[8], int row_chunks, float *const (&pool)[3],
+                                      int pool_chunks, cudaStream_t stream) {
+    return a.d == 32 ? launch_weights<32, 4>(a, rows, row_chunks, pool, pool_chunks, stream)
+                     : launch_weights<64, 8>(a, rows, row_chunks, pool, pool_chunks, stream);
+}
+
+}  // namespace placeto

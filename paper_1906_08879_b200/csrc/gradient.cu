@@ -69,7 +69,9 @@ grad_messages_kernel(const GradArgs a) {
 }
 
 // ------------------------------------------------------------- 2. head / pool
-// One block per state (grid-stride). Shared memory: the state's vectors.
+// One block per state (grid-stride). Shared memory: the state's vectors. kPooled: the sums arrive per chunk of
+// nodes and what is pushed back stops at them and at the current node's embedding (grad_pool.cu does the rows).
+template <bool kPooled>
 __global__ void __launch_bounds__(kThreads)
 grad_head_kernel(const GradArgs a) {
     extern __shared__ __align__(16) float smem[];
@@ -88,7 +90,7 @@ grad_head_kernel(const GradArgs a) {
     float *wl = erow + G * ((E + 3) & ~3); // [3][E * d + d]: the three l_i (weights, then bias)
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int lsz = E * d + d;
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; !kPooled && i < 3; ++i) {
         for (int t = threadIdx.x; t < E * d; t += kThreads) wl[i * lsz + t] = a.l[i].W1[t];
         for (int t = threadIdx.x; t < d; t += kThreads) wl[i * lsz + E * d + t] = a.l[i].b1[t];
     }
@@ -97,7 +99,7 @@ grad_head_kernel(const GradArgs a) {
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
         const int c = a.cur[b];
         if (c < 0 || c >= n) {             // no such node: the state contributes nothing
-            for (int i = threadIdx.x; i < n * d; i += kThreads) {
+            for (int i = threadIdx.x; !kPooled && i < n * d; i += kThreads) {
                 const size_t off = ((size_t)(i / d) * B + b) * d + (i % d);
                 a.DH[0][off] = 0.f;
                 a.DH[1][off] = 0.f;
@@ -115,9 +117,9 @@ grad_head_kernel(const GradArgs a) {
                              : a.X[((size_t)u * B + b) * F + (k - 2 * d)];
         };
         // ---- pooled sums S_i = sum_{u in set i} relu(l_i(e_u)); warp g takes nodes g, g + G, ...
-        for (int i = threadIdx.x; i < G * 3 * d; i += kThreads) part[i] = 0.f;
+        for (int i = threadIdx.x; !kPooled && i < G * 3 * d; i += kThreads) part[i] = 0.f;
         __syncthreads();
-        for (int u = g; u < n; u += G) {
+        for (int u = g; !kPooled && u < n; u += G) {
             const int set = rel[u];
             if (set > 2) continue;
             const float *W = wl + set * lsz;
@@ -133,7 +135,10 @@ grad_head_kernel(const GradArgs a) {
         __syncthreads();
         for (int i = threadIdx.x; i < 3 * d; i += kThreads) {
             float acc = 0.f;
-            for (int q = 0; q < G; ++q) acc += part[q * 3 * d + i];
+            if (kPooled)
+                for (int q = 0; q < a.pool_chunks; ++q) acc += a.pool_partial[((size_t)q * B + b) * 3 * d + i];
+            else
+                for (int q = 0; q < G; ++q) acc += part[q * 3 * d + i];
             S[i] = acc;
             a.Sbuf[(size_t)b * 3 * d + i] = acc;
         }
@@ -213,6 +218,12 @@ grad_head_kernel(const GradArgs a) {
             float acc = 0.f;
             for (int j = 0; j < d; ++j) acc = fmaf(part[set * d + j], h.W1[k * d + j], acc);
             dS[i] = acc;
+            if (kPooled) a.dS[(size_t)b * 3 * d + i] = acc;
+        }
+        if (kPooled) {
+            for (int k = threadIdx.x; k < 2 * d; k += kThreads) a.dZ[(size_t)b * 2 * d + k] = dz[k];
+            __syncthreads();
+            continue;
         }
         __syncthreads();
         // ---- through l_i to every node: dpre_l = dS_set * (pre > 0); de = dpre_l W_l^T
@@ -542,7 +553,8 @@ grad_weight_reduce_kernel(const WeightJobs jobs) {
     }
 }
 
-cudaError_t weight_grads(const WeightJobs &jobs, cudaStream_t stream) {
+// sums the jobs' chunks into their gradients, after computing them unless another kernel has (`products`)
+cudaError_t weight_grads(const WeightJobs &jobs, cudaStream_t stream, bool products) {
     if (jobs.count == 0) return cudaSuccess;
     size_t smem = 0;
     int max_chunks = 1, max_out = 1, max_tiles = 1;
@@ -554,11 +566,13 @@ cudaError_t weight_grads(const WeightJobs &jobs, cudaStream_t stream) {
         max_out = std::max(max_out, (w.K + 1) * w.J);
         max_tiles = std::max(max_tiles, (Kp / 4) * (Jp / 4));
     }
-    cudaError_t err = cudaFuncSetAttribute(grad_weight_partial_kernel,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    grad_weight_partial_kernel<<<dim3(max_chunks, (max_tiles + kThreads - 1) / kThreads, jobs.count), kThreads, smem, stream>>>(jobs);
-    count_launch();
+    if (products) {
+        const cudaError_t err = cudaFuncSetAttribute(grad_weight_partial_kernel,
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err != cudaSuccess) return err;
+        grad_weight_partial_kernel<<<dim3(max_chunks, (max_tiles + kThreads - 1) / kThreads, jobs.count), kThreads, smem, stream>>>(jobs);
+        count_launch();
+    }
     grad_weight_reduce_kernel<<<dim3((max_out + 31) / 32, jobs.count), 256, 0, stream>>>(jobs);
     count_launch();
     return cudaGetLastError();
@@ -590,7 +604,7 @@ bool policy_gradient_applicable(const GradArgs &a) {
 }
 
 // floats of workspace (every array padded to a multiple of 4 floats by the carve below)
-size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh) {
+size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh, int pool_chunks) {
     const size_t R = (size_t)n * B, Z = 5 * (size_t)d + F, E = 2 * (size_t)d + F;
     const size_t per_dir = R * ((size_t)Hf * 2 + (size_t)Hg * 2 + (size_t)d * 6);
     size_t total = 2 * per_dir + 3 * R * d;
@@ -599,7 +613,8 @@ size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int H
     const size_t widest = 2 * (((size_t)d + F + 1) * Hf + ((size_t)Hf + 1) * d + ((size_t)d + 1) * Hg + ((size_t)Hg + 1) * d) +
                           3 * ((E + 1) * (size_t)d + ((size_t)d + 1) * d) + (Z + 1) * (size_t)Hh + ((size_t)Hh + 1) * m;
     const size_t masks = 2 * R * (((size_t)d + 31) / 32) * 4;
-    return total + masks + (size_t)kGradChunks * widest + 256;
+    const size_t pooled = R * (((size_t)d + 31) / 32) + (size_t)B * 5 * d + (size_t)pool_chunks * B * 3 * d;
+    return total + masks + pooled + (size_t)kGradChunks * widest + 256;
 }
 
 cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, cudaStream_t stream) {
@@ -620,10 +635,15 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
     a.Zbuf = take((size_t)B * Z); a.HID = take((size_t)B * Hh); a.DHID = take((size_t)B * Hh);
     a.DLOG = take((size_t)B * m); a.Sbuf = take((size_t)B * 3 * d); a.DPRE_H = take((size_t)B * 3 * d);
     for (int dir = 0; dir < 2; ++dir) a.masks[dir] = reinterpret_cast<unsigned *>(take(R * (((size_t)d + 31) / 32) * 4));
+    grad_pool_chunks(n, B, di, &a.pool_chunk_nodes, &a.pool_chunks);
+    a.l_masks = reinterpret_cast<unsigned *>(take(R * (((size_t)d + 31) / 32)));
+    a.dS = take((size_t)B * 3 * d); a.dZ = take((size_t)B * 2 * d);
+    a.pool_partial = take((size_t)a.pool_chunks * B * 3 * d);
     float *partial = p;
     const bool split = grad_split_applicable(a, di);
 
-    cudaError_t err = cudaMemsetAsync(a.DPRE_L[0], 0, 3 * ((R * d + 3) & ~size_t(3)) * sizeof(float), stream);
+    cudaError_t err = cudaSuccess;
+    if (!split) err = cudaMemsetAsync(a.DPRE_L[0], 0, 3 * ((R * d + 3) & ~size_t(3)) * sizeof(float), stream);
     if (err != cudaSuccess) return err;
     // 1. messages
     if (split) {
@@ -640,15 +660,20 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
     }
     // 2. head and pooling
     {
+        if (split) err = launch_grad_pool_forward(a, di, stream);
+        if (err != cudaSuccess) return err;
         const size_t E = 2 * (size_t)d + F;
         const size_t floats = 2 * (size_t)Z + 2 * (size_t)Hh + 6 * (size_t)d + ((m + 3) & ~3) +
                               (size_t)(kThreads / 32) * 3 * d + (size_t)(kThreads / 32) * ((E + 3) & ~size_t(3)) +
-                              3 * (E * d + d);
+                              (split ? 0 : 3 * (E * d + d));
         const size_t smem = floats * sizeof(float);
-        err = cudaFuncSetAttribute(grad_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        void (*kern)(const GradArgs) = split ? grad_head_kernel<true> : grad_head_kernel<false>;
+        err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err != cudaSuccess) return err;
-        grad_head_kernel<<<std::min(B, 8 * di.sm_count), kThreads, smem, stream>>>(a);
+        kern<<<std::min(B, 8 * di.sm_count), kThreads, smem, stream>>>(a);
         count_launch();
+        if (split) err = launch_grad_pool_backward(a, di, stream);
+        if (err != cudaSuccess) return err;
     }
     // 3. reverse sweeps
     if (split) {
@@ -681,8 +706,9 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
     WeightJobs by_row, by_state;
     by_row.count = by_state.count = 0;
     auto job = [&](const float *in0, int w0, int s0, const float *in1, int w1, const float *in2, int w2,
-                   const float *dp, int dp_stride, int J, size_t rows, float *dW, float *db) {
-        WeightJobs &list = rows == R ? by_row : by_state;
+                   const float *dp, int dp_stride, int J, bool per_row, float *dW, float *db, int chunks = 0) {
+        WeightJobs &list = per_row ? by_row : by_state;
+        const size_t rows = per_row ? R : (size_t)B;
         WeightJob &w = list.job[list.count++];
         w.in[0] = in0; w.in[1] = in1; w.in[2] = in2;
         w.width[0] = w0; w.width[1] = w1; w.width[2] = w2;
@@ -691,26 +717,38 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
         w.dW = dW; w.db = db;
         w.accumulate = a.accumulate;
         w.chunks = (int)std::max<size_t>(1, std::min<size_t>(kGradChunks, (rows + kRows - 1) / kRows));
+        if (split && chunks > 0) w.chunks = chunks;
         w.partial = partial;                                  // each job its own stretch
         partial += (size_t)w.chunks * (w.K + 1) * w.J;
     };
+    // (For the shapes of grad_pool.cu the per-row jobs are only reduced here. Eight jobs share the SMs: half as many
+    // chunks as SMs put four blocks on each, while a chunk has at least four stages of rows.)
+    const int row_chunks = (int)std::max<size_t>(1, std::min<size_t>(di.sm_count / 2, R / 128));
+    const int pool_chunks = std::min(di.sm_count, n);
     for (int dir = 0; dir < 2; ++dir) {
         const int Hf = a.f[dir].hidden_dim, Hg = a.g[dir].hidden_dim;
-        job(a.H[dir], d, d, a.X, F, nullptr, 0, a.DFH[dir], Hf, Hf, R, a.gf[dir].W1, a.gf[dir].b1);
-        job(a.FH[dir], Hf, Hf, nullptr, 0, nullptr, 0, a.DPRE_F2[dir], d, d, R, a.gf[dir].W2, a.gf[dir].b2);
-        job(a.Sg[dir], d, d, nullptr, 0, nullptr, 0, a.DT1[dir], Hg, Hg, R, a.gg[dir].W1, a.gg[dir].b1);
-        job(a.T1[dir], Hg, Hg, nullptr, 0, nullptr, 0, a.DPRE_G2[dir], d, d, R, a.gg[dir].W2, a.gg[dir].b2);
+        job(a.H[dir], d, d, a.X, F, nullptr, 0, a.DFH[dir], Hf, Hf, true, a.gf[dir].W1, a.gf[dir].b1, row_chunks);
+        job(a.FH[dir], Hf, Hf, nullptr, 0, nullptr, 0, a.DPRE_F2[dir], d, d, true, a.gf[dir].W2, a.gf[dir].b2, row_chunks);
+        job(a.Sg[dir], d, d, nullptr, 0, nullptr, 0, a.DT1[dir], Hg, Hg, true, a.gg[dir].W1, a.gg[dir].b1, row_chunks);
+        job(a.T1[dir], Hg, Hg, nullptr, 0, nullptr, 0, a.DPRE_G2[dir], d, d, true, a.gg[dir].W2, a.gg[dir].b2, row_chunks);
     }
     for (int i = 0; i < 3; ++i) {
-        job(a.H[0], d, d, a.H[1], d, a.X, F, a.DPRE_L[i], d, d, R, a.gl[i].W1, a.gl[i].b1);
+        job(a.H[0], d, d, a.H[1], d, a.X, F, a.DPRE_L[i], d, d, true, a.gl[i].W1, a.gl[i].b1, pool_chunks);
         // h_i: rows are states; the inputs and gradients of set i sit at column offset i * d of [B][3][d]
-        job(a.Sbuf + i * d, d, 3 * d, nullptr, 0, nullptr, 0, a.DPRE_H + i * d, 3 * d, d, B, a.gh[i].W1, a.gh[i].b1);
+        job(a.Sbuf + i * d, d, 3 * d, nullptr, 0, nullptr, 0, a.DPRE_H + i * d, 3 * d, d, false, a.gh[i].W1, a.gh[i].b1);
     }
-    job(a.Zbuf, Z, Z, nullptr, 0, nullptr, 0, a.DHID, Hh, Hh, B, a.ghead.W1, a.ghead.b1);
-    job(a.HID, Hh, Hh, nullptr, 0, nullptr, 0, a.DLOG, m, m, B, a.ghead.W2, a.ghead.b2);
-    err = weight_grads(by_row, stream);
+    job(a.Zbuf, Z, Z, nullptr, 0, nullptr, 0, a.DHID, Hh, Hh, false, a.ghead.W1, a.ghead.b1);
+    job(a.HID, Hh, Hh, nullptr, 0, nullptr, 0, a.DLOG, m, m, false, a.ghead.W2, a.ghead.b2);
+    if (split) {
+        float *rows[8], *pool[3];
+        for (int k = 0; k < 8; ++k) rows[k] = by_row.job[k].partial;
+        for (int k = 0; k < 3; ++k) pool[k] = by_row.job[8 + k].partial;
+        err = launch_grad_weights_split(a, rows, row_chunks, pool, pool_chunks, stream);
+        if (err != cudaSuccess) return err;
+    }
+    err = weight_grads(by_row, stream, !split);
     if (err != cudaSuccess) return err;
-    return weight_grads(by_state, stream);
+    return weight_grads(by_state, stream, true);
 }
 
 }  // namespace placeto

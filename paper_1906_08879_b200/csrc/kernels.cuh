@@ -194,6 +194,11 @@ struct GradArgs {
     float *DPRE_L[3], *Zbuf, *HID, *DHID, *DLOG, *Sbuf, *DPRE_H;
     unsigned *masks[2];        // one bit per ReLU of every row (grad_sweep.cu)
     int max_level_width;
+    // the passes of grad_pool.cu: sums per chunk of nodes [chunk][B][3][d], their gradients [B][3][d], the gradient of
+    // the current node's embedding [B][2 d], one bit per pooled row and column [row][d / 32]
+    int pool_chunk_nodes, pool_chunks;
+    float *pool_partial, *dS, *dZ;
+    unsigned *l_masks;
     GradOut gf[2], gg[2], gl[3], gh[3], ghead;
 };
 
@@ -303,7 +308,7 @@ cudaError_t launch_simulator(const SimArgs &a, const DeviceInfo &di, cudaStream_
 
 // gradient.cu: gradient of the policy objective with respect to all weights
 bool policy_gradient_applicable(const GradArgs &a);
-size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh);
+size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh, int pool_chunks);
 cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, cudaStream_t stream);
 
 // grad_sweep.cu: the passes over the node-state rows for d = 32 / 64 with hidden width d: forward values and masks of
@@ -311,6 +316,13 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
 bool grad_split_applicable(const GradArgs &a, const DeviceInfo &di);
 cudaError_t launch_grad_rows(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream);
 cudaError_t launch_grad_sweep_split(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream);
+
+// grad_pool.cu: the passes through the pooling networks and the per-row weight gradients of the same shapes
+void grad_pool_chunks(int n, int B, const DeviceInfo &di, int *chunk_nodes, int *chunks);
+cudaError_t launch_grad_pool_forward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream);
+cudaError_t launch_grad_pool_backward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream);
+cudaError_t launch_grad_weights_split(const GradArgs &a, float *const (&rows)[8], int row_chunks, float *const (&pool)[3],
+                                      int pool_chunks, cudaStream_t stream);
 
 // writes the d x d identity matrix followed by d zeros (an identity layer: W2 = I, b2 = 0)
 cudaError_t launch_identity_layer(float *dst, int d, cudaStream_t stream);

@@ -143,3 +143,14 @@ def test_split_sweep_over_tiles(d, m, B, layers):
     adv = adv.astype(np.float32).astype(np.float64)
     grads = gpu_gradient(cfg, actions, adv, 0.1)
     compare(cfg, grads, gradient.gradient(cfg, actions, adv, 0.1))
+
+
+@pytest.mark.parametrize("d,m,n,B", [(32, 3, 150, 2), (64, 8, 140, 3), (64, 4, 300, 1)])
+def test_pooling_passes_over_chunks_of_nodes(d, m, n, B):
+    """More chunks of nodes than one (few states), sets of fewer rows than a warp's batch and of many batches, states
+    whose current node lies in each chunk."""
+    cfg, actions, adv = small_case(d + n, n=n, m=m, d=d, B=B, p=0.02)
+    cfg["cur"] = np.linspace(0, n - 1, B).astype(np.int32)
+    adv = adv.astype(np.float32).astype(np.float64)
+    grads = gpu_gradient(cfg, actions, adv, 0.1)
+    compare(cfg, grads, gradient.gradient(cfg, actions, adv, 0.1))
