@@ -200,8 +200,10 @@ placeto_status cuda_status(cudaError_t e) {
 placeto_status run_embed(const placeto_graph *g, const placeto_weights *w, const float *X, int B,
                          float *H_down, float *H_up, char *ws, const Layout &L, uint32_t flags,
                          cudaStream_t stream, const StatusSlot &status, bool after_own_kernel = false,
-                         const CompactState *compact = nullptr, bool embeddings_returned = false) {
+                         const CompactState *compact = nullptr, bool embeddings_returned = false,
+                         EpisodeWalk walk = EpisodeWalk{nullptr, 0}) {
     EmbedArgs a;
+    a.walk = walk;
     a.status = status;
     a.compact = compact ? *compact : CompactState{};
     a.lv[0] = g->lv[0]; a.lv[1] = g->lv[1];
@@ -377,15 +379,22 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
     if (cudaDeviceGetAttribute(&g->info.sm_count, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&g->info.max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device) != cudaSuccess)
         return fail(PLACETO_ERR_CUDA);
-    // one int allocation: per direction level_ptr, order, nbr_ptr, nbr, own_slot, nbr_slot
+    // one int allocation: per direction level_ptr, order, nbr_ptr, nbr, own_slot, nbr_slot, level of a node
     // (each padded to 4 ints)
-    constexpr int kArrays = 6;
+    constexpr int kArrays = 7;
+    std::vector<int32_t> level_of[2];
+    for (int dir = 0; dir < 2; ++dir) {
+        const LevelPlan &p = g->host.dir[dir];
+        level_of[dir].resize(g->host.n);
+        for (int l = 0; l < p.n_levels; ++l)
+            for (int q = p.level_ptr[l]; q < p.level_ptr[l + 1]; ++q) level_of[dir][p.order[q]] = l;
+    }
     size_t total = 0;
     size_t offs[2][kArrays];
     for (int dir = 0; dir < 2; ++dir) {
         const LevelPlan &p = g->host.dir[dir];
         const size_t sizes[kArrays] = {p.level_ptr.size(), p.order.size(), p.nbr_ptr.size(),
-                                       p.nbr.size(), p.own_slot.size(), p.nbr_slot.size()};
+                                       p.nbr.size(), p.own_slot.size(), p.nbr_slot.size(), level_of[dir].size()};
         for (int k = 0; k < kArrays; ++k) { offs[dir][k] = total; total += (sizes[k] + 3) & ~size_t(3); }
     }
     // and, by node id: children and their entries in the parent lists (runtime simulator), parents (policy gradient)
@@ -400,7 +409,7 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
     for (int dir = 0; dir < 2; ++dir) {
         const LevelPlan &p = g->host.dir[dir];
         const std::vector<int32_t> *vecs[kArrays] = {&p.level_ptr, &p.order, &p.nbr_ptr,
-                                                     &p.nbr, &p.own_slot, &p.nbr_slot};
+                                                     &p.nbr, &p.own_slot, &p.nbr_slot, &level_of[dir]};
         for (int k = 0; k < kArrays; ++k)
             if (!vecs[k]->empty() &&
                 cudaMemcpy(g->d_ints + offs[dir][k], vecs[k]->data(), vecs[k]->size() * sizeof(int),
@@ -414,6 +423,7 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
         g->lv[dir].n_slots = p.n_slots;
         g->lv[dir].own_slot = g->d_ints + offs[dir][4];
         g->lv[dir].nbr_slot = g->d_ints + offs[dir][5];
+        g->lv[dir].level_of = g->d_ints + offs[dir][6];
         g->lv[dir].n_nbr = static_cast<int>(p.nbr.size());
     }
     {
@@ -722,6 +732,7 @@ placeto_status placeto_embed_rounds(const placeto_graph *g, const placeto_weight
     char *ws = static_cast<char *>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     EmbedArgs a;
+    a.walk = EpisodeWalk{nullptr, 0};
     a.lv[0] = g->lv[0]; a.lv[1] = g->lv[1];
     a.f[0] = to_dev(w->f_down); a.f[1] = to_dev(w->f_up);
     a.g[0] = to_dev(w->g_down); a.g[1] = to_dev(w->g_up);
@@ -812,7 +823,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
         step.logp = logp; step.actions = actions;
         for (int t = 0; s == PLACETO_OK && t < ep.n; ++t) {
             step.t = t;
-            s = run_embed(g, w, nullptr, E, Hd, Hu, ws, L, flags, st, status, true, &cs);
+            s = run_embed(g, w, nullptr, E, Hd, Hu, ws, L, flags, st, status, true, &cs, false, EpisodeWalk{order, t});
             if (s == PLACETO_OK)
                 s = run_pool(g, w, nullptr, Hd, Hu, ep.cur, E, const_cast<float *>(ep.logits), probs, ws, L, flags, st,
                              status, true, &cs, &step);
@@ -826,7 +837,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
         s = cuda_status(launch_features(ep.n, E, w->m, cost, bytes, dev, ep.cur, ep.placed, X, st));
     for (int t = 0; s == PLACETO_OK && t < ep.n; ++t) {
         // one policy evaluation of the E current states, then the transition
-        s = run_embed(g, w, X, E, Hd, Hu, ws, L, flags, st, status, true);
+        s = run_embed(g, w, X, E, Hd, Hu, ws, L, flags, st, status, true, nullptr, false, EpisodeWalk{order, t});
         if (s == PLACETO_OK)
             s = run_pool(g, w, X, Hd, Hu, ep.cur, E, const_cast<float *>(ep.logits), probs, ws, L, flags, st, status, true);
         if (s == PLACETO_OK) s = cuda_status(launch_episode_step(ep, t, st));

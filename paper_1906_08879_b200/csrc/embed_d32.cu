@@ -103,12 +103,12 @@ struct Weights32 {
 // gather -> g -> store h -> f -> store m. The R rows share the node, so the
 // schedule lookups are done once. A, Bf: the warp's exchange buffers, R rows of
 // KF floats each. All shared-memory offsets are 32-bit.
-template <int R, int KF, int L>   // L layers per network
+template <int R, int KF, int L, bool kWalk>   // L layers per network; kWalk: messages also go to memory
 __device__ __forceinline__ void run_node(const Weights32 &w, const pair_t (&wf1)[KF / 2], int pos,
                                          int q, int s0, bool last_live, int nb, int S, int F,
                                          int lane, const int4 *meta, const int *nbr_slot,
                                          float *msg, const float *xs, float *__restrict__ H,
-                                         size_t B, int b_first, float *A, float *Bf) {
+                                         float *__restrict__ M, size_t B, int b_first, float *A, float *Bf) {
     int st[R];
     float x[R], acc[R];
 #pragma unroll
@@ -181,10 +181,15 @@ after_g1:
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
-        if (r == 0 || last_live) msg[((slot * S) + st[r]) * kD + lane] = fmaxf(acc[r], 0.f);
+        if (r == 0 || last_live) {
+            const float v_m = fmaxf(acc[r], 0.f);
+            msg[((slot * S) + st[r]) * kD + lane] = v_m;
+            if constexpr (kWalk) M[((size_t)v * B + b_first + s0 + r) * kD + lane] = v_m;
+        }
 }
 
-template <int F4, bool kCompact, int L>   // feature width padded to 4 * F4; features built from compact states; layers
+// feature width padded to 4 * F4; features built from compact states; layers; a sweep of an episode
+template <int F4, bool kCompact, int L, bool kWalk>
 __global__ void __launch_bounds__(kThreads, 1)
 embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     constexpr int KF = kD + 4 * F4;      // padded input width of f's first layer
@@ -281,12 +286,23 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
         }
         __pipeline_commit();
     };
+    const int start = kWalk ? first_level(a.walk, lv, a.n) : 0;
     dependency_wait();          // the raw features may come from a kernel that is still running
-    prefetch(0);
+    prefetch(start);
+    float *__restrict__ M = a.M[dir];
+    if (kWalk && start > 0) {
+        // messages from above `start` that it or a later level reads: a slot belongs to its node until then
+        for (int e = meta[level_ptr[start]].x + warp; e < lv.n_nbr; e += kWarps) {
+            const int u = lv.nbr[e];
+            if (lv.level_of[u] >= start) continue;
+            const int slot = nbr_slot[e];
+            for (int s = 0; s < nb; ++s) msg[(slot * p.S + s) * kD + lane] = M[((size_t)u * B + b_first + s) * kD + lane];
+        }
+    }
     __pipeline_wait_prior(0);
     __syncthreads();
 
-    for (int level = 0; level < lv.n_levels; ++level) {
+    for (int level = start; level < lv.n_levels; ++level) {
         if (level + 1 < lv.n_levels) prefetch(level + 1);
         const int p0 = level_ptr[level];
         const int rows = (level_ptr[level + 1] - p0) * nb;
@@ -297,8 +313,8 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
             if (warp < rows) {
                 const int q = nb == 1 ? warp : (int)__umulhi((unsigned)warp, magic_nb);
                 const int s0 = warp - q * nb;
-                run_node<1, KF, L>(w, wf1, p0 + q, q, s0, true, nb, p.S, F, lane, meta, nbr_slot, msg,
-                                xs, H, B, b_first, A, Bf);
+                run_node<1, KF, L, kWalk>(w, wf1, p0 + q, q, s0, true, nb, p.S, F, lane, meta, nbr_slot, msg,
+                                xs, H, M, B, b_first, A, Bf);
             }
         } else {
             // two states of one node per warp pass
@@ -306,8 +322,8 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
             for (int item = warp; item < width * ppn; item += kWarps) {
                 const int q = ppn == 1 ? item : (int)__umulhi((unsigned)item, magic_ppn);
                 const int s0 = (item - q * ppn) * 2;
-                run_node<2, KF, L>(w, wf1, p0 + q, q, s0, s0 + 1 < nb, nb, p.S, F, lane, meta, nbr_slot,
-                                msg, xs, H, B, b_first, A, Bf);
+                run_node<2, KF, L, kWalk>(w, wf1, p0 + q, q, s0, s0 + 1 < nb, nb, p.S, F, lane, meta, nbr_slot,
+                                msg, xs, H, M, B, b_first, A, Bf);
             }
         }
         __pipeline_wait_prior(0);
@@ -379,12 +395,14 @@ cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStrea
     if (!plan_d32(a, di, &p)) return cudaErrorNotSupported;
     const int F4 = (a.F + 3) / 4;
     typedef void (*Kernel)(const EmbedArgs, const D32Plan);
-    static const Kernel kernels[2][2][4] = {     // [layers][compact][F4]
-        {{embed_d32_kernel<1, false, 1>, embed_d32_kernel<2, false, 1>, embed_d32_kernel<3, false, 1>, embed_d32_kernel<4, false, 1>},
-         {embed_d32_kernel<1, true, 1>, embed_d32_kernel<2, true, 1>, embed_d32_kernel<3, true, 1>, embed_d32_kernel<4, true, 1>}},
-        {{embed_d32_kernel<1, false, 2>, embed_d32_kernel<2, false, 2>, embed_d32_kernel<3, false, 2>, embed_d32_kernel<4, false, 2>},
-         {embed_d32_kernel<1, true, 2>, embed_d32_kernel<2, true, 2>, embed_d32_kernel<3, true, 2>, embed_d32_kernel<4, true, 2>}}};
-    const Kernel kern = kernels[a.f[0].n_layers - 1][a.compact.state != nullptr][F4 - 1];
+#define PLACETO_D32_KERNELS(compact, layers, walk) \
+    {embed_d32_kernel<1, compact, layers, walk>, embed_d32_kernel<2, compact, layers, walk>, \
+     embed_d32_kernel<3, compact, layers, walk>, embed_d32_kernel<4, compact, layers, walk>}
+    static const Kernel kernels[2][3][4] = {     // [layers][X, X in an episode, compact states (always an episode)][F4]
+        {PLACETO_D32_KERNELS(false, 1, false), PLACETO_D32_KERNELS(false, 1, true), PLACETO_D32_KERNELS(true, 1, true)},
+        {PLACETO_D32_KERNELS(false, 2, false), PLACETO_D32_KERNELS(false, 2, true), PLACETO_D32_KERNELS(true, 2, true)}};
+#undef PLACETO_D32_KERNELS
+    const Kernel kern = kernels[a.f[0].n_layers - 1][a.compact.state != nullptr ? 2 : a.walk.order != nullptr ? 1 : 0][F4 - 1];
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)p.smem_bytes);
     if (err != cudaSuccess) return err;

@@ -115,7 +115,11 @@ embed_generic_kernel(const EmbedArgs a, const GenericPlan p) {
 
     // In the cooperative schedule every block runs the same number of rounds.
     const int last = kCooperative ? p.level_end : min(p.level_end, lv.n_levels);
-    for (int level = p.level_begin; level < last; ++level) {
+    // A sweep of an episode starts where the features changed: the messages of the levels above are where the step
+    // before left them. With grid-wide barriers both directions start together.
+    int start = first_level(a.walk, lv, a.n);
+    if (kCooperative) start = min(start, first_level(a.walk, a.lv[1 - dir], a.n));
+    for (int level = max(p.level_begin, start); level < last; ++level) {
         if (level < lv.n_levels) {
             // a synchronous round treats all nodes as one level
             const int p0 = p.round_mode ? 0 : lv.level_ptr[level];

@@ -15,8 +15,7 @@
 //
 // A level is a serial chain (gather, four layers), so what is not arithmetic of the tile
 // is taken off it: four helper warps work a level ahead, turning the schedule into one
-// record per row and the raw features (cp.async, two levels ahead, or compact states) into
-// pieces.
+// record per row and the raw features (cp.async, two levels ahead) into pieces.
 //
 // Measured on a B200, message passing alone, against the kernels it replaced (d = 64: a pipeline of layers on TF32
 // mma.sync, a warpgroup per layer; single layers: the dimension-generic kernel), us:
@@ -80,7 +79,7 @@ struct SplitPlan {
 // a matrix's bounds: |out| <= norm * max |in| + bias (largest over the columns)
 struct Bound { float norm, bias; };
 
-template <typename C, bool kCompact>
+template <typename C, bool kWalk>     // kWalk: a sweep of an episode
 __global__ void __launch_bounds__(kThreads, 1)
 embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
     typedef typename C::SP SP;
@@ -97,6 +96,7 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
     const int b_first = blockIdx.x * S;
     const int nb = min(S, B - b_first);
     const int n_levels = lv.n_levels;
+    const int start = kWalk ? first_level(a.walk, lv, a.n) : 0;
 
     // ---- shared memory: [schedule][message slots][raw features x2][bounds][row tiles x2][tiles of every group]
     //   meta[p] = {first neighbour entry, end of neighbour entries, own slot, node id}
@@ -149,13 +149,6 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
             if (level < n_levels) {
                 const int p0 = level_ptr[level], width = level_ptr[level + 1] - p0;
                 float *dst = xstage + (size_t)(level & 1) * p.x_floats;
-                if (kCompact) {
-#pragma unroll 1
-                    for (int i = ht; i < width * nb; i += kHelperThreads) {       // one (node, state) pair per thread
-                        const int q = node_of_row(i), s = i - q * nb;
-                        compact_features(a.compact, meta[p0 + q].w, b_first + s, B, dst + (size_t)i * F);
-                    }
-                } else {
 #pragma unroll 1
                     for (int i = ht; i < width * per; i += kHelperThreads) {
                         const int q = per == 1 ? i : (int)__umulhi((unsigned)i, magic_per);
@@ -164,7 +157,6 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
                         if (vec) __pipeline_memcpy_async(dst + q * per_node + 4 * piece, src + 4 * piece, 16);
                         else __pipeline_memcpy_async(dst + q * per_node + piece, src + piece, 4);
                     }
-                }
             }
             __pipeline_commit();
         };
@@ -207,14 +199,24 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
         };
         __syncthreads();              // schedule staged
         dependency_wait();            // the raw features may come from a kernel that is still running
-        fetch(0);
-        fetch(1);
+        fetch(start);
+        fetch(start + 1);
+        if (kWalk && start > 0) {
+            // messages from above `start` that it or a later level reads: a slot belongs to its node until then
+            for (int e = meta[level_ptr[start]].x + (ht >> 5); e < lv.n_nbr; e += kHelperThreads / 32) {
+                const int u = lv.nbr[e];
+                if (lv.level_of[u] >= start) continue;
+                const int slot = nbr_slot[e];
+                for (int i = lane; i < nb * D; i += 32)
+                    msg[(slot * S + i / D) * P + i % D] = a.M[dir][((size_t)u * B + b_first) * D + i];
+            }
+        }
         __pipeline_wait_prior(1);
         group_sync<kHelperThreads>(kHelperBar);
-        publish(0);
+        publish(start);
         __syncthreads();
 #pragma unroll 1
-        for (int level = 0; level < n_levels; ++level) {
+        for (int level = start; level < n_levels; ++level) {
             if (level + 1 < n_levels) {
                 fetch(level + 2);
                 __pipeline_wait_prior(1);
@@ -441,15 +443,20 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
                 if (kept) {
                     m[col] = v[i][e];
                     m[col + 8] = v[i][2 + e];
+                    if constexpr (kWalk) {
+                        float *mg = a.M[dir] + (size_t)(unsigned)to[i][e].x * D + col;
+                        mg[0] = v[i][e];
+                        mg[8] = v[i][2 + e];
+                    }
                 }
             }
     };
 
-    int n_tiles = (level_ptr[1] * nb + kTile - 1) / kTile, first = level_ptr[1];
+    int first = level_ptr[start + 1], n_tiles = ((first - level_ptr[start]) * nb + kTile - 1) / kTile;
     const unsigned char *mine = row_tiles + group * (int)C::kRowTile;
-    __syncthreads();                                     // level 0 published
+    __syncthreads();                                     // the first level published
 #pragma unroll 1
-    for (int level = 0; level < n_levels; ++level) {
+    for (int level = start; level < n_levels; ++level) {
         const int next = level_ptr[min(level + 2, n_levels)];
         const unsigned char *info = mine + (level & 1) * p.row_bytes;
         int left = n_tiles - group;                      // this group takes every G-th tile
@@ -495,7 +502,7 @@ cudaError_t launch(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream
     p.x_floats = x_floats(p.S);
     p.row_bytes = row_bytes(p.S);
     p.smem_bytes = need(p.S);
-    auto kern = a.compact.state != nullptr ? embed_split_kernel<C, true> : embed_split_kernel<C, false>;
+    auto kern = a.walk.order != nullptr ? embed_split_kernel<C, true> : embed_split_kernel<C, false>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);
     if (err != cudaSuccess) return err;
     err = launch_overlapped(overlap, kern, dim3(p.n_slices, 2), dim3(kThreads), p.smem_bytes, stream, a, p);

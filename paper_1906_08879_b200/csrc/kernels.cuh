@@ -23,6 +23,7 @@ struct DevLevels {
     //   pos4[p]     = {first neighbour entry, end of neighbour entries, own slot, node id}
     const int4 *lvl4, *pos4;
     int max_level_nbr;               // most neighbour entries in one level
+    const int *level_of;             // [n] level of a node id
 };
 
 // One feed-forward network with device pointers.
@@ -123,6 +124,23 @@ struct EpisodeStep {
     uint8_t *actions;          // [E][n] by step, or null
 };
 
+// Consecutive sweeps of an episode batch on the same buffers: between steps t - 1 and t only the features of
+// order[t - 1] (placed) and order[t] (now current) change, so levels above both keep their embeddings and
+// messages. A sweep given a walk stores every message in M beside its slot and starts at first_level(); the
+// messages that later levels read from above come back from M.
+struct EpisodeWalk {
+    const int *order;      // [n], or null: a sweep on its own
+    int t;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ int first_level(const EpisodeWalk &w, const DevLevels &lv, int n) {
+    if (w.order == nullptr || w.t == 0) return 0;
+    const int u = w.order[w.t - 1], v = w.order[w.t];
+    if (u < 0 || u >= n || v < 0 || v >= n) return 0;
+    return min(lv.level_of[u], lv.level_of[v]);
+}
+#endif
+
 struct EmbedArgs {
     DevLevels lv[2];
     DevMlp f[2], g[2];
@@ -133,6 +151,7 @@ struct EmbedArgs {
     int max_level_width;   // widest level over both directions
     StatusSlot status;
     CompactState compact;  // compact.state != null: X is not read
+    EpisodeWalk walk;
 };
 
 struct PoolArgs {

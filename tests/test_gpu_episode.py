@@ -110,6 +110,25 @@ def test_reverse_order_and_single_episode():
     compare(cfg, order, dev0, uni, got, min_full=0)
 
 
+@pytest.mark.parametrize("d,m,layers,flags", [(32, 4, 2, 0), (32, 3, 1, 0), (32, 8, 1, 0), (64, 8, 2, 0), (64, 3, 1, 0), (8, 3, 2, 0),
+                                              (8, 2, 1, placeto.PLACETO_COOPERATIVE), (8, 2, 2, placeto.PLACETO_PER_LEVEL)])
+def test_sweeps_that_start_where_the_features_changed(d, m, layers, flags):
+    """A step of an episode redoes the levels from the changed nodes on and reads the messages above from memory:
+    long edges that skip levels, several episodes per block, visiting orders that jump up and down the graph."""
+    r = rng(d + m)
+    n = 30
+    src = list(range(n - 1)) + list(range(0, n - 9, 4)) + [0, 0, 3]
+    dst = list(range(1, n)) + [i + 9 for i in range(0, n - 9, 4)] + [n - 1, n // 2, n - 2]
+    cfg = {"n": n, "src": np.asarray(src, np.int32), "dst": np.asarray(dst, np.int32), "m": m, "d": d, "F": m + 4}
+    cfg["cost"], cfg["bytes"] = states.node_costs(r, n, normalise=True)
+    cfg["weights"] = states.policy_weights(r, d, m + 4, m, layers, 0, 0.1)
+    dev0 = r.integers(0, m, size=(80, n)).astype(np.uint8)
+    uni = r.random(size=(80, n))
+    for order in (np.arange(n), np.arange(n)[::-1].copy(), r.permutation(n)):
+        got = run_gpu(cfg, order, dev0, uni, flags)
+        compare(cfg, order, dev0, uni, got, min_full=50)
+
+
 def test_one_node_graph():
     r = rng(3)
     m, d = 4, 32
