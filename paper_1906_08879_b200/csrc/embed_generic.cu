@@ -12,7 +12,7 @@
 //                direction, ordering them with __syncthreads() only
 //   COOPERATIVE  one persistent cooperative launch; the nodes of a level are also
 //                spread over several blocks, with a grid-wide sync per level
-// This file is the dimension-generic fallback: one thread per output element,
+// This file is the dimension-generic fallback (above 32 columns; embed_small.cu below): one thread per output element,
 // weights staged in shared memory when they fit.
 #include <cooperative_groups.h>
 

@@ -1,0 +1,255 @@
+// Step 2 of the policy (Sec. 2.2 step 2 of the Placeto paper) for narrow networks: every layer of f
+// and g at most 32 wide, one or two layers, any activation:
+//   h_v = g( sum_{u in nbr(v)} m_u ),   m_u = f([h_u || x_u]).
+//
+// The widths that have no kernel of their own ran on the dimension-generic one, which takes a level
+// in eight block-wide phases and passes messages through global memory: 4 us per level of a 32-node
+// graph at d = 8, all of it latency. Here a row (node, state) belongs to 8, 16 or 32 lanes of a warp
+// from the gather to the message, a lane keeps its column of every matrix in registers, the messages
+// (slots assigned on the host) stay in shared memory, raw features arrive by cp.async two levels
+// ahead, a row's record and first neighbours are read during the level before, and a level costs one
+// block barrier. What is left is the chain gather -> g -> f of a level, about 1 us with four
+// neighbours, 0.6 us with one. Measured on a B200 (this kernel, the generic one): 32 nodes in 8
+// levels, d = 8, 16 states: 10.8, 32 us; 160 nodes in 40 levels, 1024 states: 61, 326 us; 318 nodes
+// in modules, d = 16, 256 states: 129, 455 us; d = 24, 1024 states: 600, 1684 us. The bits are the
+// generic kernel's: every sum is taken in its order.
+#include <cuda_pipeline.h>
+
+#include <algorithm>
+
+#include "kernels.cuh"
+
+namespace placeto {
+
+namespace {
+
+constexpr int kWarps = 8, kThreads = 32 * kWarps;
+constexpr int kMaxF = 16;
+constexpr int kAhead = 4;     // neighbours whose slots are read ahead
+
+struct SmallPlan {
+    int S, n_slices;
+    int x_floats;          // floats of one feature staging buffer
+    size_t smem_bytes;
+};
+
+// Floats of a row's exchange buffers: the input of g, the hidden layer, the input of f. Whatever lies behind the
+// columns that a network has stays zero.
+template <int LW> struct RowBuffer { static constexpr int kHidden = LW, kMessage = 2 * LW, kFloats = 3 * LW + kMaxF; };
+
+template <int LW>     // lanes of a row
+__global__ void __launch_bounds__(kThreads)
+embed_small_kernel(const EmbedArgs a, const SmallPlan p) {
+    constexpr int kRows = 32 / LW;                       // rows of a warp at a time
+    using Buffer = RowBuffer<LW>;
+    extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
+    const int dir = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j = lane % LW, part = lane / LW;
+    const DevLevels lv = a.lv[dir];
+    const DevMlp f = a.f[dir], g = a.g[dir];
+    const int d = a.d, F = a.F, B = a.B, S = p.S;
+    const int b_first = blockIdx.x * S, nb = min(S, B - b_first);
+
+    // ---- shared memory: [raw features x3][row buffers][schedule][message slots]
+    float *xstage = smem, *bufs = smem + 3 * (size_t)p.x_floats;
+    int *ints = reinterpret_cast<int *>(bufs + kWarps * kRows * Buffer::kFloats);
+    int4 *meta = reinterpret_cast<int4 *>(ints);         // {first neighbour entry, end, own slot, node}
+    int *level_ptr = ints + 4 * a.n, *nbr_slot = level_ptr + lv.n_levels + 1;
+    float *msg = reinterpret_cast<float *>(nbr_slot + lv.n_nbr);        // [n_slots][S][d]
+#pragma unroll 1
+    for (int i = threadIdx.x; i < a.n; i += kThreads) __pipeline_memcpy_async(meta + i, lv.pos4 + i, 16);
+#pragma unroll 1
+    for (int i = threadIdx.x; i <= lv.n_levels; i += kThreads) __pipeline_memcpy_async(level_ptr + i, lv.level_ptr + i, 4);
+#pragma unroll 1
+    for (int i = threadIdx.x; i < lv.n_nbr; i += kThreads) __pipeline_memcpy_async(nbr_slot + i, lv.nbr_slot + i, 4);
+    __pipeline_commit();
+    for (int i = threadIdx.x; i < kWarps * kRows * Buffer::kFloats; i += kThreads) bufs[i] = 0.f;
+
+    // Lane j of a row keeps column j of every matrix, zeros behind the last row and column.
+    float gW1[LW], gW2[LW], fW1[LW + kMaxF], fW2[LW];
+    const int hg = g.hidden_dim, hf = f.hidden_dim;
+    auto column = [&](const float *W, int k, int K, int N) { return k < K && j < N ? W[k * N + j] : 0.f; };
+#pragma unroll
+    for (int k = 0; k < LW; ++k) gW1[k] = column(g.W1, k, d, hg);
+#pragma unroll
+    for (int k = 0; k < LW + kMaxF; ++k) fW1[k] = column(f.W1, k, d + F, hf);
+#pragma unroll
+    for (int k = 0; k < LW; ++k) {
+        gW2[k] = g.n_layers == 2 ? column(g.W2, k, hg, d) : 0.f;
+        fW2[k] = f.n_layers == 2 ? column(f.W2, k, hf, d) : 0.f;
+    }
+    const float gb1 = j < hg ? g.b1[j] : 0.f, gb2 = g.n_layers == 2 && j < d ? g.b2[j] : 0.f;
+    const float fb1 = j < hf ? f.b1[j] : 0.f, fb2 = f.n_layers == 2 && j < d ? f.b2[j] : 0.f;
+    PLACETO_DEBUG_CHECK(a.status, nb >= 1 && b_first + nb <= B);
+    __pipeline_wait_prior(0);
+    __syncthreads();
+    const int start = first_level(a.walk, lv, a.n);
+    auto prefetch = [&](int level) {
+        if (level < lv.n_levels) {
+            const int p0 = level_ptr[level], width = level_ptr[level + 1] - p0;
+            float *dst = xstage + (size_t)(level % 3) * p.x_floats;
+            for (int q = kWarps - 1 - warp; q < width; q += kWarps) {        // the last warps have the fewest rows
+                const float *src = a.X + ((size_t)meta[p0 + q].w * B + b_first) * F;
+                for (int i = lane; i < nb * F; i += 32) __pipeline_memcpy_async(dst + q * nb * F + i, src + i, 4);
+            }
+        }
+        __pipeline_commit();
+    };
+    dependency_wait();          // the raw features may come from a kernel that is still running
+    prefetch(start);
+    prefetch(start + 1);
+    if (start > 0) {            // an episode's sweep: messages from above that a later level reads
+        for (int e = meta[level_ptr[start]].x + warp; e < lv.n_nbr; e += kWarps) {
+            const int u = lv.nbr[e];
+            if (lv.level_of[u] >= start) continue;
+            for (int i = lane; i < nb * d; i += 32)
+                msg[nbr_slot[e] * S * d + i] = a.M[dir][((size_t)u * B + b_first) * d + i];
+        }
+    }
+    __pipeline_wait_prior(1);
+    __syncthreads();
+
+    // bias + in W for this lane's column, one chain, k ascending: the bits are the generic kernel's
+    auto column_sum = [&](auto &w, float c, const float *in, int K) {
+        constexpr int kMost = sizeof(w) / sizeof(float);
+#pragma unroll
+        for (int k = 0; k < kMost; k += 4) {
+            if (k < LW || k < K) {
+                const float4 x = *reinterpret_cast<const float4 *>(in + k);
+                c = fmaf(x.x, w[k], c);
+                c = fmaf(x.y, w[k + 1], c);
+                c = fmaf(x.z, w[k + 2], c);
+                c = fmaf(x.w, w[k + 3], c);
+            }
+        }
+        return c;
+    };
+    auto act = [](bool relu, float v) { return relu ? fmaxf(v, 0.f) : v; };
+    float *sums = bufs + (warp * kRows + part) * Buffer::kFloats, *hidden = sums + Buffer::kHidden, *input = sums + Buffer::kMessage;
+    const bool g_first = g.act == 0 && (g.n_layers == 2 || g.final_act), g_last = g.act == 0 && g.final_act;
+    const bool f_first = f.act == 0 && (f.n_layers == 2 || f.final_act), f_last = f.act == 0 && f.final_act;
+    const unsigned per_state = nb > 1 ? 0xffffffffu / nb + 1 : 0;       // r / nb, exact for r < 2^32 / nb
+    // A pass's record and first neighbours depend on the schedule only: a warp's first pass of a level has them read
+    // during the level before, so that its gather starts with the messages.
+    struct Record { int r, s; int4 m; const float *first[kAhead]; };
+    auto record = [&](int p0, int rows, int base) {
+        Record c;
+        c.r = base + part < rows ? base + part : base;   // idle lanes shadow the warp's first row
+        const int q = nb > 1 ? __umulhi(c.r, per_state) : c.r;
+        c.s = c.r - q * nb;
+        c.m = meta[p0 + q];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i)
+            c.first[i] = msg + ((c.m.x + i < c.m.y ? nbr_slot[c.m.x + i] : 0) * S + c.s) * d + min(j, d - 1);
+        return c;
+    };
+    int p0 = level_ptr[start], rows = (level_ptr[start + 1] - p0) * nb;
+    Record c = record(p0, rows, min(warp * kRows, rows - 1));
+    for (int level = start; level < lv.n_levels; ++level) {
+        const float *xs = xstage + (size_t)(level % 3) * p.x_floats;
+        for (int base = warp * kRows; base < rows; base += kWarps * kRows) {
+            if (base > warp * kRows) c = record(p0, rows, base);
+            const bool live = base + part < rows;
+            const int r = c.r, s = c.s;
+            const int4 m = c.m;
+            float u[kAhead], v = 0.f;
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) u[i] = m.x + i < m.y ? *c.first[i] : 0.f;
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) v += u[i];
+            const float *from = msg + s * d + min(j, d - 1);
+            int e = m.x + kAhead;
+            for (; e + 4 <= m.y; e += 4) {
+                const float u0 = from[nbr_slot[e] * S * d], u1 = from[nbr_slot[e + 1] * S * d];
+                const float u2 = from[nbr_slot[e + 2] * S * d], u3 = from[nbr_slot[e + 3] * S * d];
+                v += u0;
+                v += u1;
+                v += u2;
+                v += u3;
+            }
+            for (; e < m.y; ++e) v += from[nbr_slot[e] * S * d];
+            if (j < d) sums[j] = v;
+#pragma unroll
+            for (int k = 0; k < kMaxF; k += LW)
+                if (j + k < F) input[d + j + k] = xs[r * F + j + k];
+            __syncwarp();
+            v = act(g_first, column_sum(gW1, gb1, sums, d));
+            if (g.n_layers == 2) {
+                if (j < hg) hidden[j] = v;
+                __syncwarp();
+                v = act(g_last, column_sum(gW2, gb2, hidden, hg));
+            }
+            const size_t row = (size_t)m.w * B + b_first + s;
+            if (j < d) {
+                input[j] = v;
+                if (live) a.H[dir][row * d + j] = v;
+            }
+            __syncwarp();
+            v = act(f_first, column_sum(fW1, fb1, input, d + F));
+            if (f.n_layers == 2) {
+                if (j < hf) hidden[j] = v;
+                __syncwarp();
+                v = act(f_last, column_sum(fW2, fb2, hidden, hf));
+            }
+            if (live && j < d && m.z >= 0) {
+                msg[(m.z * S + s) * d + j] = v;
+                if (a.walk.order != nullptr) a.M[dir][row * d + j] = v;
+            }
+            __syncwarp();
+        }
+        prefetch(level + 2);
+        if (level + 1 < lv.n_levels) {
+            p0 = level_ptr[level + 1];
+            rows = (level_ptr[level + 2] - p0) * nb;
+            c = record(p0, rows, min(warp * kRows, rows - 1));
+        }
+        __pipeline_wait_prior(1);
+        __syncthreads();
+    }
+}
+
+int widest(const EmbedArgs &a) {
+    int w = a.d;
+    for (int dir = 0; dir < 2; ++dir) w = std::max(w, std::max(a.f[dir].hidden_dim, a.g[dir].hidden_dim));
+    return w;
+}
+
+}  // namespace
+
+bool embed_small_applicable(const EmbedArgs &a) { return a.F <= kMaxF && widest(a) <= 32; }
+
+cudaError_t launch_embed_small(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap) {
+    SmallPlan p;
+    const int w = widest(a), LW = w <= 8 ? 8 : w <= 16 ? 16 : 32;
+    const size_t buffers = (size_t)kWarps * (32 / LW) * (3 * LW + kMaxF);
+    auto x_floats = [&](int S) { return (a.max_level_width * S * a.F + 3) & ~3; };
+    auto need = [&](int S) {
+        size_t worst = 0;
+        for (int dir = 0; dir < 2; ++dir) {
+            const DevLevels &lv = a.lv[dir];
+            worst = std::max(worst, (size_t)lv.n_slots * S * a.d + 4 * (size_t)a.n + lv.n_levels + 1 + lv.n_nbr);
+        }
+        return (worst + 3 * (size_t)x_floats(S) + buffers) * sizeof(float);
+    };
+    const size_t budget = (size_t)std::min(di.max_smem_optin, 227 * 1024) - 1024;
+    // A block per SM while that is at most eight states each; then two, where the registers allow it (100 a thread at 8
+    // lanes, 140 at 16, 200 at 32). 318 nodes in modules, d = 8, 256 states: 137 us with one, 141 with two; 160 nodes in
+    // 40 levels, 1024 states: 80 and 61.
+    const int per_sm = LW == 8 && a.B > 8 * (di.sm_count / 2) ? 2 : 1;
+    const int slices = std::max(1, std::min(a.B, per_sm * di.sm_count / 2));
+    p.S = (a.B + slices - 1) / slices;
+    while (p.S > 1 && need(p.S) > budget / per_sm) --p.S;
+    if (need(p.S) > budget) return cudaErrorNotSupported;
+    p.n_slices = (a.B + p.S - 1) / p.S;
+    p.x_floats = x_floats(p.S);
+    p.smem_bytes = need(p.S);
+    auto kern = LW == 8 ? embed_small_kernel<8> : LW == 16 ? embed_small_kernel<16> : embed_small_kernel<32>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);
+    if (err != cudaSuccess) return err;
+    err = launch_overlapped(overlap, kern, dim3(p.n_slices, 2), dim3(kThreads), p.smem_bytes, stream, a, p);
+    count_launch();
+    return err;
+}
+
+}  // namespace placeto

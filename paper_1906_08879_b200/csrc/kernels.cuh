@@ -379,6 +379,10 @@ bool embed_split_applicable(const EmbedArgs &a);
 bool embed_split_preferred(const EmbedArgs &a, const DeviceInfo &di);   // applicable and faster than the FMA kernels
 cudaError_t launch_embed_split(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
 
+// embed_small.cu: every layer of f and g at most 32 wide. cudaErrorNotSupported when it does not fit in shared memory.
+bool embed_small_applicable(const EmbedArgs &a);
+cudaError_t launch_embed_small(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
+
 // embed_pipe.cu: d = 64, two layers, as a pipeline of layers on mma.sync (TF32 head + tail operands, a group of warps
 // per layer of f and g). cudaErrorNotSupported when the schedule and the message slots do not fit in shared memory.
 bool embed_pipe_applicable(const EmbedArgs &a);

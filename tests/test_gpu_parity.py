@@ -341,6 +341,23 @@ def test_single_layer_networks_at_the_specialised_widths(d, m, B):
     _small_case(45, src, dst, d=d, m=m, B=B, layers=1, seed=B + d)
 
 
+@pytest.mark.parametrize("d,m,B,layers,act", [(1, 1, 1, 1, 0), (3, 2, 200, 2, 0), (8, 2, 16, 2, 0), (8, 4, 301, 1, 0), (8, 8, 900, 2, 1), (14, 2, 75, 2, 0),
+                                              (21, 8, 33, 2, 0), (31, 2, 500, 1, 0)])
+def test_narrow_sweep_kernel_keeps_the_generic_kernels_bits(d, m, B, layers, act):
+    """Networks of at most 32 columns: 8, 16 and 32 lanes per row, idle lanes, one and several rows per warp, one and
+    several states per block; and shapes that are not narrow any more. Same order of additions, so same bits."""
+    r = rng(B + d)
+    src, dst = random_dag(r, 37, 0.15)
+    cfg = {"n": 37, "src": src, "dst": dst, "m": m, "d": d, "F": m + 4}
+    cfg["cost"], cfg["bytes"] = states.node_costs(r, 37, normalise=True)
+    cfg["dev"], cfg["cur"], cfg["placed"] = states.random_states(r, 37, m, B)
+    cfg["weights"] = states.policy_weights(r, d, m + 4, m, layers, act, 0.1)
+    out = gpu_forward(cfg, 0)
+    compare(cfg, out, oracle.forward(cfg))
+    generic = gpu_forward(cfg, placeto.PLACETO_GENERIC)
+    assert torch.equal(out["H_down"], generic["H_down"]) and torch.equal(out["H_up"], generic["H_up"])
+
+
 @pytest.mark.parametrize("d,m,B,layers", [(64, 8, 1, 2), (64, 3, 90, 2), (64, 8, 600, 2), (64, 5, 300, 1), (32, 4, 1, 2), (32, 8, 1500, 2),
                                           (32, 3, 900, 1)])
 def test_split_sweep_kernel_over_tiles(d, m, B, layers):
