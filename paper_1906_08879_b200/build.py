@@ -34,7 +34,7 @@ LIB_DEBUG = os.path.join(HERE, "libplaceto_debug.so")
 LIB_TIMERS = os.path.join(HERE, "libplaceto_timers.so")
 
 SOURCES = ["api.cu", "plan.cpp", "features.cu", "embed_generic.cu", "embed_d32.cu", "embed_d64.cu", "embed_pipe.cu", "embed_split.cu", "embed_small.cu", "embed_tc.cu",
-           "policy_generic.cu", "policy_d32.cu", "policy_d64.cu", "episode.cu",
+           "policy_generic.cu", "policy_d32.cu", "pool_split.cu", "policy_d64.cu", "episode.cu",
            "embed_rounds_d32.cu", "simulator.cu", "gradient.cu", "grad_sweep.cu", "grad_pool.cu", "status.cu", "aggregator.cu", "policy_tc.cu"]
 
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo",

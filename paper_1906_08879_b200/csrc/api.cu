@@ -87,7 +87,7 @@ struct Layout {
     size_t compact;                // episode call: the compact states [n][E]
     int chunks, chunk_nodes;       // node chunks of the generic pooling kernel
     int chunks32, chunk_nodes32;   // and of the d = 32 / d = 64 kernel (0 when neither can apply)
-    int chunks_tc, chunk_nodes_tc; // and of the d = 64 tensor-core kernel (0 when it cannot apply)
+    int chunks_tc, chunk_nodes_tc; // and of the tensor-core kernel of d = 64 or 32 (0 when it cannot apply or is not faster)
 };
 
 // Workspace layout shared by every call; a call uses the leading part it needs.
@@ -126,6 +126,7 @@ Layout make_layout(const placeto_graph *g, const placeto_weights *w, int B, plac
         return L;
     }
     if (w->F <= 16) {
+        if (w->d == 32) pool_split_chunks((int)n, B, g->info, &L.chunk_nodes_tc, &L.chunks_tc);
         if (w->d == 32) pool_d32_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
         if (w->d == 64 && (w->F & 3) == 0) pool_d64_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
         if (w->d == 64) pool_tc_chunks((int)n, B, g->info, &L.chunk_nodes_tc, &L.chunks_tc);
@@ -272,7 +273,13 @@ placeto_status run_pool(const placeto_graph *g, const placeto_weights *w, const 
     a.logits = logits; a.probs = probs;
     a.n = g->host.n; a.B = B; a.F = w->F; a.d = w->d; a.m = w->m;
     const bool fast32 = pool_d32_applicable(a), fast64 = pool_d64_applicable(a);
-    if (compact != nullptr) {    // only the d = 32 kernel and the fast head kernel take compact states
+    if (!(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY)) && L.chunks_tc > 0 && pool_split_applicable(a)) {
+        a.chunks = L.chunks_tc; a.chunk_nodes = L.chunk_nodes_tc;
+        cudaError_t e = launch_pool_split(a, g->info, stream, after_own_kernel);
+        if (e == cudaSuccess) return cuda_status(launch_pool_head(a, g->info, stream));
+        if (e != cudaErrorNotSupported) return cuda_status(e);
+    }
+    if (compact != nullptr) {    // only the d = 32 kernels and the fast head kernel take compact states
         a.chunks = L.chunks32; a.chunk_nodes = L.chunk_nodes32;
         cudaError_t e = launch_pool_d32(a, g->info, stream, after_own_kernel);
         return cuda_status(e == cudaSuccess ? launch_pool_head(a, g->info, stream) : e);
