@@ -417,15 +417,12 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
         return fail(PLACETO_ERR_NO_MEMORY);
     if (cudaMalloc(&g->d_relation, g->host.relation.size()) != cudaSuccess)
         return fail(PLACETO_ERR_NO_MEMORY);
+    std::vector<int32_t> ints(std::max<size_t>(total, 4));      // one upload for all of them
     for (int dir = 0; dir < 2; ++dir) {
         const LevelPlan &p = g->host.dir[dir];
         const std::vector<int32_t> *vecs[kArrays] = {&p.level_ptr, &p.order, &p.nbr_ptr,
                                                      &p.nbr, &p.own_slot, &p.nbr_slot, &level_of[dir]};
-        for (int k = 0; k < kArrays; ++k)
-            if (!vecs[k]->empty() &&
-                cudaMemcpy(g->d_ints + offs[dir][k], vecs[k]->data(), vecs[k]->size() * sizeof(int),
-                           cudaMemcpyHostToDevice) != cudaSuccess)
-                return fail(PLACETO_ERR_CUDA);
+        for (int k = 0; k < kArrays; ++k) std::copy(vecs[k]->begin(), vecs[k]->end(), ints.begin() + offs[dir][k]);
         g->lv[dir].n_levels = p.n_levels;
         g->lv[dir].level_ptr = g->d_ints + offs[dir][0];
         g->lv[dir].order = g->d_ints + offs[dir][1];
@@ -441,12 +438,11 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
         int **dst[5] = {&g->d_child_ptr, &g->d_child, &g->d_child_entry, &g->d_parent_ptr, &g->d_parent};
         for (int k = 0; k < 5; ++k) {
             *dst[k] = g->d_ints + sim_off[k];
-            if (!extra[k]->empty() &&
-                cudaMemcpy(*dst[k], extra[k]->data(), extra[k]->size() * sizeof(int),
-                           cudaMemcpyHostToDevice) != cudaSuccess)
-                return fail(PLACETO_ERR_CUDA);
+            std::copy(extra[k]->begin(), extra[k]->end(), ints.begin() + sim_off[k]);
         }
     }
+    if (cudaMemcpy(g->d_ints, ints.data(), ints.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+        return fail(PLACETO_ERR_CUDA);
     if (cudaMemcpy(g->d_relation, g->host.relation.data(), g->host.relation.size(),
                    cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(PLACETO_ERR_CUDA);

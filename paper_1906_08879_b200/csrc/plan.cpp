@@ -3,6 +3,7 @@
 #include "plan.h"
 
 #include <algorithm>
+#include <cstring>
 #include <new>
 
 namespace placeto {
@@ -140,27 +141,40 @@ placeto_status build_plan(int32_t n, int64_t n_edges, const int32_t *src, const 
                 plan.max_level_width = std::max(
                     plan.max_level_width, plan.dir[dir].level_ptr[l + 1] - plan.dir[dir].level_ptr[l]);
 
-        // Ancestor bitsets in top-down level order: anc(v) = U_{u in par(v)} (anc(u) + u).
+        // Ancestor bitsets in top-down level order: anc(v) = U_{u in par(v)} (anc(u) + u); descendants likewise, bottom-up.
         const size_t words = (static_cast<size_t>(n) + 63) / 64;
-        std::vector<uint64_t> anc(static_cast<size_t>(n) * words, 0);
-        for (int32_t p = 0; p < n; ++p) {
-            const int32_t v = plan.dir[0].order[p];
-            uint64_t *av = &anc[static_cast<size_t>(v) * words];
-            for (int32_t u : par[v]) {
-                const uint64_t *au = &anc[static_cast<size_t>(u) * words];
-                for (size_t w = 0; w < words; ++w) av[w] |= au[w];
-                av[u >> 6] |= 1ull << (u & 63);
+        std::vector<uint64_t> reach[2];
+        for (int dir = 0; dir < 2; ++dir) {
+            const LevelPlan &p = plan.dir[dir];
+            reach[dir].assign(static_cast<size_t>(n) * words, 0);
+            for (int32_t q = 0; q < n; ++q) {
+                uint64_t *mine = &reach[dir][static_cast<size_t>(p.order[q]) * words];
+                for (int32_t e = p.nbr_ptr[q]; e < p.nbr_ptr[q + 1]; ++e) {
+                    const int32_t u = p.nbr[e];
+                    const uint64_t *theirs = &reach[dir][static_cast<size_t>(u) * words];
+                    for (size_t w = 0; w < words; ++w) mine[w] |= theirs[w];
+                    mine[u >> 6] |= 1ull << (u & 63);
+                }
             }
         }
-        plan.relation.assign(static_cast<size_t>(n) * n, 2);
+        // relation[c][u] = 0 (u can reach c), 1 (u can be reached from c), 2 (neither), 3 (u is c): a row at a time, eight
+        // bytes from eight bits of either set (writing the transposed entry beside each 0 walked the columns: 4 of 7 ms
+        // for 1987 nodes)
+        uint64_t spread[256];                    // bit i -> byte i
+        for (int b = 0; b < 256; ++b) {
+            unsigned char bytes[8];
+            for (int i = 0; i < 8; ++i) bytes[i] = b >> i & 1;
+            std::memcpy(&spread[b], bytes, 8);
+        }
+        plan.relation.resize(static_cast<size_t>(n) * n);
         for (int32_t c = 0; c < n; ++c) {
-            const uint64_t *ac = &anc[static_cast<size_t>(c) * words];
+            const uint64_t *up = &reach[0][static_cast<size_t>(c) * words], *down = &reach[1][static_cast<size_t>(c) * words];
             uint8_t *row = &plan.relation[static_cast<size_t>(c) * n];
-            for (int32_t u = 0; u < n; ++u)
-                if (ac[u >> 6] >> (u & 63) & 1) {
-                    row[u] = 0;                                         // u can reach c
-                    plan.relation[static_cast<size_t>(u) * n + c] = 1;  // u can reach c, seen from u
-                }
+            for (int32_t u = 0; u < n; u += 8) {
+                const uint64_t eight = 0x0202020202020202ull - 2 * spread[up[u >> 6] >> (u & 63) & 255] -
+                                       spread[down[u >> 6] >> (u & 63) & 255];
+                std::memcpy(row + u, &eight, std::min(8, n - u));
+            }
             row[c] = 3;
         }
     } catch (const std::bad_alloc &) {
