@@ -355,8 +355,8 @@ pool_head_kernel(const PoolArgs a, int tmp_floats, int stage_floats) {
 
 // The same finish for the common shapes (single-layer h_i of width d, two-layer
 // head) with HS states per block, HS chosen so that the blocks cover the device: a
-// small batch is spread over many SMs instead of eight states sharing one. Nothing
-// is staged: weights are read once per block straight from L2, as 128-bit loads
+// small batch is spread over many SMs instead of eight states sharing one. The head's
+// weights are read once per block straight from L2, as 128-bit loads
 // where the hidden width keeps the rows of the head's first matrix aligned for
 // them (VEC = 4), as 64- or 32-bit ones otherwise (odd device counts: F = m + 4 is
 // then no multiple of 4); a thread of the first head layer
@@ -388,40 +388,70 @@ __device__ __forceinline__ float4 load_row4(const float *__restrict__ p, int lef
 
 template <int HS, int VEC>
 __global__ void __launch_bounds__(kFastThreads, 1)
-pool_head_fast_kernel(const PoolArgs a) {
-    constexpr int SR = HS < 4 ? HS : 4;     // states of a thread tile
+pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: floats of h_i's weights kept in shared memory
+    constexpr int SR = HS < 4 ? HS : 4;     // states of a thread tile (all eight: 21.0 -> 23.5 us for 992 states, more to add up)
     constexpr int SG = HS / SR;             // state groups
     extern __shared__ __align__(16) float smem[];
     const int d = a.d, F = a.F, B = a.B, m = a.m;
     const int E = 2 * d + F, Z = 5 * d + F, Hd = a.head.hidden_dim;
     const int Hp = (Hd + 3) & ~3;                  // hidden units in whole groups of four columns
-    float *zt = smem;                              // [Z][HS]: e_c, then the three h_i outputs
+    float *hw = smem;                              // [3][d][d], the weights of h_i
+    float *zt = hw + staged_h;                     // [Z][HS]: e_c, then the three h_i outputs
     float *sum = zt + Z * HS;                      // [HS][3 d]
     float *hid = sum + HS * 3 * d;                 // [Hp][HS]
     float *lg = hid + Hp * HS;                     // [HS][m]
     float *red = lg + ((HS * m + 3) & ~3);         // [parts][Hp][HS]
     const int b0 = blockIdx.x * HS;
+    // Weights do not depend on the kernel before: those of h_i go to shared memory, this thread's first rows of the head
+    // into registers, while it runs or while the sums below are on their way. Reading them where they are used cost a
+    // round trip to L2 in each layer (a step of 16 episodes of 151 nodes: 10.6 -> 8.5 us).
+    for (int i = threadIdx.x; i < staged_h / 4; i += blockDim.x) {
+        const int set = i / (d * d / 4);
+        __pipeline_memcpy_async(hw + 4 * i, a.h[set].W1 + 4 * (i - set * (d * d / 4)), 16);
+    }
+    __pipeline_commit();
+    const int CG = Hp >> 2, tiles = SG * CG;
+    const int parts = max(1, min((int)blockDim.x / tiles, Z));
+    const int per = (Z + parts - 1) / parts;
+    const int part = threadIdx.x / tiles, cg = (threadIdx.x - part * tiles) % CG, sg = (threadIdx.x - part * tiles) / CG;
+    const int k0 = part * per, k1 = part < parts ? min(Z, k0 + per) : k0;
+    const float *__restrict__ head_W = a.head.W1 + 4 * cg;
+    float4 head_w[16];                             // sixteen rows in flight
+    auto load_head = [&](int kb) {
+#pragma unroll
+        for (int t = 0; t < 16; ++t)
+            head_w[t] = kb + t < k1 ? load_row4<VEC>(head_W + (size_t)(kb + t) * Hd, Hd - 4 * cg) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    load_head(k0);
     prefetch_l2(a.head.W1, (size_t)Z * Hd);
     prefetch_l2(a.head.W2, (size_t)Hd * m);
-    for (int i = 0; i < 3; ++i) prefetch_l2(a.h[i].W1, (size_t)d * d);
+    float uniform = 0.f;
+    int visit = -1, next_visit = -1;               // of the step: the node whose device is chosen, the one after
+    if (a.step.enabled && threadIdx.x < HS && b0 + threadIdx.x < B) {
+        if (a.step.uniforms != nullptr) uniform = a.step.uniforms[(size_t)(b0 + threadIdx.x) * a.step.n + a.step.t];
+        visit = a.step.order[a.step.t];
+        if (a.step.t + 1 < a.step.n) next_visit = a.step.order[a.step.t + 1];
+    }
     dependency_wait();          // the partial sums come from a kernel that may still be running
+    const int c_mine = threadIdx.x < HS && b0 + threadIdx.x < B ? a.cur[b0 + threadIdx.x] : -1;
     for (int i = threadIdx.x; i < HS * 3 * d; i += blockDim.x) {
         const int s = i / (3 * d), j = i - s * 3 * d;
         const int b = min(b0 + s, B - 1);          // rows past the batch repeat the last state
-        // chunks are added in ascending order; eight loads in flight at a time
+        // chunks are added in ascending order; sixteen loads in flight at a time
         const float *src = a.partial + (size_t)b * 3 * d + j;
         const size_t step = (size_t)B * 3 * d;
         float acc = 0.f;
-        for (int ch = 0; ch < a.chunks; ch += 8) {
-            float t[8];
+        for (int ch = 0; ch < a.chunks; ch += 16) {
+            float t[16];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) t[q] = ch + q < a.chunks ? src[(ch + q) * step] : 0.f;
+            for (int q = 0; q < 16; ++q) t[q] = ch + q < a.chunks ? src[(ch + q) * step] : 0.f;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) acc += t[q];
+            for (int q = 0; q < 16; ++q) acc += t[q];
         }
         sum[i] = acc;
     }
-    for (int i = threadIdx.x; i < HS * E; i += blockDim.x) {
+    // from the last thread down: a small batch has others for these than for the sums
+    for (int i = blockDim.x - 1 - threadIdx.x; i < HS * E; i += blockDim.x) {
         const int s = i / E, k = i - s * E;
         const int b = min(b0 + s, B - 1);
         const int c = a.cur[b];
@@ -433,6 +463,7 @@ pool_head_fast_kernel(const PoolArgs a) {
                                            : a.X[((size_t)c * B + b) * F + (k - 2 * d)];
         zt[k * HS + s] = v;
     }
+    __pipeline_wait_prior(0);
     __syncthreads();
     // the three h_i: thread = (state, set, four columns)
     const int dq = d >> 2;
@@ -440,23 +471,17 @@ pool_head_fast_kernel(const PoolArgs a) {
         const int s = i / (3 * dq), r = i - s * 3 * dq;
         const int set = r / dq, cq = r - set * dq;
         const DevMlp &nt = a.h[set];
-        const float *__restrict__ W = nt.W1 + 4 * cq;
+        const float *W = (staged_h > 0 ? hw + set * d * d : nt.W1) + 4 * cq;
         const float *v = sum + s * 3 * d + set * d;
         float4 acc = *reinterpret_cast<const float4 *>(nt.b1 + 4 * cq), odd = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int kb = 0; kb < d; kb += 16) {   // sixteen weight rows in flight (d is a multiple of 4)
-            float4 w[16];
-#pragma unroll
-            for (int t = 0; t < 16; ++t)
-                w[t] = kb + t < d ? __ldg(reinterpret_cast<const float4 *>(W + (size_t)(kb + t) * d))
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int t = 0; t < 16; t += 2) {      // two chains: shorter, and less rounding in each
-                const float x = kb + t < d ? v[kb + t] : 0.f, y = kb + t + 1 < d ? v[kb + t + 1] : 0.f;
-                acc.x = fmaf(x, w[t].x, acc.x); odd.x = fmaf(y, w[t + 1].x, odd.x);
-                acc.y = fmaf(x, w[t].y, acc.y); odd.y = fmaf(y, w[t + 1].y, odd.y);
-                acc.z = fmaf(x, w[t].z, acc.z); odd.z = fmaf(y, w[t + 1].z, odd.z);
-                acc.w = fmaf(x, w[t].w, acc.w); odd.w = fmaf(y, w[t + 1].w, odd.w);
-            }
+#pragma unroll 8
+        for (int k = 0; k < d; k += 2) {           // two chains: shorter, and less rounding in each (d is a multiple of 4)
+            const float4 w0 = *reinterpret_cast<const float4 *>(W + k * d), w1 = *reinterpret_cast<const float4 *>(W + (k + 1) * d);
+            const float x = v[k], y = v[k + 1];
+            acc.x = fmaf(x, w0.x, acc.x); odd.x = fmaf(y, w1.x, odd.x);
+            acc.y = fmaf(x, w0.y, acc.y); odd.y = fmaf(y, w1.y, odd.y);
+            acc.z = fmaf(x, w0.z, acc.z); odd.z = fmaf(y, w1.z, odd.z);
+            acc.w = fmaf(x, w0.w, acc.w); odd.w = fmaf(y, w1.w, odd.w);
         }
         acc.x += odd.x; acc.y += odd.y; acc.z += odd.z; acc.w += odd.w;
         if (nt.act == 0 && nt.final_act) {
@@ -468,26 +493,15 @@ pool_head_fast_kernel(const PoolArgs a) {
     }
     __syncthreads();
     // head, first layer
-    const int CG = Hp >> 2, tiles = SG * CG;
-    const int parts = max(1, min((int)blockDim.x / tiles, Z));
-    const int per = (Z + parts - 1) / parts;
-    if ((int)threadIdx.x < tiles * parts) {
-        const int part = threadIdx.x / tiles, r = threadIdx.x - part * tiles;
-        const int sg = r / CG, cg = r - sg * CG;
+    if (part < parts) {
         float acc[SR][4];
 #pragma unroll
         for (int s = 0; s < SR; ++s)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[s][c] = 0.f;
-        const int k0 = part * per, k1 = min(Z, k0 + per);
-        const float *__restrict__ W = a.head.W1 + 4 * cg;
         const float *zrow = zt + sg * SR;
-        for (int kb = k0; kb < k1; kb += 16) {   // sixteen weight rows in flight
-            float4 w[16];
-#pragma unroll
-            for (int t = 0; t < 16; ++t)
-                w[t] = kb + t < k1 ? load_row4<VEC>(W + (size_t)(kb + t) * Hd, Hd - 4 * cg)
-                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int kb = k0; kb < k1; kb += 16) {
+            if (kb > k0) load_head(kb);
 #pragma unroll
             for (int t = 0; t < 16; ++t) {
                 const bool live = kb + t < k1;
@@ -496,17 +510,15 @@ pool_head_fast_kernel(const PoolArgs a) {
                 if (SR == 4) {
                     const float4 u = *reinterpret_cast<const float4 *>(zrow + k * HS);
                     zv[0] = u.x; zv[1 % SR] = u.y; zv[2 % SR] = u.z; zv[3 % SR] = u.w;
-                } else if (SR == 2) {
+                } else {
                     const float2 u = *reinterpret_cast<const float2 *>(zrow + k * HS);
                     zv[0] = u.x; zv[1 % SR] = u.y;
-                } else {
-                    zv[0] = zrow[k * HS];
                 }
 #pragma unroll
                 for (int s = 0; s < SR; ++s) {
                     zv[s] = live ? zv[s] : 0.f;
-                    acc[s][0] = fmaf(zv[s], w[t].x, acc[s][0]); acc[s][1] = fmaf(zv[s], w[t].y, acc[s][1]);
-                    acc[s][2] = fmaf(zv[s], w[t].z, acc[s][2]); acc[s][3] = fmaf(zv[s], w[t].w, acc[s][3]);
+                    acc[s][0] = fmaf(zv[s], head_w[t].x, acc[s][0]); acc[s][1] = fmaf(zv[s], head_w[t].y, acc[s][1]);
+                    acc[s][2] = fmaf(zv[s], head_w[t].z, acc[s][2]); acc[s][3] = fmaf(zv[s], head_w[t].w, acc[s][3]);
                 }
             }
         }
@@ -541,9 +553,8 @@ pool_head_fast_kernel(const PoolArgs a) {
     if (threadIdx.x < HS && b0 + threadIdx.x < B) {
         const int b = b0 + threadIdx.x;
         const float *l = lg + threadIdx.x * m;
-        const int c = a.cur[b];
         // a current node out of range yields NaN (ReLU would swallow a NaN input)
-        const bool valid = c >= 0 && c < a.n;
+        const bool valid = c_mine >= 0 && c_mine < a.n;
         float mx = l[0];
         for (int k = 1; k < m; ++k) mx = fmaxf(mx, l[k]);
         float tot = 0.f;
@@ -563,7 +574,7 @@ pool_head_fast_kernel(const PoolArgs a) {
                 if (l[k] > top) { top = l[k]; best = k; }
             int action = best;
             if (st.uniforms != nullptr) {
-                const float u = st.uniforms[(size_t)b * st.n + st.t];
+                const float u = uniform;
                 float cum = 0.f;
                 action = m - 1;
                 for (int k = 0; k < m; ++k) {
@@ -573,9 +584,8 @@ pool_head_fast_kernel(const PoolArgs a) {
             }
             if (st.logp != nullptr) st.logp[(size_t)b * st.n + st.t] = (l[action] - mx) - logf(tot);
             if (st.actions != nullptr) st.actions[(size_t)b * st.n + st.t] = (uint8_t)action;
-            const int v = st.order[st.t];
-            if (v >= 0 && v < st.n) st.state[(size_t)v * B + b] = (uint8_t)(action | 0x80);   // placed, visited
-            if (st.t + 1 < st.n) st.cur[b] = st.order[st.t + 1];
+            if (visit >= 0 && visit < st.n) st.state[(size_t)visit * B + b] = (uint8_t)(action | 0x80);   // placed, visited
+            if (st.t + 1 < st.n) st.cur[b] = next_visit;
         }
     }
 }
@@ -596,16 +606,17 @@ cudaError_t launch_head_fast(const PoolArgs &a, cudaStream_t stream) {
     const int parts = std::max(1, std::min(kFastThreads / tiles, Z));
     const size_t floats = (size_t)Z * HS + (size_t)HS * 3 * a.d + (size_t)Hd * HS + ((HS * a.m + 3) & ~3) +
                           (size_t)parts * Hd * HS;
-    const size_t bytes = floats * sizeof(float);
-    if (bytes > 200 * 1024) return cudaErrorNotSupported;
-    void (*kern)(const PoolArgs) = (a.head.hidden_dim & 3) == 0   ? pool_head_fast_kernel<HS, 4>
+    if (floats * sizeof(float) > 200 * 1024) return cudaErrorNotSupported;
+    const int staged_h = (floats + (size_t)3 * a.d * a.d) * sizeof(float) <= 200 * 1024 ? 3 * a.d * a.d : 0;
+    const size_t bytes = (floats + staged_h) * sizeof(float);
+    void (*kern)(const PoolArgs, const int) = (a.head.hidden_dim & 3) == 0   ? pool_head_fast_kernel<HS, 4>
                                    : (a.head.hidden_dim & 1) == 0 ? pool_head_fast_kernel<HS, 2>
                                                                   : pool_head_fast_kernel<HS, 1>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (err != cudaSuccess) return err;
     // always preceded by one of this library's pooling kernels on the same stream
     err = launch_overlapped(true, kern, dim3((a.B + HS - 1) / HS), dim3(kFastThreads),
-                            bytes, stream, a);
+                            bytes, stream, a, staged_h);
     count_launch();
     return err;
 }
@@ -656,8 +667,9 @@ cudaError_t launch_policy_generic(const PoolArgs &a, const DeviceInfo &di, cudaS
 
 cudaError_t launch_pool_head(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream) {
     if (head_fast_applicable(a)) {
-        // fewest states per block that keeps the grid within two blocks per SM
-        const int limit = 2 * std::max(1, di.sm_count);
+        // fewest states per block that keeps the grid within one block per SM, what the registers allow: a second wave costs
+        // more than twice the states (512 states, d = 64: 31.0 -> 21.5 us; 400, d = 32: 14.5 -> 10.0)
+        const int limit = std::max(1, di.sm_count);
         cudaError_t e = (a.B + 1) / 2 <= limit   ? launch_head_fast<2>(a, stream)
                         : (a.B + 3) / 4 <= limit ? launch_head_fast<4>(a, stream)
                                                  : launch_head_fast<8>(a, stream);
