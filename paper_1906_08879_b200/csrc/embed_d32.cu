@@ -142,10 +142,19 @@ __device__ __forceinline__ void run_node(const Weights32 &w, const pair_t (&wf1)
             acc[r] += (t[0] + t[1]) + (t[2] + t[3]);
         }
     }
-    for (; e < e1; ++e) {
-        const int base = nbr_slot[e] * S;
+    if (e < e1) {                   // the last one to three likewise (151 nodes with 267 edges: 0.60 -> 0.54 us a level)
+        int base[3];
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] += msg[(base + st[r]) * kD + lane];
+        for (int k = 0; k < 3; ++k) base[k] = nbr_slot[min(e + k, e1 - 1)] * S;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            float t[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) t[k] = msg[(base[k] + st[r]) * kD + lane];
+            acc[r] += t[0];
+            if (e + 1 < e1) acc[r] += t[1];
+            if (e + 2 < e1) acc[r] += t[2];
+        }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) A[r * KF + lane] = acc[r];
@@ -291,13 +300,15 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     prefetch(start);
     float *__restrict__ M = a.M[dir];
     if (kWalk && start > 0) {
-        // messages from above `start` that it or a later level reads: a slot belongs to its node until then
-        for (int e = meta[level_ptr[start]].x + warp; e < lv.n_nbr; e += kWarps) {
-            const int u = lv.nbr[e];
-            if (lv.level_of[u] >= start) continue;
-            const int slot = nbr_slot[e];
-            for (int s = 0; s < nb; ++s) msg[(slot * p.S + s) * kD + lane] = M[((size_t)u * B + b_first + s) * kD + lane];
-        }
+        carried_messages(lv, meta[level_ptr[start]].x, start, warp, kWarps, lane, [&](const int (&u)[4], const int (&e)[4]) {
+            for (int s = 0; s < nb; ++s) {
+                float v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = M[((size_t)u[k] * B + b_first + s) * kD + lane];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) msg[(nbr_slot[e[k]] * p.S + s) * kD + lane] = v[k];
+            }
+        });
     }
     __pipeline_wait_prior(0);
     __syncthreads();

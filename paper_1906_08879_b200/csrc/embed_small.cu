@@ -100,12 +100,15 @@ embed_small_kernel(const EmbedArgs a, const SmallPlan p) {
     prefetch(start);
     prefetch(start + 1);
     if (start > 0) {            // an episode's sweep: messages from above that a later level reads
-        for (int e = meta[level_ptr[start]].x + warp; e < lv.n_nbr; e += kWarps) {
-            const int u = lv.nbr[e];
-            if (lv.level_of[u] >= start) continue;
-            for (int i = lane; i < nb * d; i += 32)
-                msg[nbr_slot[e] * S * d + i] = a.M[dir][((size_t)u * B + b_first) * d + i];
-        }
+        carried_messages(lv, meta[level_ptr[start]].x, start, warp, kWarps, lane, [&](const int (&u)[4], const int (&e)[4]) {
+            for (int i = lane; i < nb * d; i += 32) {
+                float v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = a.M[dir][((size_t)u[k] * B + b_first) * d + i];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) msg[nbr_slot[e[k]] * S * d + i] = v[k];
+            }
+        });
     }
     __pipeline_wait_prior(1);
     __syncthreads();

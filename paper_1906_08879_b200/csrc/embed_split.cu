@@ -202,14 +202,16 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
         fetch(start);
         fetch(start + 1);
         if (kWalk && start > 0) {
-            // messages from above `start` that it or a later level reads: a slot belongs to its node until then
-            for (int e = meta[level_ptr[start]].x + (ht >> 5); e < lv.n_nbr; e += kHelperThreads / 32) {
-                const int u = lv.nbr[e];
-                if (lv.level_of[u] >= start) continue;
-                const int slot = nbr_slot[e];
-                for (int i = lane; i < nb * D; i += 32)
-                    msg[(slot * S + i / D) * P + i % D] = a.M[dir][((size_t)u * B + b_first) * D + i];
-            }
+            carried_messages(lv, meta[level_ptr[start]].x, start, ht >> 5, kHelperThreads / 32, lane, [&](const int (&u)[4], const int (&e)[4]) {
+#pragma unroll 1
+                for (int i = lane; i < nb * D; i += 32) {
+                    float v[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] = a.M[dir][((size_t)u[k] * B + b_first) * D + i];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) msg[(nbr_slot[e[k]] * S + i / D) * P + i % D] = v[k];
+                }
+            });
         }
         __pipeline_wait_prior(1);
         group_sync<kHelperThreads>(kHelperBar);

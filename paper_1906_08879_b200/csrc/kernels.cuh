@@ -100,12 +100,14 @@ __device__ __forceinline__ float compact_feature(const CompactState &c, int v, i
 // all F = m + 4 features of node v in state b into x[0 .. F): one state byte, the node's cost and
 // size, the state's current node
 __device__ __forceinline__ void compact_features(const CompactState &c, int v, int b, int B, float *x) {
+    // all loads before the first store: the compiler cannot move them across (a round trip to L2 for each)
     const unsigned s = c.state[(size_t)v * B + b];
-    const int dev = (int)(s & 63u);
-    x[0] = c.cost[v];
-    x[1] = c.bytes[v];
+    const float cost = c.cost[v], bytes = c.bytes[v];
+    const int cur = c.cur[b], dev = (int)(s & 63u);
+    x[0] = cost;
+    x[1] = bytes;
     for (int k = 0; k < c.m; ++k) x[2 + k] = k == dev ? 1.f : 0.f;
-    x[2 + c.m] = c.cur[b] == v ? 1.f : 0.f;
+    x[2 + c.m] = cur == v ? 1.f : 0.f;
     x[3 + c.m] = (float)(s >> 7);
 }
 #endif
@@ -138,6 +140,32 @@ __device__ __forceinline__ int first_level(const EpisodeWalk &w, const DevLevels
     const int u = w.order[w.t - 1], v = w.order[w.t];
     if (u < 0 || u >= n || v < 0 || v >= n) return 0;
     return min(lv.level_of[u], lv.level_of[v]);
+}
+// The messages from levels above `start` that it or a later level reads, four rows at a time: copy(u, e) with four nodes and
+// the neighbour entries that name them (repeated when fewer are left). A slot belongs to its node until its last reader, so
+// they can all be brought in at once. `workers` warps share the entries; a lane looks at one of them, since an entry that is
+// looked at alone costs three round trips to L2 (a sweep of 16 episodes of 151 nodes: 37.8 -> 34.5 us; of 64, d = 64: 80 -> 74).
+template <typename Copy>
+__device__ __forceinline__ void carried_messages(const DevLevels &lv, int first_entry, int start, int worker, int workers, int lane,
+                                                 Copy copy) {
+#pragma unroll 1
+    for (int base = first_entry + 32 * worker; base < lv.n_nbr; base += 32 * workers) {
+        const int mine = base + lane < lv.n_nbr ? lv.nbr[base + lane] : -1;
+        unsigned left = __ballot_sync(0xffffffffu, mine >= 0 && lv.level_of[max(mine, 0)] < start);
+#pragma unroll 1
+        while (left) {
+            int u[4], e[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int at = __ffs(left) - 1;
+                if (left & (left - 1)) left &= left - 1;
+                else if (k == 3) left = 0;
+                u[k] = __shfl_sync(0xffffffffu, mine, at);
+                e[k] = base + at;
+            }
+            copy(u, e);
+        }
+    }
 }
 #endif
 
