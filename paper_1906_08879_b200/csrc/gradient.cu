@@ -69,9 +69,7 @@ grad_messages_kernel(const GradArgs a) {
 }
 
 // ------------------------------------------------------------- 2. head / pool
-// One block per state (grid-stride). Shared memory: the state's vectors. kPooled: the sums arrive per chunk of
-// nodes and what is pushed back stops at them and at the current node's embedding (grad_pool.cu does the rows).
-template <bool kPooled>
+// One block per state (grid-stride). Shared memory: the state's vectors.
 __global__ void __launch_bounds__(kThreads)
 grad_head_kernel(const GradArgs a) {
     extern __shared__ __align__(16) float smem[];
@@ -90,7 +88,7 @@ grad_head_kernel(const GradArgs a) {
     float *wl = erow + G * ((E + 3) & ~3); // [3][E * d + d]: the three l_i (weights, then bias)
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int lsz = E * d + d;
-    for (int i = 0; !kPooled && i < 3; ++i) {
+    for (int i = 0; i < 3; ++i) {
         for (int t = threadIdx.x; t < E * d; t += kThreads) wl[i * lsz + t] = a.l[i].W1[t];
         for (int t = threadIdx.x; t < d; t += kThreads) wl[i * lsz + E * d + t] = a.l[i].b1[t];
     }
@@ -99,7 +97,7 @@ grad_head_kernel(const GradArgs a) {
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
         const int c = a.cur[b];
         if (c < 0 || c >= n) {             // no such node: the state contributes nothing
-            for (int i = threadIdx.x; !kPooled && i < n * d; i += kThreads) {
+            for (int i = threadIdx.x; i < n * d; i += kThreads) {
                 const size_t off = ((size_t)(i / d) * B + b) * d + (i % d);
                 a.DH[0][off] = 0.f;
                 a.DH[1][off] = 0.f;
@@ -117,9 +115,9 @@ grad_head_kernel(const GradArgs a) {
                              : a.X[((size_t)u * B + b) * F + (k - 2 * d)];
         };
         // ---- pooled sums S_i = sum_{u in set i} relu(l_i(e_u)); warp g takes nodes g, g + G, ...
-        for (int i = threadIdx.x; !kPooled && i < G * 3 * d; i += kThreads) part[i] = 0.f;
+        for (int i = threadIdx.x; i < G * 3 * d; i += kThreads) part[i] = 0.f;
         __syncthreads();
-        for (int u = g; !kPooled && u < n; u += G) {
+        for (int u = g; u < n; u += G) {
             const int set = rel[u];
             if (set > 2) continue;
             const float *W = wl + set * lsz;
@@ -135,10 +133,7 @@ grad_head_kernel(const GradArgs a) {
         __syncthreads();
         for (int i = threadIdx.x; i < 3 * d; i += kThreads) {
             float acc = 0.f;
-            if (kPooled)
-                for (int q = 0; q < a.pool_chunks; ++q) acc += a.pool_partial[((size_t)q * B + b) * 3 * d + i];
-            else
-                for (int q = 0; q < G; ++q) acc += part[q * 3 * d + i];
+            for (int q = 0; q < G; ++q) acc += part[q * 3 * d + i];
             S[i] = acc;
             a.Sbuf[(size_t)b * 3 * d + i] = acc;
         }
@@ -218,12 +213,6 @@ grad_head_kernel(const GradArgs a) {
             float acc = 0.f;
             for (int j = 0; j < d; ++j) acc = fmaf(part[set * d + j], h.W1[k * d + j], acc);
             dS[i] = acc;
-            if (kPooled) a.dS[(size_t)b * 3 * d + i] = acc;
-        }
-        if (kPooled) {
-            for (int k = threadIdx.x; k < 2 * d; k += kThreads) a.dZ[(size_t)b * 2 * d + k] = dz[k];
-            __syncthreads();
-            continue;
         }
         __syncthreads();
         // ---- through l_i to every node: dpre_l = dS_set * (pre > 0); de = dpre_l W_l^T
@@ -263,6 +252,149 @@ grad_head_kernel(const GradArgs a) {
             }
             __syncwarp();
         }
+        __syncthreads();
+    }
+}
+
+// The same between the row kernels of grad_pool.cu: the sums arrive per chunk of nodes, and what is pushed back stops
+// at them and at the current node's embedding. A chain of small products per state, bound by the round trips to L2 for
+// their weights: one thread per sum of 332 products with four loads in flight took 111 us for 100 states at d = 64, 38 us
+// for 256 at d = 32. Sixteen in flight here, the last layer's weights in shared memory, the transposed product four
+// rows to a warp: 43 and 24 us. Sums are taken in the order of the forward pass, so the ReLU masks are the same.
+constexpr int kHeadThreads = 512;
+
+// init + sum over k < K of x[k] w[k * stride], ascending
+__device__ __forceinline__ float strided_dot(float init, const float *x, const float *__restrict__ w, int stride, int K) {
+    float acc = init;
+    int k = 0;
+    for (; k + 16 <= K; k += 16) {
+        float v[16];
+#pragma unroll
+        for (int t = 0; t < 16; ++t) v[t] = __ldg(w + (size_t)(k + t) * stride);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) acc = fmaf(x[k + t], v[t], acc);
+    }
+    for (; k < K; ++k) acc = fmaf(x[k], __ldg(w + (size_t)k * stride), acc);
+    return acc;
+}
+
+__global__ void __launch_bounds__(kHeadThreads)
+grad_head_pooled_kernel(const GradArgs a, const int staged) {      // staged: floats of the last layer's weights in shared memory
+    extern __shared__ __align__(16) float smem[];
+    const int d = a.d, F = a.F, m = a.m, n = a.n, B = a.B;
+    const int E = 2 * d + F, Z = 5 * d + F, Hh = a.head.hidden_dim;
+    float *z = smem;                       // [Z]
+    float *hid = z + Z;                    // [Hh]
+    float *dhid = hid + Hh;                // [Hh]
+    float *dz = dhid + Hh;                 // [Z]
+    float *S = dz + Z;                     // [3][d]
+    float *dpre = S + 3 * d;               // [3][d]
+    float *lg = dpre + 3 * d;              // [m] logits, then d/d(logits)
+    float *w2 = lg + m;                    // [Hh][m]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < staged; i += kHeadThreads) w2[i] = a.head.W2[i];
+    const float *W2 = staged > 0 ? w2 : a.head.W2;
+    for (int b = blockIdx.x; b < B; b += gridDim.x) {
+        const int c = a.cur[b];
+        if (c < 0 || c >= n) {             // no such node: the state contributes nothing
+            for (int k = threadIdx.x; k < Z; k += kHeadThreads) a.Zbuf[(size_t)b * Z + k] = 0.f;
+            for (int k = threadIdx.x; k < Hh; k += kHeadThreads) { a.HID[(size_t)b * Hh + k] = 0.f; a.DHID[(size_t)b * Hh + k] = 0.f; }
+            for (int k = threadIdx.x; k < m; k += kHeadThreads) a.DLOG[(size_t)b * m + k] = 0.f;
+            for (int k = threadIdx.x; k < 3 * d; k += kHeadThreads) { a.Sbuf[(size_t)b * 3 * d + k] = 0.f; a.DPRE_H[(size_t)b * 3 * d + k] = 0.f; }
+            continue;
+        }
+        for (int i = threadIdx.x; i < 3 * d; i += kHeadThreads) {
+            const float *src = a.pool_partial + (size_t)b * 3 * d + i;
+            float acc = 0.f;
+            for (int q0 = 0; q0 < a.pool_chunks; q0 += 8) {
+                float v[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) v[t] = q0 + t < a.pool_chunks ? src[(size_t)(q0 + t) * B * 3 * d] : 0.f;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) acc += v[t];
+            }
+            S[i] = acc;
+            a.Sbuf[(size_t)b * 3 * d + i] = acc;
+        }
+        for (int k = kHeadThreads - 1 - threadIdx.x; k < E; k += kHeadThreads)
+            z[k] = k < d ? a.H[0][((size_t)c * B + b) * d + k]
+                 : k < 2 * d ? a.H[1][((size_t)c * B + b) * d + (k - d)]
+                             : a.X[((size_t)c * B + b) * F + (k - 2 * d)];
+        __syncthreads();
+        // ---- a_i = relu(h_i(S_i)) into z, hidden layer, logits
+        for (int i = threadIdx.x; i < 3 * d; i += kHeadThreads) {
+            const int set = i / d, j = i - set * d;
+            z[E + i] = fmaxf(strided_dot(a.h[set].b1[j], S + set * d, a.h[set].W1 + j, d, d), 0.f);
+        }
+        __syncthreads();
+        for (int j = threadIdx.x; j < Hh; j += kHeadThreads) hid[j] = fmaxf(strided_dot(a.head.b1[j], z, a.head.W1 + j, Hh, Z), 0.f);
+        __syncthreads();
+        for (int j = threadIdx.x; j < m; j += kHeadThreads) {
+            float acc = a.head.b2[j];
+#pragma unroll 8
+            for (int k = 0; k < Hh; ++k) acc = fmaf(hid[k], W2[(size_t)k * m + j], acc);
+            lg[j] = acc;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            // d/d(logit_k) of A log p[a] + beta H = A (1[k = a] - p_k) - beta p_k (log p_k + H)
+            float mx = lg[0];
+            for (int k = 1; k < m; ++k) mx = fmaxf(mx, lg[k]);
+            float tot = 0.f;
+            for (int k = 0; k < m; ++k) tot += expf(lg[k] - mx);
+            const float lt = logf(tot);
+            float ent = 0.f;
+            for (int k = 0; k < m; ++k) {
+                const float lp = lg[k] - mx - lt;
+                ent -= expf(lp) * lp;
+            }
+            const float A = a.advantages[b];
+            const int act = a.actions[b];
+            for (int k = 0; k < m; ++k) {
+                const float lp = lg[k] - mx - lt, p = expf(lp);
+                lg[k] = A * ((k == act ? 1.f : 0.f) - p) - a.beta * p * (lp + ent);
+            }
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < Z; k += kHeadThreads) a.Zbuf[(size_t)b * Z + k] = z[k];
+        for (int j = threadIdx.x; j < m; j += kHeadThreads) a.DLOG[(size_t)b * m + j] = lg[j];
+        for (int k = threadIdx.x; k < Hh; k += kHeadThreads) {
+            float acc = 0.f;
+            for (int j = 0; j < m; ++j) acc = fmaf(lg[j], W2[(size_t)k * m + j], acc);
+            acc = hid[k] > 0.f ? acc : 0.f;
+            dhid[k] = acc;
+            a.HID[(size_t)b * Hh + k] = hid[k];
+            a.DHID[(size_t)b * Hh + k] = acc;
+        }
+        __syncthreads();
+        for (int i0 = 4 * warp; i0 < Z; i0 += 4 * (kHeadThreads / 32)) {       // a warp per four inputs: their weight rows are contiguous
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+            for (int k = lane; k < Hh; k += 32) {
+                const float x = dhid[k];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) acc[r] = fmaf(x, __ldg(a.head.W1 + (size_t)min(i0 + r, Z - 1) * Hh + k), acc[r]);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+                if (lane == 0 && i0 + r < Z) dz[i0 + r] = acc[r];
+            }
+        }
+        __syncthreads();
+        // through h_i: dpre_h = dz_a * (a > 0); dS = dpre_h W_h^T
+        for (int i = threadIdx.x; i < 3 * d; i += kHeadThreads) {
+            const float v = z[E + i] > 0.f ? dz[E + i] : 0.f;
+            dpre[i] = v;
+            a.DPRE_H[(size_t)b * 3 * d + i] = v;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 * d; i += kHeadThreads) {
+            const int set = i / d, k = i - set * d;
+            a.dS[(size_t)b * 3 * d + i] = strided_dot(0.f, dpre + set * d, a.h[set].W1 + (size_t)k * d, 1, d);
+        }
+        for (int k = threadIdx.x; k < 2 * d; k += kHeadThreads) a.dZ[(size_t)b * 2 * d + k] = dz[k];
         __syncthreads();
     }
 }
@@ -663,14 +795,22 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
         if (split) err = launch_grad_pool_forward(a, di, stream);
         if (err != cudaSuccess) return err;
         const size_t E = 2 * (size_t)d + F;
-        const size_t floats = 2 * (size_t)Z + 2 * (size_t)Hh + 6 * (size_t)d + ((m + 3) & ~3) +
-                              (size_t)(kThreads / 32) * 3 * d + (size_t)(kThreads / 32) * ((E + 3) & ~size_t(3)) +
-                              (split ? 0 : 3 * (E * d + d));
-        const size_t smem = floats * sizeof(float);
-        void (*kern)(const GradArgs) = split ? grad_head_kernel<true> : grad_head_kernel<false>;
-        err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess) return err;
-        kern<<<std::min(B, 8 * di.sm_count), kThreads, smem, stream>>>(a);
+        const size_t vectors = 2 * (size_t)Z + 2 * (size_t)Hh + 6 * (size_t)d;
+        if (split) {
+            const size_t own = vectors + m, w2 = (size_t)Hh * m;
+            const int staged = (own + w2) * sizeof(float) <= 96 * 1024 ? (int)w2 : 0;
+            const size_t smem = (own + staged) * sizeof(float);
+            err = cudaFuncSetAttribute(grad_head_pooled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (err != cudaSuccess) return err;
+            grad_head_pooled_kernel<<<std::min(B, 2 * di.sm_count), kHeadThreads, smem, stream>>>(a, staged);
+        } else {
+            const size_t floats = vectors + ((m + 3) & ~3) + (size_t)(kThreads / 32) * 3 * d +
+                                  (size_t)(kThreads / 32) * ((E + 3) & ~size_t(3)) + 3 * (E * d + d);
+            const size_t smem = floats * sizeof(float);
+            err = cudaFuncSetAttribute(grad_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (err != cudaSuccess) return err;
+            grad_head_kernel<<<std::min(B, 8 * di.sm_count), kThreads, smem, stream>>>(a);
+        }
         count_launch();
         if (split) err = launch_grad_pool_backward(a, di, stream);
         if (err != cudaSuccess) return err;
