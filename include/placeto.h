@@ -160,12 +160,12 @@ typedef struct {
 #define PLACETO_COOPERATIVE 4u /* persistent cooperative launch: a level's nodes are spread over
                                   blocks, grid-wide sync between levels (small B, wide levels) */
 #define PLACETO_GENERIC 8u     /* use only the dimension-generic kernels (no specialised ones) */
-#define PLACETO_FMA_ONLY 16u   /* keep step 2 on the FP32 FMA pipes: do not use the tensor-core
-                                  kernel (operands split into half-precision pieces whose products
+#define PLACETO_FMA_ONLY 16u   /* keep steps 2 and 3 on the FP32 FMA pipes: do not use the tensor-core
+                                  kernels (operands split into half-precision pieces whose products
                                   carry FP32 accuracy) that d = 64 and large batches otherwise take */
 #define PLACETO_TENSOR 32u     /* use the tensor-core kernel of step 2 wherever it applies (d = 32 or 64) */
-#define PLACETO_TCGEN05 64u    /* d = 64: take the kernel built on tcgen05.mma with accumulators in tensor
-                                  memory instead of the warp-level (mma.sync) tensor-core kernel that is
+#define PLACETO_TCGEN05 64u    /* d = 64: take the kernels built on tcgen05.mma with accumulators in tensor
+                                  memory instead of the warp-level (mma.sync) tensor-core kernels that are
                                   the default there (measured slower at the configured batch sizes) */
 #define PLACETO_PIPELINE 128u  /* d = 64, two layers: take the kernel that runs the four layers of g and f as a
                                   pipeline on TF32 operands (a group of warps per layer, tiles of eight rows).

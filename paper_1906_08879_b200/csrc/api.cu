@@ -87,7 +87,8 @@ struct Layout {
     size_t compact;                // episode call: the compact states [n][E]
     int chunks, chunk_nodes;       // node chunks of the generic pooling kernel
     int chunks32, chunk_nodes32;   // and of the d = 32 / d = 64 kernel (0 when neither can apply)
-    int chunks_tc, chunk_nodes_tc; // and of the tensor-core kernel of d = 64 or 32 (0 when it cannot apply or is not faster)
+    int chunks_split, chunk_nodes_split; // and of the tensor-core kernel of both (0 when it cannot apply or is not faster)
+    int chunks_tc, chunk_nodes_tc; // and of the tcgen05 kernel of d = 64 (0 when it cannot apply)
 };
 
 // Workspace layout shared by every call; a call uses the leading part it needs.
@@ -126,13 +127,13 @@ Layout make_layout(const placeto_graph *g, const placeto_weights *w, int B, plac
         return L;
     }
     if (w->F <= 16) {
-        if (w->d == 32) pool_split_chunks((int)n, B, g->info, &L.chunk_nodes_tc, &L.chunks_tc);
+        if (w->d == 32 || w->d == 64) pool_split_chunks((int)n, B, w->d, g->info, &L.chunk_nodes_split, &L.chunks_split);
         if (w->d == 32) pool_d32_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
         if (w->d == 64 && (w->F & 3) == 0) pool_d64_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
         if (w->d == 64) pool_tc_chunks((int)n, B, g->info, &L.chunk_nodes_tc, &L.chunks_tc);
     }
     if (call == PLACETO_CALL_LOGITS || (call >= PLACETO_CALL_FORWARD && call <= PLACETO_CALL_EPISODE))
-        L.partial = take((size_t)std::max(L.chunks, std::max(L.chunks32, L.chunks_tc)) * B * 3 * d * sizeof(float));
+        L.partial = take((size_t)std::max(std::max(L.chunks, L.chunks_split), std::max(L.chunks32, L.chunks_tc)) * B * 3 * d * sizeof(float));
     if (call >= PLACETO_CALL_FORWARD && call <= PLACETO_CALL_EPISODE) {
         L.X = take(n * B * F * sizeof(float));
         L.H[0] = take(n * B * d * sizeof(float));
@@ -273,8 +274,8 @@ placeto_status run_pool(const placeto_graph *g, const placeto_weights *w, const 
     a.logits = logits; a.probs = probs;
     a.n = g->host.n; a.B = B; a.F = w->F; a.d = w->d; a.m = w->m;
     const bool fast32 = pool_d32_applicable(a), fast64 = pool_d64_applicable(a);
-    if (!(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY)) && L.chunks_tc > 0 && pool_split_applicable(a)) {
-        a.chunks = L.chunks_tc; a.chunk_nodes = L.chunk_nodes_tc;
+    if (!(flags & (PLACETO_GENERIC | PLACETO_FMA_ONLY | PLACETO_TCGEN05)) && L.chunks_split > 0 && pool_split_applicable(a)) {
+        a.chunks = L.chunks_split; a.chunk_nodes = L.chunk_nodes_split;
         cudaError_t e = launch_pool_split(a, g->info, stream, after_own_kernel);
         if (e == cudaSuccess) return cuda_status(launch_pool_head(a, g->info, stream));
         if (e != cudaErrorNotSupported) return cuda_status(e);

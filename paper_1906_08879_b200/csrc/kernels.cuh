@@ -439,9 +439,9 @@ cudaError_t launch_policy_generic(const PoolArgs &a, const DeviceInfo &di, cudaS
 cudaError_t launch_pool_head(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream);
 
 // policy_d32.cu: specialised partial sums for d = 32, F <= 16, single-layer ReLU l_i
-// pool_split.cu: d = 32 pooling on the tensor cores (exact half-precision pieces)
+// pool_split.cu: d = 32 and 64 pooling on the tensor cores (exact half-precision pieces)
 bool pool_split_applicable(const PoolArgs &a);
-void pool_split_chunks(int n, int B, const DeviceInfo &di, int *chunk_nodes, int *chunks);   // *chunks = 0: the FMA kernel is faster
+void pool_split_chunks(int n, int B, int d, const DeviceInfo &di, int *chunk_nodes, int *chunks);   // *chunks = 0: the FMA kernel is faster
 cudaError_t launch_pool_split(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
 
 bool pool_d32_applicable(const PoolArgs &a);

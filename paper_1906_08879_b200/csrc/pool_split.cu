@@ -1,22 +1,25 @@
-// Step 3 of the policy (Sec. 2.2 step 3 of the Placeto paper) for d = 32 with single-layer ReLU l_i
+// Step 3 of the policy (Sec. 2.2 step 3 of the Placeto paper) for d = 32 and 64 with single-layer ReLU l_i
 // on the tensor cores: the per-set sums
 //   sum_{u in S_i(c)} l_i(e_u),   e_u = [h_down_u || h_up_u || x_u],
 // over a chunk of nodes of a state, written as the partial sums that the head kernel adds up.
 //
-// Rows (node, state) depend on nothing, so this is a throughput problem: 32 (64 + F) multiply-adds a
+// Rows (node, state) depend on nothing, so this is a throughput problem: d (2 d + F) multiply-adds a
 // row. On the FP32 units (policy_d32.cu) that is what bounds it: 219 us for 992 nodes in 992 states,
-// F = 12 (106 here; 1080 nodes x 256 states, F = 8: 63 and 37). Here sixteen rows of a (state, set) are the 16 rows of mma.sync.m16n8k16, on exact pieces of
-// three bfloat16 numbers (Bf16x3, six products), which the pipe takes in a quarter of the time.
+// d = 32, F = 12 (103 here; 1080 nodes x 256 states, F = 8: 63 and 37). Here sixteen rows of a (state, set)
+// are the 16 rows of mma.sync.m16n8k16. d = 32: on exact pieces of three bfloat16 numbers (Bf16x3, six
+// products). d = 64: on two half-precision pieces (Fp16x2, three products; a row's two embeddings and its raw features
+// scaled apart, since they are of different size): 217 us for 1987 nodes x 512 states, 244 on the tcgen05 kernel (policy_tc.cu),
+// whose producers and barriers cost 19 us on the smallest call, 6.4 here. (Fp16x2 at d = 32: 91 us, but 3e-5 of error
+// where one logit of one device is what cancellation left, above the 2e-5 that FP32 keeps.)
 //   - A warp owns items (state, chunk of nodes) and walks the three sets one by one; it compacts the
 //     relation row of the state into the set's node list and takes the list sixteen at a time.
 //   - The rows go from memory straight into A fragments: the inner index is permuted so that the four
 //     numbers a lane needs of a 16-wide step are adjacent (one 128-bit load, 64 contiguous bytes of a row per step).
 //   - The weights' pieces lie in shared memory as B fragments, split once per block; reading them costs
 //     half of what the instructions they feed take.
-// Warps never wait for one another; sixteen of them per SM cover the loads (the tensor pipe is busy 58 % of the time. Reading a
-// tile's rows during the tile before, at twelve or sixteen warps, takes registers from the chains: 108 and 114 us). Products of the leading pieces
-// are kept in two chains and the small ones in a third, since the tensor core's accumulation truncates.
-// Summation order is fixed, so results are reproducible bit for bit.
+// Warps never wait for one another; twelve or sixteen of them per SM cover the loads (d = 32: the tensor pipe is busy 58 %
+// of the time. Reading a tile's rows during the tile before, at twelve or sixteen warps, takes registers from the
+// chains: 108 and 114 us instead of 106). Summation order is fixed, so results are reproducible bit for bit.
 #include <algorithm>
 
 #include "kernels.cuh"
@@ -27,48 +30,72 @@ namespace placeto {
 namespace {
 
 using split::Bf16x3;
+using split::Fp16x2;
 
-constexpr int kD = 32, kNT = kD / 8, kKS = 2 * kD / 16 + 1;     // output tiles, 16-wide steps (the last: raw features)
-constexpr int kWarps = 16, kThreads = kWarps * 32, kTile = 16;
-constexpr int kMaxChunk = 1024;
-constexpr int kPieces = Bf16x3::kPieces;
-constexpr int kFragments = 3 * kKS * kPieces * 2 * 32;          // uint4 of weight fragments
+constexpr int kTile = 16, kMaxChunk = 1024;
+
+// Widths of a shape: output tiles, 16-wide steps of either embedding (one more for the raw features), warps of a block.
+template <int D> struct Shape {
+    typedef std::conditional_t<D == 32, Bf16x3, Fp16x2> SP;
+    static constexpr int kPieces = SP::kPieces;
+    static constexpr int NT = D / 8, KE = D / 16, KS = 2 * KE + 1;
+    static constexpr int kWarps = D == 32 ? 16 : 12, kThreads = kWarps * 32;
+    static constexpr int kFragments = 3 * KS * kPieces * (NT / 2) * 32;          // uint4 of weight fragments
+};
 
 struct PoolSplitPlan {
     int chunk_nodes, chunks, items;
 };
 
+template <int D>
 size_t smem_bytes(int chunk_nodes) {
-    return (size_t)kFragments * sizeof(uint4) + 3 * kD * sizeof(float) + (size_t)kWarps * ((chunk_nodes + 7) & ~7) * sizeof(uint16_t);
+    return (size_t)Shape<D>::kFragments * sizeof(uint4) + (3 * D + 20) * sizeof(float) +
+           (size_t)Shape<D>::kWarps * ((chunk_nodes + 7) & ~7) * sizeof(uint16_t);
 }
 
-template <bool kCompact, bool kVec>      // raw features from compact states; in rows of whole 16-byte pieces
-__global__ void __launch_bounds__(kThreads, 1)
+template <int D, bool kCompact, bool kVec>      // raw features from compact states; in rows of whole 16-byte pieces
+__global__ void __launch_bounds__(Shape<D>::kThreads, 1)
 pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
+    typedef Shape<D> C;
+    typedef typename C::SP SP;
+    constexpr int kPieces = C::kPieces;
+    constexpr int NT = C::NT, KE = C::KE, KS = C::KS, kWarps = C::kWarps, kThreads = C::kThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int n = a.n, B = a.B, F = a.F;
-    uint4 *frag = reinterpret_cast<uint4 *>(smem_raw);                  // [set][step][piece][half of the tiles][lane]
-    float *bias_s = reinterpret_cast<float *>(frag + kFragments);       // [3][32]
-    uint16_t *list = reinterpret_cast<uint16_t *>(bias_s + 3 * kD) + (size_t)warp * ((p.chunk_nodes + 7) & ~7);
+    uint4 *frag = reinterpret_cast<uint4 *>(smem_raw);                  // [set][step][piece][pair of tiles][lane]
+    float *bias_s = reinterpret_cast<float *>(frag + C::kFragments);    // [3][D]
+    float *scale_s = bias_s + 3 * D;                                    // [3][segment]: what the weights are multiplied by
+    uint16_t *list = reinterpret_cast<uint16_t *>(scale_s + 20) + (size_t)warp * ((p.chunk_nodes + 7) & ~7);
+    // the three segments of a row: h_down, h_up, raw features
+    auto segment_of = [](int ks) { return ks < KE ? 0 : ks < 2 * KE ? 1 : 2; };
 
     // ---- weights as fragments: lane (g, t) of tile nt holds rows 16 ks + 4 t .. + 3 of column 8 nt + g
-    for (int i = threadIdx.x; i < 3 * kKS * kNT * 32; i += kThreads) {
-        const int l = i & 31, nt = (i >> 5) % kNT, ks = (i >> 5) / kNT % kKS, set = (i >> 5) / (kNT * kKS);
-        const float *W = a.l[set].W1;
+    for (int i = warp; SP::kScaled && i < 9; i += kWarps) {
+        const float *W = a.l[i / 3].W1 + (i % 3) * D * D;
+        float top = 0.f;
+        for (int k = lane; k < (i % 3 == 2 ? F : D) * D; k += 32) top = fmaxf(top, fabsf(W[k]));
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        if (lane == 0) scale_s[i] = split::scale_up(top);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * KS * NT * 32; i += kThreads) {
+        const int l = i & 31, nt = (i >> 5) % NT, ks = (i >> 5) / NT % KS, set = (i >> 5) / (NT * KS);
+        const float *W = a.l[set].W1, up = SP::kScaled ? scale_s[set * 3 + segment_of(ks)] : 1.f;
         const int k0 = 16 * ks + 4 * (l & 3), col = 8 * nt + (l >> 2);
         float w[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = k0 + j < 2 * kD + F ? W[(k0 + j) * kD + col] : 0.f;
+        for (int j = 0; j < 4; ++j) w[j] = k0 + j < 2 * D + F ? W[(k0 + j) * D + col] * up : 0.f;
         unsigned lo[kPieces], hi[kPieces];
-        Bf16x3::pieces(w[0], w[1], lo);
-        Bf16x3::pieces(w[2], w[3], hi);
+        SP::pieces(w[0], w[1], lo);
+        SP::pieces(w[2], w[3], hi);
 #pragma unroll
         for (int q = 0; q < kPieces; ++q)
-            reinterpret_cast<uint2 *>(frag + (((set * kKS + ks) * kPieces + q) * 2 + nt / 2) * 32 + l)[nt & 1] = make_uint2(lo[q], hi[q]);
+            reinterpret_cast<uint2 *>(frag + (((set * KS + ks) * kPieces + q) * (NT / 2) + nt / 2) * 32 + l)[nt & 1] = make_uint2(lo[q], hi[q]);
     }
-    if (threadIdx.x < 3 * kD) bias_s[threadIdx.x] = a.l[threadIdx.x / kD].b1[threadIdx.x % kD];
+    for (int i = threadIdx.x; i < 3 * D; i += kThreads) bias_s[i] = a.l[i / D].b1[i % D];
     __syncthreads();
     dependency_wait();          // the embeddings may come from a kernel that is still running
 
@@ -79,7 +106,7 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
         const bool valid = c >= 0 && c < n;
         PLACETO_DEBUG_CHECK(a.status, valid);
         const uint8_t *rel = a.relation + (size_t)(valid ? c : 0) * n + u0;
-        float *out = a.partial + ((size_t)chunk * B + b) * 3 * kD;
+        float *out = a.partial + ((size_t)chunk * B + b) * 3 * D;
 #pragma unroll 1
         for (int set = 0; set < 3; ++set) {
             int count = 0;
@@ -90,22 +117,22 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
                 count += __popc(mask);
             }
             __syncwarp();
-            float total[kNT][2];
+            float total[NT][2];
 #pragma unroll
-            for (int nt = 0; nt < kNT; ++nt) total[nt][0] = total[nt][1] = 0.f;
-            const uint4 *fr = frag + (size_t)set * kKS * kPieces * 2 * 32 + lane;
+            for (int nt = 0; nt < NT; ++nt) total[nt][0] = total[nt][1] = 0.f;
+            const uint4 *fr = frag + (size_t)set * KS * kPieces * (NT / 2) * 32 + lane;
 #pragma unroll 1
             for (int first = 0; first < count; first += kTile) {
                 // rows past the end repeat the last one
                 const int u[2] = {u0 + list[min(first + g, count - 1)], u0 + list[min(first + 8 + g, count - 1)]};
-                float4 x[kKS][2];
+                float4 x[KS][2];
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     const size_t row = (size_t)u[r] * B + b;
 #pragma unroll
-                    for (int ks = 0; ks < kKS - 1; ++ks)
-                        x[ks][r] = *reinterpret_cast<const float4 *>(a.H[ks >= 2] + row * kD + 16 * (ks & 1) + 4 * t);
-                    float4 &f = x[kKS - 1][r];
+                    for (int ks = 0; ks < KS - 1; ++ks)
+                        x[ks][r] = *reinterpret_cast<const float4 *>(a.H[ks >= KE] + row * D + 16 * (ks % KE) + 4 * t);
+                    float4 &f = x[KS - 1][r];
                     f = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (kCompact) {
                         // [cost, bytes, one-hot_m(device), u == current, visited], this lane's four
@@ -128,97 +155,132 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
                             if (4 * t + j < F) v[j] = a.X[row * F + 4 * t + j];
                     }
                 }
-                // chains: leading products of the first steps, of the others, and all small ones
-                float acc[3][kNT][4];
+                // every segment of a row is scaled by itself (where the pieces need it)
+                unsigned A[KS][kPieces][4];
+                float down_by[3][2];
 #pragma unroll
-                for (int ks = 0; ks < kKS; ++ks) {
-                    unsigned A[kPieces][4];
-                    {
-                        unsigned q[4][kPieces];
-                        Bf16x3::pieces(x[ks][0].x, x[ks][0].y, q[0]);
-                        Bf16x3::pieces(x[ks][1].x, x[ks][1].y, q[1]);
-                        Bf16x3::pieces(x[ks][0].z, x[ks][0].w, q[2]);
-                        Bf16x3::pieces(x[ks][1].z, x[ks][1].w, q[3]);
+                for (int seg = 0; seg < 3; ++seg) {
+                    const int k0 = seg == 2 ? 2 * KE : seg * KE, k1 = seg == 2 ? KS : k0 + KE;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
+                    for (int r = 0; r < 2; ++r) {
+                        float top = 0.f, up = 1.f;
 #pragma unroll
-                            for (int k = 0; k < kPieces; ++k) A[k][i] = q[i][k];
-                    }
-                    // products (piece of the rows, piece of the weights) in the order in which the weights' pieces are read
-                    auto product = [&](auto chain, auto fresh, const unsigned (&rows)[4], const uint4 (&w)[2]) {
-                        constexpr int ch = decltype(chain)::value;
-#pragma unroll
-                        for (int nt = 0; nt < kNT; ++nt) {
-                            const unsigned b0 = (nt & 1) ? w[nt / 2].z : w[nt / 2].x, b1 = (nt & 1) ? w[nt / 2].w : w[nt / 2].y;
-                            if (decltype(fresh)::value) Bf16x3::mma_zero(acc[ch][nt], rows, b0, b1);
-                            else Bf16x3::mma(acc[ch][nt], rows, b0, b1);
+                        for (int ks = k0; SP::kScaled && ks < k1; ++ks) {
+                            const float4 v = x[ks][r];
+                            top = fmaxf(top, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
                         }
-                    };
-                    typedef std::integral_constant<int, 0> lead0;
-                    typedef std::integral_constant<int, 1> lead1;
-                    typedef std::integral_constant<int, 2> small;
-                    const uint4 *w_at = fr + ks * kPieces * 2 * 32;
-                    uint4 w[2] = {w_at[128], w_at[160]};                             // third piece
-                    if (ks == 0) product(small(), std::true_type(), A[0], w);
-                    else product(small(), std::false_type(), A[0], w);
-                    w[0] = w_at[64]; w[1] = w_at[96];                                // second
-                    product(small(), std::false_type(), A[0], w);
-                    product(small(), std::false_type(), A[1], w);
-                    w[0] = w_at[0]; w[1] = w_at[32];
-                    product(small(), std::false_type(), A[2], w);
-                    product(small(), std::false_type(), A[1], w);
-                    if (ks == 0) product(lead0(), std::true_type(), A[0], w);
-                    else if (ks == 1) product(lead0(), std::false_type(), A[0], w);
-                    else if (ks == 2) product(lead1(), std::true_type(), A[0], w);
-                    else product(lead1(), std::false_type(), A[0], w);
+                        if (SP::kScaled) {
+                            top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 1));
+                            top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
+                            up = split::scale_up(top);
+                            down_by[seg][r] = split::inverse_pow2(up);
+                        }
+#pragma unroll
+                        for (int ks = k0; ks < k1; ++ks) {
+                            const float4 v = x[ks][r];
+                            unsigned lo[kPieces], hi[kPieces];
+                            SP::pieces(v.x * up, v.y * up, lo);
+                            SP::pieces(v.z * up, v.w * up, hi);
+#pragma unroll
+                            for (int q = 0; q < kPieces; ++q) { A[ks][q][r] = lo[q]; A[ks][q][2 + r] = hi[q]; }
+                        }
+                    }
                 }
                 const bool live[2] = {first + g < count, first + 8 + g < count};
 #pragma unroll
-                for (int nt = 0; nt < kNT; ++nt) {
-                    const float2 bias = *reinterpret_cast<const float2 *>(bias_s + set * kD + 8 * nt + 2 * t);
+                for (int half = 0; half < NT / 4; ++half) {
+                    // Chains. Scaled: one per segment, small products before the leading one of a step. Not scaled: leading
+                    // products of the first steps, of the others, and all small ones (the tensor core's accumulation truncates).
+                    float acc[3][4][4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float v = ((acc[0][nt][i] + acc[1][nt][i]) + acc[2][nt][i]) + ((i & 1) ? bias.y : bias.x);
-                        total[nt][i & 1] += live[i >> 1] ? fmaxf(v, 0.f) : 0.f;
+                    for (int ks = 0; ks < KS; ++ks) {
+                        const uint4 *w_at = fr + ks * kPieces * (NT / 2) * 32 + half * 64;
+                        auto product = [&](int chain, bool zero, const unsigned (&rows)[4], const uint4 (&w)[2]) {
+#pragma unroll
+                            for (int nt = 0; nt < 4; ++nt) {
+                                const unsigned b0 = (nt & 1) ? w[nt / 2].z : w[nt / 2].x, b1 = (nt & 1) ? w[nt / 2].w : w[nt / 2].y;
+                                if (zero) SP::mma_zero(acc[chain][nt], rows, b0, b1);
+                                else SP::mma(acc[chain][nt], rows, b0, b1);
+                            }
+                        };
+                        auto weights = [&](int piece, uint4 (&w)[2]) {
+                            w[0] = w_at[piece * (NT / 2) * 32];
+                            w[1] = w_at[piece * (NT / 2) * 32 + 32];
+                        };
+                        uint4 w[2];
+                        if constexpr (SP::kScaled) {
+                            const int seg = segment_of(ks);
+                            weights(1, w);
+                            product(seg, ks == 0 || ks == KE || ks == 2 * KE, A[ks][0], w);
+                            weights(0, w);
+                            product(seg, false, A[ks][1], w);
+                            product(seg, false, A[ks][0], w);
+                        } else {
+                            weights(2, w);
+                            product(2, ks == 0, A[ks][0], w);
+                            weights(1, w);
+                            product(2, false, A[ks][0], w);
+                            product(2, false, A[ks][1], w);
+                            weights(0, w);
+                            product(2, false, A[ks][kPieces - 1], w);
+                            product(2, false, A[ks][1], w);
+                            product(ks < 2 ? 0 : 1, ks == 0 || ks == 2, A[ks][0], w);
+                        }
+                    }
+                    float back[3];              // the weights' scales undone
+#pragma unroll
+                    for (int seg = 0; seg < 3; ++seg) back[seg] = SP::kScaled ? split::inverse_pow2(scale_s[set * 3 + seg]) : 1.f;
+#pragma unroll
+                    for (int nt = 0; nt < 4; ++nt) {
+                        const float2 bias = *reinterpret_cast<const float2 *>(bias_s + set * D + 32 * half + 8 * nt + 2 * t);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int r = i >> 1;
+                            float part[3];
+#pragma unroll
+                            for (int q = 0; q < 3; ++q) part[q] = SP::kScaled ? (acc[q][nt][i] * down_by[q][r]) * back[q] : acc[q][nt][i];
+                            const float v = ((part[0] + part[1]) + part[2]) + ((i & 1) ? bias.y : bias.x);
+                            total[4 * half + nt][i & 1] += live[r] ? fmaxf(v, 0.f) : 0.f;
+                        }
                     }
                 }
             }
             __syncwarp();       // the list is read
 #pragma unroll
-            for (int nt = 0; nt < kNT; ++nt) {
+            for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) {
                     total[nt][0] += __shfl_xor_sync(0xffffffffu, total[nt][0], o);
                     total[nt][1] += __shfl_xor_sync(0xffffffffu, total[nt][1], o);
                 }
-                if (g == nt) *reinterpret_cast<float2 *>(out + set * kD + 8 * nt + 2 * t) = make_float2(total[nt][0], total[nt][1]);
+                if (g == nt) *reinterpret_cast<float2 *>(out + set * D + 8 * nt + 2 * t) = make_float2(total[nt][0], total[nt][1]);
             }
         }
     }
 }
 
-bool relu1(const DevMlp &m, int in) {
-    return m.n_layers == 1 && m.in_dim == in && m.out_dim == kD && m.act == 0 && m.final_act == 1;
+bool relu1(const DevMlp &m, int in, int d) {
+    return m.n_layers == 1 && m.in_dim == in && m.out_dim == d && m.act == 0 && m.final_act == 1;
 }
 
 }  // namespace
 
 bool pool_split_applicable(const PoolArgs &a) {
-    if (a.d != kD || a.F < 1 || a.F > 16) return false;
+    if ((a.d != 32 && a.d != 64) || a.F < 1 || a.F > 16) return false;
     for (int i = 0; i < 3; ++i)
-        if (!relu1(a.l[i], 2 * kD + a.F)) return false;
+        if (!relu1(a.l[i], 2 * a.d + a.F, a.d)) return false;
     return true;
 }
 
-// Below 4096 rows the FMA kernel, whose weights need no splitting, is faster (pooling and head together: 279 nodes x 1
+// d = 32: below 4096 rows the FMA kernel, whose weights need no splitting, is faster (pooling and head together: 279 nodes x 1
 // state 14.1 us there, 14.7 here; 300 x 16: 16.4 and 14.5; 300 x 64: 17.3 and 16.5; 279 x 256: 23.7 and 21.3).
 // A warp takes whole items, so the batch costs (items per warp, rounded up) x (tiles per item); a set's last tile is
 // half empty on average.
-void pool_split_chunks(int n, int B, const DeviceInfo &di, int *chunk_nodes, int *chunks) {
-    const long warps = (long)di.sm_count * kWarps;
+void pool_split_chunks(int n, int B, int d, const DeviceInfo &di, int *chunk_nodes, int *chunks) {
+    const long warps = (long)di.sm_count * (d == 32 ? Shape<32>::kWarps : Shape<64>::kWarps);
     double best = 0;
     *chunks = 0;
-    if ((long)n * B < 4096) return;
+    if (d == 32 && (long)n * B < 4096) return;
     for (int c = (n + kMaxChunk - 1) / kMaxChunk; c <= std::max(1, n / 16); ++c) {
         const int nodes = (n + c - 1) / c;
         if ((n + nodes - 1) / nodes != c) continue;
@@ -228,20 +290,27 @@ void pool_split_chunks(int n, int B, const DeviceInfo &di, int *chunk_nodes, int
     if (*chunks == 0) { *chunk_nodes = std::min(n, kMaxChunk); *chunks = (n + *chunk_nodes - 1) / *chunk_nodes; }
 }
 
+namespace {
+template <int D>
+cudaError_t launch(const PoolArgs &a, const PoolSplitPlan &p, const DeviceInfo &di, cudaStream_t stream, bool overlap) {
+    const size_t bytes = smem_bytes<D>(p.chunk_nodes);
+    if (bytes > (size_t)di.max_smem_optin || p.chunk_nodes > kMaxChunk) return cudaErrorNotSupported;
+    auto kern = (a.F & 3) == 0 ? pool_split_kernel<D, false, true> : pool_split_kernel<D, false, false>;
+    if (D == 32 && a.compact.state) kern = pool_split_kernel<32, true, true>;      // only episodes at d = 32 keep compact states
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (err != cudaSuccess) return err;
+    err = launch_overlapped(overlap, kern, dim3(std::min(di.sm_count, p.items)), dim3(Shape<D>::kThreads), bytes, stream, a, p);
+    count_launch();
+    return err;
+}
+}  // namespace
+
 cudaError_t launch_pool_split(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap) {
     PoolSplitPlan p;
     p.chunk_nodes = a.chunk_nodes;
     p.chunks = a.chunks;
     p.items = a.B * a.chunks;
-    const size_t bytes = smem_bytes(p.chunk_nodes);
-    if (bytes > (size_t)di.max_smem_optin || p.chunk_nodes > kMaxChunk) return cudaErrorNotSupported;
-    auto kern = a.compact.state ? pool_split_kernel<true, true> : (a.F & 3) == 0 ? pool_split_kernel<false, true> : pool_split_kernel<false, false>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (err != cudaSuccess) return err;
-    const int grid = std::min(di.sm_count, p.items);
-    err = launch_overlapped(overlap, kern, dim3(grid), dim3(kThreads), bytes, stream, a, p);
-    count_launch();
-    return err;
+    return a.d == 32 ? launch<32>(a, p, di, stream, overlap) : launch<64>(a, p, di, stream, overlap);
 }
 
 }  // namespace placeto

@@ -377,17 +377,18 @@ def test_split_sweep_kernel_over_tiles(d, m, B, layers):
     assert_close(logits, oracle.forward(cfg)["logits"], "logits")
 
 
-@pytest.mark.parametrize("n,m,B", [(9, 4, 1000), (37, 3, 900), (300, 8, 40), (1100, 5, 8)])
-def test_split_pooling_over_chunks_and_sets(n, m, B):
-    """Tensor-core pooling at d = 32: sets that are empty, of less than a tile and of several, chunks of one node list and of
+@pytest.mark.parametrize("n,m,B,d", [(9, 4, 1000, 32), (37, 3, 900, 32), (300, 8, 40, 32), (1100, 5, 8, 32), (9, 8, 5, 64), (37, 5, 300, 64),
+                                     (1100, 4, 7, 64)])
+def test_split_pooling_over_chunks_and_sets(n, m, B, d):
+    """Tensor-core pooling: sets that are empty, of less than a tile and of several, chunks of one node list and of
     several, feature rows that are and are not 16-byte aligned, a current node out of range; beside the FMA kernel."""
     r = rng(n + B)
     src, dst = random_dag(r, n, 2.5 / n)
-    cfg = {"n": n, "src": src, "dst": dst, "m": m, "d": 32, "F": m + 4}
+    cfg = {"n": n, "src": src, "dst": dst, "m": m, "d": d, "F": m + 4}
     cfg["cost"], cfg["bytes"] = states.node_costs(r, n, normalise=True)
     cfg["dev"], cfg["cur"], cfg["placed"] = states.random_states(r, n, m, B)
     cfg["cur"][:2] = 0, n - 1
-    cfg["weights"] = states.policy_weights(r, 32, m + 4, m, 2, 0, 0.1)
+    cfg["weights"] = states.policy_weights(r, d, m + 4, m, 2, 0, 0.1)
     out = gpu_forward(cfg)
     compare(cfg, out, oracle.forward(cfg))
     assert_close(out["logits"], gpu_forward(cfg, placeto.PLACETO_FMA_ONLY)["logits"].cpu().numpy(), "logits of the FMA kernel")
