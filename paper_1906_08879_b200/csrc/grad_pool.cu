@@ -50,23 +50,27 @@ __device__ __forceinline__ bool find_batch(const Lists &l, int k, int &set, int 
     return false;
 }
 
+// Warps of a block: at d = 64 the networks leave room for one block per SM, which takes the warps of two (531 nodes x 100
+// states: forward 110 -> 76 us).
+template <int D> constexpr int kPoolWarps = D == 32 ? 8 : 16;
+
 // relu(l_i(e_u)) of every row: sums per (chunk, state, set), and one bit per column, positive or not
 template <int D>
-__global__ void __launch_bounds__(kRowThreads)
+__global__ void __launch_bounds__(32 * kPoolWarps<D>)
 grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
-    constexpr int C = D / 32;
+    constexpr int C = D / 32, kWarps = kPoolWarps<D>, kThreads = 32 * kWarps;
     extern __shared__ __align__(16) float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n = a.n, B = a.B, F = a.F, E = 2 * D + F, Ep = (E + 3) & ~3;
     float *W = smem;                                     // [3][Ep][D], zero padded
     float *in = W + 3 * Ep * D + warp * kRowsPerWarp * Ep;
-    float *sums = W + 3 * Ep * D + kRowWarps * kRowsPerWarp * Ep;       // [batch][D]
+    float *sums = W + 3 * Ep * D + kWarps * kRowsPerWarp * Ep;       // [batch][D]
     const int max_batches = chunk_nodes / kRowsPerWarp + 3;
     Lists l;
     l.count = reinterpret_cast<int *>(sums + max_batches * D);
     l.node = reinterpret_cast<unsigned short *>(l.count + 4);
     for (int i = 0; i < 3; ++i)
-        for (int t = threadIdx.x; t < Ep * D; t += kRowThreads) W[i * Ep * D + t] = t < E * D ? a.l[i].W1[t] : 0.f;
+        for (int t = threadIdx.x; t < Ep * D; t += kThreads) W[i * Ep * D + t] = t < E * D ? a.l[i].W1[t] : 0.f;
     __syncthreads();
     const int items = B * chunks;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
@@ -77,17 +81,28 @@ grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
         build_lists(l, a.relation + (size_t)(valid ? c : 0) * n, u0, nu, chunk_nodes, valid, warp, lane);
         __syncthreads();
         int set, at, rows;
-        for (int k = warp; find_batch(l, k, set, at, rows); k += kRowWarps) {
+        for (int k = warp; find_batch(l, k, set, at, rows); k += kWarps) {
             __syncwarp();
+            // every row requested before the first store: the compiler cannot move a load across one (279 nodes x 256 states: 64 -> 37 us)
+            float down[kRowsPerWarp][C], up[kRowsPerWarp][C], x[kRowsPerWarp];
 #pragma unroll
             for (int r = 0; r < kRowsPerWarp; ++r) {
                 const size_t row = (size_t)l.node[set * chunk_nodes + at + min(r, rows - 1)] * B + b;
 #pragma unroll
                 for (int q = 0; q < C; ++q) {
-                    in[r * Ep + lane + 32 * q] = a.H[0][row * D + lane + 32 * q];
-                    in[r * Ep + D + lane + 32 * q] = a.H[1][row * D + lane + 32 * q];
+                    down[r][q] = a.H[0][row * D + lane + 32 * q];
+                    up[r][q] = a.H[1][row * D + lane + 32 * q];
                 }
-                if (lane < Ep - 2 * D) in[r * Ep + 2 * D + lane] = lane < F ? a.X[row * F + lane] : 0.f;
+                x[r] = lane < F ? a.X[row * F + lane] : 0.f;
+            }
+#pragma unroll
+            for (int r = 0; r < kRowsPerWarp; ++r) {
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    in[r * Ep + lane + 32 * q] = down[r][q];
+                    in[r * Ep + D + lane + 32 * q] = up[r][q];
+                }
+                if (lane < Ep - 2 * D) in[r * Ep + 2 * D + lane] = x[r];
             }
             __syncwarp();
             float acc[kRowsPerWarp][C];
@@ -113,7 +128,7 @@ grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
             }
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < 3 * D; i += kRowThreads) {
+        for (int i = threadIdx.x; i < 3 * D; i += kThreads) {
             const int s = i / D, j = i - s * D;
             int first = 0;
             for (int q = 0; q < s; ++q) first += (l.count[q] + kRowsPerWarp - 1) / kRowsPerWarp;
@@ -128,19 +143,19 @@ grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
 
 // dpre_l = dS of the row's set where the pre-activation was positive; d/dh = dpre_l W_l^T (its embedding columns)
 template <int D>
-__global__ void __launch_bounds__(kRowThreads)
+__global__ void __launch_bounds__(32 * kPoolWarps<D>)
 grad_pool_backward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
-    constexpr int C = D / 32;
+    constexpr int C = D / 32, kWarps = kPoolWarps<D>, kThreads = 32 * kWarps;
     extern __shared__ __align__(16) float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n = a.n, B = a.B;
     float *Wt = smem;                                    // [3][D][2 D]
     float *in = Wt + 3 * D * 2 * D + warp * kRowsPerWarp * D;
     Lists l;
-    l.count = reinterpret_cast<int *>(Wt + 3 * D * 2 * D + kRowWarps * kRowsPerWarp * D);
+    l.count = reinterpret_cast<int *>(Wt + 3 * D * 2 * D + kWarps * kRowsPerWarp * D);
     l.node = reinterpret_cast<unsigned short *>(l.count + 4);
     for (int i = 0; i < 3; ++i)
-        for (int t = threadIdx.x; t < 2 * D * D; t += kRowThreads) {
+        for (int t = threadIdx.x; t < 2 * D * D; t += kThreads) {
             // a warp reads 4 rows x 8 columns: whole sectors, stores to eight rows
             const int q = t >> 5, j = q % (D / 8) * 8 + (t & 7), k = q / (D / 8) * 4 + (t >> 3 & 3);
             Wt[(i * D + j) * 2 * D + k] = a.l[i].W1[k * D + j];
@@ -154,28 +169,32 @@ grad_pool_backward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
         const bool valid = c >= 0 && c < n;
         build_lists(l, a.relation + (size_t)(valid ? c : 0) * n, u0, nu, chunk_nodes, valid, warp, lane);
         // the current node's embedding enters the head directly; a state without one contributes nothing
-        if (valid && c >= u0 && c < u0 + nu && warp == kRowWarps - 1) {
+        if (valid && c >= u0 && c < u0 + nu && warp == kWarps - 1) {
 #pragma unroll
             for (int q = 0; q < 2 * C; ++q)
                 a.DH[q / C][((size_t)c * B + b) * D + lane + 32 * (q % C)] = a.dZ[(size_t)b * 2 * D + lane + 32 * q];
         }
         if (!valid)
-            for (int i = threadIdx.x; i < nu * D; i += kRowThreads) {
+            for (int i = threadIdx.x; i < nu * D; i += kThreads) {
                 const size_t at = ((size_t)(u0 + i / D) * B + b) * D + i % D;
                 a.DH[0][at] = 0.f;
                 a.DH[1][at] = 0.f;
             }
         __syncthreads();
         int set, at, rows;
-        for (int k = warp; find_batch(l, k, set, at, rows); k += kRowWarps) {
+        for (int k = warp; find_batch(l, k, set, at, rows); k += kWarps) {
             __syncwarp();
 #pragma unroll
             for (int q = 0; q < C; ++q) {
                 const float ds = a.dS[((size_t)b * 3 + set) * D + lane + 32 * q];
+                unsigned bits[kRowsPerWarp];
+#pragma unroll
+                for (int r = 0; r < kRowsPerWarp; ++r)
+                    bits[r] = a.l_masks[((size_t)l.node[set * chunk_nodes + at + min(r, rows - 1)] * B + b) * C + q];
 #pragma unroll
                 for (int r = 0; r < kRowsPerWarp; ++r) {
                     const size_t row = (size_t)l.node[set * chunk_nodes + at + min(r, rows - 1)] * B + b;
-                    const float v = a.l_masks[row * C + q] >> lane & 1 ? ds : 0.f;
+                    const float v = bits[r] >> lane & 1 ? ds : 0.f;
                     in[r * D + lane + 32 * q] = v;
                     if (r < rows) a.DPRE_L[0][row * D + lane + 32 * q] = v;
                 }
@@ -375,32 +394,34 @@ grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const pa
     if (live) write_partial<D, TK>(out + (size_t)blockIdx.x * (K + 1) * D, K, tk, tj, acc);
 }
 
-size_t forward_smem(int D, int F, int chunk_nodes) {
+template <int D>
+size_t forward_smem(int F, int chunk_nodes) {
     const int Ep = (2 * D + F + 3) & ~3;
-    return ((size_t)3 * Ep * D + (size_t)kRowWarps * kRowsPerWarp * Ep + (size_t)(chunk_nodes / kRowsPerWarp + 3) * D + 4) * sizeof(float) +
+    return ((size_t)3 * Ep * D + (size_t)kPoolWarps<D> * kRowsPerWarp * Ep + (size_t)(chunk_nodes / kRowsPerWarp + 3) * D + 4) * sizeof(float) +
            (size_t)3 * chunk_nodes * 2;
 }
-size_t backward_smem(int D, int chunk_nodes) {
-    return ((size_t)6 * D * D + (size_t)kRowWarps * kRowsPerWarp * D + 4) * sizeof(float) + (size_t)3 * chunk_nodes * 2;
+template <int D>
+size_t backward_smem(int chunk_nodes) {
+    return ((size_t)6 * D * D + (size_t)kPoolWarps<D> * kRowsPerWarp * D + 4) * sizeof(float) + (size_t)3 * chunk_nodes * 2;
 }
 
 template <int D>
 cudaError_t launch_forward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
-    const size_t smem = forward_smem(D, a.F, a.pool_chunk_nodes);
+    const size_t smem = forward_smem<D>(a.F, a.pool_chunk_nodes);
     cudaError_t err = cudaFuncSetAttribute(grad_pool_forward_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int grid = std::min(a.B * a.pool_chunks, (D == 32 ? 3 : 1) * di.sm_count);
-    grad_pool_forward_kernel<D><<<grid, kRowThreads, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
+    grad_pool_forward_kernel<D><<<grid, 32 * kPoolWarps<D>, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
     count_launch();
     return cudaGetLastError();
 }
 template <int D>
 cudaError_t launch_backward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
-    const size_t smem = backward_smem(D, a.pool_chunk_nodes);
+    const size_t smem = backward_smem<D>(a.pool_chunk_nodes);
     cudaError_t err = cudaFuncSetAttribute(grad_pool_backward_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int grid = std::min(a.B * a.pool_chunks, (D == 32 ? 4 : 1) * di.sm_count);
-    grad_pool_backward_kernel<D><<<grid, kRowThreads, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
+    grad_pool_backward_kernel<D><<<grid, 32 * kPoolWarps<D>, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
     count_launch();
     return cudaGetLastError();
 }

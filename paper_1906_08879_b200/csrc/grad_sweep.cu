@@ -54,21 +54,34 @@ grad_rows_f_kernel(const GradArgs a) {
     unsigned *masks = a.masks[dir];
     const size_t R = (size_t)a.n * a.B;
     const size_t step = (size_t)gridDim.x * kRowWarps * kRowsPerWarp;
-    for (size_t r0 = ((size_t)blockIdx.x * kRowWarps + warp) * kRowsPerWarp; r0 < R; r0 += step) {
+    // A batch's rows are requested while the batch before is computed, all before the first store: the compiler cannot
+    // move a load across one, and eight round trips in turn bound the kernel (279 nodes x 256 states, d = 32: 62 -> 40 us).
+    float h[kRowsPerWarp][C], x[kRowsPerWarp];
+    auto request = [&](size_t r0) {
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            const size_t row = min(r0 + r, R - 1);       // rows past the last repeat it
+#pragma unroll
+            for (int c = 0; c < C; ++c) h[r][c] = H[row * D + lane + 32 * c];
+            x[r] = lane < F ? a.X[row * F + lane] : 0.f;
+        }
+    };
+    const size_t first = ((size_t)blockIdx.x * kRowWarps + warp) * kRowsPerWarp;
+    if (first < R) request(first);
+    for (size_t r0 = first; r0 < R; r0 += step) {
         const int rows = (int)min((size_t)kRowsPerWarp, R - r0);
         __syncwarp();
 #pragma unroll
         for (int r = 0; r < kRowsPerWarp; ++r) {
-            const size_t row = r0 + min(r, rows - 1);    // rows past the last repeat it
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                const float h = H[row * D + lane + 32 * c];
-                in[r * K + lane + 32 * c] = h;
-                const unsigned bits = __ballot_sync(0xffffffffu, h > 0.f);
-                if (lane == 0 && r < rows) masks[(row * 4 + kMaskH) * C + c] = bits;
+                in[r * K + lane + 32 * c] = h[r][c];
+                const unsigned bits = __ballot_sync(0xffffffffu, h[r][c] > 0.f);
+                if (lane == 0 && r < rows) masks[((r0 + r) * 4 + kMaskH) * C + c] = bits;
             }
-            if (lane < K - D) in[r * K + D + lane] = lane < F ? a.X[row * F + lane] : 0.f;
+            if (lane < K - D) in[r * K + D + lane] = x[r];
         }
+        if (r0 + step < R) request(r0 + step);
         __syncwarp();
         float acc[kRowsPerWarp][C];
 #pragma unroll
@@ -126,22 +139,39 @@ grad_rows_g_kernel(const GradArgs a) {
     for (size_t r0 = ((size_t)blockIdx.x * kRowWarps + warp) * kRowsPerWarp; r0 < R; r0 += step) {
         const int rows = (int)min((size_t)kRowsPerWarp, R - r0);
         __syncwarp();
+        // sums over the neighbours, all eight rows' loads in flight where they are of one node
+        float s[kRowsPerWarp][C];
 #pragma unroll
-        for (int r = 0; r < kRowsPerWarp; ++r) {
-            const size_t row = r0 + min(r, rows - 1);
-            const int u = (int)(row / B), b = (int)(row - (size_t)u * B);
-            float s[C];
+        for (int r = 0; r < kRowsPerWarp; ++r)
 #pragma unroll
-            for (int c = 0; c < C; ++c) s[c] = 0.f;
-            for (int e = nbr_ptr[u]; e < nbr_ptr[u + 1]; ++e)
+            for (int c = 0; c < C; ++c) s[r][c] = 0.f;
+        const int u0 = (int)(r0 / B), b0 = (int)(r0 - (size_t)u0 * B);
+        if (b0 + rows <= B) {
+            const int last = nbr_ptr[u0 + 1];
+            for (int e = nbr_ptr[u0]; e < last; ++e) {
+                const float *m = M + ((size_t)nbr[e] * B + b0) * D + lane;
 #pragma unroll
-                for (int c = 0; c < C; ++c) s[c] += M[((size_t)nbr[e] * B + b) * D + lane + 32 * c];
+                for (int r = 0; r < kRowsPerWarp; ++r)
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                in[r * D + lane + 32 * c] = s[c];
-                if (r < rows) a.Sg[dir][row * D + lane + 32 * c] = s[c];
+                    for (int c = 0; c < C; ++c) s[r][c] += m[min(r, rows - 1) * D + 32 * c];
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < kRowsPerWarp; ++r) {
+                const size_t row = r0 + min(r, rows - 1);
+                const int u = (int)(row / B), b = (int)(row - (size_t)u * B);
+                for (int e = nbr_ptr[u]; e < nbr_ptr[u + 1]; ++e)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) s[r][c] += M[((size_t)nbr[e] * B + b) * D + lane + 32 * c];
             }
         }
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                in[r * D + lane + 32 * c] = s[r][c];
+                if (r < rows) a.Sg[dir][(r0 + r) * D + lane + 32 * c] = s[r][c];
+            }
         __syncwarp();
         float acc[kRowsPerWarp][C];
 #pragma unroll
@@ -477,7 +507,9 @@ bool plan_sweep(const GradArgs &a, const DeviceInfo &di, SweepPlan *out) {
 template <int D>
 cudaError_t launch_rows(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
     const size_t R = (size_t)a.n * a.B;
-    const int blocks = (int)std::min<size_t>((R + kRowWarps * kRowsPerWarp - 1) / (kRowWarps * kRowsPerWarp), 2 * (size_t)di.sm_count);
+    // two directions: two blocks of the first kernel per SM (its registers), four of the second
+    const size_t batches = (R + kRowWarps * kRowsPerWarp - 1) / (kRowWarps * kRowsPerWarp);
+    const int blocks = (int)std::min<size_t>(batches, (size_t)di.sm_count), blocks_g = (int)std::min<size_t>(batches, 2 * (size_t)di.sm_count);
     const int K = (D + a.F + 3) & ~3;
     const size_t smem_f = ((size_t)(K + D) * D + (size_t)kRowThreads / 32 * kRowsPerWarp * (K + D)) * sizeof(float);
     const size_t smem_g = ((size_t)D * D + (size_t)kRowThreads / 32 * kRowsPerWarp * D) * sizeof(float);
@@ -485,7 +517,7 @@ cudaError_t launch_rows(const GradArgs &a, const DeviceInfo &di, cudaStream_t st
     if (err != cudaSuccess) return err;
     grad_rows_f_kernel<D><<<dim3(blocks, 2), kRowThreads, smem_f, stream>>>(a);
     count_launch();
-    grad_rows_g_kernel<D><<<dim3(blocks, 2), kRowThreads, smem_g, stream>>>(a);
+    grad_rows_g_kernel<D><<<dim3(blocks_g, 2), kRowThreads, smem_g, stream>>>(a);
     count_launch();
     return cudaGetLastError();
 }
