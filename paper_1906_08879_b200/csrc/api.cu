@@ -112,9 +112,7 @@ Layout make_layout(const placeto_graph *g, const placeto_weights *w, int B, plac
         auto hidden = [](const placeto_mlp &net) { return net.n_layers == 2 ? net.hidden_dim : net.out_dim; };
         const int Hf = std::max(hidden(w->f_down), hidden(w->f_up));
         const int Hg = std::max(hidden(w->g_down), hidden(w->g_up));
-        int pool_nodes, pool_chunks;
-        grad_pool_chunks((int)n, B, g->info, &pool_nodes, &pool_chunks);
-        L.grad = take(policy_gradient_workspace_floats((int)n, B, w->d, w->F, w->m, Hf, Hg, w->head.hidden_dim, pool_chunks) *
+        L.grad = take(policy_gradient_workspace_floats((int)n, B, w->d, w->F, w->m, Hf, Hg, w->head.hidden_dim) *
                       sizeof(float));
         L.grad_extra = take(4 * 2 * (d * d + d) * sizeof(float));
         L.total = off;

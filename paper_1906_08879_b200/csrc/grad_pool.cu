@@ -54,7 +54,8 @@ __device__ __forceinline__ bool find_batch(const Lists &l, int k, int &set, int 
 // states: forward 110 -> 76 us).
 template <int D> constexpr int kPoolWarps = D == 32 ? 8 : 16;
 
-// relu(l_i(e_u)) of every row: sums per (chunk, state, set), and one bit per column, positive or not
+// relu(l_i(e_u)) of every row, and one bit per column, positive or not. The rows go where the sweep will put d/d(sums)
+// later; the head adds them up.
 template <int D>
 __global__ void __launch_bounds__(32 * kPoolWarps<D>)
 grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
@@ -64,10 +65,8 @@ grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
     const int n = a.n, B = a.B, F = a.F, E = 2 * D + F, Ep = (E + 3) & ~3;
     float *W = smem;                                     // [3][Ep][D], zero padded
     float *in = W + 3 * Ep * D + warp * kRowsPerWarp * Ep;
-    float *sums = W + 3 * Ep * D + kWarps * kRowsPerWarp * Ep;       // [batch][D]
-    const int max_batches = chunk_nodes / kRowsPerWarp + 3;
     Lists l;
-    l.count = reinterpret_cast<int *>(sums + max_batches * D);
+    l.count = reinterpret_cast<int *>(W + 3 * Ep * D + kWarps * kRowsPerWarp * Ep);
     l.node = reinterpret_cast<unsigned short *>(l.count + 4);
     for (int i = 0; i < 3; ++i)
         for (int t = threadIdx.x; t < Ep * D; t += kThreads) W[i * Ep * D + t] = t < E * D ? a.l[i].W1[t] : 0.f;
@@ -114,28 +113,16 @@ grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
             }
             row_products<D>(W + set * Ep * D, in, Ep, Ep, lane, acc);
 #pragma unroll
-            for (int q = 0; q < C; ++q) {
-                float s = 0.f;
+            for (int q = 0; q < C; ++q)
 #pragma unroll
                 for (int r = 0; r < kRowsPerWarp; ++r) {
                     const unsigned bits = __ballot_sync(0xffffffffu, acc[r][q] > 0.f);
                     if (r < rows) {
-                        s += fmaxf(acc[r][q], 0.f);
-                        if (lane == 0) a.l_masks[((size_t)l.node[set * chunk_nodes + at + r] * B + b) * C + q] = bits;
+                        const size_t row = (size_t)l.node[set * chunk_nodes + at + r] * B + b;
+                        a.pool_rows[row * D + lane + 32 * q] = fmaxf(acc[r][q], 0.f);
+                        if (lane == 0) a.l_masks[row * C + q] = bits;
                     }
                 }
-                sums[k * D + lane + 32 * q] = s;
-            }
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < 3 * D; i += kThreads) {
-            const int s = i / D, j = i - s * D;
-            int first = 0;
-            for (int q = 0; q < s; ++q) first += (l.count[q] + kRowsPerWarp - 1) / kRowsPerWarp;
-            const int last = first + (l.count[s] + kRowsPerWarp - 1) / kRowsPerWarp;
-            float total = 0.f;
-            for (int q = first; q < last; ++q) total += sums[q * D + j];
-            a.pool_partial[((size_t)chunk * B + b) * 3 * D + i] = total;
         }
         __syncthreads();
     }
@@ -397,7 +384,7 @@ grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const pa
 template <int D>
 size_t forward_smem(int F, int chunk_nodes) {
     const int Ep = (2 * D + F + 3) & ~3;
-    return ((size_t)3 * Ep * D + (size_t)kPoolWarps<D> * kRowsPerWarp * Ep + (size_t)(chunk_nodes / kRowsPerWarp + 3) * D + 4) * sizeof(float) +
+    return ((size_t)3 * Ep * D + (size_t)kPoolWarps<D> * kRowsPerWarp * Ep + 4) * sizeof(float) +
            (size_t)3 * chunk_nodes * 2;
 }
 template <int D>

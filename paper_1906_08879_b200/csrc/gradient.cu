@@ -256,11 +256,11 @@ grad_head_kernel(const GradArgs a) {
     }
 }
 
-// The same between the row kernels of grad_pool.cu: the sums arrive per chunk of nodes, and what is pushed back stops
+// The same between the row kernels of grad_pool.cu: relu(l_i(e_u)) arrives row by row, and what is pushed back stops
 // at them and at the current node's embedding. A chain of small products per state, bound by the round trips to L2 for
 // their weights: one thread per sum of 332 products with four loads in flight took 111 us for 100 states at d = 64, 38 us
 // for 256 at d = 32. Sixteen in flight here, the last layer's weights in shared memory, the transposed product four
-// rows to a warp: 43 and 24 us. Sums are taken in the order of the forward pass, so the ReLU masks are the same.
+// rows to a warp: 53 and 26 us, of which the pooled sums take 10 and 2.
 constexpr int kHeadThreads = 512;
 
 // init + sum over k < K of x[k] w[k * stride], ascending
@@ -290,7 +290,8 @@ grad_head_pooled_kernel(const GradArgs a, const int staged) {      // staged: fl
     float *S = dz + Z;                     // [3][d]
     float *dpre = S + 3 * d;               // [3][d]
     float *lg = dpre + 3 * d;              // [m] logits, then d/d(logits)
-    float *w2 = lg + m;                    // [Hh][m]
+    float *part = lg + m;                  // [8][3][d] sums over the nodes of one residue
+    float *w2 = part + 8 * 3 * d;          // [Hh][m]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < staged; i += kHeadThreads) w2[i] = a.head.W2[i];
     const float *W2 = staged > 0 ? w2 : a.head.W2;
@@ -303,23 +304,42 @@ grad_head_pooled_kernel(const GradArgs a, const int staged) {      // staged: fl
             for (int k = threadIdx.x; k < 3 * d; k += kHeadThreads) { a.Sbuf[(size_t)b * 3 * d + k] = 0.f; a.DPRE_H[(size_t)b * 3 * d + k] = 0.f; }
             continue;
         }
-        for (int i = threadIdx.x; i < 3 * d; i += kHeadThreads) {
-            const float *src = a.pool_partial + (size_t)b * 3 * d + i;
-            float acc = 0.f;
-            for (int q0 = 0; q0 < a.pool_chunks; q0 += 8) {
+        // ---- pooled sums, added up as the general kernel's eight warps do: S decides the masks of h_i and the head, and a last
+        // bit more or less in it flips one now and then (256 states: a gradient off by 2e-4 of its norm)
+        const uint8_t *rel = a.relation + (size_t)c * n;
+        for (int i = threadIdx.x; i < 8 * d; i += kHeadThreads) {
+            const int g = i / d, j = i - g * d;
+            const float *src = a.pool_rows + (size_t)b * d + j;
+            float acc[3] = {0.f, 0.f, 0.f};
+            for (int u0 = g; u0 < n; u0 += 64) {
                 float v[8];
+                int set[8];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) v[t] = q0 + t < a.pool_chunks ? src[(size_t)(q0 + t) * B * 3 * d] : 0.f;
+                for (int t = 0; t < 8; ++t) {
+                    const int u = u0 + 8 * t;
+                    set[t] = u < n ? rel[u] : 3;
+                    v[t] = u < n ? src[(size_t)u * B * d] : 0.f;
+                }
 #pragma unroll
-                for (int t = 0; t < 8; ++t) acc += v[t];
+                for (int t = 0; t < 8; ++t)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) acc[k] += set[t] == k ? v[t] : 0.f;
             }
-            S[i] = acc;
-            a.Sbuf[(size_t)b * 3 * d + i] = acc;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) part[(g * 3 + k) * d + j] = acc[k];
         }
         for (int k = kHeadThreads - 1 - threadIdx.x; k < E; k += kHeadThreads)
             z[k] = k < d ? a.H[0][((size_t)c * B + b) * d + k]
                  : k < 2 * d ? a.H[1][((size_t)c * B + b) * d + (k - d)]
                              : a.X[((size_t)c * B + b) * F + (k - 2 * d)];
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 * d; i += kHeadThreads) {
+            float acc = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc += part[q * 3 * d + i];
+            S[i] = acc;
+            a.Sbuf[(size_t)b * 3 * d + i] = acc;
+        }
         __syncthreads();
         // ---- a_i = relu(h_i(S_i)) into z, hidden layer, logits
         for (int i = threadIdx.x; i < 3 * d; i += kHeadThreads) {
@@ -736,7 +756,7 @@ bool policy_gradient_applicable(const GradArgs &a) {
 }
 
 // floats of workspace (every array padded to a multiple of 4 floats by the carve below)
-size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh, int pool_chunks) {
+size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh) {
     const size_t R = (size_t)n * B, Z = 5 * (size_t)d + F, E = 2 * (size_t)d + F;
     const size_t per_dir = R * ((size_t)Hf * 2 + (size_t)Hg * 2 + (size_t)d * 6);
     size_t total = 2 * per_dir + 3 * R * d;
@@ -745,7 +765,7 @@ size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int H
     const size_t widest = 2 * (((size_t)d + F + 1) * Hf + ((size_t)Hf + 1) * d + ((size_t)d + 1) * Hg + ((size_t)Hg + 1) * d) +
                           3 * ((E + 1) * (size_t)d + ((size_t)d + 1) * d) + (Z + 1) * (size_t)Hh + ((size_t)Hh + 1) * m;
     const size_t masks = 2 * R * (((size_t)d + 31) / 32) * 4;
-    const size_t pooled = R * (((size_t)d + 31) / 32) + (size_t)B * 5 * d + (size_t)pool_chunks * B * 3 * d;
+    const size_t pooled = R * (((size_t)d + 31) / 32) + (size_t)B * 5 * d;
     return total + masks + pooled + (size_t)kGradChunks * widest + 256;
 }
 
@@ -770,7 +790,7 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
     grad_pool_chunks(n, B, di, &a.pool_chunk_nodes, &a.pool_chunks);
     a.l_masks = reinterpret_cast<unsigned *>(take(R * (((size_t)d + 31) / 32)));
     a.dS = take((size_t)B * 3 * d); a.dZ = take((size_t)B * 2 * d);
-    a.pool_partial = take((size_t)a.pool_chunks * B * 3 * d);
+    a.pool_rows = a.DS[0];      // free until the sweep
     float *partial = p;
     const bool split = grad_split_applicable(a, di);
 
@@ -797,7 +817,7 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
         const size_t E = 2 * (size_t)d + F;
         const size_t vectors = 2 * (size_t)Z + 2 * (size_t)Hh + 6 * (size_t)d;
         if (split) {
-            const size_t own = vectors + m, w2 = (size_t)Hh * m;
+            const size_t own = vectors + m + 24 * (size_t)d, w2 = (size_t)Hh * m;
             const int staged = (own + w2) * sizeof(float) <= 96 * 1024 ? (int)w2 : 0;
             const size_t smem = (own + staged) * sizeof(float);
             err = cudaFuncSetAttribute(grad_head_pooled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

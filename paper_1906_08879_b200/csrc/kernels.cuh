@@ -244,7 +244,7 @@ struct GradArgs {
     // the passes of grad_pool.cu: sums per chunk of nodes [chunk][B][3][d], their gradients [B][3][d], the gradient of
     // the current node's embedding [B][2 d], one bit per pooled row and column [row][d / 32]
     int pool_chunk_nodes, pool_chunks;
-    float *pool_partial, *dS, *dZ;
+    float *pool_rows, *dS, *dZ;
     unsigned *l_masks;
     GradOut gf[2], gg[2], gl[3], gh[3], ghead;
 };
@@ -355,7 +355,7 @@ cudaError_t launch_simulator(const SimArgs &a, const DeviceInfo &di, cudaStream_
 
 // gradient.cu: gradient of the policy objective with respect to all weights
 bool policy_gradient_applicable(const GradArgs &a);
-size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh, int pool_chunks);
+size_t policy_gradient_workspace_floats(int n, int B, int d, int F, int m, int Hf, int Hg, int Hh);
 cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, cudaStream_t stream);
 
 // grad_sweep.cu: the passes over the node-state rows for d = 32 / 64 with hidden width d: forward values and masks of
