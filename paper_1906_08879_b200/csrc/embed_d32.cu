@@ -10,7 +10,7 @@
 //     a row (node, state) through gather -> g1 -> g2 -> f1 -> f2 on its own. With
 //     single-layer networks the second layers drop out at compile time: half
 //     the dependent chain of a level (whole path on a 279-node graph, 132 levels, 250
-//     states, two devices, B200: 106 us; 618 us on the dimension-generic kernels).
+//     states, two devices, B200: 90 us; 618 us on the dimension-generic kernels).
 //     Between layers the 32 outputs are exchanged through a per-warp shared
 //     buffer and read back as broadcast 128-bit loads: 4 FMAs per shared load,
 //     issued as two packed fma.rn.f32x2 against weights kept in register pairs.
@@ -21,7 +21,7 @@
 //     Global traffic is the compulsory part only: read x, write h.
 //   - The level schedule (order, CSR, slots) is staged in shared memory, and the
 //     raw features of the next level are copied asynchronously (cp.async) into a
-//     double-buffered staging area while the current level computes, so no DRAM
+//     staging area of two or three levels while the current level computes, so no DRAM
 //     latency sits on the level-to-level critical path.
 #include <cuda_pipeline.h>
 
@@ -35,7 +35,10 @@ namespace {
 
 constexpr int kD = 32;
 constexpr int kWarps = 8;
-constexpr int kThreads = kWarps * 32;
+// With single-layer networks a level is short: a ninth warp brings the raw features, two levels ahead (279 nodes, 250 states:
+// 80 -> 68 us). With two layers, where the registers are full and the features come in time, either costs 3 %.
+template <int L> constexpr int kStages = L == 1 ? 3 : 2;            // levels of raw features on chip
+template <int L> constexpr int kThreads = (kWarps + (L == 1)) * 32;
 
 struct D32Plan {
     int S;          // states per slice
@@ -199,7 +202,7 @@ after_g1:
 
 // feature width padded to 4 * F4; features built from compact states; layers; a sweep of an episode
 template <int F4, bool kCompact, int L, bool kWalk>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads<L>, 1)
 embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     constexpr int KF = kD + 4 * F4;      // padded input width of f's first layer
     extern __shared__ __align__(16) float smem[];
@@ -211,25 +214,25 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     const int b_first = blockIdx.x * p.S;
     const int nb = min(p.S, B - b_first);
 
-    // ---- shared memory: [schedule ints][message slots][feature staging x2][exchange buffers]
+    // ---- shared memory: [schedule ints][message slots][feature staging x2 or x3][exchange buffers]
     // one packed record per position: {first neighbour entry, end,
     // own slot (low 16 bits, 0xffff = none) | slot of the first neighbour (high 16 bits), node id}
     int4 *meta_w = reinterpret_cast<int4 *>(smem);
-    for (int i = threadIdx.x; i < a.n; i += kThreads) {
+    for (int i = threadIdx.x; i < a.n; i += kThreads<L>) {
         const int e0 = lv.nbr_ptr[i], e1 = lv.nbr_ptr[i + 1];
         const int first = e1 > e0 ? lv.nbr_slot[e0] : 0;
         meta_w[i] = make_int4(e0, e1, (lv.own_slot[i] & 0xffff) | (first << 16), lv.order[i]);
         PLACETO_DEBUG_CHECK(a.status, e0 >= 0 && e0 <= e1 && e1 <= lv.n_nbr && lv.own_slot[i] >= -1 &&
                                           lv.own_slot[i] < lv.n_slots && lv.order[i] >= 0 && lv.order[i] < a.n);
     }
-    for (int e = threadIdx.x; e < lv.n_nbr; e += kThreads)
+    for (int e = threadIdx.x; e < lv.n_nbr; e += kThreads<L>)
         PLACETO_DEBUG_CHECK(a.status, lv.nbr_slot[e] >= 0 && lv.nbr_slot[e] < lv.n_slots);
     PLACETO_DEBUG_CHECK(a.status, nb >= 1 && b_first + nb <= B);
     const int4 *meta = meta_w;
     int *ism = reinterpret_cast<int *>(smem) + 4 * a.n;
     auto stage = [&](const int *src, int count) {
         int *dst = ism;
-        for (int i = threadIdx.x; i < count; i += kThreads) dst[i] = src[i];
+        for (int i = threadIdx.x; i < count; i += kThreads<L>) dst[i] = src[i];
         ism += (count + 3) & ~3;
         return (const int *)dst;
     };
@@ -237,8 +240,8 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     const int *nbr_slot = stage(lv.nbr_slot, lv.n_nbr);
     float *fsm = reinterpret_cast<float *>(ism);
     float *msg = fsm;                                       // [n_slots][S][32]
-    float *xstage = msg + (size_t)lv.n_slots * p.S * kD;    // [2][x_floats]
-    float *xbuf = xstage + 2 * (size_t)p.x_floats + (size_t)warp * 4 * KF;
+    float *xstage = msg + (size_t)lv.n_slots * p.S * kD;    // [kStages][x_floats]
+    float *xbuf = xstage + kStages<L> * (size_t)p.x_floats + (size_t)(L == 1 ? min(warp, kWarps - 1) : warp) * 4 * KF;
     float *A = xbuf, *Bf = xbuf + 2 * KF;
 
     // ---- this lane's weight columns
@@ -275,9 +278,9 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     // The last warp (the one least often needed for rows) issues all copies, so
     // the other warps go straight to their rows.
     auto prefetch = [&](int level) {
-        if (warp != kWarps - 1) return;
+        if (warp != (L == 1 ? kWarps : kWarps - 1)) return;
         const int q0 = level_ptr[level], width = level_ptr[level + 1] - q0;
-        float *dst = xstage + (size_t)(level & 1) * p.x_floats;
+        float *dst = xstage + (size_t)(L == 1 ? level % 3 : level & 1) * p.x_floats;
         if (kCompact) {
             // no X tensor: the level's features from one byte per (node, state)
             for (int i = lane; i < width * nb; i += 32) {       // one (node, state) pair per lane
@@ -298,9 +301,10 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     const int start = kWalk ? first_level(a.walk, lv, a.n) : 0;
     dependency_wait();          // the raw features may come from a kernel that is still running
     prefetch(start);
+    if (L == 1 && start + 1 < lv.n_levels) prefetch(start + 1);
     float *__restrict__ M = a.M[dir];
     if (kWalk && start > 0) {
-        carried_messages(lv, meta[level_ptr[start]].x, start, warp, kWarps, lane, [&](const int (&u)[4], const int (&e)[4]) {
+        carried_messages(lv, meta[level_ptr[start]].x, start, warp, kThreads<L> / 32, lane, [&](const int (&u)[4], const int (&e)[4]) {
             for (int s = 0; s < nb; ++s) {
                 float v[4];
 #pragma unroll
@@ -313,11 +317,25 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
     __pipeline_wait_prior(0);
     __syncthreads();
 
+    if (L == 1 && warp == kWarps) {
+        for (int level = start; level < lv.n_levels; ++level) {
+            if (level + 2 < lv.n_levels) {
+                prefetch(level + 2);
+                __pipeline_wait_prior(1);
+            } else {
+                __pipeline_wait_prior(0);
+            }
+            __syncthreads();
+        }
+        return;
+    }
+    int stage_now = start % kStages<L>;
     for (int level = start; level < lv.n_levels; ++level) {
-        if (level + 1 < lv.n_levels) prefetch(level + 1);
+        if (L == 2 && level + 1 < lv.n_levels) prefetch(level + 1);
         const int p0 = level_ptr[level];
         const int rows = (level_ptr[level + 1] - p0) * nb;
-        const float *xs = xstage + (size_t)(level & 1) * p.x_floats;
+        const float *xs = xstage + (size_t)(L == 1 ? stage_now : level & 1) * p.x_floats;
+        if (L == 1) stage_now = stage_now == 2 ? 0 : stage_now + 1;
         const int width = level_ptr[level + 1] - p0;
         if (rows <= kWarps) {
             // narrow level: one row per warp, shortest dependent chains
@@ -337,7 +355,7 @@ embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
                                 msg, xs, H, M, B, b_first, A, Bf);
             }
         }
-        __pipeline_wait_prior(0);
+        if (L == 2) __pipeline_wait_prior(0);
         __syncthreads();
     }
 }
@@ -376,7 +394,7 @@ bool plan_d32(const EmbedArgs &a, const DeviceInfo &di, D32Plan *out) {
     const size_t xbuf = (size_t)kWarps * 4 * KF * sizeof(float);
     auto x_floats = [&](int S) { return (a.max_level_width * S * a.F + 3) & ~3; };
     auto need = [&](int S) {
-        return (size_t)max_slots * S * kD * sizeof(float) + 2 * (size_t)x_floats(S) * sizeof(float) +
+        return (size_t)max_slots * S * kD * sizeof(float) + (a.f[0].n_layers == 1 ? kStages<1> : kStages<2>) * (size_t)x_floats(S) * sizeof(float) +
                xbuf + ints * sizeof(int);
     };
     // narrower slices when the shared memory does not fit (more blocks: they queue up)
@@ -417,7 +435,7 @@ cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStrea
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)p.smem_bytes);
     if (err != cudaSuccess) return err;
-    err = launch_overlapped(overlap, kern, dim3(p.n_slices, 2), dim3(kThreads), p.smem_bytes, stream, a, p);
+    err = launch_overlapped(overlap, kern, dim3(p.n_slices, 2), dim3(a.f[0].n_layers == 1 ? kThreads<1> : kThreads<2>), p.smem_bytes, stream, a, p);
     count_launch();
     return err;
 }
