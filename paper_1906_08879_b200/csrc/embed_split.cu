@@ -524,13 +524,14 @@ bool embed_split_applicable(const EmbedArgs &a) {
 // d = 64: wherever it applies. d = 32: measured against the FMA kernel (us, two layers / one), the lines cross at 12
 // to 14 rows of a block per level: 20 rows 417 -> 308 / 295 -> 213, 12 rows 286 -> 263 / 203 -> 183, 8.5 rows
 // 96 -> 114 / 70 -> 80; with four neighbours per node (a recurrent grid with attention) the gather, which only one
-// group of warps per tile does, costs more than the products save: 26 rows 310 -> 401.
+// group of warps per tile does, costs more than the products save: 26 rows 310 -> 401. The line is at three and a half (whole
+// path, 256 states: 3.0 edges per node 118 -> 100, 3.3 184 -> 151, 4.0 349 -> 445).
 bool embed_split_preferred(const EmbedArgs &a, const DeviceInfo &di) {
     if (!embed_split_applicable(a)) return false;
     if (a.d == 64) return true;
     const int blocks = std::max(1, std::min(a.B, di.sm_count / 2)), S = (a.B + blocks - 1) / blocks;
     const long long rows = (long long)a.n * S;
-    return rows >= 12ll * a.lv[0].n_levels && rows >= 12ll * a.lv[1].n_levels && a.lv[0].n_nbr <= 2 * a.n;
+    return rows >= 12ll * a.lv[0].n_levels && rows >= 12ll * a.lv[1].n_levels && 2ll * a.lv[0].n_nbr <= 7ll * a.n;
 }
 
 cudaError_t launch_embed_split(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap) {
