@@ -19,7 +19,7 @@ struct placeto_graph {
     int device = -1;
     DeviceInfo info{};
     int *d_ints = nullptr;       // one allocation for all int arrays
-    int4 *d_packed = nullptr;    // per direction lvl4[n_levels], pos4[n] (see DevLevels)
+    int4 *d_packed = nullptr;    // per direction lvl4[n_levels], pos4[n], row4[n] (see DevLevels)
     int *d_child_ptr = nullptr, *d_child = nullptr, *d_child_entry = nullptr;   // inside d_ints
     int *d_parent_ptr = nullptr, *d_parent = nullptr;                          // inside d_ints
     uint8_t *d_relation = nullptr;
@@ -447,7 +447,7 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
         return fail(PLACETO_ERR_CUDA);
     {   // packed per-level and per-position records (kernels that stream the schedule)
         std::vector<int4> packed;
-        size_t at[2][2];
+        size_t at[2][3];
         for (int dir = 0; dir < 2; ++dir) {
             const LevelPlan &p = g->host.dir[dir];
             at[dir][0] = packed.size();
@@ -461,6 +461,10 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
             at[dir][1] = packed.size();
             for (int q = 0; q < g->host.n; ++q)
                 packed.push_back(make_int4(p.nbr_ptr[q], p.nbr_ptr[q + 1], p.own_slot[q], p.order[q]));
+            at[dir][2] = packed.size();
+            for (int l = 0; l < p.n_levels; ++l)
+                for (int q = p.level_ptr[l]; q < p.level_ptr[l + 1]; ++q)
+                    packed.push_back(make_int4(p.order[q], p.level_ptr[l], p.level_ptr[l + 1] - p.level_ptr[l], 0));
             g->lv[dir].max_level_nbr = max_nbr;
         }
         if (cudaMalloc(&g->d_packed, packed.size() * sizeof(int4)) != cudaSuccess) return fail(PLACETO_ERR_NO_MEMORY);
@@ -469,6 +473,7 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
         for (int dir = 0; dir < 2; ++dir) {
             g->lv[dir].lvl4 = g->d_packed + at[dir][0];
             g->lv[dir].pos4 = g->d_packed + at[dir][1];
+            g->lv[dir].row4 = g->d_packed + at[dir][2];
         }
     }
     g->on_device = true;

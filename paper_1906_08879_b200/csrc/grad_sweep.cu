@@ -118,20 +118,59 @@ grad_rows_f_kernel(const GradArgs a) {
     }
 }
 
+// acc[r][c] = in[r][0 .. D) . W[.][lane + 32 c] as two chains, even and odd k, added at the end
 template <int D>
-__global__ void __launch_bounds__(kRowThreads)
+__device__ __forceinline__ void paired_products(const float *W, const float *in, int lane, float (&acc)[kRowsPerWarp][D / 32]) {
+    constexpr int C = D / 32;
+    float odd[kRowsPerWarp][C];
+#pragma unroll
+    for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[r][c] = odd[r][c] = 0.f;
+    for (int k = 0; k < D; k += 4) {
+        float w[4][C];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < C; ++c) w[q][c] = W[(k + q) * D + lane + 32 * c];
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            const float4 x = *reinterpret_cast<const float4 *>(in + r * D + k);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                acc[r][c] = fmaf(x.x, w[0][c], acc[r][c]);
+                odd[r][c] = fmaf(x.y, w[1][c], odd[r][c]);
+                acc[r][c] = fmaf(x.z, w[2][c], acc[r][c]);
+                odd[r][c] = fmaf(x.w, w[3][c], odd[r][c]);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[r][c] += odd[r][c];
+}
+
+// Rows are taken in the order of the levels: row r is state r % B of the node at position r / B. The hidden layer of g has
+// the general kernel's bits, since its signs are masks and a last bit flips one now and then (256 states of a 279-node
+// graph: in one batch of 40, and a weight gradient is then off by up to 4e-3 of its norm). That kernel takes a slice's rows
+// of a level in passes of kGradPassRows and adds a product up in two chains where a pass has at most kGradShortPass
+// outputs, in one otherwise. Rows of both kinds in one batch are multiplied twice. (One chain for all rows: whole gradient
+// step 542 instead of 545 us there, 1204 instead of 1213 for 531 nodes x 100 states at d = 64.)
+template <int D>
+__global__ void __launch_bounds__(kRowThreads, D == 64 ? 4 : 3)
 grad_rows_g_kernel(const GradArgs a) {
     constexpr int C = D / 32;
     extern __shared__ __align__(16) float smem[];
     const int dir = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const DevMlp gn = a.g[dir];
+    const DevLevels lv = a.lv[dir];
     float *W1 = smem, *in = W1 + D * D + warp * kRowsPerWarp * D;
     for (int i = threadIdx.x; i < D * D; i += kRowThreads) W1[i] = gn.W1[i];
     __syncthreads();
     float b1[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) b1[c] = gn.b1[lane + 32 * c];
-    const int *nbr_ptr = dir == 0 ? a.parent_ptr : a.child_ptr, *nbr = dir == 0 ? a.parent : a.child;
     const float *M = a.M[dir];
     const int B = a.B;
     const size_t R = (size_t)a.n * B;
@@ -139,17 +178,26 @@ grad_rows_g_kernel(const GradArgs a) {
     for (size_t r0 = ((size_t)blockIdx.x * kRowWarps + warp) * kRowsPerWarp; r0 < R; r0 += step) {
         const int rows = (int)min((size_t)kRowsPerWarp, R - r0);
         __syncwarp();
+        // lane r: where row r goes, and how many rows its pass of the general kernel has
+        const unsigned mine = (unsigned)r0 + min(lane, rows - 1);
+        const int pos = (int)(mine / (unsigned)B), state = (int)(mine - (unsigned)pos * B);
+        const int4 rec = lv.row4[pos];
+        const int slice = state / a.slice_states * a.slice_states, nb = min(a.slice_states, B - slice);
+        const int at = (pos - rec.y) * nb + state - slice;
+        const int pass = min(kGradPassRows, rec.z * nb - at / kGradPassRows * kGradPassRows);
+        const unsigned paired = __ballot_sync(0xffffffffu, pass * D <= kGradShortPass);
+        const unsigned to_mine = (unsigned)rec.x * B + state;
         // sums over the neighbours, all eight rows' loads in flight where they are of one node
         float s[kRowsPerWarp][C];
 #pragma unroll
         for (int r = 0; r < kRowsPerWarp; ++r)
 #pragma unroll
             for (int c = 0; c < C; ++c) s[r][c] = 0.f;
-        const int u0 = (int)(r0 / B), b0 = (int)(r0 - (size_t)u0 * B);
+        const int p0 = (int)(r0 / B), b0 = (int)(r0 - (size_t)p0 * B);
         if (b0 + rows <= B) {
-            const int last = nbr_ptr[u0 + 1];
-            for (int e = nbr_ptr[u0]; e < last; ++e) {
-                const float *m = M + ((size_t)nbr[e] * B + b0) * D + lane;
+            const int last = lv.nbr_ptr[p0 + 1];
+            for (int e = lv.nbr_ptr[p0]; e < last; ++e) {
+                const float *m = M + ((size_t)lv.nbr[e] * B + b0) * D + lane;
 #pragma unroll
                 for (int r = 0; r < kRowsPerWarp; ++r)
 #pragma unroll
@@ -159,37 +207,49 @@ grad_rows_g_kernel(const GradArgs a) {
 #pragma unroll
             for (int r = 0; r < kRowsPerWarp; ++r) {
                 const size_t row = r0 + min(r, rows - 1);
-                const int u = (int)(row / B), b = (int)(row - (size_t)u * B);
-                for (int e = nbr_ptr[u]; e < nbr_ptr[u + 1]; ++e)
+                const int p = (int)(row / B), b = (int)(row - (size_t)p * B);
+                for (int e = lv.nbr_ptr[p]; e < lv.nbr_ptr[p + 1]; ++e)
 #pragma unroll
-                    for (int c = 0; c < C; ++c) s[r][c] += M[((size_t)nbr[e] * B + b) * D + lane + 32 * c];
+                    for (int c = 0; c < C; ++c) s[r][c] += M[((size_t)lv.nbr[e] * B + b) * D + lane + 32 * c];
             }
         }
 #pragma unroll
-        for (int r = 0; r < kRowsPerWarp; ++r)
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            const size_t to = __shfl_sync(0xffffffffu, to_mine, r);
 #pragma unroll
             for (int c = 0; c < C; ++c) {
                 in[r * D + lane + 32 * c] = s[r][c];
-                if (r < rows) a.Sg[dir][(r0 + r) * D + lane + 32 * c] = s[r][c];
+                if (r < rows) a.Sg[dir][to * D + lane + 32 * c] = s[r][c];
             }
+        }
         __syncwarp();
         float acc[kRowsPerWarp][C];
+        auto finish = [&](unsigned which) {
 #pragma unroll
-        for (int r = 0; r < kRowsPerWarp; ++r)
+            for (int r = 0; r < kRowsPerWarp; ++r) {
+                const size_t to = __shfl_sync(0xffffffffu, to_mine, r);
+                if (r >= rows || !(which >> r & 1)) continue;
 #pragma unroll
-            for (int c = 0; c < C; ++c) acc[r][c] = 0.f;
-        row_products<D>(W1, in, D, D, lane, acc);
-#pragma unroll
-        for (int r = 0; r < kRowsPerWarp; ++r)
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const float v = fmaxf(acc[r][c] + b1[c], 0.f);
-                const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
-                if (r < rows) {
-                    a.T1[dir][(r0 + r) * D + lane + 32 * c] = v;
-                    if (lane == 0) a.masks[dir][((r0 + r) * 4 + kMaskG) * C + c] = bits;
+                for (int c = 0; c < C; ++c) {
+                    const float v = fmaxf(acc[r][c] + b1[c], 0.f);
+                    const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
+                    a.T1[dir][to * D + lane + 32 * c] = v;
+                    if (lane == 0) a.masks[dir][(to * 4 + kMaskG) * C + c] = bits;
                 }
             }
+        };
+        if (paired != 0) {
+            paired_products<D>(W1, in, lane, acc);
+            finish(paired);
+        }
+        if (paired != 0xffffffffu) {
+#pragma unroll
+            for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c) acc[r][c] = 0.f;
+            row_products<D>(W1, in, D, D, lane, acc);
+            finish(~paired);
+        }
     }
 }
 

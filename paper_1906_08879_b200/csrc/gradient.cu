@@ -420,7 +420,7 @@ grad_head_pooled_kernel(const GradArgs a, const int staged) {      // staged: fl
 }
 
 // ------------------------------------------------------------------ 3. sweeps
-constexpr int kSweepRows = 64;     // rows per pass of the sweep kernel
+constexpr int kSweepRows = kGradPassRows;
 
 // out(r, j) = sum_k A[r][k] W[k][j] for rows x J outputs, all operands in shared
 // memory (A row stride lda, odd; W row stride ldw, a multiple of 4). A thread owns
@@ -428,7 +428,7 @@ constexpr int kSweepRows = 64;     // rows per pass of the sweep kernel
 template <typename Epilogue>
 __device__ __forceinline__ void tile_product(const float *A, int lda, const float *W, int ldw, int K,
                                              int J, int rows, Epilogue done) {
-    if (rows * J <= 2 * kThreads) {
+    if (rows * J <= kGradShortPass) {
         // a short pass (narrow level, few states): one output per thread keeps the chain short
         for (int i = threadIdx.x; i < rows * J; i += kThreads) {
             const int r = i / J, j = i - r * J;
@@ -797,6 +797,8 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
     cudaError_t err = cudaSuccess;
     if (!split) err = cudaMemsetAsync(a.DPRE_L[0], 0, 3 * ((R * d + 3) & ~size_t(3)) * sizeof(float), stream);
     if (err != cudaSuccess) return err;
+    const int slices = std::max(1, std::min(B, di.sm_count / 2));
+    a.slice_states = (B + slices - 1) / slices;
     // 1. messages
     if (split) {
         err = launch_grad_rows(a, di, stream);
@@ -840,8 +842,7 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
         err = launch_grad_sweep_split(a, di, stream);
         if (err != cudaSuccess) return err;
     } else {
-        const int slices = std::max(1, std::min(B, di.sm_count / 2));
-        const int S = (B + slices - 1) / slices;
+        const int S = a.slice_states;
         int W = d;
         for (int dir = 0; dir < 2; ++dir) W = std::max({W, a.f[dir].hidden_dim, a.g[dir].hidden_dim});
         size_t wfloats = 0;

@@ -21,7 +21,8 @@ struct DevLevels {
     // packed records for kernels that stream the schedule level by level:
     //   lvl4[level] = {first position, width, first neighbour entry, neighbour entries of the level}
     //   pos4[p]     = {first neighbour entry, end of neighbour entries, own slot, node id}
-    const int4 *lvl4, *pos4;
+    //   row4[p]     = {node id, first position of its level, width of its level, 0}
+    const int4 *lvl4, *pos4, *row4;
     int max_level_nbr;               // most neighbour entries in one level
     const int *level_of;             // [n] level of a node id
 };
@@ -225,6 +226,9 @@ struct SimArgs {
 
 // Policy gradient (gradient.cu): inputs, per-row intermediates in the workspace, outputs.
 constexpr int kGradChunks = 256;   // row chunks whose partial weight gradients are added in order
+// The general reverse sweep takes the rows of a level in passes, and adds the products of a pass with few outputs up in two
+// chains, the others in one. The sign of such a sum is a ReLU mask: whoever recomputes one keeps the rule.
+constexpr int kGradPassRows = 64, kGradShortPass = 512;
 struct GradOut { float *W1, *b1, *W2, *b2; };
 struct GradArgs {
     int n, B, d, F, m;
@@ -241,7 +245,8 @@ struct GradArgs {
     float *DPRE_L[3], *Zbuf, *HID, *DHID, *DLOG, *Sbuf, *DPRE_H;
     unsigned *masks[2];        // one bit per ReLU of every row (grad_sweep.cu)
     int max_level_width;
-    // the passes of grad_pool.cu: sums per chunk of nodes [chunk][B][3][d], their gradients [B][3][d], the gradient of
+    int slice_states;          // states per slice of the general reverse sweep
+    // the passes of grad_pool.cu: relu(l_i(e_u)) of every row, the gradients of the pooled sums [B][3][d], the gradient of
     // the current node's embedding [B][2 d], one bit per pooled row and column [row][d / 32]
     int pool_chunk_nodes, pool_chunks;
     float *pool_rows, *dS, *dZ;

@@ -154,3 +154,57 @@ def test_pooling_passes_over_chunks_of_nodes(d, m, n, B):
     adv = adv.astype(np.float32).astype(np.float64)
     grads = gpu_gradient(cfg, actions, adv, 0.1)
     compare(cfg, grads, gradient.gradient(cfg, actions, adv, 0.1))
+
+
+def cancelling(W, rows):
+    """The first `rows` rows of W, the second half of them the first negated: over inputs whose halves agree the exact sum is
+    zero, and what a kernel finds is what its order of summation leaves."""
+    W = W.copy()
+    W[rows // 2:rows] = -W[:rows // 2]
+    W[rows:] = 0
+    return W
+
+
+@pytest.mark.parametrize("nets", ["g", "f and l"])
+@pytest.mark.parametrize("d,m,n,B,p", [(32, 4, 60, 303, 0.05), (32, 3, 25, 1200, 0.15), (32, 4, 12, 1, 0.3), (64, 8, 40, 155, 0.06), (64, 3, 70, 500, 0.03)])
+def test_masks_are_those_of_the_general_kernels(d, m, n, B, p, nets):
+    """A ReLU's mask is the sign of a recomputed sum, so the kernels for d = 32 and 64 add up in the order of the general
+    ones. Here the sums before the first ReLU of g (of f and l_i) are nothing but rounding; one hidden unit of weight zero more
+    in f sends the same problem to the general kernels. One mask that differs moves an array by 1e-3 of its norm and more;
+    without, sums of at most n B = 35,000 terms and a few levels differ by rounding, 1e-6 (bound: 2e-5). Levels of one
+    row up to more than a pass of 64, last passes short and long, ragged last slices."""
+    cfg, actions, adv = small_case(d + n, n=n, m=m, d=d, B=B, p=p)
+    r = rng(d + B)
+    half = r.uniform(0.1, 1.0, (2, n, B, d // 2)).astype(np.float32)
+    H = np.concatenate([half, half], axis=-1)
+    w = cfg["weights"]
+    for way in ("down", "up"):
+        f, g = w["f_" + way], w["g_" + way]
+        if nets == "g":
+            g["W1"], g["b1"] = cancelling(g["W1"], d), np.zeros(d, np.float32)
+            f["W2"][:, d // 2:], f["b2"][d // 2:] = f["W2"][:, :d // 2], f["b2"][:d // 2]      # messages: two equal halves
+        else:
+            f["W1"], f["b1"] = cancelling(f["W1"], d), np.zeros(d, np.float32)
+    for l in w["l"] if nets != "g" else []:
+        l["W1"][:d], l["W1"][d:2 * d] = cancelling(l["W1"][:d], d), cancelling(l["W1"][d:2 * d], d)
+        l["W1"][2 * d:], l["b1"] = 0, np.zeros(d, np.float32)
+
+    def gradient_of(weights):
+        graph = placeto.Graph(cfg["n"], cfg["src"], cfg["dst"])
+        cur = dev_t(cfg["cur"])
+        X = placeto.placeto_build_features(graph, dev_t(cfg["cost"]), dev_t(cfg["bytes"]), dev_t(cfg["dev"]), cur,
+                                           dev_t(cfg["placed"]), m)
+        grads = placeto.binding.zero_gradients(weights)
+        placeto.placeto_policy_gradient(graph, placeto.Weights(weights), X, dev_t(H[0]), dev_t(H[1]), cur,
+                                        dev_t(actions.astype(np.int32)), dev_t(adv.astype(np.float32)), 0.1, grads)
+        return {k: t.cpu().numpy().astype(np.float64) for k, t in grads.tensors.items()}
+
+    got = gradient_of(w)
+    f = w["f_down"]
+    wider = dict(f, hidden_dim=d + 1, W1=np.pad(f["W1"], ((0, 0), (0, 1))), b1=np.pad(f["b1"], (0, 1)), W2=np.pad(f["W2"], ((0, 1), (0, 0))))
+    want = gradient_of(dict(w, f_down=wider))
+    for (name, idx, key), a in got.items():
+        if nets == "g" and name in ("f_down", "f_up") and key in ("W1", "b1"):
+            continue               # equal halves of messages, negated halves of g's weights: f's hidden layer has no gradient but rounding
+        b = want[name, idx, key][tuple(slice(0, k) for k in a.shape)]
+        assert np.linalg.norm(a - b) <= 2e-5 * np.linalg.norm(b), (name, idx, key, np.linalg.norm(a - b), np.linalg.norm(b))
