@@ -209,6 +209,7 @@ grad_pool_backward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
 // partial[chunk][K + 1][J] = sum over rows of [in || 1]^T dp. A thread owns TK x 4 outputs; the rows arrive in stages
 // of 32 by cp.async while the stage before is multiplied.
 constexpr int kStageRows = 32;
+constexpr int kListStates = 1024;      // states of a node whose rows are listed at a time: the list must not grow with the batch
 
 // One stage of the product: the staged rows' inputs [32][Kp] and gradients [32][D].
 template <int D, int TK>
@@ -309,7 +310,7 @@ grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const pa
     const int tiles_j = D / 4;
     const int tk = threadIdx.x / tiles_j, tj = threadIdx.x % tiles_j;
     const bool live = TK * tk < Kp;
-    int *list = reinterpret_cast<int *>(smem + 2 * stage);           // rows waiting: fewer than 32 left over, then a node's
+    int *list = reinterpret_cast<int *>(smem + 2 * stage);           // rows waiting: fewer than 32 left over, then a node's of kListStates states
     __shared__ int have_s;
     for (int i = threadIdx.x; i < 2 * kStageRows * (Kp - K); i += threads) {
         const int r = i / (Kp - K), k = i - r * (Kp - K);
@@ -335,15 +336,17 @@ grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const pa
     for (int i = 0; i < TK; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
     const int per = (n + chunks - 1) / chunks;
     const int u0 = blockIdx.x * per, u1 = min(n, u0 + per);
+    const int parts = (B + kListStates - 1) / kListStates;
     int have = 0;
-    for (int u = u0; u < u1; ++u) {
+    for (int item = u0 * parts; item < u1 * parts; ++item) {
+        const int u = item / parts, b0 = (item - u * parts) * kListStates, b1 = min(B, b0 + kListStates);
         if (warp == 0) {
             int cnt = have;
-            for (int base = 0; base < B; base += 128) {          // four loads in flight
+            for (int base = b0; base < b1; base += 128) {        // four loads in flight
                 int s[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const int b = base + 32 * q + lane, c = b < B ? a.cur[b] : -1;
+                    const int b = base + 32 * q + lane, c = b < b1 ? a.cur[b] : -1;
                     s[q] = c >= 0 && c < n ? a.relation[(size_t)c * n + u] : 3;
                 }
 #pragma unroll
@@ -357,7 +360,7 @@ grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const pa
         }
         __syncthreads();
         have = have_s;
-        const int use = u + 1 < u1 ? have / kStageRows * kStageRows : have;
+        const int use = item + 1 < u1 * parts ? have / kStageRows * kStageRows : have;
         if (use > 0) load(0, min(kStageRows, use), 0);
         int buffer = 0;
         for (int r0 = 0; r0 < use; r0 += kStageRows, buffer ^= 1) {
@@ -431,7 +434,7 @@ cudaError_t launch_weights(const GradArgs &a, float *const (&rows)[8], int row_c
     if (err != cudaSuccess) return err;
     grad_weight_rows_kernel<D, TK><<<dim3(row_chunks, 8), threads, smem, stream>>>(jobs, (size_t)a.n * a.B, a.F, row_chunks);
     count_launch();
-    smem = (size_t)2 * kStageRows * (Lp + D) * sizeof(float) + (size_t)(a.B + kStageRows) * sizeof(int);
+    smem = (size_t)2 * kStageRows * (Lp + D) * sizeof(float) + (size_t)(std::min(a.B, kListStates) + kStageRows) * sizeof(int);
     err = cudaFuncSetAttribute(grad_weight_pool_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     grad_weight_pool_kernel<D, TK><<<dim3(pool_chunks, 3), pool_threads, smem, stream>>>(a, pool[0], pool[1], pool[2], pool_chunks);

@@ -156,6 +156,16 @@ def test_pooling_passes_over_chunks_of_nodes(d, m, n, B):
     compare(cfg, grads, gradient.gradient(cfg, actions, adv, 0.1))
 
 
+@pytest.mark.parametrize("d,m,n,B", [(32, 4, 3, 52500), (64, 5, 4, 1025), (32, 2, 5, 2079)])
+def test_pooling_weights_of_large_batches(d, m, n, B):
+    """The rows of a node are listed a part of the batch at a time: more states than a list in shared memory could hold,
+    parts of one state, remainders of a stage carried from part to part and from node to node."""
+    cfg, actions, adv = small_case(n + B, n=n, m=m, d=d, B=B, p=0.7)
+    adv = adv.astype(np.float32).astype(np.float64)
+    grads = gpu_gradient(cfg, actions, adv, 0.1)
+    compare(cfg, grads, gradient.gradient(cfg, actions, adv, 0.1))
+
+
 def cancelling(W, rows):
     """The first `rows` rows of W, the second half of them the first negated: over inputs whose halves agree the exact sum is
     zero, and what a kernel finds is what its order of summation leaves."""
