@@ -98,9 +98,19 @@ Layout make_layout(const placeto_graph *g, const placeto_weights *w, int B, plac
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
     L.status = take(kStatusBytes);
-    int chunks = pool_chunks((int)n, B, g->info);
-    L.chunk_nodes = ((int)n + chunks - 1) / chunks;
-    L.chunks = ((int)n + L.chunk_nodes - 1) / L.chunk_nodes;
+    // placeto_policy_logits_static takes a batch whose partial sums fit its array with the general kernel's coarse chunks
+    // and, where the raw features come in whole 16-byte pieces, with those of the d = 32 kernel and of the d = 64 tcgen05
+    // kernel. The kernels and chunks that the library prefers to these may need more room: for such a batch they make do
+    // with what there is, in placeto_policy_logits too, which has the same bits.
+    const size_t chunk_bytes = (size_t)B * 3 * d * sizeof(float);
+    const long long scratch_chunks = (long long)((PLACETO_STATIC_SCRATCH_BYTES - kStatusBytes) / chunk_bytes);
+    auto generic_chunks = [&](bool fine) {
+        const int chunks = pool_chunks((int)n, B, g->info, fine);
+        L.chunk_nodes = ((int)n + chunks - 1) / chunks;
+        L.chunks = ((int)n + L.chunk_nodes - 1) / L.chunk_nodes;
+    };
+    generic_chunks(false);
+    bool bounded = call == PLACETO_CALL_LOGITS && L.chunks <= scratch_chunks;
     if (call == PLACETO_CALL_EMBED || call == PLACETO_CALL_EMBED_ROUNDS ||
         (call >= PLACETO_CALL_FORWARD && call <= PLACETO_CALL_EPISODE)) {
         L.msg[0] = take(n * B * d * sizeof(float));
@@ -125,11 +135,20 @@ Layout make_layout(const placeto_graph *g, const placeto_weights *w, int B, plac
         return L;
     }
     if (w->F <= 16) {
-        if (w->d == 32 || w->d == 64) pool_split_chunks((int)n, B, w->d, g->info, &L.chunk_nodes_split, &L.chunks_split);
         if (w->d == 32) pool_d32_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
         if (w->d == 64 && (w->F & 3) == 0) pool_d64_chunks((int)n, B, w->F, g->info, &L.chunk_nodes32, &L.chunks32);
         if (w->d == 64) pool_tc_chunks((int)n, B, g->info, &L.chunk_nodes_tc, &L.chunks_tc);
+        if ((w->F & 3) == 0) {
+            bounded = bounded && std::max(L.chunks32, L.chunks_tc) <= scratch_chunks;
+        } else if (bounded) {
+            if (L.chunks32 > scratch_chunks) L.chunks32 = 0;
+            if (L.chunks_tc > scratch_chunks) L.chunks_tc = 0;
+        }
+        if (w->d == 32 || w->d == 64)
+            pool_split_chunks((int)n, B, w->d, g->info, bounded ? scratch_chunks : (long long)n, &L.chunk_nodes_split, &L.chunks_split);
     }
+    generic_chunks(true);
+    if (bounded && L.chunks > scratch_chunks) generic_chunks(false);
     if (call == PLACETO_CALL_LOGITS || (call >= PLACETO_CALL_FORWARD && call <= PLACETO_CALL_EPISODE))
         L.partial = take((size_t)std::max(std::max(L.chunks, L.chunks_split), std::max(L.chunks32, L.chunks_tc)) * B * 3 * d * sizeof(float));
     if (call >= PLACETO_CALL_FORWARD && call <= PLACETO_CALL_EPISODE) {

@@ -438,17 +438,18 @@ cudaError_t launch_simple_aggregator(const DevMlp &l, const DevMlp &h, const Dev
                                      cudaStream_t stream);
 
 // policy_generic.cu: pooling partial sums, then per-state finalisation + head + softmax.
-int pool_chunks(int n, int B, const DeviceInfo &di);
+int pool_chunks(int n, int B, const DeviceInfo &di, bool fine);
 cudaError_t launch_policy_generic(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream);
 // adds the chunk partial sums, applies h_i, the head and the softmax (one block per state)
 cudaError_t launch_pool_head(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream);
 
-// policy_d32.cu: specialised partial sums for d = 32, F <= 16, single-layer ReLU l_i
 // pool_split.cu: d = 32 and 64 pooling on the tensor cores (exact half-precision pieces)
 bool pool_split_applicable(const PoolArgs &a);
-void pool_split_chunks(int n, int B, int d, const DeviceInfo &di, int *chunk_nodes, int *chunks);   // *chunks = 0: the FMA kernel is faster
+// at most max_chunks; *chunks = 0: the FMA kernel is faster, or that many are not enough
+void pool_split_chunks(int n, int B, int d, const DeviceInfo &di, long long max_chunks, int *chunk_nodes, int *chunks);
 cudaError_t launch_pool_split(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
 
+// policy_d32.cu: specialised partial sums for d = 32, F <= 16, single-layer ReLU l_i
 bool pool_d32_applicable(const PoolArgs &a);
 bool pool_d32_fits(const PoolArgs &a, const DeviceInfo &di);      // applicable (a.chunk_nodes set) and within shared memory
 void pool_d32_chunks(int n, int B, int F, const DeviceInfo &di, int *chunk_nodes, int *chunks);

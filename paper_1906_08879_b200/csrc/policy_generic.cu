@@ -625,14 +625,14 @@ cudaError_t launch_head_fast(const PoolArgs &a, cudaStream_t stream) {
 
 bool pool_head_takes_compact(const PoolArgs &a) { return head_fast_applicable(a); }
 
-int pool_chunks(int n, int B, const DeviceInfo &di) {
+int pool_chunks(int n, int B, const DeviceInfo &di, bool fine) {
     // enough (chunk, state-group) blocks to fill the device a few times over
     const int state_blocks = (B + kPoolWarps - 1) / kPoolWarps;
-    int chunks = (4 * di.sm_count + state_blocks - 1) / state_blocks;
-    // chunks of eight nodes, or, on a small graph, of fewer: a node is a round trip to L2 for its warp, sixteen chunks
-    // are one for the head (32 nodes, 16 states, d = 8: pooling 16.7 -> 8.5 us)
-    chunks = std::max(1, std::min(chunks, std::max((n + 7) / 8, std::min(16, (n + 1) / 2))));
-    return chunks;
+    const int chunks = (4 * di.sm_count + state_blocks - 1) / state_blocks;
+    // chunks of eight nodes, or (`fine`), on a small graph, of fewer: a node is a round trip to L2 for its warp, sixteen
+    // chunks are one for the head (32 nodes, 16 states, d = 8: pooling 16.7 -> 8.5 us)
+    const int most = fine ? std::max((n + 7) / 8, std::min(16, (n + 1) / 2)) : (n + 7) / 8;
+    return std::max(1, std::min(chunks, most));
 }
 
 cudaError_t launch_policy_generic(const PoolArgs &a, const DeviceInfo &di, cudaStream_t stream) {

@@ -276,12 +276,14 @@ bool pool_split_applicable(const PoolArgs &a) {
 // state 14.1 us there, 14.7 here; 300 x 16: 16.4 and 14.5; 300 x 64: 17.3 and 16.5; 279 x 256: 23.7 and 21.3).
 // A warp takes whole items, so the batch costs (items per warp, rounded up) x (tiles per item); a set's last tile is
 // half empty on average.
-void pool_split_chunks(int n, int B, int d, const DeviceInfo &di, int *chunk_nodes, int *chunks) {
+void pool_split_chunks(int n, int B, int d, const DeviceInfo &di, long long max_chunks, int *chunk_nodes, int *chunks) {
     const long warps = (long)di.sm_count * (d == 32 ? Shape<32>::kWarps : Shape<64>::kWarps);
     double best = 0;
     *chunks = 0;
     if (d == 32 && (long)n * B < 4096) return;
-    for (int c = (n + kMaxChunk - 1) / kMaxChunk; c <= std::max(1, n / 16); ++c) {
+    const int fewest = (n + kMaxChunk - 1) / kMaxChunk;
+    if (fewest > max_chunks) return;
+    for (int c = fewest; c <= std::max(1, n / 16) && c <= max_chunks; ++c) {
         const int nodes = (n + c - 1) / c;
         if ((n + nodes - 1) / nodes != c) continue;
         const double cost = (double)(((long)B * c + warps - 1) / warps) * (nodes / (double)kTile + 1.5 + 0.5);

@@ -176,3 +176,22 @@ def test_workspace_bytes_on_host_graph():
         ctypes.c_size_t(0), ctypes.c_uint32(0), None)
     assert rc == 1
     del ws
+
+
+@pytest.mark.parametrize("d,F", [(8, 6), (48, 8), (128, 8), (32, 6), (32, 7), (64, 6), (64, 8), (32, 8)])
+def test_batches_within_the_built_in_scratch_stay_within_it(d, F):
+    """placeto_policy_logits_static takes a batch whose partial sums fit with chunks of eight nodes, at most four blocks
+    of eight states per SM (d = 32 and 64 with F a multiple of 4 have chunks of their own: graphs of up to 24 nodes fit
+    them in one to three). Kernels and chunks that are preferred to those must not ask for more than there is."""
+    sms, limit, checked = 148, placeto.binding.STATIC_SCRATCH_BYTES, 0
+    own = d in (32, 64) and F % 4 == 0
+    for n in (3, 8, 12, 16, 20, 24) if own else (3, 8, 12, 20, 32, 64, 151, 279, 531, 1000, 2130):
+        g = placeto.Graph(n, np.arange(n - 1), np.arange(1, n), host_only=True)
+        w = placeto.Weights({"d": d, "F": F, "m": 4}, device="cpu")
+        for B in (1, 100, 250, 300, 500, 600, 800, 992, 1500, 2000, 3000, 4096, 5000, 8192, 10000):
+            chunks = max(1, min((4 * sms + (B + 7) // 8 - 1) // ((B + 7) // 8), (n + 7) // 8))
+            if 256 + chunks * B * 3 * d * 4 > limit - 256:
+                continue
+            assert placeto.placeto_workspace_bytes(g, w, B, placeto.CALL_LOGITS) <= limit, (n, B)
+            checked += 1
+    assert checked > 20

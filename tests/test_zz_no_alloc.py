@@ -15,7 +15,8 @@ import pytest
 import torch
 
 import paper_1906_08879_b200 as placeto
-from gen import configs
+from gen import configs, states
+from tests.helpers import rng
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +67,20 @@ def test_static_scratch_call_rejects_a_batch_beyond_its_array():
     assert "scratch" in str(e.value)
     torch.cuda.synchronize()
     assert (logits == 0).all()                         # nothing was launched
+
+
+@pytest.mark.parametrize("n,d,m,B", [(279, 32, 2, 4096), (1500, 64, 2, 992), (20, 128, 2, 400)])
+def test_static_scratch_call_where_the_preferred_chunks_need_more(n, d, m, B):
+    """The preferred kernel's (or chunks') partial sums would exceed the array, the general ones fit: the call goes
+    through, with the bits of the workspace call."""
+    r = rng(n)
+    cfg = {"n": n, "src": np.arange(n - 1, dtype=np.int32), "dst": np.arange(1, n, dtype=np.int32), "m": m, "B": B}
+    cfg["cost"], cfg["bytes"] = states.node_costs(r, n, normalise=True)
+    cfg["dev"], cfg["cur"], cfg["placed"] = states.random_states(r, n, m, B)
+    cfg["weights"] = states.policy_weights(r, d, m + 4, m, 2, 0, 0.1)
+    g, w, X, Hd, Hu, cur = _inputs(cfg)
+    logits, probs = torch.full((B, m), float("nan"), device="cuda"), torch.full((B, m), float("nan"), device="cuda")
+    placeto.placeto_policy_logits_static(g, w, X, Hd, Hu, cur, logits, probs)
+    want_logits, want_probs = placeto.placeto_policy_logits(g, w, X, Hd, Hu, cur)
+    torch.cuda.synchronize()
+    assert torch.isfinite(logits).all() and torch.equal(logits, want_logits) and torch.equal(probs, want_probs)
