@@ -310,7 +310,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
  * time per device bus, overlapping with compute; an operation becomes runnable when
  * all parents have finished and their outputs have arrived on its device; an
  * operation takes cost[v], a transfer bytes[u] / bandwidth; the result is the time
- * stamp of the last operation to finish. One thread simulates one placement.
+ * stamp of the last operation to finish. A group of 8 to 32 lanes simulates one placement.
  * Readings where the paper is silent: one run time per operation whatever the
  * device; a tensor is sent once to each distinct device that hosts a child; a free
  * device or bus starts the head of its queue at once; equal time stamps are handled
@@ -319,7 +319,8 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
  * cost, bytes : DEVICE float[n].          dev : DEVICE uint8[P][n], devices < m.
  * bandwidth   : > 0, in units of bytes[] per unit of cost[].
  * runtime     : DEVICE double[P]; NaN for a placement that names a device >= m.
- * workspace   : DEVICE, at least placeto_simulator_workspace_bytes(g, P, m).
+ * workspace   : DEVICE, at least placeto_simulator_workspace_bytes(g, P, m), which grows with P up to what the device
+ *               simulates at once and no further (such calls take several launches).
  * Times are IEEE doubles added and divided in the model's order: reproducible.
  */
 size_t placeto_simulator_workspace_bytes(const placeto_graph *g, int32_t P, int32_t m);

@@ -877,7 +877,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
 
 size_t placeto_simulator_workspace_bytes(const placeto_graph *g, int32_t P, int32_t m) {
     if (!g || P < 1 || m < 1 || m > PLACETO_MAX_M) return 0;
-    return sim_workspace_bytes(g->host.n, (int)g->host.n_edges, P, g->on_device ? g->info : DeviceInfo{148, 227 * 1024});
+    return sim_workspace_bytes(g->host.n, (int)g->host.n_edges, m, P, g->on_device ? g->info : DeviceInfo{148, 227 * 1024});
 }
 
 placeto_status placeto_simulate_placements(const placeto_graph *g, const float *cost, const float *bytes,
@@ -895,7 +895,7 @@ placeto_status placeto_simulate_placements(const placeto_graph *g, const float *
         (runtime && !aligned16(runtime)) || (peak_memory && !aligned16(peak_memory)) ||
         (penalised && !aligned16(penalised)))
         return PLACETO_ERR_INVALID_ARG;
-    if (workspace_bytes < sim_workspace_bytes(g->host.n, (int)g->host.n_edges, P, g->info))
+    if (workspace_bytes < sim_workspace_bytes(g->host.n, (int)g->host.n_edges, m, P, g->info))
         return PLACETO_ERR_WORKSPACE;
     SimArgs a;
     a.n = g->host.n; a.n_edges = (int)g->host.n_edges; a.m = m; a.P = P;

@@ -355,7 +355,7 @@ cudaError_t launch_episode_end_compact(int n, int E, const uint8_t *state, uint8
 bool pool_head_takes_compact(const PoolArgs &a);
 
 // simulator.cu: event-based run time of P placements, a group of lanes each
-size_t sim_workspace_bytes(int n, int n_edges, int P, const DeviceInfo &di);
+size_t sim_workspace_bytes(int n, int n_edges, int m, int P, const DeviceInfo &di);
 cudaError_t launch_simulator(const SimArgs &a, const DeviceInfo &di, cudaStream_t stream);
 
 // gradient.cu: gradient of the policy objective with respect to all weights

@@ -17,8 +17,8 @@
 // earliest event is found with a butterfly over the group, and the children
 // (parents) of the operation are looked at one per lane. Queues are linked lists
 // threaded through per-placement arrays of 16-bit ids, which live in shared memory
-// together with the graph; what does not fit there (large graphs) keeps the arrays in the
-// workspace as 32-bit words. All times are doubles and are added and divided in
+// together with the graph; what does not fit there (large graphs, many placements) keeps
+// the arrays in the workspace as 32-bit words. All times are doubles and are added and divided in
 // the order the model states, so results are reproducible bit for bit.
 //
 // Measured on a B200 (279-node graph of multi-branch modules, 4096 placements on 4 devices, about
@@ -401,43 +401,82 @@ simulate_kernel(const SimArgs a, const SimPlan plan) {
 }  // namespace
 
 namespace {
-// placements per block whose arrays fit in shared memory beside the graph; 0: the arrays go to the workspace
-int sim_shared_fit(int n, int n_edges, const DeviceInfo &di) {
-    if (n_edges >= 0xffff) return 0;
-    const int budget = std::min(di.max_smem_optin, 227 * 1024) - 1024;
-    const int fit = (budget - sim_graph_bytes(n, n_edges)) / sim_state_bytes(n, n_edges);
-    return fit >= 4 ? fit : 0;
+int sim_group(int m) { return m <= 8 ? 8 : m <= 16 ? 16 : 32; }
+
+// Placements of a block and blocks of a launch: at most `most` placements a block, the blocks spread evenly over the SMs, and
+// over the waves of blocks where one does not hold them.
+int sim_per_block(int P, int most, const DeviceInfo &di) {
+    const long long wave = (long long)most * di.sm_count, waves = (P + wave - 1) / wave;
+    return (int)((P + waves * di.sm_count - 1) / (waves * di.sm_count));
 }
+
+// Fills `plan` for arrays in shared memory; false where they go to the workspace. A placement takes 1.2 to 1.45 times as
+// long with its arrays there, but an SM then has as many of them in flight as the registers allow (four blocks: 128, 64 or 32
+// by the width of a group). So they stay in shared memory (at least four a block) where that holds half as many, or holds
+// all of the call's at once, in as few blocks per SM as possible. ms, shared and workspace: 1948 nodes on 8 devices (four an
+// SM): 512 placements 5.5, 7.5; 1024: 10.9, 7.5; 8192: 64.5, 10.7. 351 nodes, 8 devices (32 of 128): 4096: 1.07, 1.47; 8192: 2.10,
+// 1.75; on 12 devices (32 of 64): 40000: 9.4, 10.3; 306 nodes, 12 devices (26 of 64): 19.1, 11.9. The line lies at a
+// number of placements, so that a smaller call never needs a larger workspace.
+bool sim_shared_plan(int n, int n_edges, int m, int P, const DeviceInfo &di, SimPlan *plan) {
+    if (n_edges >= 0xffff) return false;
+    const int block = std::min(di.max_smem_optin, 227 * 1024), threads_hold = kMaxThreads / sim_group(m);
+    plan->graph_bytes = sim_graph_bytes(n, n_edges);
+    plan->state_bytes = sim_state_bytes(n, n_edges);
+    int most[5];
+    for (int k = 1; k <= 4; ++k) {               // blocks of an SM, which has 1 KB more, a KB of each block being the system's
+        const int fit = ((block + 1024) / k - (k == 1 ? 2048 : 1024) - plan->graph_bytes) / plan->state_bytes;
+        if (k == 1 && fit < 4) return false;
+        most[k] = std::min(fit, threads_hold);
+    }
+    for (int k = 1; k <= 4; ++k)
+        if (P <= k * most[k] * di.sm_count) {
+            plan->per_block = (P + k * di.sm_count - 1) / (k * di.sm_count);
+            return true;
+        }
+    int best = 1;
+    for (int k = 2; k <= 4; ++k)
+        if (k * most[k] > best * most[best]) best = k;
+    if (2 * best * most[best] < 4 * threads_hold) return false;
+    plan->per_block = sim_per_block(P, most[best], di);
+    return true;
+}
+
+// Placements of one launch with their arrays in the workspace: twice what the device holds at once, so that the workspace
+// does not grow with their number beyond that and the end of a launch costs little.
+int sim_launch_placements(int m, int P, const DeviceInfo &di) { return std::min(P, 8 * (kMaxThreads / sim_group(m)) * di.sm_count); }
 }  // namespace
 
-size_t sim_workspace_bytes(int n, int n_edges, int P, const DeviceInfo &di) {
-    if (sim_shared_fit(n, n_edges, di) > 0) return 256;
-    return std::max<size_t>(sim_ints(n, n_edges) * (size_t)P * sizeof(int), 256);
+size_t sim_workspace_bytes(int n, int n_edges, int m, int P, const DeviceInfo &di) {
+    SimPlan plan;
+    if (sim_shared_plan(n, n_edges, m, P, di, &plan)) return 256;
+    return std::max<size_t>(sim_ints(n, n_edges) * (size_t)sim_launch_placements(m, P, di) * sizeof(int), 256);
 }
 
 cudaError_t launch_simulator(const SimArgs &a, const DeviceInfo &di, cudaStream_t stream) {
     SimPlan plan;
-    plan.graph_bytes = sim_graph_bytes(a.n, a.n_edges);
-    plan.state_bytes = sim_state_bytes(a.n, a.n_edges);
-    const int group = a.m <= 8 ? 8 : a.m <= 16 ? 16 : 32;
-    const int fit = sim_shared_fit(a.n, a.n_edges, di);
-    const bool shared = fit > 0;
-    const int most = shared ? std::min(fit, kMaxThreads / group) : kMaxThreads / group;
-    // the placements spread evenly over the SMs, and over the waves of blocks where one does not hold them
-    const int waves = (a.P + most * di.sm_count - 1) / (most * di.sm_count);
-    plan.per_block = (a.P + waves * di.sm_count - 1) / (waves * di.sm_count);
-    const int grid = (a.P + plan.per_block - 1) / plan.per_block;
-    const int threads = (plan.per_block * group + 31) & ~31;
-    const size_t smem = shared ? (size_t)plan.graph_bytes + (size_t)plan.per_block * plan.state_bytes : 0;
+    const int group = sim_group(a.m);
+    const bool shared = sim_shared_plan(a.n, a.n_edges, a.m, a.P, di, &plan);
     typedef void (*Kernel)(const SimArgs, const SimPlan);
     const Kernel kernels[2][4] = {
         {simulate_kernel<false, 8, 1>, simulate_kernel<false, 16, 1>, simulate_kernel<false, 32, 1>, simulate_kernel<false, 32, 2>},
         {simulate_kernel<true, 8, 1>, simulate_kernel<true, 16, 1>, simulate_kernel<true, 32, 1>, simulate_kernel<true, 32, 2>}};
     const Kernel kern = kernels[shared][a.m <= 8 ? 0 : a.m <= 16 ? 1 : a.m <= 32 ? 2 : 3];
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    kern<<<grid, threads, smem, stream>>>(a, plan);
-    count_launch();
+    const int step = shared ? a.P : sim_launch_placements(a.m, a.P, di);
+    for (int first = 0; first < a.P; first += step) {
+        SimArgs part = a;
+        part.P = std::min(step, a.P - first);
+        part.dev += (size_t)first * a.n;
+        if (part.runtime) part.runtime += first;
+        if (part.peak_memory) part.peak_memory += (size_t)first * a.m;
+        if (part.penalised) part.penalised += first;
+        if (!shared) plan.per_block = sim_per_block(part.P, kMaxThreads / group, di);
+        const size_t smem = shared ? (size_t)plan.graph_bytes + (size_t)plan.per_block * plan.state_bytes : 0;
+        const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err != cudaSuccess) return err;
+        kern<<<(part.P + plan.per_block - 1) / plan.per_block, (plan.per_block * group + 31) & ~31, smem, stream>>>(part, plan);
+        count_launch();
+        if (first > a.P - step) break;           // (the counter must not pass INT_MAX)
+    }
     return cudaGetLastError();
 }
 

@@ -169,3 +169,24 @@ def test_devices_per_lane_fan_out_and_arrays_in_the_workspace(n, m, P, p):
     np.testing.assert_array_equal(rt.cpu().numpy()[sel], want_rt)
     np.testing.assert_array_equal(peak.cpu().numpy()[sel], want_peak)
     np.testing.assert_array_equal(pen.cpu().numpy()[sel], want_pen)
+
+
+@pytest.mark.parametrize("n,m,P,p", [(12, 3, 18945, 0.3), (220, 3, 37889, 0.02), (120, 3, 16000, 0.02), (340, 12, 19000, 0.01), (300, 9, 4000, 0.01),
+                                     (900, 40, 9500, 0.002)])
+def test_more_placements_than_shared_memory_or_one_launch_holds(n, m, P, p):
+    """Small graphs keep any number of placements in shared memory, others what four blocks per SM hold; beyond that the
+    arrays go to the workspace, in launches of at most 37888, 18944 and 9472 placements by the width of a group."""
+    r = rng(P)
+    src, dst = random_dag(r, n, p)
+    cost = r.integers(1, 5, n).astype(np.float32)
+    size = r.integers(1, 5, n).astype(np.float32)
+    devs = r.integers(0, m, size=(P, n))
+    g = placeto.Graph(n, src, dst)
+    rt, peak, pen = placeto.placeto_simulate_placements(g, dev_t(cost), dev_t(size), dev_t(devs.astype(np.uint8)), m, 2.0, 6.0, 2.0)
+    torch.cuda.synchronize()
+    assert torch.isfinite(rt).all()
+    sel = np.unique(np.concatenate([np.arange(0, P, P // 12), np.arange(P - 8, P)]))
+    want_rt, want_peak, want_pen = simulator.placements(n, src, dst, cost, size, devs[sel], m, 2.0, 6.0, 2.0)
+    np.testing.assert_array_equal(rt.cpu().numpy()[sel], want_rt)
+    np.testing.assert_array_equal(peak.cpu().numpy()[sel], want_peak)
+    np.testing.assert_array_equal(pen.cpu().numpy()[sel], want_pen)

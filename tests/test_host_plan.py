@@ -195,3 +195,16 @@ def test_batches_within_the_built_in_scratch_stay_within_it(d, F):
             assert placeto.placeto_workspace_bytes(g, w, B, placeto.CALL_LOGITS) <= limit, (n, B)
             checked += 1
     assert checked > 20
+
+
+@pytest.mark.parametrize("n,m", [(160, 3), (351, 12), (351, 8), (1000, 2), (1948, 40)])
+def test_simulator_workspace_grows_with_the_placements_up_to_what_the_device_holds(n, m):
+    """A workspace made for a large call serves every smaller one, and its size is bounded however many the placements."""
+    r = rng(n)
+    src = np.repeat(np.arange(n - 1), 2)
+    dst = np.minimum(src + r.integers(1, 4, len(src)), n - 1)
+    g = placeto.Graph(n, src, dst, host_only=True)
+    need = placeto.binding._lib.placeto_simulator_workspace_bytes
+    sizes = [need(g.handle, ctypes.c_int32(P), ctypes.c_int32(m)) for P in list(range(1, 3000, 37)) + list(range(3000, 40000, 997)) + [1 << 20]]
+    assert sizes == sorted(sizes)
+    assert 4 * n * 4 * 1000 < sizes[-1] == sizes[-2] <= 8 * 32 * 148 * (4 * n + 5 * 2 * n) * 4
