@@ -176,7 +176,10 @@ after_g1:
         acc[r] = fmaxf(acc[r], 0.f);
         if (r == 0 || last_live) hrow[r * kD] = acc[r];
     }
-    if (slot < 0) return;                   // nobody consumes this node's message
+    if (slot < 0) {                         // nobody consumes this node's message
+        if constexpr (L == 1) __syncwarp();     // the next node writes A, which the only product may still be reading
+        return;
+    }
     float *in = L == 2 ? A : Bf;            // the buffer that the last product did not read
 #pragma unroll
     for (int r = 0; r < R; ++r) {

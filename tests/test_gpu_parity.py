@@ -341,6 +341,17 @@ def test_single_layer_networks_at_the_specialised_widths(d, m, B):
     _small_case(45, src, dst, d=d, m=m, B=B, layers=1, seed=B + d)
 
 
+@pytest.mark.parametrize("B", [1, 90, 300])
+def test_single_layer_networks_with_many_unread_messages(B):
+    """A warp that takes several nodes of a level one after the other, all of them with several neighbours and none with a
+    consumer: between two of them only the exchange buffer of the single product is passed on."""
+    r = rng(B)
+    sinks = [(s, 4 + k) for k in range(60) for s in r.choice(4, size=2 + k % 3, replace=False)]
+    src, dst = np.asarray(sinks, dtype=np.int32).T.copy()
+    for way in ((src, dst), (63 - dst, 63 - src)):
+        _small_case(64, *way, d=32, m=4, B=B, layers=1, seed=B)
+
+
 @pytest.mark.parametrize("d,m,B,layers,act", [(1, 1, 1, 1, 0), (3, 2, 200, 2, 0), (8, 2, 16, 2, 0), (8, 4, 301, 1, 0), (8, 8, 900, 2, 1), (14, 2, 75, 2, 0),
                                               (21, 8, 33, 2, 0), (31, 2, 500, 1, 0)])
 def test_narrow_sweep_kernel_keeps_the_generic_kernels_bits(d, m, B, layers, act):
