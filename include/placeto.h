@@ -161,8 +161,14 @@ typedef struct {
                                   blocks, grid-wide sync between levels (small B, wide levels) */
 #define PLACETO_GENERIC 8u     /* use only the dimension-generic kernels (no specialised ones) */
 #define PLACETO_FMA_ONLY 16u   /* keep steps 2 and 3 on the FP32 FMA pipes: do not use the tensor-core
-                                  kernels (operands split into half-precision pieces whose products
-                                  carry FP32 accuracy) that d = 64 and large batches otherwise take */
+                                  kernels (operands split into half-precision pieces) that d = 64 and
+                                  large batches otherwise take. Their products carry FP32 accuracy, at
+                                  d = 32 and of raw features that of every entry, of embeddings and
+                                  hidden layers at d = 64 that of the largest entry of a row (of 16
+                                  columns of a matrix): an entry below 2^-17 of it, by the bound that
+                                  the kernel has, keeps an absolute error of 2^-40 of that bound. A
+                                  network that makes such entries decisive by weights of the inverse
+                                  size needs this flag */
 #define PLACETO_TENSOR 32u     /* use the tensor-core kernel of step 2 wherever it applies (d = 32 or 64) */
 #define PLACETO_TCGEN05 64u    /* d = 64: take the kernels built on tcgen05.mma with accumulators in tensor
                                   memory instead of the warp-level (mma.sync) tensor-core kernels that are

@@ -19,7 +19,7 @@
 //
 // Measured on a B200, message passing alone, against the kernels it replaced (d = 64: a pipeline of layers on TF32
 // mma.sync, a warpgroup per layer; single layers: the dimension-generic kernel), us:
-//   d = 64, 1987 nodes in 741 levels:  64 states 884 -> 758, 256 states 1272 -> 951, 512 states 1932 -> 1350,
+//   d = 64, 1987 nodes in 741 levels:  64 states 884 -> 758, 256 states 1272 -> 951, 512 states 1932 -> 1370 (1355 with one scale for all raw features of a row),
 //   single-layer networks, 512 states: 12180 -> 839.  d = 32, 992 nodes in 249 levels, 992 states (against the FMA
 //   kernel): 826 -> 711.
 // What bounds it: the chain of a level, about 2000 cycles for one tile at d = 64 (gather 450, a layer 300: 30 for the
@@ -61,7 +61,8 @@ struct Config {
     static constexpr unsigned kSlot = 2 * kBuffer + kTile * 4;           // one tile in flight: two buffers, the rows' scales
     static constexpr unsigned kGroupBytes = 2 * kSlot;
     // per row of a level, written by the helper warps: a record, the raw features' pieces (16 columns, zero
-    // padded) and their scale
+    // padded) and their scale. (Scaled: a feature is first multiplied by the power of two that its weights are divided by,
+    // since features - byte counts beside ones and zeros - differ by any factor and the weights make up for it.)
     static constexpr int kXStride = 32;
     static constexpr unsigned kXPiece = kTile * kXStride;
     static constexpr unsigned kXTile = SP::kPieces * kXPiece;
@@ -98,7 +99,7 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
     const int n_levels = lv.n_levels;
     const int start = kWalk ? first_level(a.walk, lv, a.n) : 0;
 
-    // ---- shared memory: [schedule][message slots][raw features x2][bounds][row tiles x2][tiles of every group]
+    // ---- shared memory: [schedule][message slots][raw features x2][bounds][features' weights][row tiles x2][tiles of every group]
     //   meta[p] = {first neighbour entry, end of neighbour entries, own slot, node id}
     int *ism = reinterpret_cast<int *>(smem);
     int4 *meta_w = reinterpret_cast<int4 *>(ism);
@@ -126,8 +127,9 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
     const int *nbr_slot = stage_ints(lv.nbr_slot, lv.n_nbr);
     float *msg = smem + p.int_floats[dir];                      // [n_slots][S][P]
     float *xstage = msg + (size_t)lv.n_slots * S * P;           // [2][x_floats]
-    Bound *bounds = reinterpret_cast<Bound *>(xstage + 2 * (size_t)p.x_floats);     // [5 matrices][W]
-    unsigned char *row_tiles = reinterpret_cast<unsigned char *>(bounds + 5 * 4);   // [2][tiles of the widest level]
+    Bound *bounds = reinterpret_cast<Bound *>(xstage + 2 * (size_t)p.x_floats);     // [4 matrices][W]
+    float *x_weight = reinterpret_cast<float *>(bounds + 4 * 4);                    // [16] power of two above a feature's weights
+    unsigned char *row_tiles = reinterpret_cast<unsigned char *>(x_weight + 16);    // [2][tiles of the widest level]
     unsigned char *tiles = row_tiles + 2 * (size_t)p.row_bytes + (group < C::G ? group : 0) * C::kGroupBytes;
     float *__restrict__ H = a.H[dir];
 
@@ -160,6 +162,7 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
             }
             __pipeline_commit();
         };
+        float2 x_up = make_float2(1.f, 1.f);                // x_weight of this thread's two features
         auto publish = [&](int level) {
             const int p0 = level_ptr[level], rows = (level_ptr[level + 1] - p0) * nb;
             unsigned char *out = row_tiles + (size_t)(level & 1) * p.row_bytes;
@@ -182,11 +185,13 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
                 float x = k < F ? xs[r * F + k] : 0.f, y = k + 1 < F ? xs[r * F + k + 1] : 0.f;
                 unsigned char *tile = out + (r / kTile) * C::kRowTile;
                 if constexpr (SP::kScaled) {
-                    float top = fmaxf(fabsf(x), fabsf(y));
+                    x *= x_up.x;
+                    y *= x_up.y;
+                    float bound = fabsf(x) + fabsf(y);           // of the features' part of f's first product
 #pragma unroll
-                    for (int o = 1; o < 8; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-                    const float up = scale_up(top);
-                    if (k == 0) reinterpret_cast<float *>(tile + C::kXTile + kTile * 16)[r % kTile] = up;
+                    for (int o = 1; o < 8; o <<= 1) bound += __shfl_xor_sync(0xffffffffu, bound, o);
+                    const float up = scale_up(bound);
+                    if (k == 0) reinterpret_cast<float *>(tile + C::kXTile + kTile * 16)[r % kTile] = 0.5f * up;
                     x *= up;
                     y *= up;
                 }
@@ -197,7 +202,17 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
                     *reinterpret_cast<unsigned *>(tile + q * C::kXPiece + (r % kTile) * C::kXStride + 2 * k) = pc[q];
             }
         };
+        if constexpr (SP::kScaled) {                        // the power of two above the largest weight of each, eight lanes a feature
+            static_assert(kHelperThreads == 8 * 16, "sixteen features");
+            const int k = ht >> 3;
+            float top = 0x1p-126f;
+            for (int c = ht & 7; k < F && c < D; c += 8) top = fmaxf(top, fabsf(a.f[dir].W1[(D + k) * D + c]));
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+            if ((ht & 7) == 0) x_weight[k] = fminf(pow2_above(top), 0x1p126f);
+        }
         __syncthreads();              // schedule staged
+        if constexpr (SP::kScaled) x_up = *reinterpret_cast<const float2 *>(x_weight + 2 * (ht & 7));
         dependency_wait();            // the raw features may come from a kernel that is still running
         fetch(start);
         fetch(start + 1);
@@ -254,26 +269,28 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
         }
         bias_of(fn.b1, bf1);
         record(2, wf1.load(c0, lane, [&](int k, int c) { return fn.W1[k * D + c]; }), bf1);
-        record(3, wx.load(c0, lane, [&](int k, int c) { return k < F ? fn.W1[(D + k) * D + c] : 0.f; }), bf1);
+        if constexpr (!SP::kScaled) wx.load(c0, lane, [&](int k, int c) { return k < F ? fn.W1[(D + k) * D + c] : 0.f; });
         if constexpr (L == 2) {
             bias_of(fn.b2, bf2);
-            record(4, wf2.load(c0, lane, [&](int k, int c) { return fn.W2[k * D + c]; }), bf2);
+            record(3, wf2.load(c0, lane, [&](int k, int c) { return fn.W2[k * D + c]; }), bf2);
         }
     }
-    __syncthreads();              // schedule and bounds staged
+    __syncthreads();              // schedule, bounds and the features' weights staged
+    if constexpr (SP::kScaled)
+        wx.load(c0, lane, [&](int k, int c) { return k < F ? fn.W1[(D + k) * D + c] * inverse_pow2(x_weight[k]) : 0.f; });
     // Fp16x2: a row's activations are carried multiplied by a power of two. With b a bound of the row's input of
     // g that is at least the largest bias, b * prod (norm_i + 1) bounds every later layer, so the powers of two
     // of the layers are the input's times constants of the launch (rounded up to powers of two):
-    //   after g's layers: row scale * ug[i];  after f's first: min(row scale * uh, scale of x * ux)
+    //   after g's layers: row scale * ug[i];  after f's first: min(row scale * uh, half the scale of the features)
     // (The bound of the gathered row is its largest entry, found with shuffles: carrying a bound with every message
     // is loose by another 2^4 .. 2^6 per level, four times the error.)
-    float floor_b = 0.f, ug[2] = {1.f, 1.f}, uh = 1.f, ux = 1.f;
+    float floor_b = 0.f, ug[2] = {1.f, 1.f}, uh = 1.f;
     if constexpr (SP::kScaled) {
-        float grow[5];
+        float grow[4];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) {
+        for (int i = 0; i < 4; ++i) {
             float norm = 0.f;
-            if (L == 2 || (i != 1 && i != 4))
+            if (L == 2 || (i != 1 && i != 3))
                 for (int q = 0; q < C::W; ++q) {
                     norm = fmaxf(norm, bounds[i * C::W + q].norm);
                     floor_b = fmaxf(floor_b, bounds[i * C::W + q].bias);
@@ -283,13 +300,13 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
         ug[0] = grow[0];
         ug[1] = L == 2 ? ug[0] * grow[1] : ug[0];
         uh = 0.5f * ug[1] * grow[2];
-        ux = 0.5f * grow[3];
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             bg1[c] *= ug[0];
             bg2[c] = L == 2 ? bg2[c] * ug[1] : 0.f;
         }
         wg1.inv *= ug[0];
+        wx.inv *= 0.5f;                                  // the features' scale is stored halved
         if constexpr (L == 2) wg2.inv *= grow[1];
         wf1.inv *= inverse_pow2(ug[1]);
     }
@@ -413,7 +430,7 @@ embed_split_kernel(const EmbedArgs a, const SplitPlan p) {
             for (int e = 0; e < 2; ++e) {
                 if constexpr (SP::kScaled) {
                     // (L = 1: this is the message, unscaled)
-                    const float uf = L == 1 ? 1.f : fminf(up[i][e] * uh, upx[i][e] * ux);
+                    const float uf = L == 1 ? 1.f : fminf(up[i][e] * uh, upx[i][e]);
                     const float fh = back[i][e] * wf1.inv * uf, fx = inverse_pow2(upx[i][e]) * wx.inv * uf;
                     v[i][e] = fmaxf(fmaf(v[i][e], fh, fmaf(x[i][e], fx, bf1[0] * uf)), 0.f);
                     v[i][2 + e] = fmaxf(fmaf(v[i][2 + e], fh, fmaf(x[i][2 + e], fx, bf1[1] * uf)), 0.f);
@@ -491,7 +508,7 @@ cudaError_t launch(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream
         size_t worst = 0;
         for (int dir = 0; dir < 2; ++dir)
             worst = std::max(worst, (size_t)p.int_floats[dir] + (size_t)a.lv[dir].n_slots * S * C::P);
-        return (worst + 2 * (size_t)x_floats(S)) * sizeof(float) + 5 * 4 * sizeof(Bound) + 2 * (size_t)row_bytes(S) +
+        return (worst + 2 * (size_t)x_floats(S)) * sizeof(float) + 4 * 4 * sizeof(Bound) + 16 * sizeof(float) + 2 * (size_t)row_bytes(S) +
                (size_t)C::G * C::kGroupBytes;
     };
     while (p.S > 1 && need(p.S) > budget) --p.S;

@@ -7,8 +7,9 @@
 // row. On the FP32 units (policy_d32.cu) that is what bounds it: 219 us for 992 nodes in 992 states,
 // d = 32, F = 12 (103 here; 1080 nodes x 256 states, F = 8: 63 and 37). Here sixteen rows of a (state, set)
 // are the 16 rows of mma.sync.m16n8k16. d = 32: on exact pieces of three bfloat16 numbers (Bf16x3, six
-// products). d = 64: on two half-precision pieces (Fp16x2, three products; a row's two embeddings and its raw features
-// scaled apart, since they are of different size): 217 us for 1987 nodes x 512 states, 244 on the tcgen05 kernel (policy_tc.cu),
+// products). d = 64: on two half-precision pieces (Fp16x2, three products; a row's two embeddings scaled apart, since they
+// are of different size) and the raw features, whose sizes differ within a row by any factor, on exact pieces (8 us of
+// the whole): 225 us for 1987 nodes x 512 states, 244 on the tcgen05 kernel (policy_tc.cu),
 // whose producers and barriers cost 19 us on the smallest call, 6.4 here. (Fp16x2 at d = 32: 91 us, but 3e-5 of error
 // where one logit of one device is what cancellation left, above the 2e-5 that FP32 keeps.)
 //   - A warp owns items (state, chunk of nodes) and walks the three sets one by one; it compacts the
@@ -40,7 +41,9 @@ template <int D> struct Shape {
     static constexpr int kPieces = SP::kPieces;
     static constexpr int NT = D / 8, KE = D / 16, KS = 2 * KE + 1;
     static constexpr int kWarps = D == 32 ? 16 : 12, kThreads = kWarps * 32;
-    static constexpr int kFragments = 3 * KS * kPieces * (NT / 2) * 32;          // uint4 of weight fragments
+    typedef Bf16x3 XP;                              // of the raw features: those of one row may differ by any factor
+    static constexpr int kSetPieces = (KS - 1) * kPieces + XP::kPieces;
+    static constexpr int kFragments = 3 * kSetPieces * (NT / 2) * 32;            // uint4 of weight fragments
 };
 
 struct PoolSplitPlan {
@@ -58,24 +61,23 @@ __global__ void __launch_bounds__(Shape<D>::kThreads, 1)
 pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
     typedef Shape<D> C;
     typedef typename C::SP SP;
-    constexpr int kPieces = C::kPieces;
+    typedef typename C::XP XP;
+    constexpr int kPieces = C::kPieces, kXPieces = XP::kPieces;
     constexpr int NT = C::NT, KE = C::KE, KS = C::KS, kWarps = C::kWarps, kThreads = C::kThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int n = a.n, B = a.B, F = a.F;
-    uint4 *frag = reinterpret_cast<uint4 *>(smem_raw);                  // [set][step][piece][pair of tiles][lane]
+    uint4 *frag = reinterpret_cast<uint4 *>(smem_raw);                  // [set][step and piece][pair of tiles][lane]
     float *bias_s = reinterpret_cast<float *>(frag + C::kFragments);    // [3][D]
-    float *scale_s = bias_s + 3 * D;                                    // [3][segment]: what the weights are multiplied by
+    float *scale_s = bias_s + 3 * D;                                    // [3][embedding]: what the weights are multiplied by
     uint16_t *list = reinterpret_cast<uint16_t *>(scale_s + 20) + (size_t)warp * ((p.chunk_nodes + 7) & ~7);
-    // the three segments of a row: h_down, h_up, raw features
-    auto segment_of = [](int ks) { return ks < KE ? 0 : ks < 2 * KE ? 1 : 2; };
 
     // ---- weights as fragments: lane (g, t) of tile nt holds rows 16 ks + 4 t .. + 3 of column 8 nt + g
-    for (int i = warp; SP::kScaled && i < 9; i += kWarps) {
-        const float *W = a.l[i / 3].W1 + (i % 3) * D * D;
+    for (int i = warp; SP::kScaled && i < 6; i += kWarps) {
+        const float *W = a.l[i / 2].W1 + (i % 2) * D * D;
         float top = 0.f;
-        for (int k = lane; k < (i % 3 == 2 ? F : D) * D; k += 32) top = fmaxf(top, fabsf(W[k]));
+        for (int k = lane; k < D * D; k += 32) top = fmaxf(top, fabsf(W[k]));
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
         if (lane == 0) scale_s[i] = split::scale_up(top);
@@ -83,17 +85,22 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * KS * NT * 32; i += kThreads) {
         const int l = i & 31, nt = (i >> 5) % NT, ks = (i >> 5) / NT % KS, set = (i >> 5) / (NT * KS);
-        const float *W = a.l[set].W1, up = SP::kScaled ? scale_s[set * 3 + segment_of(ks)] : 1.f;
+        const float *W = a.l[set].W1, up = SP::kScaled && ks < KS - 1 ? scale_s[set * 2 + ks / KE] : 1.f;
         const int k0 = 16 * ks + 4 * (l & 3), col = 8 * nt + (l >> 2);
         float w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) w[j] = k0 + j < 2 * D + F ? W[(k0 + j) * D + col] * up : 0.f;
-        unsigned lo[kPieces], hi[kPieces];
-        SP::pieces(w[0], w[1], lo);
-        SP::pieces(w[2], w[3], hi);
+        auto store = [&](auto split) {
+            typedef decltype(split) S;
+            unsigned lo[S::kPieces], hi[S::kPieces];
+            S::pieces(w[0], w[1], lo);
+            S::pieces(w[2], w[3], hi);
 #pragma unroll
-        for (int q = 0; q < kPieces; ++q)
-            reinterpret_cast<uint2 *>(frag + (((set * KS + ks) * kPieces + q) * (NT / 2) + nt / 2) * 32 + l)[nt & 1] = make_uint2(lo[q], hi[q]);
+            for (int q = 0; q < S::kPieces; ++q)
+                reinterpret_cast<uint2 *>(frag + ((set * C::kSetPieces + ks * kPieces + q) * (NT / 2) + nt / 2) * 32 + l)[nt & 1] = make_uint2(lo[q], hi[q]);
+        };
+        if (ks < KS - 1) store(SP());
+        else store(XP());
     }
     for (int i = threadIdx.x; i < 3 * D; i += kThreads) bias_s[i] = a.l[i / D].b1[i % D];
     __syncthreads();
@@ -120,7 +127,7 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
             float total[NT][2];
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) total[nt][0] = total[nt][1] = 0.f;
-            const uint4 *fr = frag + (size_t)set * KS * kPieces * (NT / 2) * 32 + lane;
+            const uint4 *fr = frag + (size_t)set * C::kSetPieces * (NT / 2) * 32 + lane;
 #pragma unroll 1
             for (int first = 0; first < count; first += kTile) {
                 // rows past the end repeat the last one
@@ -155,17 +162,16 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
                             if (4 * t + j < F) v[j] = a.X[row * F + 4 * t + j];
                     }
                 }
-                // every segment of a row is scaled by itself (where the pieces need it)
-                unsigned A[KS][kPieces][4];
-                float down_by[3][2];
+                // each embedding of a row is scaled by itself (where the pieces need it), the raw features not at all
+                unsigned A[KS - 1][kPieces][4], Ax[kXPieces][4];
+                float down_by[2][2];
 #pragma unroll
-                for (int seg = 0; seg < 3; ++seg) {
-                    const int k0 = seg == 2 ? 2 * KE : seg * KE, k1 = seg == 2 ? KS : k0 + KE;
+                for (int emb = 0; emb < 2; ++emb) {
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         float top = 0.f, up = 1.f;
 #pragma unroll
-                        for (int ks = k0; SP::kScaled && ks < k1; ++ks) {
+                        for (int ks = emb * KE; SP::kScaled && ks < (emb + 1) * KE; ++ks) {
                             const float4 v = x[ks][r];
                             top = fmaxf(top, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
                         }
@@ -173,10 +179,10 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
                             top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 1));
                             top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
                             up = split::scale_up(top);
-                            down_by[seg][r] = split::inverse_pow2(up);
+                            down_by[emb][r] = split::inverse_pow2(up);
                         }
 #pragma unroll
-                        for (int ks = k0; ks < k1; ++ks) {
+                        for (int ks = emb * KE; ks < (emb + 1) * KE; ++ks) {
                             const float4 v = x[ks][r];
                             unsigned lo[kPieces], hi[kPieces];
                             SP::pieces(v.x * up, v.y * up, lo);
@@ -186,50 +192,69 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
                         }
                     }
                 }
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float4 v = x[KS - 1][r];
+                    unsigned lo[kXPieces], hi[kXPieces];
+                    XP::pieces(v.x, v.y, lo);
+                    XP::pieces(v.z, v.w, hi);
+#pragma unroll
+                    for (int q = 0; q < kXPieces; ++q) { Ax[q][r] = lo[q]; Ax[q][2 + r] = hi[q]; }
+                }
                 const bool live[2] = {first + g < count, first + 8 + g < count};
 #pragma unroll
                 for (int half = 0; half < NT / 4; ++half) {
-                    // Chains. Scaled: one per segment, small products before the leading one of a step. Not scaled: leading
-                    // products of the first steps, of the others, and all small ones (the tensor core's accumulation truncates).
+                    // Chains. Scaled: one per embedding and one for the features, small products before the leading one of a
+                    // step. Not scaled: leading products of the first steps, of the others, and all small ones (the tensor
+                    // core's accumulation truncates).
                     float acc[3][4][4];
 #pragma unroll
                     for (int ks = 0; ks < KS; ++ks) {
                         const uint4 *w_at = fr + ks * kPieces * (NT / 2) * 32 + half * 64;
-                        auto product = [&](int chain, bool zero, const unsigned (&rows)[4], const uint4 (&w)[2]) {
+                        auto product = [&](auto split, int chain, bool zero, const unsigned (&rows)[4], const uint4 (&w)[2]) {
+                            typedef decltype(split) S;
 #pragma unroll
                             for (int nt = 0; nt < 4; ++nt) {
                                 const unsigned b0 = (nt & 1) ? w[nt / 2].z : w[nt / 2].x, b1 = (nt & 1) ? w[nt / 2].w : w[nt / 2].y;
-                                if (zero) SP::mma_zero(acc[chain][nt], rows, b0, b1);
-                                else SP::mma(acc[chain][nt], rows, b0, b1);
+                                if (zero) S::mma_zero(acc[chain][nt], rows, b0, b1);
+                                else S::mma(acc[chain][nt], rows, b0, b1);
                             }
                         };
                         auto weights = [&](int piece, uint4 (&w)[2]) {
                             w[0] = w_at[piece * (NT / 2) * 32];
                             w[1] = w_at[piece * (NT / 2) * 32 + 32];
                         };
-                        uint4 w[2];
-                        if constexpr (SP::kScaled) {
-                            const int seg = segment_of(ks);
-                            weights(1, w);
-                            product(seg, ks == 0 || ks == KE || ks == 2 * KE, A[ks][0], w);
-                            weights(0, w);
-                            product(seg, false, A[ks][1], w);
-                            product(seg, false, A[ks][0], w);
-                        } else {
+                        // exact pieces: the small products into one chain, the leading one into another (or the same)
+                        auto exact = [&](const unsigned (&rows)[3][4], int small, bool zero_small, int lead, bool zero_lead) {
+                            uint4 w[2];
                             weights(2, w);
-                            product(2, ks == 0, A[ks][0], w);
+                            product(Bf16x3(), small, zero_small, rows[0], w);
                             weights(1, w);
-                            product(2, false, A[ks][0], w);
-                            product(2, false, A[ks][1], w);
+                            product(Bf16x3(), small, false, rows[0], w);
+                            product(Bf16x3(), small, false, rows[1], w);
                             weights(0, w);
-                            product(2, false, A[ks][kPieces - 1], w);
-                            product(2, false, A[ks][1], w);
-                            product(ks < 2 ? 0 : 1, ks == 0 || ks == 2, A[ks][0], w);
+                            product(Bf16x3(), small, false, rows[2], w);
+                            product(Bf16x3(), small, false, rows[1], w);
+                            product(Bf16x3(), lead, zero_lead, rows[0], w);
+                        };
+                        if constexpr (SP::kScaled) {
+                            if (ks == KS - 1) {
+                                exact(Ax, 2, true, 2, false);
+                            } else {
+                                uint4 w[2];
+                                weights(1, w);
+                                product(SP(), ks / KE, ks % KE == 0, A[ks][0], w);
+                                weights(0, w);
+                                product(SP(), ks / KE, false, A[ks][1], w);
+                                product(SP(), ks / KE, false, A[ks][0], w);
+                            }
+                        } else {
+                            exact(ks == KS - 1 ? Ax : A[ks], 2, ks == 0, ks < 2 ? 0 : 1, ks == 0 || ks == 2);
                         }
                     }
-                    float back[3];              // the weights' scales undone
+                    float back[2];              // the weights' scales undone
 #pragma unroll
-                    for (int seg = 0; seg < 3; ++seg) back[seg] = SP::kScaled ? split::inverse_pow2(scale_s[set * 3 + seg]) : 1.f;
+                    for (int emb = 0; emb < 2; ++emb) back[emb] = SP::kScaled ? split::inverse_pow2(scale_s[set * 2 + emb]) : 1.f;
 #pragma unroll
                     for (int nt = 0; nt < 4; ++nt) {
                         const float2 bias = *reinterpret_cast<const float2 *>(bias_s + set * D + 32 * half + 8 * nt + 2 * t);
@@ -238,7 +263,7 @@ pool_split_kernel(const PoolArgs a, const PoolSplitPlan p) {
                             const int r = i >> 1;
                             float part[3];
 #pragma unroll
-                            for (int q = 0; q < 3; ++q) part[q] = SP::kScaled ? (acc[q][nt][i] * down_by[q][r]) * back[q] : acc[q][nt][i];
+                            for (int q = 0; q < 3; ++q) part[q] = SP::kScaled && q < 2 ? (acc[q][nt][i] * down_by[q & 1][r]) * back[q & 1] : acc[q][nt][i];
                             const float v = ((part[0] + part[1]) + part[2]) + ((i & 1) ? bias.y : bias.x);
                             total[4 * half + nt][i & 1] += live[r] ? fmaxf(v, 0.f) : 0.f;
                         }

@@ -6,12 +6,14 @@
 //
 //   Bf16x3 : x = h + m + l in bfloat16, exact (8 + 8 + 8 bits, the exponent range of FP32). Six
 //            products (hh, hm, mh, mm, hl, lh); what is dropped is below 2^-26 of a term.
-//   Fp16x2 : x = h + l in half precision, within 2^-24 of x (half an ulp of FP32). Three products
-//            (hh, hl, lh); ll is below 2^-24 of a term, as in a TF32 head + tail split. Half the
-//            instructions of Bf16x3, but five exponent bits: a row of activations (and a warp's
-//            block of weights) is multiplied by a power of two that puts a bound of its entries
-//            at 2^15; entries down to 2^-17 of the bound keep all bits, smaller ones an absolute
-//            error of 2^-40 of the bound.
+//   Fp16x2 : x = h + l in half precision. Three products (hh, hl, lh); ll is below 2^-24 of a term,
+//            as in a TF32 head + tail split. Half the instructions of Bf16x3, but five exponent bits:
+//            a row of activations (and a warp's block of weights) is multiplied by a power of two
+//            that puts a bound of its entries at 2^15. Entries down to 2^-17 of the bound are then
+//            within 2^-24 of themselves (half an ulp of FP32), smaller ones within 2^-40 of the
+//            bound. A layer's bound is that of its input times prod(norm + 1) of the layers between,
+//            2^3 to 2^5 a layer above what comes out: entries below 2^-5 to 2^-8 of a row's largest
+//            lose bits in f's second product, a hundredth of the rounding of a row's largest entry.
 //
 // The product is computed transposed: the instruction's 16 rows are 16 output columns of a layer
 // (weights, A fragments, in registers), its 8 columns a tile's 8 data rows (B fragments, read with

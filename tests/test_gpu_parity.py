@@ -409,6 +409,66 @@ def test_split_pooling_over_chunks_and_sets(n, m, B, d):
     assert torch.isnan(logits[3]).all() and torch.equal(logits[4:], out["logits"][4:])
 
 
+@pytest.mark.parametrize("d,m,layers,B,flags", [(64, 8, 2, 90, 0), (64, 3, 1, 300, 0), (64, 4, 2, 90, placeto.PLACETO_TENSOR), (32, 4, 2, 900, 0)])
+def test_features_of_any_size_against_weights_of_the_inverse_size(d, m, layers, B, flags):
+    """Byte counts of 1e8 beside costs of 1 with weights to match (a power of two apart from the scaled problem) leave every
+    product as it is: embeddings and logits keep their bits."""
+    r = rng(d + m)
+    src, dst = random_dag(r, 40, 0.1)
+    w = states.policy_weights(r, d, m + 4, m, layers, 0, 0.1)
+    cost, size = states.node_costs(r, 40, normalise=True)
+    devs, cur, placed = states.random_states(r, 40, m, B)
+    out = []
+    for scale in (1.0, 2.0 ** 27):
+        for net, row in [(w["f_down"], d + 1), (w["f_up"], d + 1), (w["head"], 2 * d + 1)] + [(l, 2 * d + 1) for l in w["l"]]:
+            net["W1"][row] /= scale
+        g, wt, c = placeto.Graph(40, src, dst), placeto.Weights(w), dev_t(cur)
+        X = placeto.placeto_build_features(g, dev_t(cost), dev_t(size * np.float32(scale)), dev_t(devs), c, dev_t(placed), m)
+        Hd, Hu = placeto.placeto_embed_forward(g, wt, X, flags=flags)
+        fwd, _ = placeto.placeto_policy_forward(g, wt, dev_t(cost), dev_t(size * np.float32(scale)), dev_t(devs), c, dev_t(placed), flags=flags)
+        out.append((Hd, Hu, placeto.placeto_policy_logits(g, wt, X, Hd, Hu, c, flags=flags)[0], fwd))
+    torch.cuda.synchronize()
+    for a, b in zip(*out):
+        assert torch.isfinite(a).all() and torch.equal(a, b)
+
+
+@pytest.mark.parametrize("d", [32, 64])
+def test_pooling_reads_a_small_feature_beside_a_large_one(d):
+    """Costs of 1e-3 beside byte counts of 1e8 that half of the columns give no weight to: those columns' sums carry the
+    costs to FP32 accuracy. On a chain the sets of a state are the nodes before and after its current one."""
+    r = rng(d)
+    n, m, B = 300, 4, 40
+    F = m + 4
+    w = states.policy_weights(r, d, F, m, 1, 0, 0.0)
+    for i in range(3):
+        l, h = w["l"][i]["W1"], w["h"][i]["W1"]
+        l[2 * d + 1, : d // 2] = 0                       # no weight on the bytes ...
+        l[2 * d + 2:, : d // 2] = 0
+        h[d // 2:] = 0                                   # ... and only those columns matter
+        h[: d // 2] *= 100
+    cost, size = r.lognormal(-7, 1, n).astype(np.float32), r.lognormal(18, 1, n).astype(np.float32)
+    devs, cur, placed = states.random_states(r, n, m, B)
+    g, wt, c = placeto.Graph(n, np.arange(n - 1), np.arange(1, n)), placeto.Weights(w), dev_t(cur)
+    X = placeto.placeto_build_features(g, dev_t(cost), dev_t(size), dev_t(devs), c, dev_t(placed), m)
+    X[:, :, 1][c.long(), torch.arange(B, device="cuda")] = 0            # (the current node's own features enter the head)
+    zero = torch.zeros((n, B, d), device="cuda")
+    logits, _ = placeto.placeto_policy_logits(g, wt, X, zero, zero, c)
+    x64 = X.cpu().numpy().astype(np.float64)
+    a = np.zeros((B, 3, d))
+    for i in range(2):
+        rows = np.maximum(x64 @ w["l"][i]["W1"][2 * d:].astype(np.float64), 0)
+        for b in range(B):
+            a[b, i] = np.maximum((rows[: cur[b], b] if i == 0 else rows[cur[b] + 1:, b]).sum(axis=0) @ w["h"][i]["W1"].astype(np.float64), 0)
+    z = np.concatenate([np.zeros((B, 2 * d)), x64[cur, np.arange(B)], a.reshape(B, 3 * d)], axis=1)
+    z[:, 2 * d + 2: 2 * d + F] = x64[cur, np.arange(B)][:, 2:]
+    head = w["head"]
+    ref = np.maximum(z @ head["W1"], 0) @ head["W2"]
+    head_only = np.maximum(np.where(np.arange(z.shape[1]) < 2 * d + F, z, 0) @ head["W1"], 0) @ head["W2"]
+    got = logits.cpu().numpy().astype(np.float64)
+    assert np.abs(ref - head_only).max() > 0.1          # the sums decide the logits
+    assert np.abs(got - ref).max() <= 2e-5 * np.abs(ref).max()
+
+
 def test_identity_activation_and_path_counting():
     one = net([[1.0], [1.0]], [0.0], act=1)
     idn = net([[1.0]], [0.0], act=1)
