@@ -34,6 +34,7 @@ if ROOT not in sys.path:
 METRIC = "placement-state evaluations/sec (full-graph embed + logits)"
 UNIT = "evaluations/s"
 FP32_LANES_PER_SM = 128           # FMA lanes per SM
+SMS = 148
 L2_FLUSH_BYTES = 256 << 20        # > 126 MB L2
 
 
@@ -276,6 +277,26 @@ def error_against_checker(cfg, logits, Hd, Hu, samples: int = 16):
             "reference": "fp64 CPU checker (oracle/), same seeded inputs"}
 
 
+def sweep_of_the_step(g, cfg, flags: int):
+    """(flags, arithmetic) with which placeto_embed_forward runs the sweep that the whole path takes. That call keeps
+    the kernels whose bits its callers have; PLACETO_TENSOR gives it the tensor-core sweep that placeto_policy_forward picks
+    by itself at d = 64, and at d = 32 from twelve rows of a block per level on, up to three and a half neighbours per node."""
+    import paper_1906_08879_b200 as placeto
+    other = (placeto.PLACETO_PER_LEVEL | placeto.PLACETO_COOPERATIVE | placeto.PLACETO_GENERIC | placeto.PLACETO_FMA_ONLY)
+    d, n, info = cfg["d"], cfg["n"], g.info()
+    if d == 64 and not flags & other and flags & placeto.PLACETO_TCGEN05:
+        return flags, "fp32 accumulate on tcgen05.mma, TF32 head+tail operands (4 products per instruction)"
+    if d == 64 and not flags & other and flags & placeto.PLACETO_PIPELINE:
+        return flags, "fp32 accumulate on mma.sync, TF32 head+tail operands (3 products)"
+    states = -(-cfg["B"] // max(1, min(cfg["B"], SMS // 2)))
+    levels = max(info["n_levels_down"], info["n_levels_up"])
+    split = flags & placeto.PLACETO_TENSOR or (d == 64 or n * states >= 12 * levels and 2 * info["n_edges"] <= 7 * n)
+    if d in (32, 64) and not flags & other and split:
+        return flags | placeto.PLACETO_TENSOR, ("fp32 accumulate on mma.sync, operands as two scaled fp16 pieces (3 products)" if d == 64 else
+                                                "fp32 accumulate on mma.sync, operands as three bf16 pieces (6 products)")
+    return flags, "fp32 fma"
+
+
 def measure_workload(name: str, steps: int, warmup: int, flags: int, sm_count: int, peak_tflops: float):
     """Short measurement of one workload on the current device: whole path and
     the message-passing launch alone, L2 flushed before every timed call."""
@@ -312,10 +333,11 @@ def measure_workload(name: str, steps: int, warmup: int, flags: int, sm_count: i
 
     step_ms = timed(lambda: placeto.placeto_policy_forward(g, w, cost, nbytes, devs, cur, placed, logits, probs,
                                                            ws, flags, stream))
-    embed_ms = timed(lambda: placeto.placeto_embed_forward(g, w, X, Hd, Hu, ws, flags, stream))
+    sweep_flags, arithmetic = sweep_of_the_step(g, cfg, flags)
+    embed_ms = timed(lambda: placeto.placeto_embed_forward(g, w, X, Hd, Hu, ws, sweep_flags, stream))
     achieved = flops_embed(cfg) / (embed_ms * 1e-3) / 1e12
     out = {"n_nodes": n, "depth": cfg["depth"], "d": d, "states": B, "ms_per_step": step_ms,
-           "value": B / (step_ms * 1e-3), "embed_ms": embed_ms,
+           "value": B / (step_ms * 1e-3), "embed_ms": embed_ms, "embed_arithmetic": arithmetic,
            "roofline_frac": achieved / peak_tflops if d >= 32 else None}
     out.update(error_against_checker(cfg, logits, Hd, Hu))
     del out["reference"]
@@ -443,7 +465,8 @@ def run_b200(args):
     else:
         assert torch.equal(h_logits.cuda(), logits), "host and device entry points disagree"
 
-    # the dominant kernel alone: the message-passing launch(es) of embed_forward
+    # the dominant kernel alone: the message-passing launch(es) that the step runs
+    sweep_flags, arithmetic = sweep_of_the_step(g, cfg, args.flags)
     X = placeto.placeto_build_features(g, cost, nbytes, devs, cur, placed, m)
     Hd = torch.empty((n, B, d), dtype=torch.float32, device="cuda")
     Hu = torch.empty((n, B, d), dtype=torch.float32, device="cuda")
@@ -454,7 +477,7 @@ def run_b200(args):
         if args.rounds > 0:
             placeto.placeto_embed_rounds(g, w, X, args.rounds, Hd, Hu, ws_rounds, stream)
             return
-        placeto.placeto_embed_forward(g, w, X, Hd, Hu, ws, args.flags, stream)
+        placeto.placeto_embed_forward(g, w, X, Hd, Hu, ws, sweep_flags, stream)
 
     def pool_only():
         placeto.placeto_policy_logits(g, w, X, Hd, Hu, cur, logits, probs, ws, args.flags, stream)
@@ -490,10 +513,7 @@ def run_b200(args):
                            if args.rounds > 0 else "message passing (embed_forward, %d launch(es))" % embed_launches),
                 "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s", "frac": achieved / peak_tflops,
                 "traffic": traffic, "traffic_source": traffic_from,
-                "arithmetic": ("fp32 accumulate on tcgen05.mma, TF32 head+tail operands (4 products per instruction)"
-                               if d == 64 and (args.flags & 64) and not (args.flags & 24)
-                               else "fp32 accumulate on mma.sync, operands as two scaled fp16 pieces (3 products)"
-                               if d == 64 and not (args.flags & 24) else "fp32 fma"),
+                "arithmetic": arithmetic if args.rounds == 0 else "fp32 fma",
                 "algorithmic_bytes": (4 * F + 8 * d) * n * B,
                 "hbm": {"achieved": (4 * F + 8 * d) * n * B / (embed_ms * 1e-3) / 1e9, "peak": hbm_peak,
                         "unit": "GB/s", "frac": (4 * F + 8 * d) * n * B / (embed_ms * 1e-3) / 1e9 / hbm_peak,
