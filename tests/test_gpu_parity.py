@@ -261,6 +261,31 @@ def test_pipeline_kernel_on_a_deep_chain_and_a_wide_level():
     _small_case(53, src, dst, d=64, m=12, B=1480, seed=31, schedule=placeto.PLACETO_PIPELINE)
 
 
+@pytest.mark.parametrize("width,B,m", [(3, 592, 8), (5, 440, 3), (2, 1400, 4)])
+def test_pipeline_kernel_repeats_itself_with_every_ring_full(width, B, m):
+    """Levels of three and more tiles keep every slot of every ring in use: a slot written before its last reader is
+    through shows as runs that differ, or as rows far from the FMA kernel's."""
+    r = rng(width)
+    levels = 120
+    src = [(lv * width + a, (lv + 1) * width + b) for lv in range(levels - 1) for a in range(width) for b in {a, (a + 1) % width}]
+    src, dst = np.asarray(src, dtype=np.int32).T.copy()
+    n = levels * width
+    w = states.policy_weights(r, 64, m + 4, m, 2, 0, 0.1)
+    for way in ("down", "up"):
+        w["g_" + way]["W2"] *= 0.5
+    cost, size = states.node_costs(r, n, normalise=True)
+    devs, cur, placed = states.random_states(r, n, m, B)
+    g, wt = placeto.Graph(n, src, dst), placeto.Weights(w)
+    X = placeto.placeto_build_features(g, dev_t(cost), dev_t(size), dev_t(devs), dev_t(cur), dev_t(placed), m)
+    first = placeto.placeto_embed_forward(g, wt, X, flags=placeto.PLACETO_PIPELINE)
+    fma = placeto.placeto_embed_forward(g, wt, X, flags=placeto.PLACETO_FMA_ONLY)
+    for a, b in zip(first, fma):
+        assert_close(a, b.cpu().numpy(), "embeddings")
+    for _ in range(10):
+        again = placeto.placeto_embed_forward(g, wt, X, flags=placeto.PLACETO_PIPELINE)
+        assert torch.equal(again[0], first[0]) and torch.equal(again[1], first[1])
+
+
 def test_tcgen05_kernel_on_a_deep_chain_and_a_wide_level():
     n = 1500
     src = list(range(n - 1)) + list(range(0, n - 40, 37))
