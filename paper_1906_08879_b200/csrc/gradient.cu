@@ -793,6 +793,12 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
     a.pool_rows = a.DS[0];      // free until the sweep
     float *partial = p;
     const bool split = grad_split_applicable(a, di);
+    if (split) {
+        // One array holds the gradients of all three l_i, since a row belongs to one set, and d/d(sums) stays on chip: three of
+        // the arrays are the general kernels' alone. (The workspace is sized for either: which of them run depends on the graph.)
+        a.DPRE_L[1] = a.DPRE_L[2] = nullptr;
+        a.DS[1] = nullptr;
+    }
 
     cudaError_t err = cudaSuccess;
     if (!split) err = cudaMemsetAsync(a.DPRE_L[0], 0, 3 * ((R * d + 3) & ~size_t(3)) * sizeof(float), stream);
