@@ -18,7 +18,7 @@
 //     numbers a lane needs of a 16-wide step are adjacent (one 128-bit load, 64 contiguous bytes of a row per step).
 //   - The weights' pieces lie in shared memory as B fragments, split once per block; reading them costs
 //     half of what the instructions they feed take.
-// Warps never wait for one another; twelve or sixteen of them per SM cover the loads (d = 32: the tensor pipe is busy 58 %
+// Warps never wait for one another; twelve or sixteen of them per SM cover the loads (d = 32: the tensor pipe is busy 60 %
 // of the time. Reading a tile's rows during the tile before, at twelve or sixteen warps, takes registers from the
 // chains: 108 and 114 us instead of 106). Summation order is fixed, so results are reproducible bit for bit.
 #include <algorithm>
