@@ -121,6 +121,29 @@ typedef struct {
 placeto_status placeto_graph_host_view(const placeto_graph *g, placeto_level_view *down,
                                        placeto_level_view *up, const uint8_t **relation);
 
+/*
+ * Read-only HOST view of one direction's queues for `walkers` = 1, 2, 4 or 8 warps per state, valid until
+ * placeto_graph_destroy; meant for inspection and tests. Items are the nodes, queue by queue, each queue in the
+ * order in which its warp takes them.
+ *   ptr[walkers+1]        : each queue's items
+ *   node[n], own_slot[n]  : by item, the node and the message slot that it writes (-1: nobody reads it)
+ *   nbr_ptr[n+1], nbr[], nbr_slot[] : by item, the neighbours (ascending) and their slots
+ *   need[n*walkers], waits[n], publishes[n] : by item, how many items of each queue must be done before it (0: no
+ *                           matter, or implied by an earlier item of its queue); whether it has any such entry;
+ *                           whether it is the last one of another item's entry
+ *   key[n]                : by node, step << 16 | rank in an order that has every node behind its neighbours
+ *   first[n*walkers]      : by rank, the items of each queue that come before it in that order
+ */
+typedef struct {
+    int32_t walkers, n_steps, n_slots;
+    const int32_t *ptr, *node, *own_slot, *nbr_ptr, *nbr, *nbr_slot;
+    const uint16_t *need;
+    const uint8_t *waits, *publishes;
+    const int32_t *key;
+    const uint16_t *first;
+} placeto_queue_view;
+placeto_status placeto_graph_queue_view(const placeto_graph *g, int32_t dir, int32_t walkers, placeto_queue_view *view);
+
 /* Releases the plan (device memory is freed with the creating device current). NULL is a no-op. */
 void placeto_graph_destroy(placeto_graph *g);
 

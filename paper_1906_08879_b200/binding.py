@@ -28,7 +28,7 @@ CALL_EMBED, CALL_LOGITS, CALL_FORWARD, CALL_FORWARD_HOST, CALL_EPISODE, CALL_EMB
 
 EXPORTS = (
     "placeto_status_string", "placeto_graph_create", "placeto_graph_info",
-    "placeto_graph_host_view", "placeto_graph_destroy", "placeto_workspace_bytes",
+    "placeto_graph_host_view", "placeto_graph_queue_view", "placeto_graph_destroy", "placeto_workspace_bytes",
     "placeto_build_features", "placeto_embed_forward", "placeto_policy_logits",
     "placeto_policy_forward", "placeto_policy_forward_host", "placeto_policy_logits_static",
     "placeto_episode_rollout", "placeto_embed_rounds", "placeto_simulator_workspace_bytes", "placeto_simulate_runtime",
@@ -70,6 +70,14 @@ class _LevelView(ctypes.Structure):
                 ("nbr_slot", ctypes.POINTER(ctypes.c_int32))]
 
 
+class _QueueView(ctypes.Structure):
+    _fields_ = ([(k, ctypes.c_int32) for k in ("walkers", "n_steps", "n_slots")] +
+                [(k, ctypes.POINTER(ctypes.c_int32)) for k in ("ptr", "node", "own_slot", "nbr_ptr", "nbr", "nbr_slot")] +
+                [("need", ctypes.POINTER(ctypes.c_uint16)), ("waits", ctypes.POINTER(ctypes.c_uint8)),
+                 ("publishes", ctypes.POINTER(ctypes.c_uint8)), ("key", ctypes.POINTER(ctypes.c_int32)),
+                 ("first", ctypes.POINTER(ctypes.c_uint16))])
+
+
 def _load() -> ctypes.CDLL:
     if not os.path.exists(LIB_PATH):
         raise ImportError(
@@ -83,7 +91,7 @@ def _load() -> ctypes.CDLL:
     lib.placeto_workspace_bytes.restype = ctypes.c_size_t
     lib.placeto_last_launch_count.restype = ctypes.c_int32
     lib.placeto_simulator_workspace_bytes.restype = ctypes.c_size_t
-    for name in ("placeto_graph_create", "placeto_graph_info", "placeto_graph_host_view",
+    for name in ("placeto_graph_create", "placeto_graph_info", "placeto_graph_host_view", "placeto_graph_queue_view",
                  "placeto_build_features", "placeto_embed_forward", "placeto_policy_logits",
                  "placeto_policy_forward", "placeto_policy_forward_host",
                  "placeto_policy_logits_static", "placeto_episode_rollout", "placeto_embed_rounds", "placeto_simulate_runtime", "placeto_policy_gradient",
@@ -172,6 +180,19 @@ class Graph:
                              if nbr_ptr[-1] > 0 else np.zeros(0, np.int32)),
             }
         out["relation"] = np.ctypeslib.as_array(rel, shape=(n, n)).copy()
+        return out
+
+    def queue_view(self, direction: int, walkers: int) -> dict:
+        """Copies of one direction's queues for `walkers` warps per state (for inspection and tests)."""
+        v, n = _QueueView(), self.n
+        _check(_lib.placeto_graph_queue_view(self._h, ctypes.c_int32(direction), ctypes.c_int32(walkers), ctypes.byref(v)),
+               "placeto_graph_queue_view")
+        edges = v.nbr_ptr[n]
+        shapes = {"ptr": (walkers + 1,), "nbr_ptr": (n + 1,), "nbr": (edges,), "nbr_slot": (edges,), "need": (n, walkers), "first": (n, walkers)}
+        out = {"n_steps": v.n_steps, "n_slots": v.n_slots}
+        for k in ("ptr", "node", "own_slot", "nbr_ptr", "nbr", "nbr_slot", "need", "waits", "publishes", "key", "first"):
+            shape = shapes.get(k, (n,))
+            out[k] = np.ctypeslib.as_array(getattr(v, k), shape=shape).copy() if shape[0] else np.zeros(shape, np.int32)
         return out
 
     def close(self) -> None:

@@ -8,6 +8,7 @@
 #include <new>
 #include <vector>
 
+#include "embed_d32.cuh"
 #include "kernels.cuh"
 #include "plan.h"
 
@@ -18,12 +19,11 @@ struct placeto_graph {
     bool on_device = false;
     int device = -1;
     DeviceInfo info{};
-    int *d_ints = nullptr;       // one allocation for all int arrays
-    int4 *d_packed = nullptr;    // per direction lvl4[n_levels], pos4[n], row4[n] (see DevLevels)
-    int *d_child_ptr = nullptr, *d_child = nullptr, *d_child_entry = nullptr;   // inside d_ints
-    int *d_parent_ptr = nullptr, *d_parent = nullptr;                          // inside d_ints
-    uint8_t *d_relation = nullptr;
+    int4 *d_plan = nullptr;      // one allocation for all that follows
+    const int *d_child_ptr = nullptr, *d_child = nullptr, *d_child_entry = nullptr, *d_parent_ptr = nullptr, *d_parent = nullptr;
+    const uint8_t *d_relation = nullptr;
     DevLevels lv[2]{};
+    DevQueues queues[2][kQueuePlanCount]{};
     mutable std::atomic<int> calls{0};   // number of the latest forward call (see StatusSlot)
 };
 
@@ -84,7 +84,7 @@ struct Layout {
     size_t status;                 // 256 bytes at the start: the status word of the call
     size_t msg[2], msg_alt[2], partial, X, H[2], cost, bytes, dev, placed, cur, logits, probs, total;
     size_t grad, grad_extra;       // gradient call: its intermediates; identity layers of single-layer f, g
-    size_t compact;                // episode call: the compact states [n][E]
+    size_t compact, steps;         // episode call: the compact states [n][E], what the sweep of each step starts with
     int chunks, chunk_nodes;       // node chunks of the generic pooling kernel
     int chunks32, chunk_nodes32;   // and of the d = 32 / d = 64 kernel (0 when neither can apply)
     int chunks_split, chunk_nodes_split; // and of the tensor-core kernel of both (0 when it cannot apply or is not faster)
@@ -167,6 +167,7 @@ Layout make_layout(const placeto_graph *g, const placeto_weights *w, int B, plac
     }
     if (call == PLACETO_CALL_EPISODE) {
         L.compact = take(n * B);
+        L.steps = take(n * sizeof(int4));
         L.placed = take(n * B);
         L.cur = take((size_t)B * sizeof(int32_t));
         L.logits = take((size_t)B * m * sizeof(float));
@@ -201,6 +202,90 @@ const void *device_alias(const void *p) {
     return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
 
+// The device copy of a graph's plan: everything is laid out in one host array first, goes to one allocation with one copy (and
+// the relation, which need not be copied on the host, with another), and then the pointers are set.
+struct PlanUpload {
+    std::vector<int4> all;
+    std::vector<std::pair<const void **, size_t>> where;
+    static size_t quads(size_t bytes) { return (bytes + sizeof(int4) - 1) / sizeof(int4); }
+
+    template <typename T> void start(const T *&device) { where.push_back({reinterpret_cast<const void **>(&device), all.size()}); }
+    template <typename T> void put(const T *&device, const void *src, size_t bytes) {
+        start(device);
+        all.resize(all.size() + quads(bytes));
+        if (bytes > 0) std::memcpy(&all[where.back().second], src, bytes);
+    }
+    void put(const int *&device, const std::vector<int32_t> &v) { put(device, v.data(), v.size() * sizeof(int)); }
+};
+
+void put_levels(const HostPlan &host, int dir, DevLevels &d, PlanUpload &up) {
+    const LevelPlan &p = host.dir[dir];
+    d.n_levels = p.n_levels;
+    d.n_slots = p.n_slots;
+    d.n_nbr = static_cast<int>(p.nbr.size());
+    up.put(d.level_ptr, p.level_ptr);
+    up.put(d.order, p.order);
+    up.put(d.nbr_ptr, p.nbr_ptr);
+    up.put(d.nbr, p.nbr);
+    up.put(d.own_slot, p.own_slot);
+    up.put(d.nbr_slot, p.nbr_slot);
+    std::vector<int32_t> level_of(host.n);
+    for (int l = 0; l < p.n_levels; ++l)
+        for (int q = p.level_ptr[l]; q < p.level_ptr[l + 1]; ++q) level_of[p.order[q]] = l;
+    up.put(d.level_of, level_of);
+    // packed per-level and per-position records (kernels that stream the schedule)
+    up.start(d.lvl4);
+    d.max_level_nbr = 0;
+    for (int l = 0; l < p.n_levels; ++l) {
+        const int p0 = p.level_ptr[l], p1 = p.level_ptr[l + 1];
+        const int e0 = p.nbr_ptr[p0], e1 = p.nbr_ptr[p1];
+        up.all.push_back(make_int4(p0, p1 - p0, e0, e1 - e0));
+        d.max_level_nbr = std::max(d.max_level_nbr, e1 - e0);
+    }
+    up.start(d.pos4);
+    for (int q = 0; q < host.n; ++q) up.all.push_back(make_int4(p.nbr_ptr[q], p.nbr_ptr[q + 1], p.own_slot[q], p.order[q]));
+    up.start(d.row4);
+    for (int l = 0; l < p.n_levels; ++l)
+        for (int q = p.level_ptr[l]; q < p.level_ptr[l + 1]; ++q)
+            up.all.push_back(make_int4(p.order[q], p.level_ptr[l], p.level_ptr[l + 1] - p.level_ptr[l], 0));
+}
+
+void put_queues(const QueuePlan &q, int n, DevQueues &d, PlanUpload &up) {
+    const int4 last = make_int4(0, 0xffff, 0, kQueueEnd);
+    for (int w = 0; w <= 8; ++w) {
+        d.ptr[w] = q.ptr[std::min(w, q.walkers)];
+        d.entry_ptr[w] = q.entry_ptr[std::min(w, q.walkers)];
+    }
+    d.n_slots = q.n_slots;
+    d.n_steps = q.n_steps;
+    up.start(d.record);
+    const size_t start = up.all.size(), n_records = (size_t)n + kQueuePad * q.walkers;
+    std::vector<uint16_t> info(12, 0xffff);              // of an end: waits that never end, a group of slots
+    info.reserve(12 + 12 * (size_t)n + q.nbr.size());
+    for (int i = 0, w = 0; i < n; ++i) {
+        for (; i >= q.ptr[w + 1]; ++w) up.all.insert(up.all.end(), kQueuePad, last);
+        const int e0 = q.nbr_ptr[i], count = q.nbr_ptr[i + 1] - e0;
+        const bool plain = count == 1 && !q.waits[i] && !q.publishes[i] && q.own_slot[i] >= 0;
+        up.all.push_back(make_int4(q.node[i], (q.own_slot[i] & 0xffff) | (count > 0 ? q.nbr_slot[e0] << 16 : 0), (int)(info.size() / 4),
+                                   count | (q.publishes[i] ? kQueuePublishes : 0) | (plain ? kQueuePlain : 0)));
+        if (plain) continue;
+        const uint16_t *need = &q.need[(size_t)i * q.walkers];
+        for (int w8 = 0; w8 < 8; ++w8) info.push_back(w8 < q.walkers ? need[w8] : (uint16_t)0);
+        for (int e = e0; e < e0 + count; ++e) info.push_back((uint16_t)q.nbr_slot[e]);
+        for (int e = count; e == 0 || e % 4 != 0; ++e) info.push_back((uint16_t)q.n_slots);
+    }
+    up.all.resize(start + n_records, last);              // the ends of the queues left
+    up.all.resize(start + n_records + PlanUpload::quads(2 * info.size()));
+    std::memcpy(&up.all[start + n_records], info.data(), 2 * info.size());
+    d.n_quads = (int)(up.all.size() - start);
+    up.put(d.entry, q.nbr_ptr);
+    up.put(d.nbr, q.nbr);
+    up.put(d.nbr_slot, q.nbr_slot);
+    up.put(d.nbr_rank, q.nbr_rank);
+    up.put(d.key, q.key);
+    up.put(d.first, q.first.data(), 2 * q.first.size());
+}
+
 // The report slot of a new call on `g`: the record at the start of the workspace (or of the
 // built-in scratch) tagged with the call's number.
 StatusSlot new_status_slot(const placeto_graph *g, char *ws, const Layout &L) {
@@ -220,12 +305,13 @@ placeto_status run_embed(const placeto_graph *g, const placeto_weights *w, const
                          float *H_down, float *H_up, char *ws, const Layout &L, uint32_t flags,
                          cudaStream_t stream, const StatusSlot &status, bool after_own_kernel = false,
                          const CompactState *compact = nullptr, bool embeddings_returned = false,
-                         EpisodeWalk walk = EpisodeWalk{nullptr, 0}) {
+                         EpisodeWalk walk = EpisodeWalk{nullptr, 0, nullptr}) {
     EmbedArgs a;
     a.walk = walk;
     a.status = status;
     a.compact = compact ? *compact : CompactState{};
     a.lv[0] = g->lv[0]; a.lv[1] = g->lv[1];
+    a.queues = g->queues;
     a.f[0] = to_dev(w->f_down); a.f[1] = to_dev(w->f_up);
     a.g[0] = to_dev(w->g_down); a.g[1] = to_dev(w->g_up);
     a.X = X;
@@ -398,9 +484,7 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
     if (flags & PLACETO_GRAPH_HOST_ONLY) { *out = g; return PLACETO_OK; }
 
     auto fail = [&](placeto_status st) {
-        if (g->d_ints) cudaFree(g->d_ints);
-        if (g->d_packed) cudaFree(g->d_packed);
-        if (g->d_relation) cudaFree(g->d_relation);
+        if (g->d_plan) cudaFree(g->d_plan);
         delete g;
         return st;
     };
@@ -408,93 +492,26 @@ placeto_status placeto_graph_create(int32_t n, int64_t n_edges, const int32_t *s
     if (cudaDeviceGetAttribute(&g->info.sm_count, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&g->info.max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device) != cudaSuccess)
         return fail(PLACETO_ERR_CUDA);
-    // one int allocation: per direction level_ptr, order, nbr_ptr, nbr, own_slot, nbr_slot, level of a node
-    // (each padded to 4 ints)
-    constexpr int kArrays = 7;
-    std::vector<int32_t> level_of[2];
+    PlanUpload up;
+    static_assert(kQueuePlanCount == kQueuePlans, "one form on the device for each on the host");
     for (int dir = 0; dir < 2; ++dir) {
-        const LevelPlan &p = g->host.dir[dir];
-        level_of[dir].resize(g->host.n);
-        for (int l = 0; l < p.n_levels; ++l)
-            for (int q = p.level_ptr[l]; q < p.level_ptr[l + 1]; ++q) level_of[dir][p.order[q]] = l;
+        put_levels(g->host, dir, g->lv[dir], up);
+        for (int k = 0; k < kQueuePlanCount; ++k) put_queues(g->host.queues[dir][k], g->host.n, g->queues[dir][k], up);
     }
-    size_t total = 0;
-    size_t offs[2][kArrays];
-    for (int dir = 0; dir < 2; ++dir) {
-        const LevelPlan &p = g->host.dir[dir];
-        const size_t sizes[kArrays] = {p.level_ptr.size(), p.order.size(), p.nbr_ptr.size(),
-                                       p.nbr.size(), p.own_slot.size(), p.nbr_slot.size(), level_of[dir].size()};
-        for (int k = 0; k < kArrays; ++k) { offs[dir][k] = total; total += (sizes[k] + 3) & ~size_t(3); }
-    }
-    // and, by node id: children and their entries in the parent lists (runtime simulator), parents (policy gradient)
-    const std::vector<int32_t> *extra[5] = {&g->host.child_ptr, &g->host.child, &g->host.child_entry,
-                                            &g->host.parent_ptr, &g->host.parent};
-    size_t sim_off[5];
-    for (int k = 0; k < 5; ++k) { sim_off[k] = total; total += (extra[k]->size() + 3) & ~size_t(3); }
-    if (cudaMalloc(&g->d_ints, std::max<size_t>(total, 4) * sizeof(int)) != cudaSuccess)
-        return fail(PLACETO_ERR_NO_MEMORY);
-    if (cudaMalloc(&g->d_relation, g->host.relation.size()) != cudaSuccess)
-        return fail(PLACETO_ERR_NO_MEMORY);
-    std::vector<int32_t> ints(std::max<size_t>(total, 4));      // one upload for all of them
-    for (int dir = 0; dir < 2; ++dir) {
-        const LevelPlan &p = g->host.dir[dir];
-        const std::vector<int32_t> *vecs[kArrays] = {&p.level_ptr, &p.order, &p.nbr_ptr,
-                                                     &p.nbr, &p.own_slot, &p.nbr_slot, &level_of[dir]};
-        for (int k = 0; k < kArrays; ++k) std::copy(vecs[k]->begin(), vecs[k]->end(), ints.begin() + offs[dir][k]);
-        g->lv[dir].n_levels = p.n_levels;
-        g->lv[dir].level_ptr = g->d_ints + offs[dir][0];
-        g->lv[dir].order = g->d_ints + offs[dir][1];
-        g->lv[dir].nbr_ptr = g->d_ints + offs[dir][2];
-        g->lv[dir].nbr = g->d_ints + offs[dir][3];
-        g->lv[dir].n_slots = p.n_slots;
-        g->lv[dir].own_slot = g->d_ints + offs[dir][4];
-        g->lv[dir].nbr_slot = g->d_ints + offs[dir][5];
-        g->lv[dir].level_of = g->d_ints + offs[dir][6];
-        g->lv[dir].n_nbr = static_cast<int>(p.nbr.size());
-    }
-    {
-        int **dst[5] = {&g->d_child_ptr, &g->d_child, &g->d_child_entry, &g->d_parent_ptr, &g->d_parent};
-        for (int k = 0; k < 5; ++k) {
-            *dst[k] = g->d_ints + sim_off[k];
-            std::copy(extra[k]->begin(), extra[k]->end(), ints.begin() + sim_off[k]);
-        }
-    }
-    if (cudaMemcpy(g->d_ints, ints.data(), ints.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+    // by node id: children and their entries in the parent lists (runtime simulator), parents (policy gradient)
+    up.put(g->d_child_ptr, g->host.child_ptr);
+    up.put(g->d_child, g->host.child);
+    up.put(g->d_child_entry, g->host.child_entry);
+    up.put(g->d_parent_ptr, g->host.parent_ptr);
+    up.put(g->d_parent, g->host.parent);
+    const size_t bytes = up.all.size() * sizeof(int4);
+    if (cudaMalloc(&g->d_plan, bytes + g->host.relation.size()) != cudaSuccess) return fail(PLACETO_ERR_NO_MEMORY);
+    for (const auto &w : up.where) *w.first = g->d_plan + w.second;
+    uint8_t *relation = reinterpret_cast<uint8_t *>(g->d_plan) + bytes;
+    g->d_relation = relation;
+    if (cudaMemcpy(g->d_plan, up.all.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(relation, g->host.relation.data(), g->host.relation.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(PLACETO_ERR_CUDA);
-    if (cudaMemcpy(g->d_relation, g->host.relation.data(), g->host.relation.size(),
-                   cudaMemcpyHostToDevice) != cudaSuccess)
-        return fail(PLACETO_ERR_CUDA);
-    {   // packed per-level and per-position records (kernels that stream the schedule)
-        std::vector<int4> packed;
-        size_t at[2][3];
-        for (int dir = 0; dir < 2; ++dir) {
-            const LevelPlan &p = g->host.dir[dir];
-            at[dir][0] = packed.size();
-            int max_nbr = 0;
-            for (int l = 0; l < p.n_levels; ++l) {
-                const int p0 = p.level_ptr[l], p1 = p.level_ptr[l + 1];
-                const int e0 = p.nbr_ptr[p0], e1 = p.nbr_ptr[p1];
-                packed.push_back(make_int4(p0, p1 - p0, e0, e1 - e0));
-                max_nbr = std::max(max_nbr, e1 - e0);
-            }
-            at[dir][1] = packed.size();
-            for (int q = 0; q < g->host.n; ++q)
-                packed.push_back(make_int4(p.nbr_ptr[q], p.nbr_ptr[q + 1], p.own_slot[q], p.order[q]));
-            at[dir][2] = packed.size();
-            for (int l = 0; l < p.n_levels; ++l)
-                for (int q = p.level_ptr[l]; q < p.level_ptr[l + 1]; ++q)
-                    packed.push_back(make_int4(p.order[q], p.level_ptr[l], p.level_ptr[l + 1] - p.level_ptr[l], 0));
-            g->lv[dir].max_level_nbr = max_nbr;
-        }
-        if (cudaMalloc(&g->d_packed, packed.size() * sizeof(int4)) != cudaSuccess) return fail(PLACETO_ERR_NO_MEMORY);
-        if (cudaMemcpy(g->d_packed, packed.data(), packed.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess)
-            return fail(PLACETO_ERR_CUDA);
-        for (int dir = 0; dir < 2; ++dir) {
-            g->lv[dir].lvl4 = g->d_packed + at[dir][0];
-            g->lv[dir].pos4 = g->d_packed + at[dir][1];
-            g->lv[dir].row4 = g->d_packed + at[dir][2];
-        }
-    }
     g->on_device = true;
     *out = g;
     return PLACETO_OK;
@@ -532,15 +549,24 @@ placeto_status placeto_graph_host_view(const placeto_graph *g, placeto_level_vie
     return PLACETO_OK;
 }
 
+placeto_status placeto_graph_queue_view(const placeto_graph *g, int32_t dir, int32_t walkers, placeto_queue_view *view) {
+    if (!g || !view || (dir != 0 && dir != 1)) return PLACETO_ERR_INVALID_ARG;
+    for (const QueuePlan &q : g->host.queues[dir]) {
+        if (q.walkers != walkers) continue;
+        *view = {q.walkers, q.n_steps, q.n_slots, q.ptr.data(), q.node.data(), q.own_slot.data(), q.nbr_ptr.data(), q.nbr.data(),
+                 q.nbr_slot.data(), q.need.data(), q.waits.data(), q.publishes.data(), q.key.data(), q.first.data()};
+        return PLACETO_OK;
+    }
+    return PLACETO_ERR_INVALID_ARG;
+}
+
 void placeto_graph_destroy(placeto_graph *g) {
     if (!g) return;
     if (g->on_device) {
         int prev = -1;
         cudaGetDevice(&prev);
         if (prev != g->device) cudaSetDevice(g->device);
-        cudaFree(g->d_ints);
-        cudaFree(g->d_packed);
-        cudaFree(g->d_relation);
+        cudaFree(g->d_plan);
         if (prev != g->device && prev >= 0) cudaSetDevice(prev);
     }
     delete g;
@@ -762,8 +788,9 @@ placeto_status placeto_embed_rounds(const placeto_graph *g, const placeto_weight
     char *ws = static_cast<char *>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     EmbedArgs a;
-    a.walk = EpisodeWalk{nullptr, 0};
+    a.walk = EpisodeWalk{nullptr, 0, nullptr};
     a.lv[0] = g->lv[0]; a.lv[1] = g->lv[1];
+    a.queues = g->queues;
     a.f[0] = to_dev(w->f_down); a.f[1] = to_dev(w->f_up);
     a.g[0] = to_dev(w->g_down); a.g[1] = to_dev(w->g_up);
     a.X = X;
@@ -824,20 +851,25 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
     // and the fast head kernel), the episodes run without a feature tensor: one byte per (node,
     // episode) is the whole state, and the head kernel makes the transition itself.
     bool compact_path = false;
+    EmbedArgs ea;
+    ea.lv[0] = g->lv[0]; ea.lv[1] = g->lv[1];
+    ea.queues = g->queues;
+    ea.walk = EpisodeWalk{order, 0, nullptr};
+    ea.f[0] = to_dev(w->f_down); ea.f[1] = to_dev(w->f_up);
+    ea.g[0] = to_dev(w->g_down); ea.g[1] = to_dev(w->g_up);
+    ea.n = g->host.n; ea.B = E; ea.F = w->F; ea.d = w->d;
+    ea.max_level_width = g->host.max_level_width;
+    int4 *steps = reinterpret_cast<int4 *>(ws + L.steps);
+    D32Plan plan;
+    const bool d32 = embed_d32_plan(ea, g->info, &plan);
     if (!(flags & (PLACETO_GENERIC | PLACETO_TENSOR | PLACETO_PER_LEVEL | PLACETO_COOPERATIVE)) && w->m < 63 &&
         L.chunks32 > 0 && (w->F & 3) == 0) {
-        EmbedArgs ea;
-        ea.lv[0] = g->lv[0]; ea.lv[1] = g->lv[1];
-        ea.f[0] = to_dev(w->f_down); ea.f[1] = to_dev(w->f_up);
-        ea.g[0] = to_dev(w->g_down); ea.g[1] = to_dev(w->g_up);
-        ea.n = g->host.n; ea.B = E; ea.F = w->F; ea.d = w->d;
-        ea.max_level_width = g->host.max_level_width;
         PoolArgs pa;
         for (int i = 0; i < 3; ++i) { pa.l[i] = to_dev(w->l[i]); pa.h[i] = to_dev(w->h[i]); }
         pa.head = to_dev(w->head);
         pa.n = g->host.n; pa.B = E; pa.F = w->F; pa.d = w->d; pa.m = w->m;
         pa.chunks = L.chunks32; pa.chunk_nodes = L.chunk_nodes32;
-        compact_path = embed_d32_fits(ea, g->info) && pool_d32_fits(pa, g->info) && pool_head_takes_compact(pa);
+        compact_path = d32 && pool_d32_fits(pa, g->info) && pool_head_takes_compact(pa);
     }
     if (compact_path) {
         CompactState cs;
@@ -845,7 +877,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
         uint8_t *state = reinterpret_cast<uint8_t *>(ws + L.compact);
         cs.state = state;
         cs.cur = ep.cur;
-        s = cuda_status(launch_episode_begin_compact(ep.n, E, order, dev, state, ep.cur, st));
+        s = cuda_status(launch_episode_begin_compact(ep.n, E, order, dev, state, ep.cur, plan, steps, st));
         EpisodeStep step;
         step.enabled = 1; step.n = ep.n;
         step.order = order; step.uniforms = uniforms;
@@ -853,7 +885,7 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
         step.logp = logp; step.actions = actions;
         for (int t = 0; s == PLACETO_OK && t < ep.n; ++t) {
             step.t = t;
-            s = run_embed(g, w, nullptr, E, Hd, Hu, ws, L, flags, st, status, true, &cs, false, EpisodeWalk{order, t});
+            s = run_embed(g, w, nullptr, E, Hd, Hu, ws, L, flags, st, status, true, &cs, false, EpisodeWalk{order, t, steps});
             if (s == PLACETO_OK)
                 s = run_pool(g, w, nullptr, Hd, Hu, ep.cur, E, const_cast<float *>(ep.logits), probs, ws, L, flags, st,
                              status, true, &cs, &step);
@@ -861,13 +893,13 @@ placeto_status placeto_episode_rollout(const placeto_graph *g, const placeto_wei
         if (s == PLACETO_OK) s = cuda_status(launch_episode_end_compact(ep.n, E, state, dev, st));
         return s;
     }
-    s = cuda_status(launch_episode_begin(ep, st));
+    s = cuda_status(launch_episode_begin(ep, d32 ? &plan : nullptr, steps, st));
     // the features of the initial states; every later step patches them in place
     if (s == PLACETO_OK)
         s = cuda_status(launch_features(ep.n, E, w->m, cost, bytes, dev, ep.cur, ep.placed, X, st));
     for (int t = 0; s == PLACETO_OK && t < ep.n; ++t) {
         // one policy evaluation of the E current states, then the transition
-        s = run_embed(g, w, X, E, Hd, Hu, ws, L, flags, st, status, true, nullptr, false, EpisodeWalk{order, t});
+        s = run_embed(g, w, X, E, Hd, Hu, ws, L, flags, st, status, true, nullptr, false, EpisodeWalk{order, t, steps});
         if (s == PLACETO_OK)
             s = run_pool(g, w, X, Hd, Hu, ep.cur, E, const_cast<float *>(ep.logits), probs, ws, L, flags, st, status, true);
         if (s == PLACETO_OK) s = cuda_status(launch_episode_step(ep, t, st));

@@ -3,49 +3,45 @@
 // or two layers of hidden width 32:
 //   h_v = g( sum_{u in nbr(v)} m_u ),   m_u = f([h_u || x_u]).
 //
-// Design (one block = one direction x one slice of the state batch, walking all
-// levels with __syncthreads() between levels; states never interact):
+// Design (a block = one direction and a few states of the batch; states never interact):
 //   - Lane j of every warp keeps column j of all four weight matrices of the
 //     direction in registers (32 + 32 + (32 + F) + 32 values), so a warp carries
 //     a row (node, state) through gather -> g1 -> g2 -> f1 -> f2 on its own. With
-//     single-layer networks the second layers drop out at compile time: half
-//     the dependent chain of a level (whole path on a 279-node graph, 132 levels, 250
-//     states, two devices, B200: 90 us; 618 us on the dimension-generic kernels).
+//     single-layer networks the second layers drop out at compile time.
 //     Between layers the 32 outputs are exchanged through a per-warp shared
 //     buffer and read back as broadcast 128-bit loads: 4 FMAs per shared load,
 //     issued as two packed fma.rn.f32x2 against weights kept in register pairs.
-//   - Two states of a node are in flight per warp (one on narrow levels), with
-//     four dependent accumulator chains per row.
-//   - Messages never leave the SM: m_u lives in a shared-memory slot from the
-//     level of u until its last consumer's level (slots assigned on the host).
-//     Global traffic is the compulsory part only: read x, write h.
-//   - The level schedule (order, CSR, slots) is staged in shared memory, and the
-//     raw features of the next level are copied asynchronously (cp.async) into a
-//     staging area of two or three levels while the current level computes, so no DRAM
-//     latency sits on the level-to-level critical path.
-#include <cuda_pipeline.h>
-
+//   - No levels: 1, 2, 4 or 8 warps share a state, and each of them takes the nodes of its
+//     queue in order (QueuePlan in plan.h). A warp waits only where a message comes
+//     from another queue, for the count of items that the other warp has done; the
+//     links of a chain stay in one queue, where nothing separates them.
+//   - Messages never leave the SM: m_u lives in a shared-memory slot until its last reader
+//     (slots assigned on the host). Global traffic is the compulsory part only: read x, write h.
+//   - The queues lie in shared memory; raw features are copied asynchronously (cp.async) into a ring of the
+//     warp's own, two items ahead. (Requested into registers instead, a load shares one of a warp's few
+//     scoreboards with the shared-memory loads of the products, whose wait then is the load's: 100 cycles each.)
+//   - An item with one neighbour, in the same queue, whose message others read and nobody waits for
+//     (most links of a chain) has a loop body without a branch; each of the general body's questions costs 50
+//     cycles and more of the 475 that four layers take.
+//   - Four dependent accumulator chains per row; sums are added up in the same order in all forms.
+//
+// What bounds it is the chain of dependent layers of an item (B200, a chain of 400 nodes, one state: 590 cycles a node with
+// two layers, 390 with one; 845 and 670 with a block barrier per level). 279 nodes in 132 levels, two layers: one state
+// 58 -> 42 us, 256 states 96 -> 77; 1080 nodes of four neighbours, 256 states: 307 -> 262.
 #include <algorithm>
+#include <climits>
+#include <type_traits>
 
-#include "kernels.cuh"
+#include "embed_d32.cuh"
 
 namespace placeto {
 
 namespace {
 
 constexpr int kD = 32;
-constexpr int kWarps = 8;
-// With single-layer networks a level is short: a ninth warp brings the raw features, two levels ahead (279 nodes, 250 states:
-// 80 -> 68 us). With two layers, where the registers are full and the features come in time, either costs 3 %.
-template <int L> constexpr int kStages = L == 1 ? 3 : 2;            // levels of raw features on chip
-template <int L> constexpr int kThreads = (kWarps + (L == 1)) * 32;
-
-struct D32Plan {
-    int S;          // states per slice
-    int n_slices;
-    int x_floats;   // floats of one feature staging buffer (widest level x S x F, padded)
-    size_t smem_bytes;
-};
+constexpr int kLogWarps = 3, kWarps = 1 << kLogWarps, kThreads = kWarps * 32;
+constexpr int kFeatures = 4;             // items whose raw features are on chip
+constexpr int kMaxPolls = 1 << 22;       // of a wait for another warp, which in a valid plan always ends
 
 typedef unsigned long long pair_t;   // two FP32 values in one 64-bit register pair
 
@@ -64,27 +60,27 @@ __device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ pair_t mul2(pair_t a, pair_t b) {
+    pair_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 
 // out[r] = bias + in[r] . w for R rows whose K inputs are read as broadcast
 // 128-bit loads from shared memory. The weights are kept as pairs (w[2i],
 // w[2i + 1]) so that every load feeds two packed FMAs; two pair accumulators per
-// row, i.e. four dependent chains of K / 4 FMAs.
+// row, i.e. four dependent chains of K / 4 FMAs. bias: {bias, 0}.
 template <int R, int K>
-__device__ __forceinline__ void matvec(const pair_t (&w)[K / 2], float bias, const float *in,
+__device__ __forceinline__ void matvec(const pair_t (&w)[K / 2], const pair_t (&bias)[1], const float *in,
                                        int row_stride, float (&out)[R]) {
     pair_t acc[R][2];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        acc[r][0] = pack2(bias, 0.f);
-        acc[r][1] = 0ull;
-    }
 #pragma unroll
     for (int k = 0; k < K; k += 4) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(in + r * row_stride + k);
-            acc[r][0] = fma2(u.x, w[k / 2], acc[r][0]);
-            acc[r][1] = fma2(u.y, w[k / 2 + 1], acc[r][1]);
+            acc[r][0] = fma2(u.x, w[k / 2], k == 0 ? bias[0] : acc[r][0]);
+            acc[r][1] = k == 0 ? mul2(u.y, w[1]) : fma2(u.y, w[k / 2 + 1], acc[r][1]);
         }
     }
 #pragma unroll
@@ -96,270 +92,388 @@ __device__ __forceinline__ void matvec(const pair_t (&w)[K / 2], float bias, con
     }
 }
 
-struct Weights32 {
-    pair_t g1[kD / 2], g2[kD / 2], f2[kD / 2];   // column `lane`, rows in pairs
-    float bg1, bg2, bf1, bf2;
-};
-
-// Carries R states (s0 .. s0 + R - 1 of the slice; the last may be missing and
-// then repeats s0) of the node at position `pos` through
-// gather -> g -> store h -> f -> store m. The R rows share the node, so the
-// schedule lookups are done once. A, Bf: the warp's exchange buffers, R rows of
-// KF floats each. All shared-memory offsets are 32-bit.
-template <int R, int KF, int L, bool kWalk>   // L layers per network; kWalk: messages also go to memory
-__device__ __forceinline__ void run_node(const Weights32 &w, const pair_t (&wf1)[KF / 2], int pos,
-                                         int q, int s0, bool last_live, int nb, int S, int F,
-                                         int lane, const int4 *meta, const int *nbr_slot,
-                                         float *msg, const float *xs, float *__restrict__ H,
-                                         float *__restrict__ M, size_t B, int b_first, float *A, float *Bf) {
-    int st[R];
-    float x[R], acc[R];
+// The same product with half of the inner dimension and two columns per lane: lane (h, c) keeps columns 2c and 2c + 1
+// of the rows k with (k >> 1 & 1) == h, whose inputs lie together in the buffer (position() below), so that a 128-bit load feeds
+// twice as many FMAs. The halves are the chains of the form above: one exchange gives column 2c + h the same sum, bit for bit.
+template <int R, int K>
+__device__ __forceinline__ void matvec_halves(const pair_t (&w)[K / 2], const pair_t (&bias)[2], const float *in, int row_stride,
+                                              int lane, float (&out)[R]) {
+    const int h = lane >> 4;
+    const float *mine = in + h * (K / 2);
+    pair_t acc[R][2];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        st[r] = (r == 0 || last_live) ? s0 + r : s0;
-        x[r] = lane < F ? xs[(q * nb + st[r]) * F + lane] : 0.f;
-        acc[r] = 0.f;
-    }
-    const int4 m = meta[pos];       // {first neighbour entry, end, own | first neighbour slot, node}
-    const int e1 = m.y, v = m.w;
-    const int slot = (m.z & 0xffff) == 0xffff ? -1 : (m.z & 0xffff);
-    int e = m.x;
-    if (e1 - e == 1) {
-        // One neighbour (most nodes of chain-like graphs): its message row is the
-        // input of g as it stands, so the first layer reads the slot directly and
-        // the gather, the store and the warp barrier are skipped.
-        const float *row = msg + ((int)((unsigned)m.z >> 16) * S + st[0]) * kD;
-        matvec<R, kD>(w.g1, w.bg1, row, (R > 1 && last_live) ? kD : 0, acc);
-        __syncwarp();               // the previous node's last reads of Bf are done
-        goto after_g1;
-    }
-    for (; e + 4 <= e1; e += 4) {   // four neighbours at a time: the loads overlap
-        int base[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) base[k] = nbr_slot[e + k] * S;
+    for (int k = 0; k < K / 2; k += 4) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            float t[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) t[k] = msg[(base[k] + st[r]) * kD + lane];
-            acc[r] += (t[0] + t[1]) + (t[2] + t[3]);
+            const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(mine + r * row_stride + k);
+            acc[r][0] = fma2(u.x, w[k / 2], k == 0 ? bias[0] : acc[r][0]);
+            acc[r][1] = fma2(u.x, w[K / 4 + k / 2], k == 0 ? bias[1] : acc[r][1]);
+            acc[r][0] = fma2(u.y, w[k / 2 + 1], acc[r][0]);
+            acc[r][1] = fma2(u.y, w[K / 4 + k / 2 + 1], acc[r][1]);
         }
     }
-    if (e < e1) {                   // the last one to three likewise (151 nodes with 267 edges: 0.60 -> 0.54 us a level)
-        int base[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) base[k] = nbr_slot[min(e + k, e1 - 1)] * S;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float t[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) t[k] = msg[(base[k] + st[r]) * kD + lane];
-            acc[r] += t[0];
-            if (e + 1 < e1) acc[r] += t[1];
-            if (e + 2 < e1) acc[r] += t[2];
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) A[r * KF + lane] = acc[r];
-    __syncwarp();
-    matvec<R, kD>(w.g1, w.bg1, A, KF, acc);
-after_g1:
-    if constexpr (L == 2) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
-        __syncwarp();
-        matvec<R, kD>(w.g2, w.bg2, Bf, KF, acc);
-    }
-    float *hrow = H + ((size_t)v * B + b_first + s0) * kD + lane;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        acc[r] = fmaxf(acc[r], 0.f);
-        if (r == 0 || last_live) hrow[r * kD] = acc[r];
+        float a, b, c, d;
+        unpack2(acc[r][0], a, b);
+        unpack2(acc[r][1], c, d);
+        a += b;
+        c += d;
+        out[r] = (h ? c : a) + __shfl_xor_sync(0xffffffffu, h ? a : c, 16);
     }
-    if (slot < 0) {                         // nobody consumes this node's message
-        if constexpr (L == 1) __syncwarp();     // the next node writes A, which the only product may still be reading
-        return;
-    }
-    float *in = L == 2 ? A : Bf;            // the buffer that the last product did not read
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        in[r * KF + lane] = acc[r];
-        if (lane < KF - kD) in[r * KF + kD + lane] = x[r];
-    }
-    __syncwarp();
-    matvec<R, KF>(wf1, w.bf1, in, KF, acc);
-    if constexpr (L == 2) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
-        __syncwarp();
-        matvec<R, kD>(w.f2, w.bf2, Bf, KF, acc);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (r == 0 || last_live) {
-            const float v_m = fmaxf(acc[r], 0.f);
-            msg[((slot * S) + st[r]) * kD + lane] = v_m;
-            if constexpr (kWalk) M[((size_t)v * B + b_first + s0 + r) * kD + lane] = v_m;
-        }
 }
 
-// feature width padded to 4 * F4; features built from compact states; layers; a sweep of an episode
-template <int F4, bool kCompact, int L, bool kWalk>
-__global__ void __launch_bounds__(kThreads<L>, 1)
-embed_d32_kernel(const EmbedArgs a, const D32Plan p) {
-    constexpr int KF = kD + 4 * F4;      // padded input width of f's first layer
-    extern __shared__ __align__(16) float smem[];
-    dependents_may_start();
-    const int dir = blockIdx.y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const DevLevels lv = a.lv[dir];
-    const int B = a.B, F = a.F;
-    const int b_first = blockIdx.x * p.S;
-    const int nb = min(p.S, B - b_first);
-
-    // ---- shared memory: [schedule ints][message slots][feature staging x2 or x3][exchange buffers]
-    // one packed record per position: {first neighbour entry, end,
-    // own slot (low 16 bits, 0xffff = none) | slot of the first neighbour (high 16 bits), node id}
-    int4 *meta_w = reinterpret_cast<int4 *>(smem);
-    for (int i = threadIdx.x; i < a.n; i += kThreads<L>) {
-        const int e0 = lv.nbr_ptr[i], e1 = lv.nbr_ptr[i + 1];
-        const int first = e1 > e0 ? lv.nbr_slot[e0] : 0;
-        meta_w[i] = make_int4(e0, e1, (lv.own_slot[i] & 0xffff) | (first << 16), lv.order[i]);
-        PLACETO_DEBUG_CHECK(a.status, e0 >= 0 && e0 <= e1 && e1 <= lv.n_nbr && lv.own_slot[i] >= -1 &&
-                                          lv.own_slot[i] < lv.n_slots && lv.order[i] >= 0 && lv.order[i] < a.n);
+// How a warp lays out a row: which column a lane owns, where input k of a K-wide product lies. One state per warp takes whole
+// columns (the exchange would lie on the chain of layers: 95 -> 97 us with one state), two take halves (the shared loads).
+template <bool kHalves> struct Layout32 {
+    typedef pair_t Bias[kHalves ? 2 : 1];       // the first addends of a lane's chains
+    static __device__ __forceinline__ int column(int lane) { return kHalves ? 2 * (lane & 15) + (lane >> 4) : lane; }
+    template <int K> static __device__ __forceinline__ int position(int k) {
+        return kHalves ? (k >> 1 & 1) * (K / 2) + (k >> 2) * 2 + (k & 1) : k;
     }
-    for (int e = threadIdx.x; e < lv.n_nbr; e += kThreads<L>)
-        PLACETO_DEBUG_CHECK(a.status, lv.nbr_slot[e] >= 0 && lv.nbr_slot[e] < lv.n_slots);
-    PLACETO_DEBUG_CHECK(a.status, nb >= 1 && b_first + nb <= B);
-    const int4 *meta = meta_w;
-    int *ism = reinterpret_cast<int *>(smem) + 4 * a.n;
-    auto stage = [&](const int *src, int count) {
-        int *dst = ism;
-        for (int i = threadIdx.x; i < count; i += kThreads<L>) dst[i] = src[i];
-        ism += (count + 3) & ~3;
-        return (const int *)dst;
-    };
-    const int *level_ptr = stage(lv.level_ptr, lv.n_levels + 1);
-    const int *nbr_slot = stage(lv.nbr_slot, lv.n_nbr);
-    float *fsm = reinterpret_cast<float *>(ism);
-    float *msg = fsm;                                       // [n_slots][S][32]
-    float *xstage = msg + (size_t)lv.n_slots * p.S * kD;    // [kStages][x_floats]
-    float *xbuf = xstage + kStages<L> * (size_t)p.x_floats + (size_t)(L == 1 ? min(warp, kWarps - 1) : warp) * 4 * KF;
-    float *A = xbuf, *Bf = xbuf + 2 * KF;
+    // this lane's part of W [K rows, those from `rows` on zero][32]
+    template <int K> static __device__ __forceinline__ void load(pair_t (&w)[K / 2], const float *W, int rows, int lane) {
+        auto at = [&](int k, int col) { return k < rows ? W[k * kD + col] : 0.f; };
+        if constexpr (kHalves) {
+            const int h = lane >> 4, c = lane & 15;
+#pragma unroll
+            for (int i = 0; i < K / 4; ++i) {
+                w[i] = pack2(at(4 * i + 2 * h, 2 * c), at(4 * i + 2 * h + 1, 2 * c));
+                w[K / 4 + i] = pack2(at(4 * i + 2 * h, 2 * c + 1), at(4 * i + 2 * h + 1, 2 * c + 1));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; k += 2) w[k / 2] = pack2(at(k, lane), at(k + 1, lane));
+        }
+    }
+    static __device__ __forceinline__ void load_bias(Bias &b, const float *bias, int lane) {
+        if constexpr (kHalves) {
+            b[0] = pack2(lane < 16 ? bias[2 * (lane & 15)] : 0.f, 0.f);
+            b[1] = pack2(lane < 16 ? bias[2 * (lane & 15) + 1] : 0.f, 0.f);
+        } else {
+            b[0] = pack2(bias[lane], 0.f);
+        }
+    }
+    template <int R, int K>
+    static __device__ __forceinline__ void product(const pair_t (&w)[K / 2], const Bias &bias, const float *in, int stride, int lane,
+                                                   float (&out)[R]) {
+        if constexpr (kHalves) matvec_halves<R, K>(w, bias, in, stride, lane, out);
+        else matvec<R, K>(w, bias, in, stride, out);
+    }
+};
+
+__device__ __forceinline__ void copy4(unsigned dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_end_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// p + v * stride, the product of two 32-bit numbers in 64 bits
+template <typename T> __device__ __forceinline__ T *row_of(T *p, int v, unsigned stride_bytes) {
+    return reinterpret_cast<T *>(reinterpret_cast<uintptr_t>(p) + (unsigned long long)(unsigned)v * stride_bytes);
+}
+
+__device__ __forceinline__ int load_acquire(const int *p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_addr(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_release_if(bool on, int *p, int v) {       // without a branch
+    asm volatile("{\n.reg .pred p;\nsetp.ne.s32 p, %2, 0;\n@p st.release.cta.shared.b32 [%0], %1;\n}" ::"r"(smem_addr(p)), "r"(v), "r"((int)on) : "memory");
+}
+
+// Floats of a warp's buffers: two rows per state between the products, the ring of raw features (a word per lane)
+__device__ __host__ constexpr int warp_floats(int R) { return 2 * R * (kD + 16) + kFeatures * 32; }
+
+// F4: raw features, in groups of four; kSource: 0 features from X, 1 the same in a step of an episode, 2 an episode's compact
+// states; L layers per network; R states of a node that a warp carries together
+template <int F4, int kSource, int L, int R>
+__global__ void __launch_bounds__(kThreads, 1)
+embed_d32_kernel(const EmbedArgs a, const __grid_constant__ D32Plan p) {
+    constexpr bool kWalk = kSource > 0, kCompact = kSource == 2, kHalves = R == 2;
+    constexpr int KF = kHalves ? kD + 8 * ((F4 + 1) / 2) : kD + 4 * F4;      // padded input width of f's first layer
+    typedef Layout32<kHalves> Rows;
+    extern __shared__ __align__(16) float smem[];
+    __shared__ int progress[kWarps];                    // items that a warp has done, as far as others have to know
+    dependents_may_start();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int B = a.B;
+
+    // ---- this block's direction, its warps per state, and where the sweep starts
+    int dir, k, nb, rank = 0;
+    if (kWalk && a.walk.t > 0) {         // (the kernel that wrote the starts may still be running in step 0)
+        const int4 step = a.walk.steps[a.walk.t];
+        dir = (int)blockIdx.x >= step.x;
+        nb = dir ? gridDim.x - step.x : step.x;
+        k = (dir ? step.z : step.y) >> 16;
+        rank = (dir ? step.z : step.y) & 0xffff;
+    } else {
+        nb = gridDim.x / 2;
+        dir = (int)blockIdx.x >= nb;
+        k = p.form;
+    }
+    const DevQueues &q = p.q[dir][k];
+    // the first queues of all teams come first: a block's warps are dealt to the schedulers in turn
+    const int W = 1 << k, me = warp >> (kLogWarps - k), team = warp & ((kWarps >> k) - 1), teams = p.teams[k];
+    const int block = (int)blockIdx.x - (dir ? (int)gridDim.x - nb : 0);
+    const int g0 = (int)((long long)p.groups * block / nb) + team, g1 = (int)((long long)p.groups * (block + 1) / nb);
+    const int end = q.ptr[me + 1] - q.ptr[me];
+    const int first = kWalk && rank > 0 ? (int)q.first[rank * W + me] : 0;
+    const unsigned h_stride = (unsigned)B * kD * sizeof(float);
+    const bool busy = team < teams && g0 < g1;
+
+    // ---- shared memory: [records][waits and neighbours][message slots of every team, and one of zeros][buffers of every warp]
+    int4 *const records = reinterpret_cast<int4 *>(smem);
+    for (int i = threadIdx.x; i < q.n_quads; i += kThreads) records[i] = q.record[i];
+    const int4 *const queue = records + q.ptr[me] + me * kQueuePad;
+    const uint2 *const info = reinterpret_cast<const uint2 *>(records + a.n + W * kQueuePad);
+    float *const slots = smem + 4 * q.n_quads;
+    const int row = (q.n_slots + 1) * kD;                // floats of a state's slots
+    float *const msg = slots + (size_t)team * R * row;
+    float *const A = slots + (size_t)teams * R * row + warp * warp_floats(R), *const Bf = A + R * KF;
+    const float *const xring = A + 2 * R * (kD + 16);    // [kFeatures][32]
+    if (me == 0 && team < teams)
+        for (int r = 0; r < R; ++r) msg[r * row + q.n_slots * kD + lane] = 0.f;
+    const int col = Rows::column(lane), at32 = Rows::template position<kD>(col), at_h = Rows::template position<KF>(col);
+    const int at_x = Rows::template position<KF>(min(kD + lane, KF - 1));
 
     // ---- this lane's weight columns
     const DevMlp f = a.f[dir], g = a.g[dir];
-    Weights32 w;
-    pair_t wf1[KF / 2];
-#pragma unroll
-    for (int k = 0; k < kD; k += 2) {
-        w.g1[k / 2] = pack2(g.W1[k * kD + lane], g.W1[(k + 1) * kD + lane]);
-        if constexpr (L == 2) {
-            w.g2[k / 2] = pack2(g.W2[k * kD + lane], g.W2[(k + 1) * kD + lane]);
-            w.f2[k / 2] = pack2(f.W2[k * kD + lane], f.W2[(k + 1) * kD + lane]);
-        }
+    pair_t wg1[kD / 2], wg2[L == 2 ? kD / 2 : 1], wf1[KF / 2], wf2[L == 2 ? kD / 2 : 1];
+    typename Rows::Bias bg1, bg2, bf1, bf2;
+    Rows::template load<kD>(wg1, g.W1, kD, lane);
+    Rows::template load<KF>(wf1, f.W1, kD + a.F, lane);
+    Rows::load_bias(bg1, g.b1, lane);
+    Rows::load_bias(bf1, f.b1, lane);
+    if constexpr (L == 2) {
+        Rows::template load<kD>(wg2, g.W2, kD, lane);
+        Rows::template load<kD>(wf2, f.W2, kD, lane);
+        Rows::load_bias(bg2, g.b2, lane);
+        Rows::load_bias(bf2, f.b2, lane);
     }
-#pragma unroll
-    for (int k = 0; k < KF; k += 2)
-        wf1[k / 2] = pack2(k < kD + F ? f.W1[k * kD + lane] : 0.f,
-                           k + 1 < kD + F ? f.W1[(k + 1) * kD + lane] : 0.f);
-    w.bg1 = g.b1[lane]; w.bf1 = f.b1[lane];
-    if constexpr (L == 2) { w.bg2 = g.b2[lane]; w.bf2 = f.b2[lane]; }
-    const float *__restrict__ X = a.X;
     float *__restrict__ H = a.H[dir];
-    __syncthreads();
+    float *__restrict__ M = a.M[dir];
+    if (lane == 0) progress[warp] = first;
+    const int *const others = &progress[team + (min(lane & 7, W - 1) << (kLogWarps - k))];
+    // the entries of this queue from `first` on: the first 32 are looked at while the kernel before may still be running
+    const int entry_end = q.entry_ptr[me + 1];
+    int carry = kWalk && rank > 0 && busy && first < end ? q.entry[q.ptr[me] + first] : entry_end;
+    int carry_node = 0, carry_slot = 0, carry_rank = INT_MAX;
+    auto look = [&]() {
+        const bool in = carry + lane < entry_end;
+        carry_node = in ? q.nbr[carry + lane] : 0;
+        carry_slot = in ? q.nbr_slot[carry + lane] : 0;
+        carry_rank = in ? q.nbr_rank[carry + lane] : INT_MAX;
+    };
+    if constexpr (kWalk) look();
+    const int carry_first = carry;
+    __syncthreads();             // the queues, the zeros and the counts are there
+    if (!busy) return;
+#ifdef PLACETO_DEBUG
+    for (int i = lane; i < end; i += 32) {
+        const int4 r = queue[i];
+        PLACETO_DEBUG_CHECK(a.status, r.x >= 0 && r.x < a.n && ((r.y & 0xffff) == 0xffff || (r.y & 0xffff) < q.n_slots) &&
+                                          ((unsigned)r.y >> 16) <= (unsigned)q.n_slots && 2 * (a.n + W * kQueuePad) + r.z + 3 <= 2 * q.n_quads);
+    }
+    PLACETO_DEBUG_CHECK(a.status, g0 >= 0 && g1 <= p.groups && queue[end].w == kQueueEnd);
+#endif
+    dependency_wait();          // the raw features may come from a kernel that is still running
 
-    // Asynchronous copy of one level's raw features (rows of the slice) into a
-    // staging buffer, so that the next level's x is on chip when it is needed.
-    // exact division of small non-negative numbers by a per-block constant
-    auto magic_of = [](int d) { return (unsigned)((0x100000000ull + d - 1) / d); };
-    const unsigned magic_nb = magic_of(nb), magic_ppn = magic_of((nb + 1) >> 1);
-    const int per_node = nb * F;             // floats per node, contiguous in X
-    const bool vec = (F & 3) == 0;
-    const int per = vec ? per_node >> 2 : per_node;     // copy pieces per node
-    const unsigned magic_per = magic_of(per);
-    // The last warp (the one least often needed for rows) issues all copies, so
-    // the other warps go straight to their rows.
-    auto prefetch = [&](int level) {
-        if (warp != (L == 1 ? kWarps : kWarps - 1)) return;
-        const int q0 = level_ptr[level], width = level_ptr[level + 1] - q0;
-        float *dst = xstage + (size_t)(L == 1 ? level % 3 : level & 1) * p.x_floats;
-        if (kCompact) {
-            // no X tensor: the level's features from one byte per (node, state)
-            for (int i = lane; i < width * nb; i += 32) {       // one (node, state) pair per lane
-                const int q = nb == 1 ? i : (int)__umulhi((unsigned)i, magic_nb), s = i - q * nb;
-                compact_features(a.compact, meta[q0 + q].w, b_first + s, (int)B, dst + (size_t)i * F);
+#pragma unroll 1
+    for (int group = g0; group < g1; group += teams) {
+        int b[R];                // the states; a missing last one repeats the first
+#pragma unroll
+        for (int r = 0; r < R; ++r) b[r] = r == 0 || group * R + r < B ? group * R + r : group * R;
+        const bool last_live = R == 1 || b[R - 1] != b[0];
+        int current[R];
+        if constexpr (kCompact) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) current[r] = a.compact.cur[b[r]];
+        }
+        // What each lane copies for an item: a word of its raw features, or of the operation's time and size and the aligned
+        // words around the states' bytes (lanes beyond repeat another's).
+        const char *x_src;
+        unsigned x_stride;               // bytes between nodes
+        int byte_at[R] = {};             // of node 0's state byte in its word
+        if constexpr (kCompact) {
+            x_src = lane == 0 ? reinterpret_cast<const char *>(a.compact.cost)
+                  : lane == 1 ? reinterpret_cast<const char *>(a.compact.bytes)
+                              : reinterpret_cast<const char *>(a.compact.state) + b[lane == 3 ? R - 1 : 0];
+            x_stride = lane < 2 ? 4 : B;
+#pragma unroll
+            for (int i = 0; i < R; ++i) byte_at[i] = (int)(reinterpret_cast<uintptr_t>(a.compact.state + b[i]) & 3);
+        } else {
+            x_src = reinterpret_cast<const char *>(a.X + (size_t)b[lane >= 16 ? R - 1 : 0] * a.F + min(lane & 15, a.F - 1));
+            x_stride = (unsigned)B * a.F * sizeof(float);
+        }
+        const unsigned x_dst = smem_addr(xring + lane);
+        auto copy_features = [&](int i, int node) {
+            const char *src = row_of(x_src, node, x_stride);
+            if (kCompact) src = reinterpret_cast<const char *>(reinterpret_cast<uintptr_t>(src) & ~uintptr_t(3));
+            copy4(x_dst + (i & (kFeatures - 1)) * 128, src);
+            copies_end_group();
+        };
+        int4 item = queue[first];
+        int ahead = queue[first + 2].x;
+        copy_features(first, item.x);
+        copy_features(first + 1, queue[first + 1].x);
+        if constexpr (kWalk) {
+            // messages of items that are skipped, which later ones of this queue read: a slot belongs to its node until its
+            // last reader (whoever takes it waits for this warp), so they can all be brought in at once
+            if (carry != carry_first) { carry = carry_first; look(); }
+#pragma unroll 1
+            while (carry < entry_end) {
+                unsigned left = __ballot_sync(0xffffffffu, carry_rank < rank);
+                while (left) {
+                    float v[4][R];
+                    int to[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int at = __ffs(left) - 1;
+                        if (left & (left - 1)) left &= left - 1;
+                        else if (i == 3) left = 0;
+                        to[i] = __shfl_sync(0xffffffffu, carry_slot, at) * kD + at32;
+                        const float *src = M + (size_t)__shfl_sync(0xffffffffu, carry_node, at) * B * kD + col;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) v[i][r] = src[(size_t)b[r] * kD];
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int r = 0; r < R; ++r) msg[r * row + to[i]] = v[i][r];
+                }
+                carry += 32;
+                if (carry < entry_end) look();
             }
+        }
+        copies_wait<1>();
+        __syncwarp();
+        float *const h_to = H + (size_t)b[0] * kD + col, *const m_to = kWalk ? M + (size_t)b[0] * kD + col : nullptr;
+
+        // One item; kPlain: a single neighbour in this queue, a message that others read and nobody waits for. False at the
+        // end of the queue, or when a wait ran out.
+        bool timeout = false;
+        int4 item_next;
+        int ahead_next;
+        auto run = [&](auto plain, int i) -> bool {
+            constexpr bool kPlain = decltype(plain)::value;
+            copy_features(i + 2, ahead);
+            float acc[R];
+            const float *in = msg + (int)((unsigned)item.y >> 16) * kD;
+            if constexpr (!kPlain) {
+                // neighbours come in groups of four, the last one filled up with the slot of zeros
+                const uint2 *more = info + item.z + 2;
+                uint2 four = more[0];
+                const int wanted = reinterpret_cast<const unsigned short *>(more - 2)[lane & 7];
+                if (!__all_sync(0xffffffffu, load_acquire(others) >= wanted)) {
+                    if (item.w & kQueueEnd) return false;            // (its wait is for more items than there are)
+                    int polls = 0;
+                    while (!__all_sync(0xffffffffu, load_acquire(others) >= wanted))
+                        if (++polls > kMaxPolls) { timeout = true; return false; }
+                }
+                __syncwarp();
+                int left = item.w & 0xffffff;
+#pragma unroll
+                for (int r = 0; r < R; ++r) acc[r] = 0.f;
+#pragma unroll 1
+                while (true) {
+                    const unsigned word[2] = {four.x, four.y};
+                    float t[4][R];
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        const float *m = msg + ((word[n >> 1] >> (16 * (n & 1))) & 0xffffu) * kD + at32;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) t[n][r] = m[r * row];
+                    }
+                    // four are added up in pairs, a last one to three in turn (zeros do no harm)
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float pairs = acc[r] + ((t[0][r] + t[1][r]) + (t[2][r] + t[3][r])), turn = ((acc[r] + t[0][r]) + t[1][r]) + t[2][r];
+                        acc[r] = left >= 4 ? pairs : turn;
+                    }
+                    left -= 4;
+                    if (left <= 0) break;
+                    four = *++more;
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) A[r * KF + at32] = acc[r];
+                __syncwarp();
+                in = A;
+            }
+            // the next record, and this item's raw features
+            item_next = queue[i + 1];
+            ahead_next = queue[i + 3].x;
+            const float *xs = xring + (i & (kFeatures - 1)) * 32;
+            float x[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if constexpr (kCompact) {
+                    // the state's byte moves through its word from node to node
+                    const unsigned at = (byte_at[r] + (unsigned)item.x * (unsigned)B) & 3;
+                    const unsigned s = __float_as_uint(xs[2 + r]) >> (8 * at) & 255u;
+                    const float one = lane < a.F - 2 ? ((int)(s & 63u) == lane - 2 ? 1.f : 0.f)
+                                    : lane == a.F - 2 ? (current[r] == item.x ? 1.f : 0.f) : (float)(s >> 7);
+                    x[r] = lane < 2 ? xs[lane] : one;
+                } else {
+                    x[r] = xs[r * 16 + (lane & 15)];
+                }
+                if (lane >= a.F) x[r] = 0.f;
+            }
+            Rows::template product<R, kD>(wg1, bg1, in, kPlain ? row : KF, lane, acc);
+            if constexpr (L == 2) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) Bf[r * KF + at32] = fmaxf(acc[r], 0.f);
+                __syncwarp();
+                Rows::template product<R, kD>(wg2, bg2, Bf, KF, lane, acc);
+            }
+            float *h_row = row_of(h_to, item.x, h_stride);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                acc[r] = fmaxf(acc[r], 0.f);
+                if (r == 0 || last_live) h_row[r * kD] = acc[r];
+            }
+            const int own = item.y & 0xffff;
+            if (kPlain || own != 0xffff) {
+                float *fin = L == 2 ? A : Bf;            // the buffer that the last product did not read
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    fin[r * KF + at_h] = acc[r];
+                    if (lane < KF - kD) fin[r * KF + at_x] = x[r];
+                }
+                __syncwarp();
+                Rows::template product<R, KF>(wf1, bf1, fin, KF, lane, acc);
+                if constexpr (L == 2) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) Bf[r * KF + at32] = fmaxf(acc[r], 0.f);
+                    __syncwarp();
+                    Rows::template product<R, kD>(wf2, bf2, Bf, KF, lane, acc);
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    acc[r] = fmaxf(acc[r], 0.f);
+                    msg[r * row + own * kD + at32] = acc[r];
+                    if (kWalk && (r == 0 || last_live)) row_of(m_to, item.x, h_stride)[r * kD] = acc[r];
+                }
+            }
+            copies_wait<1>();
+            __syncwarp();                                // the message is there, the buffers are free, the next copies have come
+            if constexpr (!kPlain) store_release_if((item.w & kQueuePublishes) && lane == 0, &progress[warp], i + 1);
+            item = item_next;
+            ahead = ahead_next;
+            return true;
+        };
+        int i = first;
+#pragma unroll 1
+        do {                                             // (one branch per link of a chain)
+#pragma unroll 1
+            for (; item.w & kQueuePlain; ++i) run(std::true_type{}, i);
+        } while (run(std::false_type{}, i++));
+        copies_wait<0>();
+        __syncwarp();
+        if (timeout) {
+            if (lane == 0) report_status(a.status, PLACETO_ERR_TIMEOUT);
             return;
         }
-        for (int i = lane; i < width * per; i += 32) {
-            const int q = per == 1 ? i : (int)__umulhi((unsigned)i, magic_per);
-            const int piece = i - q * per;
-            const float *src = X + ((size_t)meta[q0 + q].w * B + b_first) * F;
-            if (vec) __pipeline_memcpy_async(dst + q * per_node + 4 * piece, src + 4 * piece, 16);
-            else __pipeline_memcpy_async(dst + q * per_node + piece, src + piece, 4);
-        }
-        __pipeline_commit();
-    };
-    const int start = kWalk ? first_level(a.walk, lv, a.n) : 0;
-    dependency_wait();          // the raw features may come from a kernel that is still running
-    prefetch(start);
-    if (L == 1 && start + 1 < lv.n_levels) prefetch(start + 1);
-    float *__restrict__ M = a.M[dir];
-    if (kWalk && start > 0) {
-        carried_messages(lv, meta[level_ptr[start]].x, start, warp, kThreads<L> / 32, lane, [&](const int (&u)[4], const int (&e)[4]) {
-            for (int s = 0; s < nb; ++s) {
-                float v[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) v[k] = M[((size_t)u[k] * B + b_first + s) * kD + lane];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) msg[(nbr_slot[e[k]] * p.S + s) * kD + lane] = v[k];
-            }
-        });
-    }
-    __pipeline_wait_prior(0);
-    __syncthreads();
-
-    if (L == 1 && warp == kWarps) {
-        for (int level = start; level < lv.n_levels; ++level) {
-            if (level + 2 < lv.n_levels) {
-                prefetch(level + 2);
-                __pipeline_wait_prior(1);
-            } else {
-                __pipeline_wait_prior(0);
-            }
-            __syncthreads();
-        }
-        return;
-    }
-    int stage_now = start % kStages<L>;
-    for (int level = start; level < lv.n_levels; ++level) {
-        if (L == 2 && level + 1 < lv.n_levels) prefetch(level + 1);
-        const int p0 = level_ptr[level];
-        const int rows = (level_ptr[level + 1] - p0) * nb;
-        const float *xs = xstage + (size_t)(L == 1 ? stage_now : level & 1) * p.x_floats;
-        if (L == 1) stage_now = stage_now == 2 ? 0 : stage_now + 1;
-        const int width = level_ptr[level + 1] - p0;
-        if (rows <= kWarps) {
-            // narrow level: one row per warp, shortest dependent chains
-            if (warp < rows) {
-                const int q = nb == 1 ? warp : (int)__umulhi((unsigned)warp, magic_nb);
-                const int s0 = warp - q * nb;
-                run_node<1, KF, L, kWalk>(w, wf1, p0 + q, q, s0, true, nb, p.S, F, lane, meta, nbr_slot, msg,
-                                xs, H, M, B, b_first, A, Bf);
-            }
-        } else {
-            // two states of one node per warp pass
-            const int ppn = (nb + 1) >> 1;
-            for (int item = warp; item < width * ppn; item += kWarps) {
-                const int q = ppn == 1 ? item : (int)__umulhi((unsigned)item, magic_ppn);
-                const int s0 = (item - q * ppn) * 2;
-                run_node<2, KF, L, kWalk>(w, wf1, p0 + q, q, s0, s0 + 1 < nb, nb, p.S, F, lane, meta, nbr_slot,
-                                msg, xs, H, M, B, b_first, A, Bf);
-            }
-        }
-        if (L == 2) __pipeline_wait_prior(0);
-        __syncthreads();
     }
 }
 
@@ -378,67 +492,82 @@ bool embed_d32_applicable(const EmbedArgs &a) {
 }
 
 namespace {
-// slice size and shared-memory layout; false when not even one state per block fits
-bool plan_d32(const EmbedArgs &a, const DeviceInfo &di, D32Plan *out) {
-    D32Plan p;
-    const int target = std::max(1, di.sm_count / 2);            // blocks per direction
-    const int want = std::max(1, std::min(a.B, target));
-    p.S = (a.B + want - 1) / want;
-    const int F4 = (a.F + 3) / 4;
-    const int KF = kD + 4 * F4;
+struct D32Launch {
+    D32Plan plan;
+    int pair;                // states that a warp carries together
+    size_t smem_bytes;
+};
+
+// Warps per state, blocks and shared memory; false when not even one state per block fits.
+bool plan_d32(const EmbedArgs &a, const DeviceInfo &di, D32Launch *out) {
+    if (a.B >= 1 << 25) return false;        // bytes between two nodes' rows in 32 bits
     const size_t budget = (size_t)std::min(di.max_smem_optin, 227 * 1024) - 1024;
-    const int max_slots = std::max(a.lv[0].n_slots, a.lv[1].n_slots);
-    if (max_slots >= 0xffff) return false;   // slot ids are packed into 16 bits
-    size_t ints = 0;
-    for (int dir = 0; dir < 2; ++dir) {
-        const DevLevels &lv = a.lv[dir];
-        ints = std::max(ints, (size_t)4 * a.n + ((lv.n_levels + 1 + 3) & ~3) + ((lv.n_nbr + 3) & ~3));
-    }
-    const size_t xbuf = (size_t)kWarps * 4 * KF * sizeof(float);
-    auto x_floats = [&](int S) { return (a.max_level_width * S * a.F + 3) & ~3; };
-    auto need = [&](int S) {
-        return (size_t)max_slots * S * kD * sizeof(float) + (a.f[0].n_layers == 1 ? kStages<1> : kStages<2>) * (size_t)x_floats(S) * sizeof(float) +
-               xbuf + ints * sizeof(int);
+    const int half = std::max(1, di.sm_count / 2);               // blocks per direction
+    auto row_bytes = [&](int k) { return (size_t)(std::max(a.queues[0][k].n_slots, a.queues[1][k].n_slots) + 1) * kD * sizeof(float); };
+    auto queue_bytes = [&](int k) { return (size_t)std::max(a.queues[0][k].n_quads, a.queues[1][k].n_quads) * sizeof(int4); };
+    for (int dir = 0; dir < 2; ++dir)
+        for (int k = 0; k < kQueuePlanCount; ++k) out->plan.q[dir][k] = a.queues[dir][k];
+    auto buffers = [](int pair) { return (size_t)kWarps * warp_floats(pair) * sizeof(float); };
+    auto fits = [&](int k, int pair) {
+        const size_t fixed = buffers(pair) + queue_bytes(k);
+        return fixed > budget ? 0 : (int)std::min<size_t>(kWarps >> k, (budget - fixed) / (pair * row_bytes(k)));
     };
-    // narrower slices when the shared memory does not fit (more blocks: they queue up)
-    while (p.S > 1 && need(p.S) > budget) --p.S;
-    if (need(p.S) > budget) return false;
-    // more slices than one wave of blocks: spread the batch evenly over the waves it takes
-    {
-        const int waves = ((a.B + p.S - 1) / p.S + want - 1) / want;
-        p.S = std::min(p.S, (a.B + want * waves - 1) / (want * waves));
+    // One or two states per warp, by the steps that the longer direction takes; an item of two takes 1.25 to 1.45 times as long
+    // (us, one and two: 279 nodes of 2.1 a level, 256 states 82, 80, 148 states 55, 67, 592 states 143, 115; 1080 of
+    // 6.6: 354, 270; 207, 180; 694, 475).
+    D32Plan &p = out->plan;
+    const bool walk = a.walk.order != nullptr;
+    long long best = -1;
+    for (int pair = 1; pair <= 2; ++pair) {
+        int teams[kQueuePlanCount];
+        for (int k = 0; k < kQueuePlanCount; ++k) teams[k] = fits(k, pair);
+        if (teams[0] < 1) continue;
+        const int groups = (a.B + pair - 1) / pair, most = (groups + std::min(half, groups) - 1) / std::min(half, groups);
+        const int k = form_for(most, teams);
+        const long long cost = (long long)std::max(a.queues[0][k].n_steps, a.queues[1][k].n_steps) * ((most + teams[k] - 1) / teams[k]) * (pair == 2 ? 13 : 10);
+        if (best >= 0 && cost >= best) continue;
+        best = cost;
+        out->pair = pair;
+        p.groups = groups;
+        std::copy(teams, teams + kQueuePlanCount, p.teams);
+        p.form = k;
     }
-    p.n_slices = (a.B + p.S - 1) / p.S;
-    p.x_floats = x_floats(p.S);
-    p.smem_bytes = need(p.S);
-    *out = p;
+    if (best < 0) return false;
+    p.blocks = 2 * std::min(half, p.groups);
+    size_t most = 0;
+    for (int k = 0; k < kQueuePlanCount; ++k)
+        if (p.teams[k] > 0 && (walk || k == p.form)) most = std::max(most, queue_bytes(k) + out->pair * p.teams[k] * row_bytes(k));
+    out->smem_bytes = most + buffers(out->pair);
     return true;
 }
 }  // namespace
 
-bool embed_d32_fits(const EmbedArgs &a, const DeviceInfo &di) {
-    D32Plan p;
-    return embed_d32_applicable(a) && plan_d32(a, di, &p);
+bool embed_d32_plan(const EmbedArgs &a, const DeviceInfo &di, D32Plan *plan) {
+    D32Launch l;
+    if (!embed_d32_applicable(a) || !plan_d32(a, di, &l)) return false;
+    *plan = l.plan;
+    return true;
 }
 
 cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream,
                              bool overlap) {
-    D32Plan p;
-    if (!plan_d32(a, di, &p)) return cudaErrorNotSupported;
+    D32Launch l;
+    if (!plan_d32(a, di, &l)) return cudaErrorNotSupported;
     const int F4 = (a.F + 3) / 4;
     typedef void (*Kernel)(const EmbedArgs, const D32Plan);
-#define PLACETO_D32_KERNELS(compact, layers, walk) \
-    {embed_d32_kernel<1, compact, layers, walk>, embed_d32_kernel<2, compact, layers, walk>, \
-     embed_d32_kernel<3, compact, layers, walk>, embed_d32_kernel<4, compact, layers, walk>}
-    static const Kernel kernels[2][3][4] = {     // [layers][X, X in an episode, compact states (always an episode)][F4]
-        {PLACETO_D32_KERNELS(false, 1, false), PLACETO_D32_KERNELS(false, 1, true), PLACETO_D32_KERNELS(true, 1, true)},
-        {PLACETO_D32_KERNELS(false, 2, false), PLACETO_D32_KERNELS(false, 2, true), PLACETO_D32_KERNELS(true, 2, true)}};
+#define PLACETO_D32_KERNELS(source, layers, pair) \
+    {embed_d32_kernel<1, source, layers, pair>, embed_d32_kernel<2, source, layers, pair>, \
+     embed_d32_kernel<3, source, layers, pair>, embed_d32_kernel<4, source, layers, pair>}
+#define PLACETO_D32_SOURCES(layers, pair) \
+    {PLACETO_D32_KERNELS(0, layers, pair), PLACETO_D32_KERNELS(1, layers, pair), PLACETO_D32_KERNELS(2, layers, pair)}
+    static const Kernel kernels[2][2][3][4] = {     // [states per warp][layers][source][F4]
+        {PLACETO_D32_SOURCES(1, 1), PLACETO_D32_SOURCES(2, 1)}, {PLACETO_D32_SOURCES(1, 2), PLACETO_D32_SOURCES(2, 2)}};
+#undef PLACETO_D32_SOURCES
 #undef PLACETO_D32_KERNELS
-    const Kernel kern = kernels[a.f[0].n_layers - 1][a.compact.state != nullptr ? 2 : a.walk.order != nullptr ? 1 : 0][F4 - 1];
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)p.smem_bytes);
+    const Kernel kern = kernels[l.pair - 1][a.f[0].n_layers - 1][a.compact.state != nullptr ? 2 : a.walk.order != nullptr ? 1 : 0][F4 - 1];
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem_bytes);
     if (err != cudaSuccess) return err;
-    err = launch_overlapped(overlap, kern, dim3(p.n_slices, 2), dim3(a.f[0].n_layers == 1 ? kThreads<1> : kThreads<2>), p.smem_bytes, stream, a, p);
+    err = launch_overlapped(overlap, kern, dim3(l.plan.blocks), dim3(kThreads), l.smem_bytes, stream, a, l.plan);
     count_launch();
     return err;
 }

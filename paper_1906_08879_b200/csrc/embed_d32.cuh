@@ -1,0 +1,67 @@
+// What the d = 32 sweep (embed_d32.cu) is launched with, and the starts of an episode's sweeps, which the kernel that begins
+// the episodes works out (episode.cu).
+#pragma once
+#include "kernels.cuh"
+
+namespace placeto {
+
+struct D32Plan {
+    DevQueues q[2][kQueuePlanCount];
+    int teams[kQueuePlanCount];     // warps-per-state forms: states (pairs) of a block at a time, 0: not to be used
+    int groups;                     // states of the batch, or pairs of them
+    int form;                       // of a sweep on its own, which gives both directions the same number of blocks
+    int blocks;
+};
+
+// Log2 of the warps per state for `states` states (or pairs) of a block: as many as there are warps for.
+__device__ __host__ __forceinline__ int form_for(int states, const int (&teams)[kQueuePlanCount]) {
+    int k = kQueuePlanCount - 1;
+    while (k > 0 && teams[k] < states) --k;
+    return k;
+}
+
+#ifdef __CUDACC__
+// What the sweep of step t of an episode starts with, worked out by a warp: {blocks of the top-down direction, and by
+// direction the rank it starts at | its form << 16}. A sweep starts where the features changed: at the top of the graph one
+// direction has all of its steps left and the other next to none, in the middle they have the same. Every lane weighs one
+// split, by the longer direction. (Looked up and weighed in the sweep itself this took 2.3 us of every step.)
+__device__ __forceinline__ void write_d32_step(const D32Plan &p, const int *order, int n, int t, int lane, int4 *steps) {
+    const int blocks = p.blocks;
+    int left[2][kQueuePlanCount], from[2][kQueuePlanCount];
+    const int u = t > 0 ? order[t - 1] : -1, v = order[t];
+    const bool known = u >= 0 && u < n && v >= 0 && v < n;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < kQueuePlanCount; ++j) {
+            const int key = known ? min(p.q[i][j].key[u], p.q[i][j].key[v]) : 0;
+            from[i][j] = key & 0xffff;
+            left[i][j] = p.q[i][j].n_steps - (key >> 16);
+        }
+    int down;
+    if (lane < 8) down = (p.groups + lane) / (lane + 1);                          // lane + 1 states per block top-down,
+    else if (lane < 16) down = blocks - (p.groups + lane - 8) / (lane - 7);       // bottom-up,
+    else down = blocks * (lane - 15) / 17;                                        // or a proportion
+    down = max(1, min(blocks - 1, down));
+    unsigned worst = 0;
+    int start[2];
+#pragma unroll
+    for (int dir = 0; dir < 2; ++dir) {
+        const int nb = dir == 0 ? down : blocks - down, states = (p.groups + nb - 1) / nb;
+        const int k = form_for(states, p.teams), rounds = (states + p.teams[k] - 1) / p.teams[k];
+        int step = 0;
+#pragma unroll
+        for (int i = 0; i < kQueuePlanCount; ++i)
+            if (i == k) { step = left[dir][i]; start[dir] = from[dir][i] | i << 16; }
+        const int busy = min(states, p.teams[k]) << k;                            // warps at work slow each other down
+        worst = max(worst, (unsigned)(rounds * step) * (unsigned)(16 + busy));
+    }
+    const unsigned best = __reduce_min_sync(0xffffffffu, worst);
+    if (lane == __ffs(__ballot_sync(0xffffffffu, worst == best)) - 1) steps[t] = make_int4(down, start[0], start[1], 0);
+}
+#endif
+
+// false when not even one state fits in shared memory
+bool embed_d32_plan(const EmbedArgs &a, const DeviceInfo &di, D32Plan *plan);
+
+}  // namespace placeto

@@ -17,7 +17,7 @@
 // place and the feature tensor is built once per episode, not once per step.
 #include <cmath>
 
-#include "kernels.cuh"
+#include "embed_d32.cuh"
 
 namespace placeto {
 
@@ -25,9 +25,18 @@ namespace {
 
 constexpr int kThreads = 128;
 
+// the starts of the sweeps of all steps, a warp each
+__device__ __forceinline__ void write_steps(const D32Plan &plan, const int *order, int n, int4 *steps) {
+    const int warps = gridDim.x * (kThreads / 32);
+    for (int t = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); t < n; t += warps)
+        write_d32_step(plan, order, n, t, threadIdx.x & 31, steps);
+}
+
 // placed[e][:] = 0 and cur[e] = order[0] for every episode
 __global__ void episode_begin_kernel(int n, int E, const int *__restrict__ order,
-                                     uint8_t *__restrict__ placed, int *__restrict__ cur) {
+                                     uint8_t *__restrict__ placed, int *__restrict__ cur,
+                                     const __grid_constant__ D32Plan plan, int4 *__restrict__ steps) {
+    if (steps != nullptr) write_steps(plan, order, n, steps);
     const size_t total = (size_t)E * n;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (size_t)gridDim.x * blockDim.x)
@@ -85,7 +94,9 @@ __global__ void episode_step_kernel(EpisodeArgs a, int t) {
 // carries: its one-hot is all zero), nothing visited; cur[e] = order[0]
 __global__ void episode_begin_compact_kernel(int n, int E, const int *__restrict__ order,
                                              const uint8_t *__restrict__ dev, uint8_t *__restrict__ state,
-                                             int *__restrict__ cur) {
+                                             int *__restrict__ cur, const __grid_constant__ D32Plan plan,
+                                             int4 *__restrict__ steps) {
+    write_steps(plan, order, n, steps);
     const size_t total = (size_t)E * n;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const size_t v = i / E, e = i - v * E;
@@ -111,10 +122,10 @@ __global__ void episode_end_compact_kernel(int n, int E, const uint8_t *__restri
 }  // namespace
 
 cudaError_t launch_episode_begin_compact(int n, int E, const int *order, const uint8_t *dev, uint8_t *state,
-                                         int *cur, cudaStream_t stream) {
+                                         int *cur, const D32Plan &plan, int4 *steps, cudaStream_t stream) {
     const int blocks = std::max(1, std::min(2048, (int)(((size_t)E * n + kThreads - 1) / kThreads)));
     const int need = (E + kThreads - 1) / kThreads;       // every episode needs its thread
-    episode_begin_compact_kernel<<<std::max(blocks, need), kThreads, 0, stream>>>(n, E, order, dev, state, cur);
+    episode_begin_compact_kernel<<<std::max(blocks, need), kThreads, 0, stream>>>(n, E, order, dev, state, cur, plan, steps);
     count_launch();
     return cudaGetLastError();
 }
@@ -127,10 +138,11 @@ cudaError_t launch_episode_end_compact(int n, int E, const uint8_t *state, uint8
     return err;
 }
 
-cudaError_t launch_episode_begin(const EpisodeArgs &a, cudaStream_t stream) {
+cudaError_t launch_episode_begin(const EpisodeArgs &a, const D32Plan *plan, int4 *steps, cudaStream_t stream) {
     const int blocks = std::max(1, std::min(1024, (int)(((size_t)a.E * a.n + kThreads - 1) / kThreads)));
     const int need = (a.E + kThreads - 1) / kThreads;       // every episode needs its thread
-    episode_begin_kernel<<<std::max(blocks, need), kThreads, 0, stream>>>(a.n, a.E, a.order, a.placed, a.cur);
+    episode_begin_kernel<<<std::max(blocks, need), kThreads, 0, stream>>>(a.n, a.E, a.order, a.placed, a.cur,
+                                                                              plan ? *plan : D32Plan{}, plan ? steps : nullptr);
     count_launch();
     return cudaGetLastError();
 }

@@ -27,6 +27,25 @@ struct DevLevels {
     const int *level_of;             // [n] level of a node id
 };
 
+// One direction's queues for 1, 2, 4 or 8 warps per state in device memory (see QueuePlan in plan.h). Kernels take `record`
+// on chip as a whole: every queue's records and kQueuePad with kQueueEnd (of node 0), then what the records point to.
+//   record[i] = {node id, own slot (0xffff: none) | slot of the first neighbour << 16, where its waits are (in eight bytes),
+//                neighbours | kQueuePublishes, kQueuePlain (one neighbour, a message that is read, no waits, not published)}
+//   of a record that is not plain: eight 16-bit counts of items to wait for, one a queue; the slots of its neighbours,
+//   16 bits each, filled up to a multiple of four (but not zero) of them with slot n_slots, which holds zeros. What a
+//   kQueueEnd waits for never comes.
+constexpr int kQueuePlanCount = 4, kQueuePad = 4, kQueueEnd = 1 << 30, kQueuePublishes = 1 << 29, kQueuePlain = 1 << 28;
+struct DevQueues {
+    int ptr[9], entry_ptr[9];        // by queue: items, neighbour entries
+    int n_slots, n_steps;
+    int n_quads;                     // of 16 bytes that `record` has in all
+    const int4 *record;
+    const int *entry;                // [n] by item: first neighbour entry
+    const int *nbr, *nbr_slot, *nbr_rank;
+    const int *key;                  // [n] by node: step << 16 | rank
+    const unsigned short *first;     // [n][walkers] by rank: a queue's items of smaller rank
+};
+
 // One feed-forward network with device pointers.
 struct DevMlp {
     int n_layers, in_dim, hidden_dim, out_dim, act, final_act;
@@ -134,6 +153,7 @@ struct EpisodeStep {
 struct EpisodeWalk {
     const int *order;      // [n], or null: a sweep on its own
     int t;
+    const int4 *steps;     // [n] of the d = 32 sweep: see write_d32_step
 };
 #ifdef __CUDACC__
 __device__ __forceinline__ int first_level(const EpisodeWalk &w, const DevLevels &lv, int n) {
@@ -181,6 +201,7 @@ struct EmbedArgs {
     StatusSlot status;
     CompactState compact;  // compact.state != null: X is not read
     EpisodeWalk walk;
+    const DevQueues (*queues)[kQueuePlanCount];    // host: the graph's queues, [direction][log2 of the warps per state]
 };
 
 struct PoolArgs {
@@ -344,12 +365,13 @@ cudaError_t launch_stage_inputs(const void *const (&src)[5], void *const (&dst)[
                                 const size_t (&bytes)[5], int sm_count, cudaStream_t stream);
 
 // episode.cu: the MDP transition between two policy evaluations of an episode
-cudaError_t launch_episode_begin(const EpisodeArgs &a, cudaStream_t stream);
+struct D32Plan;            // of the sweeps that follow, if they are those of embed_d32.cu: their starts go to steps [n]
+cudaError_t launch_episode_begin(const EpisodeArgs &a, const D32Plan *plan, int4 *steps, cudaStream_t stream);
 cudaError_t launch_episode_step(const EpisodeArgs &a, int t, cudaStream_t stream);
 // compact states: state[v][e] from the initial placement dev[e][v] (nothing visited), cur[e] = order[0];
 // and back: dev[e][v] = the device of state[v][e]
 cudaError_t launch_episode_begin_compact(int n, int E, const int *order, const uint8_t *dev, uint8_t *state,
-                                         int *cur, cudaStream_t stream);
+                                         int *cur, const D32Plan &plan, int4 *steps, cudaStream_t stream);
 cudaError_t launch_episode_end_compact(int n, int E, const uint8_t *state, uint8_t *dev, cudaStream_t stream);
 // true when an episode step on these shapes runs on kernels that take compact states
 bool pool_head_takes_compact(const PoolArgs &a);
@@ -397,7 +419,6 @@ cudaError_t launch_embed_rounds_d32(const EmbedArgs &a, const DeviceInfo &di, in
 // layer or of two with hidden width 32; returns cudaErrorNotSupported when the shapes or
 // the shared-memory budget do not fit (the caller then uses the generic kernel).
 bool embed_d32_applicable(const EmbedArgs &a);
-bool embed_d32_fits(const EmbedArgs &a, const DeviceInfo &di);   // applicable and within shared memory
 cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream,
                              bool overlap = false);
 

@@ -10,22 +10,41 @@ namespace placeto {
 
 namespace {
 
-// Longest-path layering along one direction. `nbrs[v]` are the nodes v waits
-// for (parents for the top-down pass), `rev[v]` the nodes waiting for v.
-// Returns false if the graph has a cycle.
-bool layer(int32_t n, const std::vector<std::vector<int32_t>> &nbrs,
-           const std::vector<std::vector<int32_t>> &rev, std::vector<int32_t> &level) {
+// Lists by node id, ascending, without repeats: list[ptr[v] .. ptr[v + 1]) from the pairs (key, value).
+void lists(int32_t n, int64_t n_pairs, const int32_t *key, const int32_t *value, std::vector<int32_t> &ptr, std::vector<int32_t> &list) {
+    std::vector<int64_t> start(n + 1, 0);            // (a caller may repeat edges)
+    for (int64_t e = 0; e < n_pairs; ++e) ++start[key[e] + 1];
+    for (int32_t v = 0; v < n; ++v) start[v + 1] += start[v];
+    list.resize(n_pairs);
+    std::vector<int64_t> at(start.begin(), start.end() - 1);
+    for (int64_t e = 0; e < n_pairs; ++e) list[at[key[e]]++] = value[e];
+    ptr.assign(n + 1, 0);
+    auto kept = list.begin();
+    for (int32_t v = 0; v < n; ++v) {
+        const auto first = list.begin() + start[v], end = list.begin() + start[v + 1];
+        std::sort(first, end);
+        kept = std::copy(first, std::unique(first, end), kept);
+        ptr[v + 1] = static_cast<int32_t>(kept - list.begin());
+    }
+    list.resize(ptr[n]);
+}
+
+// Longest-path layering along one direction. nbr are the nodes that v waits for (parents for the top-down pass), rev
+// the nodes waiting for v. Returns false if the graph has a cycle.
+bool layer(int32_t n, const std::vector<int32_t> &nbr_ptr, const std::vector<int32_t> &rev_ptr, const std::vector<int32_t> &rev,
+           std::vector<int32_t> &level) {
     std::vector<int32_t> pending(n);
     std::vector<int32_t> queue;
     queue.reserve(n);
     level.assign(n, 0);
     for (int32_t v = 0; v < n; ++v) {
-        pending[v] = static_cast<int32_t>(nbrs[v].size());
+        pending[v] = nbr_ptr[v + 1] - nbr_ptr[v];
         if (pending[v] == 0) queue.push_back(v);
     }
     for (size_t head = 0; head < queue.size(); ++head) {
         const int32_t u = queue[head];
-        for (int32_t v : rev[u]) {
+        for (int32_t e = rev_ptr[u]; e < rev_ptr[u + 1]; ++e) {
+            const int32_t v = rev[e];
             level[v] = std::max(level[v], level[u] + 1);
             if (--pending[v] == 0) queue.push_back(v);
         }
@@ -33,8 +52,8 @@ bool layer(int32_t n, const std::vector<std::vector<int32_t>> &nbrs,
     return static_cast<int32_t>(queue.size()) == n;
 }
 
-void bucket(int32_t n, const std::vector<int32_t> &level,
-            const std::vector<std::vector<int32_t>> &nbrs, LevelPlan &out) {
+void bucket(int32_t n, const std::vector<int32_t> &level, const std::vector<int32_t> &nbr_ptr, const std::vector<int32_t> &nbr,
+            LevelPlan &out) {
     int32_t n_levels = 0;
     for (int32_t v = 0; v < n; ++v) n_levels = std::max(n_levels, level[v] + 1);
     out.n_levels = n_levels;
@@ -46,9 +65,10 @@ void bucket(int32_t n, const std::vector<int32_t> &level,
     for (int32_t v = 0; v < n; ++v) out.order[fill[level[v]]++] = v;  // ascending id per level
     out.nbr_ptr.assign(n + 1, 0);
     out.nbr.clear();
+    out.nbr.reserve(nbr.size());
     for (int32_t p = 0; p < n; ++p) {
-        const auto &list = nbrs[out.order[p]];
-        out.nbr.insert(out.nbr.end(), list.begin(), list.end());
+        const int32_t v = out.order[p];
+        out.nbr.insert(out.nbr.end(), nbr.begin() + nbr_ptr[v], nbr.begin() + nbr_ptr[v + 1]);
         out.nbr_ptr[p + 1] = static_cast<int32_t>(out.nbr.size());
     }
 }
@@ -91,50 +111,34 @@ placeto_status build_plan(int32_t n, int64_t n_edges, const int32_t *src, const 
     if (n < 1 || n > PLACETO_MAX_NODES || n_edges < 0) return PLACETO_ERR_INVALID_ARG;
     if (n_edges > 0 && (src == nullptr || dst == nullptr)) return PLACETO_ERR_INVALID_ARG;
     try {
-        std::vector<std::vector<int32_t>> par(n), chi(n);
         for (int64_t e = 0; e < n_edges; ++e) {
             const int32_t u = src[e], v = dst[e];
             if (u < 0 || u >= n || v < 0 || v >= n || u == v) return PLACETO_ERR_NOT_DAG;
-            par[v].push_back(u);
-            chi[u].push_back(v);
         }
-        int64_t distinct = 0;
+        lists(n, n_edges, dst, src, plan.parent_ptr, plan.parent);
+        lists(n, n_edges, src, dst, plan.child_ptr, plan.child);
         int32_t max_degree = 0;
-        for (int32_t v = 0; v < n; ++v) {
-            for (auto *list : {&par[v], &chi[v]}) {
-                std::sort(list->begin(), list->end());
-                list->erase(std::unique(list->begin(), list->end()), list->end());
-                max_degree = std::max(max_degree, static_cast<int32_t>(list->size()));
-            }
-            distinct += static_cast<int64_t>(par[v].size());
-        }
+        for (int32_t v = 0; v < n; ++v)
+            for (auto *ptr : {&plan.parent_ptr, &plan.child_ptr}) max_degree = std::max(max_degree, (*ptr)[v + 1] - (*ptr)[v]);
         std::vector<int32_t> level_down, level_up;
-        if (!layer(n, par, chi, level_down)) return PLACETO_ERR_NOT_DAG;
-        if (!layer(n, chi, par, level_up)) return PLACETO_ERR_NOT_DAG;
+        if (!layer(n, plan.parent_ptr, plan.child_ptr, plan.child, level_down)) return PLACETO_ERR_NOT_DAG;
+        if (!layer(n, plan.child_ptr, plan.parent_ptr, plan.parent, level_up)) return PLACETO_ERR_NOT_DAG;
         plan.n = n;
-        plan.n_edges = distinct;
+        plan.n_edges = static_cast<int64_t>(plan.parent.size());
         plan.max_degree = max_degree;
-        bucket(n, level_down, par, plan.dir[0]);
-        bucket(n, level_up, chi, plan.dir[1]);
+        bucket(n, level_down, plan.parent_ptr, plan.parent, plan.dir[0]);
+        bucket(n, level_up, plan.child_ptr, plan.child, plan.dir[1]);
         assign_slots(n, level_down, plan.dir[0]);
         assign_slots(n, level_up, plan.dir[1]);
-        plan.child_ptr.assign(n + 1, 0);
-        plan.child.clear();
-        for (int32_t v = 0; v < n; ++v) {
-            plan.child.insert(plan.child.end(), chi[v].begin(), chi[v].end());
-            plan.child_ptr[v + 1] = static_cast<int32_t>(plan.child.size());
-        }
-        plan.parent_ptr.assign(n + 1, 0);
-        plan.parent.clear();
-        for (int32_t v = 0; v < n; ++v) {
-            plan.parent.insert(plan.parent.end(), par[v].begin(), par[v].end());
-            plan.parent_ptr[v + 1] = static_cast<int32_t>(plan.parent.size());
-        }
         // parents are visited in ascending order by every child: walking the children in ascending
         // order fills each parent's child list front to back
         plan.child_entry.assign(plan.child.size(), 0);
         std::vector<int32_t> at(plan.child_ptr.begin(), plan.child_ptr.end() - 1);
         for (int32_t e = 0; e < static_cast<int32_t>(plan.parent.size()); ++e) plan.child_entry[at[plan.parent[e]]++] = e;
+        for (int q = 0; q < kQueuePlans; ++q) {
+            build_queues(n, plan.parent_ptr, plan.parent, plan.child_ptr, plan.child, plan.dir[0], level_up, 1 << q, plan.queues[0][q]);
+            build_queues(n, plan.child_ptr, plan.child, plan.parent_ptr, plan.parent, plan.dir[1], level_down, 1 << q, plan.queues[1][q]);
+        }
         plan.max_level_width = 0;
         for (int dir = 0; dir < 2; ++dir)
             for (int32_t l = 0; l < plan.dir[dir].n_levels; ++l)

@@ -24,12 +24,34 @@ struct LevelPlan {
     std::vector<int32_t> nbr_slot;   // [nbr.size()] slot of each neighbour
 };
 
+// The same pass as queues of nodes, one for each of `walkers` warps that share a state: every warp takes its queue's
+// nodes in order and waits only where a neighbour's message comes from another queue (or the slot that it is about to
+// write is still read by another), so no barrier separates the levels. Any order of the nodes that has neighbours first
+// would do; `key` is the one the queues were filled in, and an episode's sweep starts at the smallest key whose features changed.
+struct QueuePlan {
+    int32_t walkers = 1;
+    int32_t n_steps = 0;             // steps that take one node of every queue at most
+    int32_t n_slots = 0;             // message slots per state
+    std::vector<int32_t> ptr, entry_ptr;    // [walkers + 1] items, and their neighbour entries, by queue
+    std::vector<int32_t> node;       // [n] by item
+    std::vector<int32_t> own_slot;   // [n] by item, -1 if nobody reads the message
+    std::vector<int32_t> nbr_ptr;    // [n + 1] by item
+    std::vector<int32_t> nbr, nbr_slot, nbr_rank;   // by entry, neighbours ascending; rank in filling order
+    std::vector<uint16_t> need;      // [n][walkers] items of each queue that must be done before this one
+    std::vector<uint8_t> waits, publishes;  // [n] an entry of `need` that is not implied by an earlier wait; is such an entry of another item
+    std::vector<uint16_t> first;     // [n][walkers] by rank: a queue's items of smaller rank
+    std::vector<int32_t> key;        // [n] by node: step << 16 | rank
+};
+
+constexpr int kQueuePlans = 4;       // 1, 2, 4 and 8 walkers
+
 struct HostPlan {
     int32_t n = 0;
     int64_t n_edges = 0;             // distinct edges
     int32_t max_level_width = 0;     // over both directions
     int32_t max_degree = 0;          // largest neighbour set, both directions
     LevelPlan dir[2];                // 0 top-down, 1 bottom-up
+    QueuePlan queues[2][kQueuePlans];
     std::vector<uint8_t> relation;   // [n * n], see placeto_graph_host_view
     // by node id, ascending, for the runtime simulator and the policy gradient's gathers: children and parents;
     // child_entry[e] is the entry in `parent` of the edge at entry e of `child`
@@ -41,5 +63,12 @@ struct HostPlan {
 // PLACETO_ERR_INVALID_ARG, PLACETO_ERR_NOT_DAG or PLACETO_ERR_NO_MEMORY.
 placeto_status build_plan(int32_t n, int64_t n_edges, const int32_t *src, const int32_t *dst,
                           HostPlan &plan);
+
+// Fills the queues of one direction for `walkers` warps: nbr / rev are the lists of the nodes that a node waits for and
+// that wait for it, by node id, `levels` the direction's levels and `ahead` the other direction's level of a node (the
+// length of the longest path on from it).
+void build_queues(int32_t n, const std::vector<int32_t> &nbr_ptr, const std::vector<int32_t> &nbr,
+                  const std::vector<int32_t> &rev_ptr, const std::vector<int32_t> &rev, const LevelPlan &levels,
+                  const std::vector<int32_t> &ahead, int32_t walkers, QueuePlan &out);
 
 }  // namespace placeto

@@ -1,0 +1,194 @@
+// Host plan of a pass over the DAG as queues of nodes, one per warp of a state (see plan.h). Pure C++, no CUDA.
+#include <algorithm>
+
+#include "plan.h"
+
+namespace placeto {
+
+namespace {
+
+// The nodes in filling order with their step and queue. One queue: level order. Several: in every step each queue takes one
+// node whose neighbours are done. Where the graph is on average no wider than the queues, those with the longest path ahead
+// go first, and a node that becomes available belongs to the queue that did the last of its neighbours (its message is
+// at hand, nobody waits); a queue without one takes the best of the queue that has most. On wider graphs the lowest
+// levels go first, which keeps the number of messages in use small, and any queue takes any node, its own neighbour's if it can.
+void fill_order(int32_t n, const std::vector<int32_t> &nbr_ptr, const std::vector<int32_t> &rev_ptr,
+                const std::vector<int32_t> &rev, const LevelPlan &levels, const std::vector<int32_t> &ahead, int32_t walkers,
+                std::vector<int32_t> &order, std::vector<int32_t> &step, std::vector<int32_t> &queue) {
+    step.assign(n, 0);
+    queue.assign(n, 0);
+    if (walkers == 1) {
+        order = levels.order;
+        for (int32_t p = 0; p < n; ++p) step[order[p]] = p;
+        return;
+    }
+    const bool wide = n > static_cast<int64_t>(walkers) * levels.n_levels;
+    std::vector<int32_t> better(n), pending(n), after(n, -1);    // larger first; the neighbour that was done last
+    if (wide) {
+        for (int32_t l = 0; l < levels.n_levels; ++l)
+            for (int32_t p = levels.level_ptr[l]; p < levels.level_ptr[l + 1]; ++p) better[levels.order[p]] = -l;
+    } else {
+        better = ahead;
+    }
+    auto worse = [&](int32_t u, int32_t v) { return better[u] != better[v] ? better[u] < better[v] : u > v; };
+    std::vector<int32_t> ready[8];                       // heaps; one for all of a wide graph
+    auto add = [&](int32_t q, int32_t v) { ready[q].push_back(v); std::push_heap(ready[q].begin(), ready[q].end(), worse); };
+    for (int32_t v = 0, q = 0; v < n; ++v) {
+        pending[v] = nbr_ptr[v + 1] - nbr_ptr[v];
+        if (pending[v] == 0) { add(q, v); q = wide ? 0 : (q + 1) % walkers; }
+    }
+    auto best = [&](std::vector<int32_t> &heap) {
+        std::pop_heap(heap.begin(), heap.end(), worse);
+        const int32_t v = heap.back();
+        heap.pop_back();
+        return v;
+    };
+    order.clear();
+    order.reserve(n);
+    for (int32_t t = 0; static_cast<int32_t>(order.size()) < n; ++t) {
+        int32_t taken[8];
+        std::fill(taken, taken + walkers, -1);
+        if (wide) {
+            int32_t loose[8], k = 0;
+            for (int32_t i = 0; i < walkers && !ready[0].empty(); ++i) {
+                const int32_t v = best(ready[0]), u = after[v];
+                if (u >= 0 && taken[queue[u]] < 0) taken[queue[u]] = v;
+                else loose[k++] = v;
+            }
+            for (int32_t q = 0; k > 0; ++q)
+                if (taken[q] < 0) taken[q] = loose[--k];
+        } else {
+            for (int32_t q = 0; q < walkers; ++q)
+                if (!ready[q].empty()) taken[q] = best(ready[q]);
+            for (int32_t q = 0; q < walkers; ++q) {
+                if (taken[q] >= 0) continue;
+                int32_t most = 0;
+                for (int32_t x = 1; x < walkers; ++x)
+                    if (ready[x].size() > ready[most].size()) most = x;
+                if (ready[most].empty()) break;
+                taken[q] = best(ready[most]);
+            }
+        }
+        const size_t from = order.size();
+        for (int32_t q = 0; q < walkers; ++q)
+            if (taken[q] >= 0) { order.push_back(taken[q]); step[taken[q]] = t; queue[taken[q]] = q; }
+        for (size_t i = from; i < order.size(); ++i)
+            for (int32_t e = rev_ptr[order[i]]; e < rev_ptr[order[i] + 1]; ++e)
+                if (--pending[rev[e]] == 0) { after[rev[e]] = order[i]; add(wide ? 0 : queue[order[i]], rev[e]); }
+    }
+}
+
+}  // namespace
+
+void build_queues(int32_t n, const std::vector<int32_t> &nbr_ptr, const std::vector<int32_t> &nbr,
+                  const std::vector<int32_t> &rev_ptr, const std::vector<int32_t> &rev, const LevelPlan &levels,
+                  const std::vector<int32_t> &ahead, int32_t walkers, QueuePlan &out) {
+    const int32_t W = walkers;
+    std::vector<int32_t> order, step, queue;
+    fill_order(n, nbr_ptr, rev_ptr, rev, levels, ahead, W, order, step, queue);
+    out.walkers = W;
+    out.n_steps = step[order[n - 1]] + 1;
+
+    // items: the nodes by queue, in filling order; at[v] = index of v inside its queue
+    std::vector<int32_t> at(n), rank(n);
+    out.ptr.assign(W + 1, 0);
+    out.first.resize(static_cast<size_t>(n) * W);
+    out.key.resize(n);
+    for (int32_t r = 0; r < n; ++r) {
+        const int32_t v = order[r];
+        for (int32_t w = 0; w < W; ++w) out.first[static_cast<size_t>(r) * W + w] = static_cast<uint16_t>(out.ptr[w + 1]);
+        rank[v] = r;
+        at[v] = out.ptr[queue[v] + 1]++;
+        out.key[v] = step[v] << 16 | r;
+    }
+    for (int32_t w = 0; w < W; ++w) out.ptr[w + 1] += out.ptr[w];
+
+    // Slots, in filling order. A slot is free again after the last node that reads it. One whose readers were all in one
+    // queue goes back to that queue, which may take it at once (a node may even write the slot that it has read): its warp
+    // has nothing to wait for. Any other queue takes it kSlack steps later, so that it seldom has to wait.
+    constexpr int32_t kSlack = 3;
+    std::vector<int32_t> last(n, -1), slot_of(n, -1), holder;      // last: latest reader in filling order
+    std::vector<int8_t> readers(n, -1);                            // the queue of all readers, W if they are in several
+    for (int32_t r = 0; r < n; ++r)
+        for (int32_t e = nbr_ptr[order[r]]; e < nbr_ptr[order[r] + 1]; ++e) {
+            const int32_t u = nbr[e], q = queue[order[r]];
+            last[u] = r;
+            readers[u] = static_cast<int8_t>(readers[u] < 0 || readers[u] == q ? q : W);
+        }
+    std::vector<int32_t> before(n, -1);                            // who had the slot before
+    std::vector<int32_t> done_head(n, -1), done_link(n, -1);       // nodes by their last reader
+    for (int32_t v = 0; v < n; ++v)
+        if (last[v] >= 0) { done_link[v] = done_head[last[v]]; done_head[last[v]] = v; }
+    std::vector<std::pair<int32_t, int32_t>> free_slots[9];        // {step of the last reader, slot} by queue; W: several
+    size_t oldest[9] = {};                                         // taken from the front by others
+    for (int32_t r = 0; r < n; ++r) {
+        const int32_t v = order[r], q = queue[v];
+        for (int32_t u = done_head[r]; u >= 0; u = done_link[u]) free_slots[readers[u]].push_back({step[v], slot_of[u]});
+        if (last[v] < 0) continue;
+        int32_t from = -1;
+        if (free_slots[q].size() > oldest[q]) {
+            slot_of[v] = free_slots[q].back().second;
+            free_slots[q].pop_back();
+        } else {
+            for (int32_t x = W; x >= 0 && from < 0; --x)
+                if (free_slots[x].size() > oldest[x] && free_slots[x][oldest[x]].first + kSlack < step[v]) from = x;
+            slot_of[v] = from < 0 ? static_cast<int32_t>(holder.size()) : free_slots[from][oldest[from]++].second;
+            if (from < 0) holder.push_back(-1);
+        }
+        before[v] = holder[slot_of[v]];
+        holder[slot_of[v]] = v;
+    }
+    out.n_slots = static_cast<int32_t>(holder.size());
+
+    // What a node waits for: its neighbours, and the readers of the message that its slot held before. clock[v] = the items
+    // of each queue that are known to be done once v is (an item waits only for what no earlier wait implies).
+    out.need.assign(static_cast<size_t>(n) * W, 0);
+    out.waits.assign(n, 0);
+    out.publishes.assign(n, 0);
+    out.node.resize(n);
+    out.own_slot.resize(n);
+    std::vector<uint16_t> clock(static_cast<size_t>(n) * W, 0);
+    std::vector<int32_t> previous(W, -1);
+    for (int32_t r = 0; r < n; ++r) {
+        const int32_t v = order[r], q = queue[v], item = out.ptr[q] + at[v];
+        out.node[item] = v;
+        out.own_slot[item] = slot_of[v];
+        if (W == 1) continue;
+        uint16_t *need = &out.need[static_cast<size_t>(item) * W], *mine = &clock[static_cast<size_t>(v) * W];
+        if (previous[q] >= 0) std::copy_n(&clock[static_cast<size_t>(previous[q]) * W], W, mine);
+        previous[q] = v;
+        auto after = [&](int32_t u) {
+            if (queue[u] != q) need[queue[u]] = std::max<uint16_t>(need[queue[u]], static_cast<uint16_t>(at[u] + 1));
+        };
+        for (int32_t e = nbr_ptr[v]; e < nbr_ptr[v + 1]; ++e) after(nbr[e]);
+        if (before[v] >= 0)
+            for (int32_t e = rev_ptr[before[v]]; e < rev_ptr[before[v] + 1]; ++e) after(rev[e]);
+        uint16_t known[8];
+        std::copy_n(mine, W, known);
+        for (int32_t w = 0; w < W; ++w) {
+            if (need[w] <= known[w]) { need[w] = 0; continue; }
+            out.waits[item] = 1;
+            const int32_t whom = out.ptr[w] + need[w] - 1;
+            out.publishes[whom] = 1;
+            const uint16_t *theirs = &clock[static_cast<size_t>(out.node[whom]) * W];
+            for (int32_t x = 0; x < W; ++x) mine[x] = std::max(mine[x], theirs[x]);
+        }
+        mine[q] = static_cast<uint16_t>(at[v] + 1);
+    }
+    out.nbr_ptr.assign(n + 1, 0);
+    out.nbr.clear(); out.nbr_slot.clear(); out.nbr_rank.clear();
+    out.nbr.reserve(nbr.size()); out.nbr_slot.reserve(nbr.size()); out.nbr_rank.reserve(nbr.size());
+    for (int32_t i = 0; i < n; ++i) {
+        const int32_t v = out.node[i];
+        for (int32_t e = nbr_ptr[v]; e < nbr_ptr[v + 1]; ++e) {
+            out.nbr.push_back(nbr[e]);
+            out.nbr_slot.push_back(slot_of[nbr[e]]);
+            out.nbr_rank.push_back(rank[nbr[e]]);
+        }
+        out.nbr_ptr[i + 1] = static_cast<int32_t>(out.nbr.size());
+    }
+    out.entry_ptr.assign(W + 1, 0);
+    for (int32_t w = 0; w <= W; ++w) out.entry_ptr[w] = out.nbr_ptr[out.ptr[w]];
+}
+
+}  // namespace placeto

@@ -1,0 +1,126 @@
+"""The queues that the d = 32 sweep walks without levels (placeto_graph_queue_view): replayed on the CPU with the warps of a
+state taking their steps in an arbitrary order, as they may on the device. No GPU involved."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import paper_1906_08879_b200 as placeto
+from gen import configs
+from tests.helpers import random_dag, rng
+
+
+def _check_form(n, q, walkers, nbrs):
+    items = [range(q["ptr"][w], q["ptr"][w + 1]) for w in range(walkers)]
+    assert sorted(q["node"].tolist()) == list(range(n)) and q["ptr"][0] == 0 and q["ptr"][-1] == n
+    rank, step = q["key"] & 0xffff, q["key"] >> 16
+    assert sorted(rank.tolist()) == list(range(n)) and step.max() + 1 == q["n_steps"]
+    for v in range(n):
+        assert all(rank[u] < rank[v] and step[u] < step[v] for u in nbrs[v])
+    for w in range(walkers):
+        ranks = rank[q["node"][items[w].start:items[w].stop]]
+        assert (np.diff(ranks) > 0).all()                    # a queue is taken in filling order
+        for r in range(n):
+            assert q["first"][r, w] == (ranks < r).sum()
+    for i in range(n):
+        assert q["nbr"][q["nbr_ptr"][i]:q["nbr_ptr"][i + 1]].tolist() == nbrs[q["node"][i]]
+        assert bool(q["waits"][i]) == bool(q["need"][i].any())
+
+
+def _replay(n, q, walkers, start, pick):
+    """Every warp takes its items of rank >= start in order; `pick` says which of those that need not wait goes next. A message
+    is read where it was written, a slot is never taken from a reader that is still to come, and everybody arrives."""
+    node_rank = q["key"] & 0xffff
+    done = [int(q["first"][start, w]) for w in range(walkers)]
+    seen = list(done)                                        # what the others have been told
+    holder = np.full(max(1, q["n_slots"]), -1)
+    written = node_rank < start
+    for w in range(walkers):                                 # messages carried over the start
+        for i in range(q["ptr"][w] + done[w], q["ptr"][w + 1]):
+            for e in range(q["nbr_ptr"][i], q["nbr_ptr"][i + 1]):
+                if written[q["nbr"][e]]:
+                    s = q["nbr_slot"][e]
+                    assert holder[s] in (-1, q["nbr"][e])
+                    holder[s] = q["nbr"][e]
+    left = n - sum(done)
+    while left:
+        able = [w for w in range(walkers) if q["ptr"][w] + done[w] < q["ptr"][w + 1] and
+                (not q["waits"][q["ptr"][w] + done[w]] or all(seen[x] >= q["need"][q["ptr"][w] + done[w], x] for x in range(walkers)))]
+        assert able, "nobody can go on"
+        w = pick(able)
+        i = q["ptr"][w] + done[w]
+        for e in range(q["nbr_ptr"][i], q["nbr_ptr"][i + 1]):
+            assert written[q["nbr"][e]] and holder[q["nbr_slot"][e]] == q["nbr"][e]
+        v, s = q["node"][i], q["own_slot"][i]
+        written[v] = True
+        if s >= 0:
+            assert s < q["n_slots"]
+            holder[s] = v
+        done[w] += 1
+        if q["publishes"][i]:
+            seen[w] = done[w]
+        left -= 1
+
+
+def _check(n, src, dst, r, starts=3):
+    g = placeto.Graph(n, src, dst, host_only=True)
+    view = g.host_view()
+    for direction, name in ((0, "down"), (1, "up")):
+        v = view[name]
+        nbrs = [None] * n
+        for p in range(n):
+            nbrs[v["order"][p]] = v["nbr"][v["nbr_ptr"][p]:v["nbr_ptr"][p + 1]].tolist()
+        readers = np.zeros(n, dtype=bool)
+        readers[v["nbr"]] = True
+        for walkers in (1, 2, 4, 8):
+            q = g.queue_view(direction, walkers)
+            _check_form(n, q, walkers, nbrs)
+            assert ((q["own_slot"] >= 0) == readers[q["node"]]).all()
+            for start in [0] + [int(r.integers(0, n)) for _ in range(starts)]:
+                for pick in (min, max, lambda able: int(r.choice(able))):       # one warp as far ahead as it can, or any
+                    _replay(n, q, walkers, start, pick)
+    g.close()
+
+
+def test_small_shapes():
+    e, r = np.zeros(0, np.int32), rng(1)
+    _check(1, e, e, r)
+    _check(9, e, e, r)                                         # isolated nodes
+    _check(20, np.arange(19), np.arange(1, 20), r)             # chain
+    _check(40, np.zeros(39, np.int32), np.arange(1, 40), r)    # star out: more neighbours than a warp has lanes
+    _check(40, np.arange(1, 40), np.zeros(39, np.int32), r)    # star in
+    _check(4, [0, 0, 1, 2, 0], [1, 2, 3, 3, 3], r)             # diamond and a long edge past it
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_random_graphs(seed):
+    r = rng(500 + seed)
+    n = int(r.integers(2, 70))
+    src, dst = random_dag(r, n, float(r.uniform(0.02, 0.4)))
+    _check(n, src, dst, r)
+
+
+@pytest.mark.parametrize("name", ["tiny", "inception"])
+def test_workload_graphs(name):
+    cfg = configs.make(name, B=1)
+    _check(cfg["n"], cfg["src"], cfg["dst"], rng(7), starts=2)
+
+
+def test_chains_stay_in_their_queue():
+    """Six parallel chains between a fork and a join: of 8 warps six walk one each, and wait where they meet only."""
+    ids = np.arange(60).reshape(6, 10) + 1
+    src = np.concatenate([np.zeros(6, np.int64), ids[:, :-1].ravel(), ids[:, -1]])
+    dst = np.concatenate([ids[:, 0], ids[:, 1:].ravel(), np.full(6, 61)])
+    g = placeto.Graph(62, src, dst, host_only=True)
+    q = g.queue_view(0, 8)
+    assert q["n_steps"] == 12 and q["waits"].sum() == 6 and q["publishes"].sum() == 6 and q["n_slots"] <= 7
+    assert g.queue_view(0, 1)["waits"].sum() == 0
+    g.close()
+
+
+def test_bad_arguments():
+    g = placeto.Graph(3, [0, 1], [1, 2], host_only=True)
+    for direction, walkers in ((2, 1), (-1, 1), (0, 3), (0, 0), (1, 16)):
+        with pytest.raises(placeto.PlacetoError):
+            g.queue_view(direction, walkers)
+    g.close()
