@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(32 * kPoolWarps<D>)
 grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
     constexpr int C = D / 32, kWarps = kPoolWarps<D>, kThreads = 32 * kWarps;
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n = a.n, B = a.B, F = a.F, E = 2 * D + F, Ep = (E + 3) & ~3;
     float *W = smem;                                     // [3][Ep][D], zero padded
@@ -70,6 +71,7 @@ grad_pool_forward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
     l.node = reinterpret_cast<unsigned short *>(l.count + 4);
     for (int i = 0; i < 3; ++i)
         for (int t = threadIdx.x; t < Ep * D; t += kThreads) W[i * Ep * D + t] = t < E * D ? a.l[i].W1[t] : 0.f;
+    dependency_wait();          // (weights are the caller's)
     __syncthreads();
     const int items = B * chunks;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
@@ -134,6 +136,7 @@ __global__ void __launch_bounds__(32 * kPoolWarps<D>)
 grad_pool_backward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
     constexpr int C = D / 32, kWarps = kPoolWarps<D>, kThreads = 32 * kWarps;
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n = a.n, B = a.B;
     float *Wt = smem;                                    // [3][D][2 D]
@@ -147,6 +150,7 @@ grad_pool_backward_kernel(const GradArgs a, int chunk_nodes, int chunks) {
             const int q = t >> 5, j = q % (D / 8) * 8 + (t & 7), k = q / (D / 8) * 4 + (t >> 3 & 3);
             Wt[(i * D + j) * 2 * D + k] = a.l[i].W1[k * D + j];
         }
+    dependency_wait();
     __syncthreads();
     const int items = B * chunks;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
@@ -252,6 +256,7 @@ template <int D, int TK>
 __global__ void __launch_bounds__(D == 64 ? 192 : 128)
 grad_weight_rows_kernel(const RowJobs jobs, size_t R, int F, int chunks) {
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
     const RowJob w = jobs.job[blockIdx.y];
     const int K = D + (w.x ? F : 0), Kp = (K + TK) / TK * TK;
     const int stage = kStageRows * (Kp + D);
@@ -283,6 +288,7 @@ grad_weight_rows_kernel(const RowJobs jobs, size_t R, int F, int chunks) {
     float acc[TK][4];
 #pragma unroll
     for (int i = 0; i < TK; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+    dependency_wait();
     if (r_begin < r_end) load(r_begin, 0);
     int buffer = 0;
     for (size_t r0 = r_begin; r0 < r_end; r0 += kStageRows, buffer ^= 1) {
@@ -303,6 +309,7 @@ template <int D, int TK>
 __global__ void __launch_bounds__(D == 64 ? 320 : 192)
 grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const partial1, float *const partial2, int chunks) {
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
     const int set = blockIdx.y;
     const int n = a.n, B = a.B, F = a.F, K = 2 * D + F, Kp = (K + TK) / TK * TK;
     const int stage = kStageRows * (Kp + D);
@@ -337,6 +344,7 @@ grad_weight_pool_kernel(const GradArgs a, float *const partial0, float *const pa
     const int per = (n + chunks - 1) / chunks;
     const int u0 = blockIdx.x * per, u1 = min(n, u0 + per);
     const int parts = (B + kListStates - 1) / kListStates;
+    dependency_wait();
     int have = 0;
     for (int item = u0 * parts; item < u1 * parts; ++item) {
         const int u = item / parts, b0 = (item - u * parts) * kListStates, b1 = min(B, b0 + kListStates);
@@ -395,15 +403,17 @@ size_t backward_smem(int chunk_nodes) {
     return ((size_t)6 * D * D + (size_t)kPoolWarps<D> * kRowsPerWarp * D + 4) * sizeof(float) + (size_t)3 * chunk_nodes * 2;
 }
 
+// Only kernels of one block per SM start before the one in front has ended: blocks of a kernel with several per SM crowd onto
+// the SMs that run out of work first and stay there (all kernels of the gradient: 529 -> 645 us at d = 32).
 template <int D>
 cudaError_t launch_forward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
     const size_t smem = forward_smem<D>(a.F, a.pool_chunk_nodes);
     cudaError_t err = cudaFuncSetAttribute(grad_pool_forward_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int grid = std::min(a.B * a.pool_chunks, (D == 32 ? 3 : 1) * di.sm_count);
-    grad_pool_forward_kernel<D><<<grid, 32 * kPoolWarps<D>, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
+    err = launch_overlapped(D == 64, grad_pool_forward_kernel<D>, dim3(grid), dim3(32 * kPoolWarps<D>), smem, stream, a, a.pool_chunk_nodes, a.pool_chunks);
     count_launch();
-    return cudaGetLastError();
+    return err;
 }
 template <int D>
 cudaError_t launch_backward(const GradArgs &a, const DeviceInfo &di, cudaStream_t stream) {
@@ -411,9 +421,9 @@ cudaError_t launch_backward(const GradArgs &a, const DeviceInfo &di, cudaStream_
     cudaError_t err = cudaFuncSetAttribute(grad_pool_backward_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int grid = std::min(a.B * a.pool_chunks, (D == 32 ? 4 : 1) * di.sm_count);
-    grad_pool_backward_kernel<D><<<grid, 32 * kPoolWarps<D>, smem, stream>>>(a, a.pool_chunk_nodes, a.pool_chunks);
+    err = launch_overlapped(D == 64, grad_pool_backward_kernel<D>, dim3(grid), dim3(32 * kPoolWarps<D>), smem, stream, a, a.pool_chunk_nodes, a.pool_chunks);
     count_launch();
-    return cudaGetLastError();
+    return err;
 }
 
 template <int D, int TK>
@@ -432,14 +442,15 @@ cudaError_t launch_weights(const GradArgs &a, float *const (&rows)[8], int row_c
     size_t smem = (size_t)2 * kStageRows * (Kp + D) * sizeof(float);
     cudaError_t err = cudaFuncSetAttribute(grad_weight_rows_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    grad_weight_rows_kernel<D, TK><<<dim3(row_chunks, 8), threads, smem, stream>>>(jobs, (size_t)a.n * a.B, a.F, row_chunks);
+    err = launch_overlapped(false, grad_weight_rows_kernel<D, TK>, dim3(row_chunks, 8), dim3(threads), smem, stream, jobs, (size_t)a.n * a.B, a.F, row_chunks);
+    if (err != cudaSuccess) return err;
     count_launch();
     smem = (size_t)2 * kStageRows * (Lp + D) * sizeof(float) + (size_t)(std::min(a.B, kListStates) + kStageRows) * sizeof(int);
     err = cudaFuncSetAttribute(grad_weight_pool_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    grad_weight_pool_kernel<D, TK><<<dim3(pool_chunks, 3), pool_threads, smem, stream>>>(a, pool[0], pool[1], pool[2], pool_chunks);
+    err = launch_overlapped(false, grad_weight_pool_kernel<D, TK>, dim3(pool_chunks, 3), dim3(pool_threads), smem, stream, a, pool[0], pool[1], pool[2], pool_chunks);
     count_launch();
-    return cudaGetLastError();
+    return err;
 }
 
 }  // namespace

@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(kRowThreads)
 grad_rows_f_kernel(const GradArgs a) {
     constexpr int C = D / 32;
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
     const int dir = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const DevMlp f = a.f[dir];
     const int F = a.F, K = (D + F + 3) & ~3;
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(kRowThreads, D == 64 ? 4 : 3)
 grad_rows_g_kernel(const GradArgs a) {
     constexpr int C = D / 32;
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
     const int dir = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const DevMlp gn = a.g[dir];
     const DevLevels lv = a.lv[dir];
@@ -171,6 +173,7 @@ grad_rows_g_kernel(const GradArgs a) {
     float b1[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) b1[c] = gn.b1[lane + 32 * c];
+    dependency_wait();          // the messages come from a kernel that may still be running
     const float *M = a.M[dir];
     const int B = a.B;
     const size_t R = (size_t)a.n * B;
@@ -347,6 +350,7 @@ grad_sweep_split_kernel(const GradArgs a, const SweepPlan p) {
     typedef SweepConfig<D> C;
     constexpr int KS = C::KS, P = C::P;
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int group = warp / C::W, c0 = 16 * (warp % C::W);
     const int gt = threadIdx.x % C::kGroupThreads;
@@ -412,6 +416,7 @@ grad_sweep_split_kernel(const GradArgs a, const SweepPlan p) {
             __pipeline_commit();
         };
         __syncthreads();              // schedule staged
+        dependency_wait();
         publish(0);
         publish(1);
         __pipeline_wait_prior(1);
@@ -441,6 +446,7 @@ grad_sweep_split_kernel(const GradArgs a, const SweepPlan p) {
     const int rr = gt / kLanes, c4 = 4 * (gt % kLanes);
     unsigned char *gather_to = tiles + rr * C::kStride + 2 * c4;
     __syncthreads();                  // schedule and third pieces staged
+    dependency_wait();
 
     auto run = [&](const unsigned char *info) {
         // ---- this lane's d/dh from the pooling, asked for well before it is used
@@ -577,9 +583,11 @@ cudaError_t launch_rows(const GradArgs &a, const DeviceInfo &di, cudaStream_t st
     if (err != cudaSuccess) return err;
     grad_rows_f_kernel<D><<<dim3(blocks, 2), kRowThreads, smem_f, stream>>>(a);
     count_launch();
-    grad_rows_g_kernel<D><<<dim3(blocks_g, 2), kRowThreads, smem_g, stream>>>(a);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    err = launch_overlapped(true, grad_rows_g_kernel<D>, dim3(blocks_g, 2), dim3(kRowThreads), smem_g, stream, a);
     count_launch();
-    return cudaGetLastError();
+    return err;
 }
 
 template <int D>
@@ -588,9 +596,9 @@ cudaError_t launch_sweep(const GradArgs &a, const DeviceInfo &di, cudaStream_t s
     if (!plan_sweep<D>(a, di, &p)) return cudaErrorNotSupported;
     cudaError_t err = cudaFuncSetAttribute(grad_sweep_split_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);
     if (err != cudaSuccess) return err;
-    grad_sweep_split_kernel<D><<<dim3(p.n_slices, 2), kThreads, p.smem_bytes, stream>>>(a, p);
+    err = launch_overlapped(true, grad_sweep_split_kernel<D>, dim3(p.n_slices, 2), dim3(kThreads), p.smem_bytes, stream, a, p);
     count_launch();
-    return cudaGetLastError();
+    return err;
 }
 
 }  // namespace

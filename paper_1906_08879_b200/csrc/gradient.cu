@@ -274,7 +274,14 @@ __device__ __forceinline__ float strided_dot(float init, const float *x, const f
 #pragma unroll
         for (int t = 0; t < 16; ++t) acc = fmaf(x[k + t], v[t], acc);
     }
-    for (; k < K; ++k) acc = fmaf(x[k], __ldg(w + (size_t)k * stride), acc);
+    if (k < K) {                           // the rest together too: one by one each was a round trip to L2
+        float v[16];
+#pragma unroll
+        for (int t = 0; t < 16; ++t) v[t] = k + t < K ? __ldg(w + (size_t)(k + t) * stride) : 0.f;
+#pragma unroll
+        for (int t = 0; t < 16; ++t)
+            if (k + t < K) acc = fmaf(x[k + t], v[t], acc);
+    }
     return acc;
 }
 
@@ -293,7 +300,9 @@ grad_head_pooled_kernel(const GradArgs a, const int staged) {      // staged: fl
     float *part = lg + m;                  // [8][3][d] sums over the nodes of one residue
     float *w2 = part + 8 * 3 * d;          // [Hh][m]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    dependents_may_start();
     for (int i = threadIdx.x; i < staged; i += kHeadThreads) w2[i] = a.head.W2[i];
+    dependency_wait();
     const float *W2 = staged > 0 ? w2 : a.head.W2;
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
         const int c = a.cur[b];
@@ -619,6 +628,8 @@ struct WeightJobs {
 __global__ void __launch_bounds__(kThreads)
 grad_weight_partial_kernel(const WeightJobs jobs) {
     extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
+    dependency_wait();
     const WeightJob &w = jobs.job[blockIdx.z];
     const int K = w.K, J = w.J;
     const int Kp = (K + 1 + 3) & ~3, Jp = (J + 3) & ~3;      // padded with zeros to whole 4 x 4 tiles
@@ -640,19 +651,19 @@ grad_weight_partial_kernel(const WeightJobs jobs) {
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     for (size_t r0 = r_begin; r0 < r_end; r0 += kRows) {
         const int rows = (int)min((size_t)kRows, r_end - r0);
-        for (int i = threadIdx.x; i < rows * Kp; i += kThreads) {
-            const int r = i / Kp, k = i - r * Kp;
-            float v = k == K ? 1.f : 0.f;
-            if (k < K) {
-                int kk = k, part = 0;
-                while (kk >= w.width[part]) { kk -= w.width[part]; ++part; }
-                v = w.in[part][(r0 + r) * w.stride[part] + kk];
+        // a warp per row: looked up element by element (a division, a search for its part) the loads of the head's 332 columns
+        // took most of the kernel
+        for (int r = threadIdx.x >> 5; r < rows; r += kThreads / 32) {
+            float *to = in + r * Kp;
+            for (int part = 0, at = 0; at < K; at += w.width[part], ++part) {
+                const float *from = w.in[part] + (r0 + r) * w.stride[part];
+#pragma unroll 4
+                for (int k = threadIdx.x & 31; k < w.width[part]; k += 32) to[at + k] = from[k];
             }
-            in[i] = v;
-        }
-        for (int i = threadIdx.x; i < rows * Jp; i += kThreads) {
-            const int r = i / Jp, j = i - r * Jp;
-            dp[i] = j < J ? w.dp[(r0 + r) * w.dp_stride + j] : 0.f;
+            for (int k = K + (threadIdx.x & 31); k < Kp; k += 32) to[k] = k == K ? 1.f : 0.f;
+            const float *from = w.dp + (r0 + r) * w.dp_stride;
+#pragma unroll 4
+            for (int j = threadIdx.x & 31; j < Jp; j += 32) dp[r * Jp + j] = j < J ? from[j] : 0.f;
         }
         __syncthreads();
         if (live) {
@@ -683,51 +694,79 @@ grad_weight_partial_kernel(const WeightJobs jobs) {
 
 // Adds the chunk partials: a block owns 32 outputs; eight thread groups each add
 // every eighth chunk (ascending), then the eight sums are added in group order.
+// Chunk partials added up in a fixed order: eight sums of every eighth chunk, then those (with at most eight chunks that is the
+// chunks in turn, which a thread does alone).
 __global__ void __launch_bounds__(256)
 grad_weight_reduce_kernel(const WeightJobs jobs) {
     __shared__ float sums[8][32];
+    dependents_may_start();
+    dependency_wait();
     const WeightJob &w = jobs.job[blockIdx.y];
     const int n_out = (w.K + 1) * w.J;
-    if ((int)blockIdx.x * 32 >= n_out) return;
+    const bool few = w.chunks <= 8;
+    if ((int)blockIdx.x * (few ? 256 : 32) >= n_out) return;
     const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    const int o = blockIdx.x * 32 + lane;
+    const int o = few ? blockIdx.x * 256 + threadIdx.x : blockIdx.x * 32 + lane;
+    auto store = [&](float total) {
+        float *dst = o < w.K * w.J ? w.dW + o : w.db + (o - w.K * w.J);
+        *dst = w.accumulate ? *dst + total : total;
+    };
     float acc = 0.f;
     if (o < n_out)
-        for (int c = grp; c < w.chunks; c += 8) acc += w.partial[(size_t)c * n_out + o];
+        for (int c0 = few ? 0 : grp; c0 < w.chunks; c0 += few ? 8 : 64) {       // eight loads in flight
+            float v[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const int c = c0 + t * (few ? 1 : 8);
+                v[t] = c < w.chunks ? w.partial[(size_t)c * n_out + o] : 0.f;
+            }
+#pragma unroll
+            for (int t = 0; t < 8; ++t) acc += v[t];
+        }
+    if (few) {
+        if (o < n_out) store(acc);
+        return;
+    }
     sums[grp][lane] = acc;
     __syncthreads();
     if (grp == 0 && o < n_out) {
         float total = 0.f;
 #pragma unroll
         for (int q = 0; q < 8; ++q) total += sums[q][lane];
-        float *dst = o < w.K * w.J ? w.dW + o : w.db + (o - w.K * w.J);
-        *dst = w.accumulate ? *dst + total : total;
+        store(total);
     }
 }
 
 // sums the jobs' chunks into their gradients, after computing them unless another kernel has (`products`)
-cudaError_t weight_grads(const WeightJobs &jobs, cudaStream_t stream, bool products) {
+// the products of a list of jobs; their partials are added up by reduce_weight_grads
+cudaError_t weight_products(const WeightJobs &jobs, cudaStream_t stream, bool overlap) {
     if (jobs.count == 0) return cudaSuccess;
     size_t smem = 0;
-    int max_chunks = 1, max_out = 1, max_tiles = 1;
+    int max_chunks = 1, max_tiles = 1;
     for (int i = 0; i < jobs.count; ++i) {
         const WeightJob &w = jobs.job[i];
         const int Kp = (w.K + 1 + 3) & ~3, Jp = (w.J + 3) & ~3;
         smem = std::max(smem, (size_t)kRows * (Kp + Jp) * sizeof(float));
         max_chunks = std::max(max_chunks, w.chunks);
-        max_out = std::max(max_out, (w.K + 1) * w.J);
         max_tiles = std::max(max_tiles, (Kp / 4) * (Jp / 4));
     }
-    if (products) {
-        const cudaError_t err = cudaFuncSetAttribute(grad_weight_partial_kernel,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess) return err;
-        grad_weight_partial_kernel<<<dim3(max_chunks, (max_tiles + kThreads - 1) / kThreads, jobs.count), kThreads, smem, stream>>>(jobs);
-        count_launch();
-    }
-    grad_weight_reduce_kernel<<<dim3((max_out + 31) / 32, jobs.count), 256, 0, stream>>>(jobs);
+    cudaError_t err = cudaFuncSetAttribute(grad_weight_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    err = launch_overlapped(overlap, grad_weight_partial_kernel, dim3(max_chunks, (max_tiles + kThreads - 1) / kThreads, jobs.count),
+                            dim3(kThreads), smem, stream, jobs);
     count_launch();
-    return cudaGetLastError();
+    return err;
+}
+
+cudaError_t reduce_weight_grads(const WeightJobs &jobs, cudaStream_t stream) {
+    int blocks = 1;
+    for (int i = 0; i < jobs.count; ++i) {
+        const int per = jobs.job[i].chunks <= 8 ? 256 : 32;
+        blocks = std::max(blocks, ((jobs.job[i].K + 1) * jobs.job[i].J + per - 1) / per);
+    }
+    const cudaError_t err = launch_overlapped(true, grad_weight_reduce_kernel, dim3(blocks, jobs.count), dim3(256), 0, stream, jobs);
+    count_launch();
+    return err;
 }
 
 }  // namespace
@@ -830,7 +869,8 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
             const size_t smem = (own + staged) * sizeof(float);
             err = cudaFuncSetAttribute(grad_head_pooled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (err != cudaSuccess) return err;
-            grad_head_pooled_kernel<<<std::min(B, 2 * di.sm_count), kHeadThreads, smem, stream>>>(a, staged);
+            err = launch_overlapped(true, grad_head_pooled_kernel, dim3(std::min(B, 2 * di.sm_count)), dim3(kHeadThreads), smem, stream, a, staged);
+            if (err != cudaSuccess) return err;
         } else {
             const size_t floats = vectors + ((m + 3) & ~3) + (size_t)(kThreads / 32) * 3 * d +
                                   (size_t)(kThreads / 32) * ((E + 3) & ~size_t(3)) + 3 * (E * d + d);
@@ -913,9 +953,14 @@ cudaError_t launch_policy_gradient(GradArgs a, const DeviceInfo &di, float *ws, 
         err = launch_grad_weights_split(a, rows, row_chunks, pool, pool_chunks, stream);
         if (err != cudaSuccess) return err;
     }
-    err = weight_grads(by_row, stream, !split);
+    if (!split) err = weight_products(by_row, stream, false);
     if (err != cudaSuccess) return err;
-    return weight_grads(by_state, stream, true);
+    err = weight_products(by_state, stream, true);
+    if (err != cudaSuccess) return err;
+    WeightJobs all = by_row;
+    std::copy(by_state.job, by_state.job + by_state.count, all.job + all.count);
+    all.count += by_state.count;
+    return reduce_weight_grads(all, stream);
 }
 
 }  // namespace placeto
