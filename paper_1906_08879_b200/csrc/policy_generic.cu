@@ -388,7 +388,8 @@ __device__ __forceinline__ float4 load_row4(const float *__restrict__ p, int lef
 
 template <int HS, int VEC>
 __global__ void __launch_bounds__(kFastThreads, 1)
-pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: floats of h_i's weights kept in shared memory
+pool_head_fast_kernel(const PoolArgs a, const int staged_h, const int staged_w2) {   // floats of h_i's weights and of the head's
+                                                                                   // last matrix kept in shared memory
     constexpr int SR = HS < 4 ? HS : 4;     // states of a thread tile (all eight: 21.0 -> 23.5 us for 992 states, more to add up)
     constexpr int SG = HS / SR;             // state groups
     extern __shared__ __align__(16) float smem[];
@@ -400,15 +401,23 @@ pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: 
     float *sum = zt + Z * HS;                      // [HS][3 d]
     float *hid = sum + HS * 3 * d;                 // [Hp][HS]
     float *lg = hid + Hp * HS;                     // [HS][m]
-    float *red = lg + ((HS * m + 3) & ~3);         // [parts][Hp][HS]
+    float *share = lg + HS * m;                    // [HS][m], the softmax
+    float *bh = share + HS * m;                    // [3][d] biases of h_i, [Hd] and [m] of the head, the head's last matrix transposed
+    float *b1 = bh + 3 * d, *b2 = b1 + Hd, *w2 = b2 + m;                 // w2[m][Hd]
+    float *red = lg + ((2 * HS * m + 3 * d + Hd + m + staged_w2 + 3) & ~3);     // [parts][Hp][HS]
     const int b0 = blockIdx.x * HS;
     // Weights do not depend on the kernel before: those of h_i go to shared memory, this thread's first rows of the head
-    // into registers, while it runs or while the sums below are on their way. Reading them where they are used cost a
-    // round trip to L2 in each layer (a step of 16 episodes of 151 nodes: 10.6 -> 8.5 us).
+    // into registers, while it runs or while the sums below are on their way; so do the biases and the last matrix. Reading
+    // them where they are used cost a round trip to L2 in each layer (a step of 16 episodes of 151 nodes: 10.6 -> 8.5 us, the
+    // whole step 46.4 -> 45.2 with biases and last matrix).
     for (int i = threadIdx.x; i < staged_h / 4; i += blockDim.x) {
         const int set = i / (d * d / 4);
         __pipeline_memcpy_async(hw + 4 * i, a.h[set].W1 + 4 * (i - set * (d * d / 4)), 16);
     }
+    for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) __pipeline_memcpy_async(bh + i, a.h[i / d].b1 + i % d, 4);
+    for (int i = threadIdx.x; i < Hd; i += blockDim.x) __pipeline_memcpy_async(b1 + i, a.head.b1 + i, 4);
+    for (int i = threadIdx.x; i < m; i += blockDim.x) __pipeline_memcpy_async(b2 + i, a.head.b2 + i, 4);
+    for (int i = threadIdx.x; i < staged_w2; i += blockDim.x) __pipeline_memcpy_async(w2 + (i % m) * Hd + i / m, a.head.W2 + i, 4);
     __pipeline_commit();
     const int CG = Hp >> 2, tiles = SG * CG;
     const int parts = max(1, min((int)blockDim.x / tiles, Z));
@@ -424,7 +433,6 @@ pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: 
     };
     load_head(k0);
     prefetch_l2(a.head.W1, (size_t)Z * Hd);
-    prefetch_l2(a.head.W2, (size_t)Hd * m);
     float uniform = 0.f;
     int visit = -1, next_visit = -1;               // of the step: the node whose device is chosen, the one after
     if (a.step.enabled && threadIdx.x < HS && b0 + threadIdx.x < B) {
@@ -473,7 +481,8 @@ pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: 
         const DevMlp &nt = a.h[set];
         const float *W = (staged_h > 0 ? hw + set * d * d : nt.W1) + 4 * cq;
         const float *v = sum + s * 3 * d + set * d;
-        float4 acc = *reinterpret_cast<const float4 *>(nt.b1 + 4 * cq), odd = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float *bias = bh + set * d + 4 * cq;
+        float4 acc = make_float4(bias[0], bias[1], bias[2], bias[3]), odd = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
         for (int k = 0; k < d; k += 2) {           // two chains: shorter, and less rounding in each (d is a multiple of 4)
             const float4 w0 = *reinterpret_cast<const float4 *>(W + k * d), w1 = *reinterpret_cast<const float4 *>(W + (k + 1) * d);
@@ -531,7 +540,7 @@ pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: 
     __syncthreads();
     const bool relu = a.head.act == 0;
     for (int i = threadIdx.x; i < Hd * HS; i += blockDim.x) {
-        float acc = a.head.b1[i / HS];
+        float acc = b1[i / HS];
         for (int q = 0; q < parts; ++q) acc += red[(size_t)q * Hp * HS + i];
         hid[i] = relu ? fmaxf(acc, 0.f) : acc;
     }
@@ -542,10 +551,10 @@ pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: 
         for (int item = warp; item < HS * m; item += nw) {
             const int s = item / m, j = item - s * m;
             float acc = 0.f;
-            for (int k = lane; k < Hd; k += 32) acc = fmaf(hid[k * HS + s], a.head.W2[(size_t)k * m + j], acc);
+            for (int k = lane; k < Hd; k += 32) acc = fmaf(hid[k * HS + s], staged_w2 > 0 ? w2[j * Hd + k] : a.head.W2[(size_t)k * m + j], acc);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            acc += a.head.b2[j];
+            acc += b2[j];
             if (lane == 0) lg[s * m + j] = (relu && a.head.final_act) ? fmaxf(acc, 0.f) : acc;
         }
     }
@@ -558,10 +567,15 @@ pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: 
         float mx = l[0];
         for (int k = 1; k < m; ++k) mx = fmaxf(mx, l[k]);
         float tot = 0.f;
-        for (int k = 0; k < m; ++k) tot += expf(l[k] - mx);
+        float *p = share + threadIdx.x * m;
         for (int k = 0; k < m; ++k) {
+            p[k] = expf(l[k] - mx);
+            tot += p[k];
+        }
+        for (int k = 0; k < m; ++k) {
+            p[k] /= tot;
             a.logits[(size_t)b * m + k] = valid ? l[k] : nanf("");
-            if (a.probs) a.probs[(size_t)b * m + k] = valid ? expf(l[k] - mx) / tot : nanf("");
+            if (a.probs) a.probs[(size_t)b * m + k] = valid ? p[k] : nanf("");
         }
         if (a.step.enabled) {
             // The MDP transition of episode b (Sec. 2.1), fused here: greedy takes the largest
@@ -578,7 +592,7 @@ pool_head_fast_kernel(const PoolArgs a, const int staged_h) {      // staged_h: 
                 float cum = 0.f;
                 action = m - 1;
                 for (int k = 0; k < m; ++k) {
-                    cum += expf(l[k] - mx) / tot;
+                    cum += p[k];
                     if (cum > u) { action = k; break; }
                 }
             }
@@ -607,16 +621,23 @@ cudaError_t launch_head_fast(const PoolArgs &a, cudaStream_t stream) {
     const size_t floats = (size_t)Z * HS + (size_t)HS * 3 * a.d + (size_t)Hd * HS + ((HS * a.m + 3) & ~3) +
                           (size_t)parts * Hd * HS;
     if (floats * sizeof(float) > 200 * 1024) return cudaErrorNotSupported;
-    const int staged_h = (floats + (size_t)3 * a.d * a.d) * sizeof(float) <= 200 * 1024 ? 3 * a.d * a.d : 0;
-    const size_t bytes = (floats + staged_h) * sizeof(float);
-    void (*kern)(const PoolArgs, const int) = (a.head.hidden_dim & 3) == 0   ? pool_head_fast_kernel<HS, 4>
+    // (the softmax and the biases always fit on top of that; the weights where there is room)
+    size_t all = floats + HS * a.m + 3 * a.d + a.head.hidden_dim + a.m + 4;
+    auto stage = [&](size_t more) {
+        if ((all + more) * sizeof(float) > 200 * 1024) return 0;
+        all += more;
+        return (int)more;
+    };
+    const int staged_h = stage((size_t)3 * a.d * a.d), staged_w2 = stage((size_t)a.head.hidden_dim * a.m);
+    const size_t bytes = all * sizeof(float);
+    void (*kern)(const PoolArgs, const int, const int) = (a.head.hidden_dim & 3) == 0   ? pool_head_fast_kernel<HS, 4>
                                    : (a.head.hidden_dim & 1) == 0 ? pool_head_fast_kernel<HS, 2>
                                                                   : pool_head_fast_kernel<HS, 1>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (err != cudaSuccess) return err;
     // always preceded by one of this library's pooling kernels on the same stream
     err = launch_overlapped(true, kern, dim3((a.B + HS - 1) / HS), dim3(kFastThreads),
-                            bytes, stream, a, staged_h);
+                            bytes, stream, a, staged_h, staged_w2);
     count_launch();
     return err;
 }
