@@ -33,7 +33,7 @@ LIB = os.path.join(HERE, "libplaceto.so")
 LIB_DEBUG = os.path.join(HERE, "libplaceto_debug.so")
 LIB_TIMERS = os.path.join(HERE, "libplaceto_timers.so")
 
-SOURCES = ["api.cu", "plan.cpp", "queues.cpp", "features.cu", "embed_generic.cu", "embed_d32.cu", "embed_d64.cu", "embed_pipe.cu", "embed_split.cu", "embed_small.cu", "embed_tc.cu",
+SOURCES = ["api.cu", "plan.cpp", "queues.cpp", "features.cu", "embed_generic.cu", "embed_d32.cu", "embed_levels_d32.cu", "embed_d64.cu", "embed_pipe.cu", "embed_split.cu", "embed_small.cu", "embed_tc.cu",
            "policy_generic.cu", "policy_d32.cu", "pool_split.cu", "policy_d64.cu", "episode.cu",
            "embed_rounds_d32.cu", "simulator.cu", "gradient.cu", "grad_sweep.cu", "grad_pool.cu", "status.cu", "aggregator.cu", "policy_tc.cu"]
 

@@ -345,7 +345,10 @@ placeto_status run_embed(const placeto_graph *g, const placeto_weights *w, const
         if (e != cudaErrorNotSupported) return cuda_status(e);
     }
     if (!(flags & PLACETO_GENERIC) && schedule == PLACETO_SLICED && embed_d32_applicable(a)) {
-        cudaError_t e = launch_embed_d32(a, g->info, stream, after_own_kernel);
+        const bool levels = walk.order == nullptr && embed_levels_d32_preferred(a, g->info);
+        cudaError_t e = levels ? launch_embed_levels_d32(a, g->info, stream, after_own_kernel) : launch_embed_d32(a, g->info, stream, after_own_kernel);
+        if (e == cudaErrorNotSupported)          // either's plan of the graph may be too large for shared memory
+            e = levels ? launch_embed_d32(a, g->info, stream, after_own_kernel) : launch_embed_levels_d32(a, g->info, stream, after_own_kernel);
         if (e != cudaErrorNotSupported) return cuda_status(e);
     }
     if (!(flags & PLACETO_GENERIC) && schedule == PLACETO_SLICED && embed_d64_applicable(a)) {

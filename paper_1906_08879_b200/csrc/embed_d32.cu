@@ -123,8 +123,9 @@ __device__ __forceinline__ void matvec_halves(const pair_t (&w)[K / 2], const pa
     }
 }
 
-// How a warp lays out a row: which column a lane owns, where input k of a K-wide product lies. One state per warp takes whole
-// columns (the exchange would lie on the chain of layers: 95 -> 97 us with one state), two take halves (the shared loads).
+// How a warp lays out a row: which column a lane owns, where input k of a K-wide product lies. Where a
+// few warps work the exchange would lie on the chain of layers (an episode's steps 46 -> 49 us): whole columns. Where all eight do, the
+// shared loads are what they wait for: halves (279 nodes, 256 states: whole forward 101.4 -> 98.4 us; always with two states).
 template <bool kHalves> struct Layout32 {
     typedef pair_t Bias[kHalves ? 2 : 1];       // the first addends of a lane's chains
     static __device__ __forceinline__ int column(int lane) { return kHalves ? 2 * (lane & 15) + (lane >> 4) : lane; }
@@ -187,10 +188,10 @@ __device__ __host__ constexpr int warp_floats(int R) { return 2 * R * (kD + 16) 
 
 // F4: raw features, in groups of four; kSource: 0 features from X, 1 the same in a step of an episode, 2 an episode's compact
 // states; L layers per network; R states of a node that a warp carries together
-template <int F4, int kSource, int L, int R>
+template <int F4, int kSource, int L, int R, bool kHalves = R == 2>
 __global__ void __launch_bounds__(kThreads, 1)
 embed_d32_kernel(const EmbedArgs a, const __grid_constant__ D32Plan p) {
-    constexpr bool kWalk = kSource > 0, kCompact = kSource == 2, kHalves = R == 2;
+    constexpr bool kWalk = kSource > 0, kCompact = kSource == 2;
     constexpr int KF = kHalves ? kD + 8 * ((F4 + 1) / 2) : kD + 4 * F4;      // padded input width of f's first layer
     typedef Layout32<kHalves> Rows;
     extern __shared__ __align__(16) float smem[];
@@ -278,8 +279,23 @@ embed_d32_kernel(const EmbedArgs a, const __grid_constant__ D32Plan p) {
 #endif
     dependency_wait();          // the raw features may come from a kernel that is still running
 
+    // more states than teams: in rounds, whose counts of items go on from each other
+    const int other_items = q.ptr[min(lane & 7, W - 1) + 1] - q.ptr[min(lane & 7, W - 1)];
+    int done = 0, others_done = 0;       // in earlier rounds: this queue's items, those of the queue that this lane looks at
 #pragma unroll 1
-    for (int group = g0; group < g1; group += teams) {
+    for (int group = g0; group < g1; group += teams, done += end, others_done += other_items) {
+        if (!kWalk && k > 0 && group != g0) {      // the slots are free again when the others are through as well
+            __syncwarp();
+            store_release_if(lane == 0, &progress[warp], done);
+            int polls = 0;
+            while (!__all_sync(0xffffffffu, load_acquire(others) >= others_done))
+                if (++polls > kMaxPolls) break;
+            if (polls > kMaxPolls) {
+                if (lane == 0) report_status(a.status, PLACETO_ERR_TIMEOUT);
+                return;
+            }
+            __syncwarp();
+        }
         int b[R];                // the states; a missing last one repeats the first
 #pragma unroll
         for (int r = 0; r < R; ++r) b[r] = r == 0 || group * R + r < B ? group * R + r : group * R;
@@ -364,7 +380,8 @@ embed_d32_kernel(const EmbedArgs a, const __grid_constant__ D32Plan p) {
                 // neighbours come in groups of four, the last one filled up with the slot of zeros
                 const uint2 *more = info + item.z + 2;
                 uint2 four = more[0];
-                const int wanted = reinterpret_cast<const unsigned short *>(more - 2)[lane & 7];
+                int wanted = reinterpret_cast<const unsigned short *>(more - 2)[lane & 7];
+                if constexpr (!kWalk) wanted += wanted > 0 ? others_done : 0;
                 if (!__all_sync(0xffffffffu, load_acquire(others) >= wanted)) {
                     if (item.w & kQueueEnd) return false;            // (its wait is for more items than there are)
                     int polls = 0;
@@ -378,6 +395,7 @@ embed_d32_kernel(const EmbedArgs a, const __grid_constant__ D32Plan p) {
 #pragma unroll 1
                 while (true) {
                     const unsigned word[2] = {four.x, four.y};
+                    four = *++more;                      // (behind the last ones lie others' or messages)
                     float t[4][R];
 #pragma unroll
                     for (int n = 0; n < 4; ++n) {
@@ -393,7 +411,6 @@ embed_d32_kernel(const EmbedArgs a, const __grid_constant__ D32Plan p) {
                     }
                     left -= 4;
                     if (left <= 0) break;
-                    four = *++more;
                 }
 #pragma unroll
                 for (int r = 0; r < R; ++r) A[r * KF + at32] = acc[r];
@@ -457,7 +474,7 @@ embed_d32_kernel(const EmbedArgs a, const __grid_constant__ D32Plan p) {
             }
             copies_wait<1>();
             __syncwarp();                                // the message is there, the buffers are free, the next copies have come
-            if constexpr (!kPlain) store_release_if((item.w & kQueuePublishes) && lane == 0, &progress[warp], i + 1);
+            if constexpr (!kPlain) store_release_if((item.w & kQueuePublishes) && lane == 0, &progress[warp], (kWalk ? 0 : done) + i + 1);
             item = item_next;
             ahead = ahead_next;
             return true;
@@ -514,7 +531,8 @@ bool plan_d32(const EmbedArgs &a, const DeviceInfo &di, D32Launch *out) {
     };
     // One or two states per warp, by the steps that the longer direction takes; an item of two takes 1.25 to 1.45 times as long
     // (us, one and two: 279 nodes of 2.1 a level, 256 states 82, 80, 148 states 55, 67, 592 states 143, 115; 1080 of
-    // 6.6: 354, 270; 207, 180; 694, 475).
+    // 6.6: 354, 270; 207, 180; 694, 475). Where there are more states than teams, or shared memory holds the slots of a few
+    // only, a form with fewer teams may take fewer steps over all its rounds (the second graph, 992 states: 1337 -> 967).
     D32Plan &p = out->plan;
     const bool walk = a.walk.order != nullptr;
     long long best = -1;
@@ -523,14 +541,17 @@ bool plan_d32(const EmbedArgs &a, const DeviceInfo &di, D32Launch *out) {
         for (int k = 0; k < kQueuePlanCount; ++k) teams[k] = fits(k, pair);
         if (teams[0] < 1) continue;
         const int groups = (a.B + pair - 1) / pair, most = (groups + std::min(half, groups) - 1) / std::min(half, groups);
-        const int k = form_for(most, teams);
-        const long long cost = (long long)std::max(a.queues[0][k].n_steps, a.queues[1][k].n_steps) * ((most + teams[k] - 1) / teams[k]) * (pair == 2 ? 13 : 10);
-        if (best >= 0 && cost >= best) continue;
-        best = cost;
-        out->pair = pair;
-        p.groups = groups;
-        std::copy(teams, teams + kQueuePlanCount, p.teams);
-        p.form = k;
+        for (int k = kQueuePlanCount - 1; k >= 0; --k) {
+            if (teams[k] < 1 || (walk && k != form_for(most, teams))) continue;
+            const int rounds = (most + teams[k] - 1) / teams[k];
+            const long long cost = (long long)std::max(a.queues[0][k].n_steps, a.queues[1][k].n_steps) * rounds * (pair == 2 ? 13 : 10);
+            if (best >= 0 && cost >= best) continue;
+            best = cost;
+            out->pair = pair;
+            p.groups = groups;
+            std::copy(teams, teams + kQueuePlanCount, p.teams);
+            p.form = k;
+        }
     }
     if (best < 0) return false;
     p.blocks = 2 * std::min(half, p.groups);
@@ -564,7 +585,12 @@ cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStrea
         {PLACETO_D32_SOURCES(1, 1), PLACETO_D32_SOURCES(2, 1)}, {PLACETO_D32_SOURCES(1, 2), PLACETO_D32_SOURCES(2, 2)}};
 #undef PLACETO_D32_SOURCES
 #undef PLACETO_D32_KERNELS
-    const Kernel kern = kernels[l.pair - 1][a.f[0].n_layers - 1][a.compact.state != nullptr ? 2 : a.walk.order != nullptr ? 1 : 0][F4 - 1];
+    // one or two warps per state: all eight are at work (form 2 and 3 on narrow graphs leave some idle)
+    static const Kernel halves[2][4] = {
+        {embed_d32_kernel<1, 0, 1, 1, true>, embed_d32_kernel<2, 0, 1, 1, true>, embed_d32_kernel<3, 0, 1, 1, true>, embed_d32_kernel<4, 0, 1, 1, true>},
+        {embed_d32_kernel<1, 0, 2, 1, true>, embed_d32_kernel<2, 0, 2, 1, true>, embed_d32_kernel<3, 0, 2, 1, true>, embed_d32_kernel<4, 0, 2, 1, true>}};
+    const bool half = l.pair == 1 && l.plan.form <= 1 && a.walk.order == nullptr;
+    const Kernel kern = half ? halves[a.f[0].n_layers - 1][F4 - 1] : kernels[l.pair - 1][a.f[0].n_layers - 1][a.compact.state != nullptr ? 2 : a.walk.order != nullptr ? 1 : 0][F4 - 1];
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem_bytes);
     if (err != cudaSuccess) return err;
     err = launch_overlapped(overlap, kern, dim3(l.plan.blocks), dim3(kThreads), l.smem_bytes, stream, a, l.plan);

@@ -1,0 +1,391 @@
+// Step 2 of the policy (Sec. 2.2 step 2 of the Placeto paper), d = 32, ReLU networks of one layer or of two: the arithmetic
+// and the bits of embed_d32.cu with a block barrier between the levels of the graph, for batches that its queues serve less well.
+//
+//   - A block owns one direction and a slice of the state batch and walks all levels; lane j of every warp keeps column j of all four
+//     weight matrices in registers. A level's (node, two states) items are dealt to the eight warps, so any number of states
+//     keeps them busy on a graph of several nodes per level, where the queues carry whole sets of 8 or 16 states.
+//   - Messages stay in shared-memory slots (assigned on the host, by levels); the schedule lies in shared memory, and the raw
+//     features of the next level or two come by cp.async.
+#include <cuda_pipeline.h>
+
+#include <algorithm>
+
+#include "kernels.cuh"
+
+namespace placeto {
+
+namespace {
+
+constexpr int kD = 32;
+constexpr int kWarps = 8;
+// With single-layer networks a level is short: a ninth warp brings the raw features, two levels ahead (279 nodes, 250 states:
+// 80 -> 68 us). With two layers, where the registers are full and the features come in time, either costs 3 %.
+template <int L> constexpr int kStages = L == 1 ? 3 : 2;            // levels of raw features on chip
+template <int L> constexpr int kThreads = (kWarps + (L == 1)) * 32;
+
+struct LevelsPlan {
+    int S;          // states per slice
+    int n_slices;
+    int x_floats;   // floats of one feature staging buffer (widest level x S x F, padded)
+    size_t smem_bytes;
+};
+
+typedef unsigned long long pair_t;   // two FP32 values in one 64-bit register pair
+
+__device__ __forceinline__ pair_t pack2(float lo, float hi) {
+    pair_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpack2(pair_t v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+// Two independent FP32 FMAs in one instruction (sm_100 packed arithmetic): half
+// the FMA issue slots, the same rounding as two fmaf.
+__device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c) {
+    pair_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// out[r] = bias + in[r] . w for R rows whose K inputs are read as broadcast
+// 128-bit loads from shared memory. The weights are kept as pairs (w[2i],
+// w[2i + 1]) so that every load feeds two packed FMAs; two pair accumulators per
+// row, i.e. four dependent chains of K / 4 FMAs.
+template <int R, int K>
+__device__ __forceinline__ void matvec(const pair_t (&w)[K / 2], float bias, const float *in,
+                                       int row_stride, float (&out)[R]) {
+    pair_t acc[R][2];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        acc[r][0] = pack2(bias, 0.f);
+        acc[r][1] = 0ull;
+    }
+#pragma unroll
+    for (int k = 0; k < K; k += 4) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(in + r * row_stride + k);
+            acc[r][0] = fma2(u.x, w[k / 2], acc[r][0]);
+            acc[r][1] = fma2(u.y, w[k / 2 + 1], acc[r][1]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float a, b, c, d;
+        unpack2(acc[r][0], a, b);
+        unpack2(acc[r][1], c, d);
+        out[r] = (a + b) + (c + d);
+    }
+}
+
+struct Weights32 {
+    pair_t g1[kD / 2], g2[kD / 2], f2[kD / 2];   // column `lane`, rows in pairs
+    float bg1, bg2, bf1, bf2;
+};
+
+// Carries R states (s0 .. s0 + R - 1 of the slice; the last may be missing and
+// then repeats s0) of the node at position `pos` through
+// gather -> g -> store h -> f -> store m. The R rows share the node, so the
+// schedule lookups are done once. A, Bf: the warp's exchange buffers, R rows of
+// KF floats each. All shared-memory offsets are 32-bit.
+template <int R, int KF, int L>   // L layers per network
+__device__ __forceinline__ void run_node(const Weights32 &w, const pair_t (&wf1)[KF / 2], int pos,
+                                         int q, int s0, bool last_live, int nb, int S, int F,
+                                         int lane, const int4 *meta, const int *nbr_slot,
+                                         float *msg, const float *xs, float *__restrict__ H,
+                                         size_t B, int b_first, float *A, float *Bf) {
+    int st[R];
+    float x[R], acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        st[r] = (r == 0 || last_live) ? s0 + r : s0;
+        x[r] = lane < F ? xs[(q * nb + st[r]) * F + lane] : 0.f;
+        acc[r] = 0.f;
+    }
+    const int4 m = meta[pos];       // {first neighbour entry, end, own | first neighbour slot, node}
+    const int e1 = m.y, v = m.w;
+    const int slot = (m.z & 0xffff) == 0xffff ? -1 : (m.z & 0xffff);
+    int e = m.x;
+    if (e1 - e == 1) {
+        // One neighbour (most nodes of chain-like graphs): its message row is the
+        // input of g as it stands, so the first layer reads the slot directly and
+        // the gather, the store and the warp barrier are skipped.
+        const float *row = msg + ((int)((unsigned)m.z >> 16) * S + st[0]) * kD;
+        matvec<R, kD>(w.g1, w.bg1, row, (R > 1 && last_live) ? kD : 0, acc);
+        __syncwarp();               // the previous node's last reads of Bf are done
+        goto after_g1;
+    }
+    for (; e + 4 <= e1; e += 4) {   // four neighbours at a time: the loads overlap
+        int base[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) base[k] = nbr_slot[e + k] * S;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            float t[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] = msg[(base[k] + st[r]) * kD + lane];
+            acc[r] += (t[0] + t[1]) + (t[2] + t[3]);
+        }
+    }
+    if (e < e1) {                   // the last one to three likewise (151 nodes with 267 edges: 0.60 -> 0.54 us a level)
+        int base[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) base[k] = nbr_slot[min(e + k, e1 - 1)] * S;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            float t[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) t[k] = msg[(base[k] + st[r]) * kD + lane];
+            acc[r] += t[0];
+            if (e + 1 < e1) acc[r] += t[1];
+            if (e + 2 < e1) acc[r] += t[2];
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) A[r * KF + lane] = acc[r];
+    __syncwarp();
+    matvec<R, kD>(w.g1, w.bg1, A, KF, acc);
+after_g1:
+    if constexpr (L == 2) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
+        __syncwarp();
+        matvec<R, kD>(w.g2, w.bg2, Bf, KF, acc);
+    }
+    float *hrow = H + ((size_t)v * B + b_first + s0) * kD + lane;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        acc[r] = fmaxf(acc[r], 0.f);
+        if (r == 0 || last_live) hrow[r * kD] = acc[r];
+    }
+    if (slot < 0) {                         // nobody consumes this node's message
+        if constexpr (L == 1) __syncwarp();     // the next node writes A, which the only product may still be reading
+        return;
+    }
+    float *in = L == 2 ? A : Bf;            // the buffer that the last product did not read
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        in[r * KF + lane] = acc[r];
+        if (lane < KF - kD) in[r * KF + kD + lane] = x[r];
+    }
+    __syncwarp();
+    matvec<R, KF>(wf1, w.bf1, in, KF, acc);
+    if constexpr (L == 2) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) Bf[r * KF + lane] = fmaxf(acc[r], 0.f);
+        __syncwarp();
+        matvec<R, kD>(w.f2, w.bf2, Bf, KF, acc);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (r == 0 || last_live) {
+            const float v_m = fmaxf(acc[r], 0.f);
+            msg[((slot * S) + st[r]) * kD + lane] = v_m;
+        }
+}
+
+// feature width padded to 4 * F4; layers
+template <int F4, int L>
+__global__ void __launch_bounds__(kThreads<L>, 1)
+embed_levels_d32_kernel(const EmbedArgs a, const LevelsPlan p) {
+    constexpr int KF = kD + 4 * F4;      // padded input width of f's first layer
+    extern __shared__ __align__(16) float smem[];
+    dependents_may_start();
+    const int dir = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const DevLevels lv = a.lv[dir];
+    const int B = a.B, F = a.F;
+    const int b_first = blockIdx.x * p.S;
+    const int nb = min(p.S, B - b_first);
+
+    // ---- shared memory: [schedule ints][message slots][feature staging x2 or x3][exchange buffers]
+    // one packed record per position: {first neighbour entry, end,
+    // own slot (low 16 bits, 0xffff = none) | slot of the first neighbour (high 16 bits), node id}
+    int4 *meta_w = reinterpret_cast<int4 *>(smem);
+    for (int i = threadIdx.x; i < a.n; i += kThreads<L>) {
+        const int e0 = lv.nbr_ptr[i], e1 = lv.nbr_ptr[i + 1];
+        const int first = e1 > e0 ? lv.nbr_slot[e0] : 0;
+        meta_w[i] = make_int4(e0, e1, (lv.own_slot[i] & 0xffff) | (first << 16), lv.order[i]);
+        PLACETO_DEBUG_CHECK(a.status, e0 >= 0 && e0 <= e1 && e1 <= lv.n_nbr && lv.own_slot[i] >= -1 &&
+                                          lv.own_slot[i] < lv.n_slots && lv.order[i] >= 0 && lv.order[i] < a.n);
+    }
+    for (int e = threadIdx.x; e < lv.n_nbr; e += kThreads<L>)
+        PLACETO_DEBUG_CHECK(a.status, lv.nbr_slot[e] >= 0 && lv.nbr_slot[e] < lv.n_slots);
+    PLACETO_DEBUG_CHECK(a.status, nb >= 1 && b_first + nb <= B);
+    const int4 *meta = meta_w;
+    int *ism = reinterpret_cast<int *>(smem) + 4 * a.n;
+    auto stage = [&](const int *src, int count) {
+        int *dst = ism;
+        for (int i = threadIdx.x; i < count; i += kThreads<L>) dst[i] = src[i];
+        ism += (count + 3) & ~3;
+        return (const int *)dst;
+    };
+    const int *level_ptr = stage(lv.level_ptr, lv.n_levels + 1);
+    const int *nbr_slot = stage(lv.nbr_slot, lv.n_nbr);
+    float *fsm = reinterpret_cast<float *>(ism);
+    float *msg = fsm;                                       // [n_slots][S][32]
+    float *xstage = msg + (size_t)lv.n_slots * p.S * kD;    // [kStages][x_floats]
+    float *xbuf = xstage + kStages<L> * (size_t)p.x_floats + (size_t)(L == 1 ? min(warp, kWarps - 1) : warp) * 4 * KF;
+    float *A = xbuf, *Bf = xbuf + 2 * KF;
+
+    // ---- this lane's weight columns
+    const DevMlp f = a.f[dir], g = a.g[dir];
+    Weights32 w;
+    pair_t wf1[KF / 2];
+#pragma unroll
+    for (int k = 0; k < kD; k += 2) {
+        w.g1[k / 2] = pack2(g.W1[k * kD + lane], g.W1[(k + 1) * kD + lane]);
+        if constexpr (L == 2) {
+            w.g2[k / 2] = pack2(g.W2[k * kD + lane], g.W2[(k + 1) * kD + lane]);
+            w.f2[k / 2] = pack2(f.W2[k * kD + lane], f.W2[(k + 1) * kD + lane]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < KF; k += 2)
+        wf1[k / 2] = pack2(k < kD + F ? f.W1[k * kD + lane] : 0.f,
+                           k + 1 < kD + F ? f.W1[(k + 1) * kD + lane] : 0.f);
+    w.bg1 = g.b1[lane]; w.bf1 = f.b1[lane];
+    if constexpr (L == 2) { w.bg2 = g.b2[lane]; w.bf2 = f.b2[lane]; }
+    const float *__restrict__ X = a.X;
+    float *__restrict__ H = a.H[dir];
+    __syncthreads();
+
+    // Asynchronous copy of one level's raw features (rows of the slice) into a
+    // staging buffer, so that the next level's x is on chip when it is needed.
+    // exact division of small non-negative numbers by a per-block constant
+    auto magic_of = [](int d) { return (unsigned)((0x100000000ull + d - 1) / d); };
+    const unsigned magic_nb = magic_of(nb), magic_ppn = magic_of((nb + 1) >> 1);
+    const int per_node = nb * F;             // floats per node, contiguous in X
+    const bool vec = (F & 3) == 0;
+    const int per = vec ? per_node >> 2 : per_node;     // copy pieces per node
+    const unsigned magic_per = magic_of(per);
+    // The last warp (the one least often needed for rows) issues all copies, so
+    // the other warps go straight to their rows.
+    auto prefetch = [&](int level) {
+        if (warp != (L == 1 ? kWarps : kWarps - 1)) return;
+        const int q0 = level_ptr[level], width = level_ptr[level + 1] - q0;
+        float *dst = xstage + (size_t)(L == 1 ? level % 3 : level & 1) * p.x_floats;
+        for (int i = lane; i < width * per; i += 32) {
+            const int q = per == 1 ? i : (int)__umulhi((unsigned)i, magic_per);
+            const int piece = i - q * per;
+            const float *src = X + ((size_t)meta[q0 + q].w * B + b_first) * F;
+            if (vec) __pipeline_memcpy_async(dst + q * per_node + 4 * piece, src + 4 * piece, 16);
+            else __pipeline_memcpy_async(dst + q * per_node + piece, src + piece, 4);
+        }
+        __pipeline_commit();
+    };
+    dependency_wait();          // the raw features may come from a kernel that is still running
+    prefetch(0);
+    if (L == 1 && lv.n_levels > 1) prefetch(1);
+    __pipeline_wait_prior(0);
+    __syncthreads();
+
+    if (L == 1 && warp == kWarps) {
+        for (int level = 0; level < lv.n_levels; ++level) {
+            if (level + 2 < lv.n_levels) {
+                prefetch(level + 2);
+                __pipeline_wait_prior(1);
+            } else {
+                __pipeline_wait_prior(0);
+            }
+            __syncthreads();
+        }
+        return;
+    }
+    int stage_now = 0;
+    for (int level = 0; level < lv.n_levels; ++level) {
+        if (L == 2 && level + 1 < lv.n_levels) prefetch(level + 1);
+        const int p0 = level_ptr[level];
+        const int rows = (level_ptr[level + 1] - p0) * nb;
+        const float *xs = xstage + (size_t)(L == 1 ? stage_now : level & 1) * p.x_floats;
+        if (L == 1) stage_now = stage_now == 2 ? 0 : stage_now + 1;
+        const int width = level_ptr[level + 1] - p0;
+        if (rows <= kWarps) {
+            // narrow level: one row per warp, shortest dependent chains
+            if (warp < rows) {
+                const int q = nb == 1 ? warp : (int)__umulhi((unsigned)warp, magic_nb);
+                const int s0 = warp - q * nb;
+                run_node<1, KF, L>(w, wf1, p0 + q, q, s0, true, nb, p.S, F, lane, meta, nbr_slot, msg,
+                                xs, H, B, b_first, A, Bf);
+            }
+        } else {
+            // two states of one node per warp pass
+            const int ppn = (nb + 1) >> 1;
+            for (int item = warp; item < width * ppn; item += kWarps) {
+                const int q = ppn == 1 ? item : (int)__umulhi((unsigned)item, magic_ppn);
+                const int s0 = (item - q * ppn) * 2;
+                run_node<2, KF, L>(w, wf1, p0 + q, q, s0, s0 + 1 < nb, nb, p.S, F, lane, meta, nbr_slot,
+                                msg, xs, H, B, b_first, A, Bf);
+            }
+        }
+        if (L == 2) __pipeline_wait_prior(0);
+        __syncthreads();
+    }
+}
+
+// slice size and shared-memory layout; false when not even one state per block fits
+bool plan_levels(const EmbedArgs &a, const DeviceInfo &di, LevelsPlan *out) {
+    LevelsPlan p;
+    const int target = std::max(1, di.sm_count / 2);            // blocks per direction
+    const int want = std::max(1, std::min(a.B, target));
+    p.S = (a.B + want - 1) / want;
+    const int F4 = (a.F + 3) / 4;
+    const int KF = kD + 4 * F4;
+    const size_t budget = (size_t)std::min(di.max_smem_optin, 227 * 1024) - 1024;
+    const int max_slots = std::max(a.lv[0].n_slots, a.lv[1].n_slots);
+    if (max_slots >= 0xffff) return false;   // slot ids are packed into 16 bits
+    size_t ints = 0;
+    for (int dir = 0; dir < 2; ++dir) {
+        const DevLevels &lv = a.lv[dir];
+        ints = std::max(ints, (size_t)4 * a.n + ((lv.n_levels + 1 + 3) & ~3) + ((lv.n_nbr + 3) & ~3));
+    }
+    const size_t xbuf = (size_t)kWarps * 4 * KF * sizeof(float);
+    auto x_floats = [&](int S) { return (a.max_level_width * S * a.F + 3) & ~3; };
+    auto need = [&](int S) {
+        return (size_t)max_slots * S * kD * sizeof(float) + (a.f[0].n_layers == 1 ? kStages<1> : kStages<2>) * (size_t)x_floats(S) * sizeof(float) +
+               xbuf + ints * sizeof(int);
+    };
+    // narrower slices when the shared memory does not fit (more blocks: they queue up)
+    while (p.S > 1 && need(p.S) > budget) --p.S;
+    if (need(p.S) > budget) return false;
+    // more slices than one wave of blocks: spread the batch evenly over the waves it takes
+    {
+        const int waves = ((a.B + p.S - 1) / p.S + want - 1) / want;
+        p.S = std::min(p.S, (a.B + want * waves - 1) / (want * waves));
+    }
+    p.n_slices = (a.B + p.S - 1) / p.S;
+    p.x_floats = x_floats(p.S);
+    p.smem_bytes = need(p.S);
+    *out = p;
+    return true;
+}
+}  // namespace
+
+// us of the sweep, queues and levels, two layers: with 9 to 11 states per block (two per warp, every state one warp) the queues leave
+// warps idle: 992 nodes of 4.0 a level, 10 states 723, 608; 120 of 4.3 105, 91; 706 of 2.2 565, 524, while 279 of 2.1 take 201, 208 and
+// full sets of 16 win everywhere (992 nodes 704, 797). Likewise past 16. Five or six states where nodes have more than three
+// neighbours: 1080 nodes 472, 443; 540 nodes 245, 228; with fewer neighbours 396, 410.
+bool embed_levels_d32_preferred(const EmbedArgs &a, const DeviceInfo &di) {
+    const int blocks = std::max(1, std::min(a.B, di.sm_count / 2)), S = (a.B + blocks - 1) / blocks;
+    if (S <= 8) return (S == 5 || S == 6) && a.lv[0].n_nbr > 3ll * a.n;
+    const bool wide = 20ll * a.n >= 43ll * a.lv[0].n_levels;
+    return wide && 10ll * S <= 7ll * 16 * ((S + 15) / 16);
+}
+
+cudaError_t launch_embed_levels_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap) {
+    LevelsPlan p;
+    if (a.walk.order != nullptr || !plan_levels(a, di, &p)) return cudaErrorNotSupported;
+    typedef void (*Kernel)(const EmbedArgs, const LevelsPlan);
+    static const Kernel kernels[2][4] = {
+        {embed_levels_d32_kernel<1, 1>, embed_levels_d32_kernel<2, 1>, embed_levels_d32_kernel<3, 1>, embed_levels_d32_kernel<4, 1>},
+        {embed_levels_d32_kernel<1, 2>, embed_levels_d32_kernel<2, 2>, embed_levels_d32_kernel<3, 2>, embed_levels_d32_kernel<4, 2>}};
+    const Kernel kern = kernels[a.f[0].n_layers - 1][(a.F + 3) / 4 - 1];
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);
+    if (err != cudaSuccess) return err;
+    err = launch_overlapped(overlap, kern, dim3(p.n_slices, 2), dim3(a.f[0].n_layers == 1 ? kThreads<1> : kThreads<2>), p.smem_bytes, stream, a, p);
+    count_launch();
+    return err;
+}
+
+}  // namespace placeto

@@ -538,17 +538,19 @@ bool embed_split_applicable(const EmbedArgs &a) {
     return true;
 }
 
-// d = 64: wherever it applies. d = 32: measured against the FMA kernel (us, two layers / one), the lines cross at 12
-// to 14 rows of a block per level: 20 rows 417 -> 308 / 295 -> 213, 12 rows 286 -> 263 / 203 -> 183, 8.5 rows
-// 96 -> 114 / 70 -> 80; with four neighbours per node (a recurrent grid with attention) the gather, which only one
-// group of warps per tile does, costs more than the products save: 26 rows 310 -> 401. The line is at three and a half (whole
-// path, 256 states: 3.0 edges per node 118 -> 100, 3.3 184 -> 151, 4.0 349 -> 445).
+// d = 64: wherever it applies. d = 32: measured against the FMA kernel (us of the sweep, FMA and this one, two layers): up to eight
+// states per block, which the FMA kernel carries in one go, the lines cross at 18 rows of a block per level (recurrent graph
+// of 4.0 nodes a level, 4 states 246, 264, 5 states 385, 307; cells of 2.3, 8 states 207, 240; 270 nodes of 6.1, 3
+// states 72, 61); beyond, it takes two states per warp and all nodes of a state in one warp, and this one wins from 12 rows or so on
+// (279 nodes of 2.1, 10 states 188, 158; 1.8 nodes a level, 10 states 233, 197). With more than three and a half
+// neighbours per node the gather, which only one group of warps per tile does, costs more than the products save (4.0 edges per
+// node, 256 states: 270, 401).
 bool embed_split_preferred(const EmbedArgs &a, const DeviceInfo &di) {
     if (!embed_split_applicable(a)) return false;
     if (a.d == 64) return true;
     const int blocks = std::max(1, std::min(a.B, di.sm_count / 2)), S = (a.B + blocks - 1) / blocks;
-    const long long rows = (long long)a.n * S;
-    return rows >= 12ll * a.lv[0].n_levels && rows >= 12ll * a.lv[1].n_levels && 2ll * a.lv[0].n_nbr <= 7ll * a.n;
+    const long long rows = 4ll * a.n * S, line = S <= 8 ? 73 : 48;         // four times the rows of a block, and per level
+    return rows >= line * a.lv[0].n_levels && rows >= line * a.lv[1].n_levels && 2ll * a.lv[0].n_nbr <= 7ll * a.n;
 }
 
 cudaError_t launch_embed_split(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap) {

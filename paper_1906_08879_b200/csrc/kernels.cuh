@@ -422,6 +422,10 @@ bool embed_d32_applicable(const EmbedArgs &a);
 cudaError_t launch_embed_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream,
                              bool overlap = false);
 
+// embed_levels_d32.cu: the same shapes and bits, level by level. cudaErrorNotSupported when its schedule does not fit.
+bool embed_levels_d32_preferred(const EmbedArgs &a, const DeviceInfo &di);     // faster than the queues (a is applicable)
+cudaError_t launch_embed_levels_d32(const EmbedArgs &a, const DeviceInfo &di, cudaStream_t stream, bool overlap = false);
+
 // embed_d64.cu: the same for d = 64 (four-warp column-split groups, both
 // directions in one block).
 bool embed_d64_applicable(const EmbedArgs &a);

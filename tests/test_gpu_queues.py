@@ -1,0 +1,100 @@
+"""The d = 32 sweep on queues of nodes: every form that its plan picks (1 to 8 warps per state, one or two states per warp, more
+states than a block holds at once, slots that leave room for a few states only), against the dimension-generic kernels."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import paper_1906_08879_b200 as placeto
+from gen import graphs, states
+from tests.helpers import rng
+
+pytestmark = pytest.mark.gpu
+
+
+def _fork_join(width, length, repeats):
+    """`repeats` times: a fork into `width` chains of `length` nodes and their join, and an edge past them."""
+    src, dst, last = [], [], 0
+    for _ in range(repeats):
+        join = last + width * length + 1
+        for c in range(width):
+            ids = [last] + list(range(last + 1 + c * length, last + 1 + (c + 1) * length)) + [join]
+            src += ids[:-1]
+            dst += ids[1:]
+        src.append(last)
+        dst.append(join)
+        last = join
+    return last + 1, np.array(src), np.array(dst)
+
+
+def _attention(steps):
+    """Two chains side by side, every node of the second reading all of the first: messages that live to the end."""
+    src = list(range(steps - 1)) + list(range(steps, 2 * steps - 1))
+    dst = [u + 1 for u in src]
+    for v in range(steps, 2 * steps):
+        src += range(steps)
+        dst += [v] * steps
+    return 2 * steps, np.array(src), np.array(dst)
+
+
+GRAPHS = {
+    "one node": (1, np.zeros(0, np.int64), np.zeros(0, np.int64)),
+    "chain": (37, np.arange(36), np.arange(1, 37)),
+    "fork and join": _fork_join(3, 4, 3),
+    "wide": graphs.layered_dag(seed=3, levels=9, width=11),
+    "attention": _attention(45),
+    "slots": _attention(220),            # more messages at once than eight states fit
+}
+
+
+def _case(name, m, layers, B, seed):
+    r = rng(seed)
+    n, src, dst = GRAPHS[name]
+    w = states.policy_weights(r, 32, m + 4, m, layers, 0, 0.1)
+    fan_in = max(1.0, len(src) / n)
+    for way in ("down", "up"):           # embeddings of order one whatever the neighbours
+        w["g_" + way]["W%d" % layers] = w["g_" + way]["W%d" % layers] / np.float32(fan_in)
+    cost, size = states.node_costs(r, n, True)
+    dev, cur, placed = states.random_states(r, n, m, B)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    return placeto.Graph(n, src, dst), placeto.Weights(w), [t(a) for a in (cost, size, dev, cur, placed)]
+
+
+@pytest.mark.parametrize("B", [1, 2, 75, 149, 223, 300, 593, 700, 1300])
+@pytest.mark.parametrize("name", sorted(GRAPHS))
+def test_every_form_of_the_sweep_against_the_generic_kernels(name, B):
+    for m, layers in ((4, 2), (1, 1), (7, 2)):
+        g, w, (cost, size, dev, cur, placed) = _case(name, m, layers, B, 17 * B + m)
+        X = placeto.placeto_build_features(g, cost, size, dev, cur, placed, m)
+        ws = placeto.workspace(g, w, B, placeto.CALL_EMBED)
+        got = placeto.placeto_embed_forward(g, w, X, ws=ws)
+        assert placeto.placeto_last_status(g, ws) == 0
+        want = placeto.placeto_embed_forward(g, w, X, flags=placeto.PLACETO_GENERIC)
+        for a, b in zip(got, want):      # 2e-5 of a row, the gate of every embedding: sums of at most 220 terms in another order
+            scale = b.abs().amax(dim=-1, keepdim=True).clamp_min(1e-30)
+            assert ((a - b).abs() / scale).max() < 2e-5, (name, B, m, layers)
+
+
+@pytest.mark.parametrize("E", [3, 60, 150, 297, 640])
+def test_steps_of_episodes_start_anywhere_in_the_queues(E):
+    """A rollout in an order that jumps through the graph (reversed, then interleaved), against the generic kernels: a choice
+    differs only where a uniform number falls within rounding of an interval's boundary, which hardly any does."""
+    n, src, dst = GRAPHS["fork and join"]
+    for m, order in ((4, np.arange(n)[::-1]), (4, np.argsort(np.arange(n) * 17 % n)), (3, np.arange(n))):
+        r = rng(E + m)
+        w = placeto.Weights(states.policy_weights(r, 32, m + 4, m, 2, 0, 0.1))
+        g = placeto.Graph(n, src, dst)
+        cost, size = states.node_costs(r, n, True)
+        t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        dev0, uni = t(r.integers(0, m, (E, n)).astype(np.uint8)), t(r.random((E, n)).astype(np.float32))
+        out = []
+        for flags in (0, placeto.PLACETO_GENERIC):
+            ws = placeto.workspace(g, w, E, placeto.CALL_EPISODE)
+            actions, logp = torch.empty((E, n), dtype=torch.uint8, device="cuda"), torch.empty((E, n), device="cuda")
+            placeto.placeto_episode_rollout(g, w, t(cost), t(size), t(order.astype(np.int32)), dev0.clone(), uni, actions, logp, ws, flags=flags)
+            assert placeto.placeto_last_status(g, ws) == 0
+            out.append((actions, logp))
+        same = (out[0][0] == out[1][0]).all(dim=1)
+        assert same.float().mean() > 0.98
+        assert (out[0][1] - out[1][1])[same].abs().max() < 2e-4
