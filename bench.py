@@ -280,7 +280,8 @@ def error_against_checker(cfg, logits, Hd, Hu, samples: int = 16):
 def sweep_of_the_step(g, cfg, flags: int):
     """(flags, arithmetic) with which placeto_embed_forward runs the sweep that the whole path takes. That call keeps
     the kernels whose bits its callers have; PLACETO_TENSOR gives it the tensor-core sweep that placeto_policy_forward picks
-    by itself at d = 64, and at d = 32 from twelve rows of a block per level on, up to three and a half neighbours per node."""
+    by itself at d = 64, and at d = 32 from eighteen rows of a block per level on (twelve past eight states of a block), up
+    to three and a half neighbours per node."""
     import paper_1906_08879_b200 as placeto
     other = (placeto.PLACETO_PER_LEVEL | placeto.PLACETO_COOPERATIVE | placeto.PLACETO_GENERIC | placeto.PLACETO_FMA_ONLY)
     d, n, info = cfg["d"], cfg["n"], g.info()
@@ -290,7 +291,7 @@ def sweep_of_the_step(g, cfg, flags: int):
         return flags, "fp32 accumulate on mma.sync, TF32 head+tail operands (3 products)"
     states = -(-cfg["B"] // max(1, min(cfg["B"], SMS // 2)))
     levels = max(info["n_levels_down"], info["n_levels_up"])
-    split = flags & placeto.PLACETO_TENSOR or (d == 64 or n * states >= 12 * levels and 2 * info["n_edges"] <= 7 * n)
+    split = flags & placeto.PLACETO_TENSOR or (d == 64 or 4 * n * states >= (73 if states <= 8 else 48) * levels and 2 * info["n_edges"] <= 7 * n)
     if d in (32, 64) and not flags & other and split:
         return flags | placeto.PLACETO_TENSOR, ("fp32 accumulate on mma.sync, operands as two scaled fp16 pieces (3 products)" if d == 64 else
                                                 "fp32 accumulate on mma.sync, operands as three bf16 pieces (6 products)")
