@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(256)
 features_kernel(int n, int B, int m, const float *__restrict__ cost,
                 const float *__restrict__ bytes, const uint8_t *__restrict__ dev,
                 const int *__restrict__ cur, const uint8_t *__restrict__ placed,
-                float *__restrict__ X) {
+                float *__restrict__ X, int *__restrict__ cur_copy) {        // cur_copy: null, or where cur goes as well
     dependents_may_start();
     __shared__ uint8_t s_dev[kTile][kTile + 4];
     __shared__ uint8_t s_placed[kTile][kTile + 4];
@@ -27,17 +27,35 @@ features_kernel(int n, int B, int m, const float *__restrict__ cost,
     const int v0 = blockIdx.x * kTile, b0 = blockIdx.y * kTile;
     const int F = m + 4;
     dependency_wait();          // the inputs may come from the gather kernel of the same call
-    for (int i = threadIdx.x; i < kTile * kTile; i += blockDim.x) {
-        const int bl = i / kTile, vl = i % kTile;
-        const int b = b0 + bl, v = v0 + vl;
-        const bool ok = b < B && v < n;
-        s_dev[bl][vl] = ok ? dev[(size_t)b * n + v] : 0;
-        s_placed[bl][vl] = ok ? placed[(size_t)b * n + v] : 0;
-    }
-    if (threadIdx.x < kTile) s_cur[threadIdx.x] = (b0 + threadIdx.x < B) ? cur[b0 + threadIdx.x] : -1;
-    if (threadIdx.x >= 32 && threadIdx.x < 32 + kTile && v0 + threadIdx.x - 32 < n) {
-        s_cost[threadIdx.x - 32] = cost[v0 + threadIdx.x - 32];
-        s_bytes[threadIdx.x - 32] = bytes[v0 + threadIdx.x - 32];
+    // every load before the first store: one round trip to memory (or across the host link), not one per pass
+    {
+        constexpr int kPasses = kTile * kTile / 256;
+        uint8_t t_dev[kPasses], t_placed[kPasses];
+        const int vl = threadIdx.x % kTile, bl = threadIdx.x / kTile, v = v0 + vl;
+#pragma unroll
+        for (int j = 0; j < kPasses; ++j) {
+            const int b = b0 + bl + j * (256 / kTile);
+            const bool ok = b < B && v < n;
+            t_dev[j] = ok ? dev[(size_t)b * n + v] : 0;
+            t_placed[j] = ok ? placed[(size_t)b * n + v] : 0;
+        }
+        int t_cur = -1;
+        float t_node = 0.f;
+        if (bl == 0 && b0 + vl < B) t_cur = cur[b0 + vl];
+        if ((bl == 1 || bl == 2) && v < n) t_node = (bl == 1 ? cost : bytes)[v];
+#pragma unroll
+        for (int j = 0; j < kPasses; ++j) {
+            s_dev[bl + j * (256 / kTile)][vl] = t_dev[j];
+            s_placed[bl + j * (256 / kTile)][vl] = t_placed[j];
+        }
+        if (bl == 0) {
+            s_cur[vl] = t_cur;
+            if (cur_copy != nullptr && blockIdx.x == 0 && b0 + vl < B) cur_copy[b0 + vl] = t_cur;
+        } else if (bl == 1) {
+            s_cost[vl] = t_node;
+        } else if (bl == 2) {
+            s_bytes[vl] = t_node;
+        }
     }
     __syncthreads();
     const int nb = min(kTile, B - b0);
@@ -126,10 +144,10 @@ cudaError_t launch_stage_inputs(const void *const (&src)[5], void *const (&dst)[
 
 cudaError_t launch_features(int n, int B, int m, const float *cost, const float *bytes,
                             const uint8_t *dev, const int *cur, const uint8_t *placed, float *X,
-                            cudaStream_t stream, bool overlap) {
+                            cudaStream_t stream, bool overlap, int *cur_copy) {
     dim3 grid((n + kTile - 1) / kTile, (B + kTile - 1) / kTile);
     cudaError_t err = launch_overlapped(overlap, features_kernel, grid, dim3(256), 0, stream, n, B, m, cost,
-                                        bytes, dev, cur, placed, X);
+                                        bytes, dev, cur, placed, X, cur_copy);
     count_launch();
     return err;
 }

@@ -1,0 +1,36 @@
+"""Small calls from page-locked host buffers, whose features are made from the buffers themselves, against the same call on device
+tensors: on both sides of the limit of 4096 (node, state) rows, with partial tiles, at odd addresses."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import paper_1906_08879_b200 as placeto
+from gen import graphs, states
+from tests.helpers import rng
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B", [1, 3, 31, 33, 102, 103])          # 40 nodes: 4080 and 4120 rows
+@pytest.mark.parametrize("d,m", [(32, 4), (64, 3), (8, 2)])
+def test_host_call_equals_the_device_call(d, m, B):
+    r = rng(10 * B + d)
+    n, src, dst = graphs.layered_dag(seed=2, levels=10, width=4)
+    g, w = placeto.Graph(n, src, dst), placeto.Weights(states.policy_weights(r, d, m + 4, m, 2, 0, 0.1))
+    cost, size = states.node_costs(r, n, True)
+    dev, cur, placed = states.random_states(r, n, m, B)
+    arrays = [np.ascontiguousarray(a) for a in (cost, size, dev, cur, placed)]
+    want = placeto.placeto_policy_forward(g, w, *[torch.from_numpy(a).cuda() for a in arrays])
+    for offset in (0, 1, 16):            # elements that the buffers start into their page-locked memory
+        pinned = []
+        for a in arrays:
+            whole = torch.empty(a.size + offset, dtype=torch.from_numpy(a).dtype, pin_memory=True)
+            part = whole[offset:].view(a.shape)
+            part.copy_(torch.from_numpy(a))
+            pinned.append(part)
+        logits, probs = torch.empty((B, m), pin_memory=True), torch.empty((B, m), pin_memory=True)
+        ws = placeto.workspace(g, w, B, placeto.CALL_FORWARD_HOST)
+        placeto.placeto_policy_forward_host(g, w, *pinned, logits, probs, ws)
+        assert torch.equal(logits, want[0].cpu()) and torch.equal(probs, want[1].cpu()), offset
